@@ -264,9 +264,10 @@ SweepArgs<T> sweep_args(dd4dv_ctx* ctx) {
   for (int v = 0; v < 3; ++v) a.isb2[v] = 1.0 / (ctx->sigma_b[v] * ctx->sigma_b[v]);
   a.lam = ctx->dec.lambda;
   a.mu = ctx->dec.mu;
+  const double scale = sizeof(T) == 8 ? a.dt : 1.0;   // the FP64 point functions take dt Bth and dt g Bth
   a.dt_s = (T)a.dt;
-  a.Bth_s = (T)a.Bth;
-  a.gBth_s = (T)a.gBth;
+  a.Bth_s = (T)(scale * a.Bth);
+  a.gBth_s = (T)(scale * a.gBth);
   a.href_s = (T)a.h_ref;
   for (int v = 0; v < 3; ++v) {
     a.isb2_s[v] = (T)a.isb2[v];

@@ -24,7 +24,7 @@
 //   adjoint    Alg. 6 (ADJ), the reversed product of step adjoints Eq. adjProd,
 //              derived by hand from the discrete forward step
 //   TLM        Alg. 6 (TLM), the linearised forward step.
-#include "common.cuh"
+#include "point.cuh"
 
 #include <cooperative_groups.h>
 
@@ -67,31 +67,6 @@ struct Geo {
   // (mdiv below) in the per-point index mappings
   unsigned mnx, mRn, mny, mnr;
 };
-
-// Division by a per-CTA constant d >= 1 through a precomputed multiplier
-// m = ceil(2^32 / d) (m = 0 encodes d = 1): floor(a / d) = floor(a m / 2^32)
-// exactly whenever a * d < 2^32.  (With m = (2^32 + e) / d, 0 <= e < d, the
-// product is a / d + a e / (d 2^32); the extra term is below 1 / d, the gap
-// from a / d up to the next integer, when a e < 2^32.)  Every dividend here is
-// an index into a CTA's shared-memory stripe, below 2^20, and every divisor
-// is a row length or a row count: a * d stays below 2^31.
-__host__ __device__ __forceinline__ unsigned magic_of(int d) {
-  return d <= 1 ? 0u : (unsigned)(0xFFFFFFFFu / (unsigned)d + 1u);
-}
-__device__ __forceinline__ int mdiv(int a, unsigned m) {
-  return m ? (int)__umulhi((unsigned)a, m) : a;
-}
-
-// Arithmetic with explicit rounding: the compiler neither contracts nor
-// reorders these, so every inlined copy of the forward step (forward sweep,
-// stage recomputation in the adjoint, checkpoint-segment recomputation,
-// tangent-linear sweep) rounds identically and the copies agree bit for bit.
-__device__ __forceinline__ double xmul(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ float xmul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double xsub(double a, double b) { return __dsub_rn(a, b); }
-__device__ __forceinline__ float xsub(float a, float b) { return __fsub_rn(a, b); }
-__device__ __forceinline__ double xfma(double a, double b, double c) { return __fma_rn(a, b, c); }
-__device__ __forceinline__ float xfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 
 __device__ __forceinline__ void split_rows(int ny, int CL, int rank, int& R0, int& Rn) {
   const int base = ny / CL, rem = ny % CL;
@@ -139,31 +114,13 @@ __device__ __forceinline__ void st3(T* Z, int o, int P, T h, T u, T v) {
 // Per-row constants staged in shared memory for rows rr = -1 .. Rn (index
 // i = rr + 1), as two 8-value records per row so that a point reads its row's
 // constants with two (FP32) or four (FP64) 16-byte loads:
-//   fw[8 i ..]: A, f, tau, B/c, g A, c of row i+1, c of row i-1, 0
-//               (tendencies and tangent-linear tendencies)
-//   bw[8 i ..]: A, f, tau, g A, B c, 1/c of row i+1, 1/c of row i-1, 2 tau
-//               (adjoint tendencies)
+//   fw[8 i ..] for the tendencies and tangent-linear tendencies, bw[8 i ..]
+//   for the adjoint tendencies (fill_records of point.cuh).
 // Wall ghost rows take the edge row's cos (mirror).
 template <typename T>
 struct RowSmem {
   T *fw, *bw;
 };
-
-template <typename T>
-__device__ __forceinline__ void load_rec8(const T* p, T (&r)[8]) {
-  if constexpr (sizeof(T) == 4) {
-    const float4 x = *reinterpret_cast<const float4*>(p);
-    const float4 y = *reinterpret_cast<const float4*>(p + 4);
-    r[0] = x.x; r[1] = x.y; r[2] = x.z; r[3] = x.w;
-    r[4] = y.x; r[5] = y.y; r[6] = y.z; r[7] = y.w;
-  } else {
-    for (int q = 0; q < 4; ++q) {
-      const double2 x = *reinterpret_cast<const double2*>(p + 2 * q);
-      r[2 * q] = x.x;
-      r[2 * q + 1] = x.y;
-    }
-  }
-}
 
 template <typename T>
 __device__ void load_rows(const SweepArgs<T>& a, const Geo<T>& g, RowSmem<T>& rs) {
@@ -174,24 +131,7 @@ __device__ void load_rows(const SweepArgs<T>& a, const Geo<T>& g, RowSmem<T>& rs
     const int js = min(max(j - 1, 0), a.nlat - 1);
     const RowConst rc = a.rows[jc];
     const double cn = a.rows[jn].c, cs = a.rows[js].c;
-    T* f = rs.fw + 8 * i;
-    f[0] = (T)rc.A;
-    f[1] = (T)rc.f;
-    f[2] = (T)rc.tau;
-    f[3] = (T)rc.BinvC;
-    f[4] = (T)rc.gA;
-    f[5] = (T)cn;
-    f[6] = (T)cs;
-    f[7] = (T)0;
-    T* b = rs.bw + 8 * i;
-    b[0] = (T)rc.A;
-    b[1] = (T)rc.f;
-    b[2] = (T)rc.tau;
-    b[3] = (T)rc.gA;
-    b[4] = (T)(a.Bth * rc.c);
-    b[5] = (T)(1.0 / cn);
-    b[6] = (T)(1.0 / cs);
-    b[7] = (T)(2.0 * rc.tau);
+    fill_records(rc, cn, cs, a.dt, a.Bth, rs.fw + 8 * i, rs.bw + 8 * i);
   }
 }
 
@@ -499,137 +439,12 @@ __device__ __forceinline__ T* stage_ptr(const SweepArgs<T>& a, const Geo<T>& g, 
 // The five stencil points of element index o in a buffer with plane stride
 // P, column stride CS and row stride RS: centre, east, west, north, south.
 template <typename T>
-struct Pt5 {
-  T h, u, v, hE, uE, vE, hW, uW, vW, hN, uN, vN, hS, uS, vS;
-};
-template <typename T>
 __device__ __forceinline__ void load5(const T* Z, int o, int P, int CS, int RS, Pt5<T>& p) {
   ld3(Z, o, P, p.h, p.u, p.v);
   ld3(Z, o + CS, P, p.hE, p.uE, p.vE);
   ld3(Z, o - CS, P, p.hW, p.uW, p.vW);
   ld3(Z, o + RS, P, p.hN, p.uN, p.vN);
   ld3(Z, o - RS, P, p.hS, p.uS, p.vS);
-}
-
-// Tendencies F(Z) at one point (Sec. 7, centred differences):
-//   F_u = -A u (uE-uW) - Bth v (uN-uS) + (f + tau u) v - gA (hE-hW)
-//   F_v = -A u (vE-vW) - Bth v (vN-vS) - (f + tau u) u - gBth (hN-hS)
-//   F_h = -A ((hu)_E - (hu)_W) - (Bth/c) ((h v c)_N - (h v c)_S)
-// On the FP32 path h = h_ref + h' and the h_ref parts of the fluxes are
-// formed from velocity differences.
-template <typename T, bool DEV>
-__device__ __forceinline__ void rhs_pt(const Pt5<T>& z, T A, T f, T tau, T BinvC, T gA, T cN, T cS, T Bth,
-                                       T gBth, T href, T& Fh, T& Fu, T& Fv) {
-  const T u = z.u, v = z.v;
-  const T dUx = xsub(z.uE, z.uW), dUy = xsub(z.uN, z.uS);
-  const T dVx = xsub(z.vE, z.vW), dVy = xsub(z.vN, z.vS);
-  const T dHx = xsub(z.hE, z.hW), dHy = xsub(z.hN, z.hS);
-  const T fu = xfma(tau, u, f);
-  const T Au = xmul(A, u), Bv = xmul(Bth, v);
-  Fu = xfma(fu, v, -xfma(Au, dUx, xfma(Bv, dUy, xmul(gA, dHx))));
-  Fv = -xfma(Au, dVx, xfma(Bv, dVy, xfma(fu, u, xmul(gBth, dHy))));
-  T flx = xfma(z.hE, z.uE, -xmul(z.hW, z.uW));
-  T fly = xfma(xmul(z.hN, z.vN), cN, -xmul(xmul(z.hS, z.vS), cS));
-  if (DEV) {
-    flx = xfma(href, dUx, flx);
-    fly = xfma(href, xfma(z.vN, cN, -xmul(z.vS, cS)), fly);
-  }
-  Fh = -xfma(A, flx, xmul(BinvC, fly));
-}
-
-// Adjoint of the tendencies: G = F'(Z)^T M at one point (derived by hand from
-// rhs_pt; M holds zero at ghost points that carry no tendency).  Wall rows add
-// the transposed ghost mirror (h, u, -v) of the edge row.
-//   G_u = mu (tau v - A dU_x) - mv (A dV_x + f + 2 tau u) + A (muE uE - muW uW)
-//         + A h (mhE - mhW) + Bth (muN vN - muS vS)
-//   G_v = mu (f + tau u - Bth dU_y) - mv Bth dV_y + A (mvE uE - mvW uW)
-//         + Bth (mvN vN - mvS vS) + (B c) h (mhN / cN - mhS / cS)
-//   G_h = gA (muE - muW) + gBth (mvN - mvS) + A u (mhE - mhW)
-//         + (B c) v (mhN / cN - mhS / cS)
-// evaluated as 42 explicitly rounded operations, 21 of them fused
-// multiply-adds.
-template <typename T, bool DEV>
-__device__ __forceinline__ void rhs_adj_pt(const Pt5<T>& z, const Pt5<T>& m, T A, T f, T tau, T gA, T BcC,
-                                           T icN, T icS, T tau2, T Bth, T gBth, T href, int wall, T& Gh,
-                                           T& Gu, T& Gv) {
-  T h = z.h;
-  if (DEV) h += href;
-  const T u = z.u, v = z.v;
-  const T mu = m.u, mv = m.v, mh = m.h;
-  const T dUx = xsub(z.uE, z.uW), dVx = xsub(z.vE, z.vW);
-  const T dUy = xsub(z.uN, z.uS), dVy = xsub(z.vN, z.vS);
-  const T dmhEW = xsub(m.hE, m.hW);
-  const T dmhNS = xfma(m.hN, icN, -xmul(m.hS, icS));
-  Gh = xfma(xmul(BcC, v), dmhNS,
-            xfma(xmul(A, u), dmhEW, xfma(gBth, xsub(m.vN, m.vS), xmul(gA, xsub(m.uE, m.uW)))));
-  const T a1 = xfma(-A, dUx, xmul(tau, v));
-  const T a2 = xfma(A, dVx, xfma(tau2, u, f));
-  const T p1 = xfma(m.uE, z.uE, -xmul(m.uW, z.uW));
-  const T p2 = xfma(m.uN, z.vN, -xmul(m.uS, z.vS));
-  Gu = xfma(Bth, p2, xfma(xmul(A, h), dmhEW, xfma(A, p1, xfma(-mv, a2, xmul(mu, a1)))));
-  const T b1 = xfma(-Bth, dUy, xfma(tau, u, f));
-  const T q1 = xfma(m.vE, z.uE, -xmul(m.vW, z.uW));
-  const T q2 = xfma(m.vN, z.vN, -xmul(m.vS, z.vS));
-  Gv = xfma(xmul(BcC, h), dmhNS, xfma(Bth, q2, xfma(A, q1, xfma(-mv, xmul(Bth, dVy), xmul(mu, b1)))));
-  if (wall == 1) {         // south wall: ghost row = (h, u, -v) of this row
-    Gu = xfma(xmul(Bth, mu), v, Gu);
-    Gv = xfma(-Bth, xfma(mv, v, xmul(h, mh)), Gv);
-    Gh = xfma(gBth, mv, xfma(-Bth, xmul(v, mh), Gh));
-  } else if (wall == 2) {  // north wall
-    Gu = xfma(-xmul(Bth, mu), v, Gu);
-    Gv = xfma(Bth, xfma(mv, v, xmul(h, mh)), Gv);
-    Gh = xfma(Bth, xmul(v, mh), xfma(-gBth, mv, Gh));
-  }
-}
-
-// Tangent-linear tendencies dF = F'(Z) dZ at one point.
-template <typename T, bool DEV>
-__device__ __forceinline__ void rhs_tl_pt(const Pt5<T>& z, const Pt5<T>& d, T A, T f, T tau, T BinvC, T gA,
-                                          T cN, T cS, T Bth, T gBth, T href, T& dFh, T& dFu, T& dFv) {
-  const T u = z.u, v = z.v;
-  const T du = d.u, dv = d.v;
-  const T uE = z.uE, uW = z.uW, uN = z.uN, uS = z.uS;
-  const T vE = z.vE, vW = z.vW, vN = z.vN, vS = z.vS;
-  T hE = z.hE, hW = z.hW, hN = z.hN, hS = z.hS;
-  if (DEV) {
-    hE += href; hW += href; hN += href; hS += href;
-  }
-  const T duE = d.uE, duW = d.uW, duN = d.uN, duS = d.uS;
-  const T dvE = d.vE, dvW = d.vW, dvN = d.vN, dvS = d.vS;
-  const T dhE = d.hE, dhW = d.hW, dhN = d.hN, dhS = d.hS;
-  dFu = -A * (du * (uE - uW) + u * (duE - duW)) - Bth * (dv * (uN - uS) + v * (duN - duS)) +
-        (f + tau * u) * dv + tau * du * v - gA * (dhE - dhW);
-  dFv = -A * (du * (vE - vW) + u * (dvE - dvW)) - Bth * (dv * (vN - vS) + v * (dvN - dvS)) -
-        (f + tau * u) * du - tau * du * u - gBth * (dhN - dhS);
-  dFh = -A * ((dhE * uE + hE * duE) - (dhW * uW + hW * duW)) -
-        BinvC * ((dhN * vN + hN * dvN) * cN - (dhS * vS + hS * dvS) * cS);
-}
-
-// The arithmetic of the transposed RK3 step at one point, shared by every
-// adjoint sweep so that all of them round alike.  A stage adjoint
-// mu_out = m + dt F'(z)^T m ...
-template <typename T, bool DEV>
-__device__ __forceinline__ void adj_stage_math(const Pt5<T>& z, const Pt5<T>& m, const T (&rc)[8], T dt, T Bth,
-                                               T gBth, T href, int wall, T& v0, T& v1, T& v2) {
-  T Gh, Gu, Gv;
-  rhs_adj_pt<T, DEV>(z, m, rc[0], rc[1], rc[2], rc[3], rc[4], rc[5], rc[6], rc[7], Bth, gBth, href, wall, Gh, Gu, Gv);
-  v0 = xfma(dt, Gh, m.h);
-  v1 = xfma(dt, Gu, m.u);
-  v2 = xfma(dt, Gv, m.v);
-}
-// ... and lambda(n) = lambda'/3 + mu2/2 + (mu1 + dt F'(x)^T mu1)/6 from the
-// stencil m of mu1, z of x, and lambda' = (ph, pu, pv), mu2 = (qh, qu, qv) at
-// the point.
-template <typename T, bool DEV>
-__device__ __forceinline__ void adj_lambda_math(const Pt5<T>& z, const Pt5<T>& m, const T (&rc)[8], T dt, T Bth,
-                                                T gBth, T href, int wall, T ph, T pu, T pv, T qh, T qu, T qv,
-                                                T& v0, T& v1, T& v2) {
-  const T c13 = (T)(1.0 / 3.0), c16 = (T)(1.0 / 6.0);
-  T Gh, Gu, Gv;
-  rhs_adj_pt<T, DEV>(z, m, rc[0], rc[1], rc[2], rc[3], rc[4], rc[5], rc[6], rc[7], Bth, gBth, href, wall, Gh, Gu, Gv);
-  v0 = xfma(c16, xfma(dt, Gh, m.h), xfma((T)0.5, qh, xmul(c13, ph)));
-  v1 = xfma(c16, xfma(dt, Gu, m.u), xfma((T)0.5, qu, xmul(c13, pu)));
-  v2 = xfma(c16, xfma(dt, Gv, m.v), xfma((T)0.5, qv, xmul(c13, pv)));
 }
 
 template <typename T>
@@ -668,37 +483,6 @@ __device__ __forceinline__ int overlap_count(const Geo<T>& g, int l, int r, int 
 
 // Observation misfit of the observations of level l whose lower corner row
 // is one of this CTA's rows: J_o += 1/2 w d^2, obs_force = lambda w d.
-// Observation term of one record with explicit rounding, so that every
-// sweep kernel that evaluates it rounds alike: the bilinear value of the
-// corner values x00, x01 (i + 1), x10 (j + 1), x11 (only the corners with
-// non-zero weight are used), d = H x - y, J_o += 1/2 w d^2; returns the
-// forcing lambda w d.
-__device__ __forceinline__ double obs_term(const ObsRec& ob, double x00, double x01, double x10, double x11,
-                                           double lam, double& Jo) {
-  const double wj0 = __dsub_rn(1.0, ob.dj), wi0 = __dsub_rn(1.0, ob.di);
-  double acc = __dmul_rn(__dmul_rn(wj0, wi0), x00);
-  if (ob.di != 0.0) acc = __fma_rn(__dmul_rn(wj0, ob.di), x01, acc);
-  if (ob.dj != 0.0) {
-    acc = __fma_rn(__dmul_rn(ob.dj, wi0), x10, acc);
-    if (ob.di != 0.0) acc = __fma_rn(__dmul_rn(ob.dj, ob.di), x11, acc);
-  }
-  const double d = __dsub_rn(acc, ob.y);
-  Jo = __fma_rn(__dmul_rn(__dmul_rn(0.5, ob.w), d), d, Jo);
-  return __dmul_rn(__dmul_rn(lam, ob.w), d);
-}
-
-// Overlap misfit of one point with overlap count c, explicitly rounded:
-// part + c ((x0 - t0)^2 i0 + (x1 - t1)^2 i1 + (x2 - t2)^2 i2).
-template <typename T>
-__device__ __forceinline__ T overlap_term(T part, int c, T x0, T x1, T x2, T t0, T t1, T t2, T i0, T i1,
-                                          T i2) {
-  const T e0 = xsub(x0, t0), e1 = xsub(x1, t1), e2 = xsub(x2, t2);
-  T sq = xmul(xmul(e0, e0), i0);
-  sq = xfma(xmul(e1, e1), i1, sq);
-  sq = xfma(xmul(e2, e2), i2, sq);
-  return xfma((T)c, sq, part);
-}
-
 template <typename T>
 __device__ void obs_level(const SweepArgs<T>& a, const Geo<T>& g, const T* X, int l, double& Jo) {
   const int o0 = a.lvl_obs[g.d.obs_lvl + l], o1 = a.lvl_obs[g.d.obs_lvl + l + 1];
@@ -880,31 +664,6 @@ __device__ __forceinline__ bool setup_geo(const SweepArgs<T>& a, cg::cluster_gro
   g.mny = magic_of(g.ny);
   g.mnr = magic_of(g.Rn + (g.rank > 0) + (g.rank < g.CL - 1));
   return true;
-}
-
-// The arithmetic of one RK3 stage at one point, out = cx X + cy (Y + dt F(Y)),
-// from the point's stencil y of Y, its row constants rc and its X values (read
-// only when cx != 0).  Every sweep (forward, stage recomputation, checkpoint
-// segments, tangent-linear, the deep-halo FP32 sweeps) calls this one
-// function, so all of them round every stage identically.
-template <typename T, bool DEV>
-__device__ __forceinline__ void stage_math(const Pt5<T>& y, const T (&rc)[8], T dt, T Bth, T gBth, T href, T cx,
-                                           T cy, T xh, T xu, T xv, T& o0, T& o1, T& o2) {
-  T Fh, Fu, Fv;
-  rhs_pt<T, DEV>(y, rc[0], rc[1], rc[2], rc[3], rc[4], rc[5], rc[6], Bth, gBth, href, Fh, Fu, Fv);
-  o0 = xfma(dt, Fh, y.h);
-  o1 = xfma(dt, Fu, y.u);
-  o2 = xfma(dt, Fv, y.v);
-  if (cy != (T)1) {
-    o0 = xmul(cy, o0);
-    o1 = xmul(cy, o1);
-    o2 = xmul(cy, o2);
-  }
-  if (cx != (T)0) {
-    o0 = xfma(cx, xh, o0);
-    o1 = xfma(cx, xu, o1);
-    o2 = xfma(cx, xv, o2);
-  }
 }
 
 // One RK3 stage at own point (rr, k): out = cx X + cy (Y + dt F(Y)); the
@@ -1636,15 +1395,21 @@ __device__ void stage_tl(const SweepArgs<T>& a, const Geo<T>& g, const RowSmem<T
   for (int idx = threadIdx.x; idx < g.Rn * g.nx; idx += blockDim.x) {
     const int rr = mdiv(idx, g.mnx), k = idx - rr * g.nx;
     const int o = pidx(g, rr, k), ri = rr + 1;
-    T Fh, Fu, Fv;
     T rc[8];
     load_rec8(rs.fw + 8 * ri, rc);
     Pt5<T> z, d;
     load5(Y, o, g.P, Lay<T>::CS, g.RS, z);
     load5(DY, o, g.P, Lay<T>::CS, g.RS, d);
-    rhs_tl_pt<T, DEV>(z, d, rc[0], rc[1], rc[2], rc[3], rc[4], rc[5], rc[6], Bth, gBth, href, Fh, Fu, Fv);
     T xh, xu, xv;
     ld3(DX, o, g.P, xh, xu, xv);
+    if constexpr (!DEV) {
+      T dh, du, dv;
+      tangent_pt64(z, d, rc, Bth, gBth, dh, du, dv);
+      st3(dout, o, g.P, cx * xh + cy * dh, cx * xu + cy * du, cx * xv + cy * dv);
+      continue;
+    }
+    T Fh, Fu, Fv;
+    rhs_tl_pt<T, DEV>(z, d, rc[0], rc[1], rc[2], rc[3], rc[4], rc[5], rc[6], Bth, gBth, href, Fh, Fu, Fv);
     st3(dout, o, g.P, cx * xh + cy * (d.h + dt * Fh), cx * xu + cy * (d.u + dt * Fu),
         cx * xv + cy * (d.v + dt * Fv));
   }
@@ -1832,24 +1597,7 @@ __device__ void load_rows2(const SweepArgs<float>& a, const G2& g, float* fw, fl
     const int js = min(max(j - 1, 0), a.nlat - 1);
     const RowConst rc = a.rows[jc];
     const double cn = a.rows[jn].c, cs = a.rows[js].c;
-    float* f = fw + 8 * i;
-    f[0] = (float)rc.A;
-    f[1] = (float)rc.f;
-    f[2] = (float)rc.tau;
-    f[3] = (float)rc.BinvC;
-    f[4] = (float)rc.gA;
-    f[5] = (float)cn;
-    f[6] = (float)cs;
-    f[7] = 0.0f;
-    float* b = bw + 8 * i;
-    b[0] = (float)rc.A;
-    b[1] = (float)rc.f;
-    b[2] = (float)rc.tau;
-    b[3] = (float)rc.gA;
-    b[4] = (float)(a.Bth * rc.c);
-    b[5] = (float)(1.0 / cn);
-    b[6] = (float)(1.0 / cs);
-    b[7] = (float)(2.0 * rc.tau);
+    fill_records(rc, cn, cs, a.dt, a.Bth, fw + 8 * i, bw + 8 * i);
   }
 }
 
