@@ -93,9 +93,11 @@ typedef struct {
  * 1/(number of subdomains containing it), the restriction weights of
  * Definition "Restriction of a function"; 0 gives weight 1.
  * cluster: CTAs per subdomain in the sweep kernels (thread-block cluster
- * size, 1..16); 0 = chosen from a model of the launch; -1 = autotune: the
- * forward and adjoint sweeps are timed at every feasible (cluster size, threads
- * per CTA) shape, with stored and with recomputed stage states when
+ * size, 1..16); 0 = chosen from a model of the launch, or no clusters at all
+ * where the boxes together have enough points (the level sweeps, see
+ * dd4dv_set_sweep_variant); -1 = autotune: the forward and adjoint sweeps are
+ * timed as level sweeps where those apply and at every feasible (cluster size,
+ * threads per CTA) shape, with stored and with recomputed stage states when
  * ckpt_k = 0, and the fastest shape of each and the faster mode are kept (see
  * dd4dv_sweep_config); if recomputation wins, the stage buffer is freed.
  * ckpt_k: trajectory storage for the adjoint.  0 = the forward sweep stores
@@ -112,7 +114,9 @@ typedef struct {
  * k > 0 = checkpointing:
  * evaluations store only the levels 0, k, 2k, ... and the adjoint
  * recomputes each k-step segment from its checkpoint before running back
- * through it (the exchange and dd4dv_trajectories still store every level);
+ * through it (the exchange and dd4dv_trajectories still store every level;
+ * the level sweeps store every level, whose buffer exists for the exchange, and
+ * recompute the stage states alone, with the same results);
  * -2 = choose by timing: after the launch shapes are set (or autotuned), one
  * evaluation is timed with stored stage states (when their buffer fits),
  * with recomputed stages and with checkpoints every 8, 16 and 32 levels, the
@@ -395,8 +399,9 @@ dd4dv_status dd4dv_profile_sweeps(dd4dv_ctx* ctx, const double* w_all, int reps,
 
 /* Launch shapes of the sweeps, shape[5] = {forward cluster size, forward
  * threads per CTA, adjoint cluster size, adjoint threads per CTA, stored stage
- * states (1) or recomputed (0)}; eval_ms (after autotuning, else 0) = the
- * measured forward + adjoint time of those shapes.  Either pointer may be NULL. */
+ * states (1) or recomputed (0)} (the cluster shapes also while level sweeps
+ * run); eval_ms (after autotuning, else 0) = the measured forward + adjoint
+ * time of what runs.  Either pointer may be NULL. */
 dd4dv_status dd4dv_sweep_config(const dd4dv_ctx* ctx, int* shape, double* eval_ms);
 
 /* Force launch shapes (e.g. ones an earlier autotuning run reported), same
@@ -439,8 +444,17 @@ dd4dv_status dd4dv_stage1_stored(const dd4dv_ctx* ctx, int* n_subs, double* pt_s
  * and the last stage reads x(n) from the trajectory level stored the step
  * before (every level stored: ckpt_k 0, -1 or -3), so two CTAs per SM fit where
  * three buffers fit one; same values bit for bit.
- * forward: 0 = deep-halo sweep wherever it applies (default), 1 = stripe
- * sweep only, 2 = the two-buffer stripe forward where it applies (else as
+ * The level sweeps advance all subdomains together, one launch per RK3 stage,
+ * with the states in HBM and L2 instead of a cluster's shared memory: the faster
+ * form where the boxes together have many points per level.  They are chosen
+ * with the decomposition (cluster 0, or -1 where they measure faster), give the
+ * same trajectories and gradients bit for bit and J up to the order of its
+ * partial sums, and give way to the cluster sweeps when a variant other than 0
+ * or a launch shape (dd4dv_set_sweep_config) is set.  The environment variable
+ * DD4DV_LEVEL_MIN_POINTS, read by dd4dv_set_decomposition, replaces the number
+ * of points from which they are chosen.
+ * forward: 0 = level sweep where chosen, else deep-halo sweep wherever it
+ * applies (default), 1 = stripe sweep only, 2 = the two-buffer stripe forward where it applies (else as
  * 1).  adjoint: 0 and 1 as for the forward (the stripe adjoint takes its
  * four-buffer form where five buffers do not fit), 2 = the four-buffer
  * stripe adjoint.  EINVAL for other values.  The autotuner (cluster = -1 in
@@ -450,7 +464,7 @@ dd4dv_status dd4dv_set_sweep_variant(dd4dv_ctx* ctx, int forward, int adjoint);
 
 /* Which kernels the current launch shapes run: kinds[0] forward, kinds[1]
  * adjoint; 1 = stripe sweep, 2 = deep-halo sweep, 3 = four-buffer stripe
- * adjoint, 4 = two-buffer stripe forward. */
+ * adjoint, 4 = two-buffer stripe forward, 5 = level sweep. */
 dd4dv_status dd4dv_sweep_kernels(const dd4dv_ctx* ctx, int* kinds);
 
 /* The cluster size (CTAs per subdomain) the sweeps use. */

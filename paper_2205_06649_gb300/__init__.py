@@ -23,7 +23,7 @@ __all__ = ["Context", "DD4DVError", "lib", "solver_defaults"]
 lib = _abi.load()
 
 # dd4dv_sweep_kernels codes
-KERNEL_NAMES = {1: "stripe", 2: "deep-halo", 3: "stripe-4buf", 4: "stripe-2buf"}
+KERNEL_NAMES = {1: "stripe", 2: "deep-halo", 3: "stripe-4buf", 4: "stripe-2buf", 5: "level"}
 
 
 class DD4DVError(RuntimeError):
@@ -190,7 +190,7 @@ class Context:
     def sweep_kernels(self) -> dict:
         """Kernels the current shapes run: 1 = stripe sweep, 2 = deep-halo
         sweep, 3 = four-buffer stripe adjoint, 4 = two-buffer stripe
-        forward."""
+        forward, 5 = level sweep."""
         k = np.zeros(2, dtype=np.int32)
         self._check(lib.dd4dv_sweep_kernels(self._h, C.c_void_p(k.ctypes.data)))
         return {"forward": int(k[0]), "adjoint": int(k[1])}

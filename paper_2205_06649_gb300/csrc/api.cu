@@ -4,7 +4,7 @@
 // step runs in this library's CUDA kernels; the host only validates inputs,
 // builds index tables and enqueues work.
 #include "dd4dvar.h"
-#include "common.cuh"
+#include "point.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -130,6 +130,15 @@ struct dd4dv_ctx {
     bool valid = false;
   } og;
   void drop_graphs();
+  // level sweeps (level.cu): tiles and scratch states; lv_f / lv_a: the forward
+  // / adjoint sweeps run them (else the cluster sweeps)
+  bool lv_f = false, lv_a = false;
+  LvPlan lv;
+  LvTile* lv_tiles = nullptr;
+  int *lv_boxes = nullptr, *lv_tile_off = nullptr;
+  void *lv_rec = nullptr, *lv_state = nullptr;
+  double *lv_acc_m = nullptr, *lv_acc_o = nullptr;
+  long long lv_elems = 0;     // elements of one level of every box
   std::vector<void*> dec_allocs;
 
   ~dd4dv_ctx();
@@ -353,10 +362,76 @@ void apply_VT(dd4dv_ctx* ctx, const double* y, const double* w, const double* sc
   KL(launch_grad_finish(ctx->subs_d, ctx->n_sub, w, ctx->vw2, scale, out, active, av, ctx->max_pts, ctx->st));
 }
 
+// Whether the forward / adjoint sweeps run as level sweeps: chosen with the
+// decomposition (level_plan), undone by an explicit launch shape or kernel
+// variant.
+bool level_forward(const dd4dv_ctx* ctx) { return ctx->lv_f && ctx->variant_f == 0; }
+bool level_adjoint(const dd4dv_ctx* ctx) {
+  // the level adjoint reads every level: under checkpoints only the level
+  // forward has stored them (it always stores every level)
+  return ctx->lv_a && ctx->variant_a == 0 && (ctx->ckpt == 0 || level_forward(ctx));
+}
+
+template <typename T>
+LvArgs<T> level_args(dd4dv_ctx* ctx, const int* active, int av) {
+  LvArgs<T> a{};
+  a.tiles = ctx->lv_tiles;
+  a.boxes = ctx->lv_boxes;
+  a.subs = ctx->subs_d;
+  a.mu_on = ctx->dec.mu != 0.0;
+  a.traj = static_cast<T*>(ctx->traj);
+  a.stg = ctx->use_stg ? static_cast<T*>(ctx->stg) : nullptr;
+  a.stg1 = ctx->use_stg ? nullptr : static_cast<T*>(ctx->stg1);
+  T* st = static_cast<T*>(ctx->lv_state);
+  a.x1s = st;
+  a.x2s = st + ctx->lv_elems;
+  a.lam = st + 2 * ctx->lv_elems;
+  a.mu2 = st + 3 * ctx->lv_elems;
+  a.mu1 = st + 4 * ctx->lv_elems;
+  a.tgt = static_cast<const T*>(ctx->tgt);
+  a.bnd = static_cast<const T*>(ctx->bnd);
+  a.fw = static_cast<const T*>(ctx->lv_rec);
+  a.bw = a.fw + 8 * (size_t)ctx->m.nlat;
+  const double scale = sizeof(T) == 8 ? ctx->m.dt : 1.0;   // as in sweep_args
+  a.dt = (T)ctx->m.dt;
+  a.Bth = (T)(scale * ctx->Bth);
+  a.gBth = (T)(scale * ctx->gBth);
+  a.href = (T)(sizeof(T) == 4 ? ctx->m.h_ref : 0.0);
+  for (int v = 0; v < 3; ++v) {
+    const double isb2 = 1.0 / (ctx->sigma_b[v] * ctx->sigma_b[v]);
+    a.isb2[v] = (T)isb2;
+    a.musb2[v] = (T)(ctx->dec.mu * isb2);
+  }
+  a.nlon = ctx->m.nlon;
+  a.nlat = ctx->m.nlat;
+  a.lam_w = ctx->dec.lambda;
+  a.obs = ctx->obs_d;
+  a.lvl_obs = ctx->lvl_obs_d;
+  a.obs_force = ctx->obs_force_d;
+  a.sc_tgt = ctx->sc_tgt_d;
+  a.sc_off = ctx->sc_off_d;
+  a.sc_obs = ctx->sc_obs_d;
+  a.lvl_sc = ctx->lvl_sc_d;
+  a.sc_w = ctx->sc_w_d;
+  a.acc_m = ctx->lv_acc_m;
+  a.acc_o = ctx->lv_acc_o;
+  a.active = active;
+  a.active_value = av;
+  a.lam_a = ctx->lam_a;
+  return a;
+}
+
 // full = true stores every level (exchange, trajectory export) even when the
-// evaluations checkpoint.
+// evaluations checkpoint, and leaves the terms of J out.
 template <typename T>
 void forward_sweep(dd4dv_ctx* ctx, const int* active, int av, bool full = false) {
+  if (level_forward(ctx)) {
+    LvArgs<T> a = level_args<T>(ctx, active, av);
+    a.terms = !full;
+    if (full) a.stg = a.stg1 = nullptr;
+    CK(launch_level_forward<T>(a, ctx->lv, ctx->st, &ctx->launches));
+    return;
+  }
   SweepArgs<T> a = sweep_args<T>(ctx);
   a.active = active;
   a.active_value = av;
@@ -370,18 +445,44 @@ void forward_sweep(dd4dv_ctx* ctx, const int* active, int av, bool full = false)
   KL(launch_forward<T>(a, ctx->cl_f, ctx->nt_f, ctx->st));
 }
 
+// J (and parts) from the terms that the last forward sweep left.
+void finalize_J(dd4dv_ctx* ctx, const double* w, double* J, double* parts, const int* active, int av) {
+  if (level_forward(ctx))
+    KL(launch_finalize_J_tiles(ctx->subs_d, ctx->n_sub, w, ctx->lv_acc_o, ctx->lv_acc_m, ctx->lv_tile_off,
+                               ctx->vconst, ctx->dec.lambda, ctx->dec.mu, J, parts, active, av, ctx->st));
+  else
+    KL(launch_finalize_J(ctx->subs_d, ctx->n_sub, w, ctx->part, ctx->cl_f, ctx->vconst, ctx->dec.lambda,
+                         ctx->dec.mu, J, parts, active, av, ctx->st));
+}
+
+// Adjoint sweep about the trajectory of the last forward sweep, forced by the
+// terms of J, by yforce (packed FP64 trajectories), or for a Gauss-Newton
+// product by the tangent-linear run in gn_dx.
+template <typename T>
+void adjoint_sweep(dd4dv_ctx* ctx, const int* active, int av, const double* yforce = nullptr, T* gn_dx = nullptr) {
+  if (level_adjoint(ctx)) {
+    LvArgs<T> a = level_args<T>(ctx, active, av);
+    a.yforce = yforce;
+    a.gn_dx = gn_dx;
+    CK(launch_level_adjoint<T>(a, ctx->lv, ctx->st, &ctx->launches));
+    return;
+  }
+  SweepArgs<T> a = sweep_args<T>(ctx);
+  a.active = active;
+  a.active_value = av;
+  a.yforce = yforce;
+  a.gn_dx = gn_dx;
+  KL(launch_adjoint<T>(a, ctx->cl, ctx->nthreads, ctx->st));
+}
+
 template <typename T>
 void eval_T(dd4dv_ctx* ctx, const double* w, double* J, double* grad, double* parts, const int* active,
             int av, const double* scale) {
   init_states<T>(ctx, w, ctx->vw, active, av);
   forward_sweep<T>(ctx, active, av);
-  KL(launch_finalize_J(ctx->subs_d, ctx->n_sub, w, ctx->part, ctx->cl_f, ctx->vconst, ctx->dec.lambda,
-                       ctx->dec.mu, J, parts, active, av, ctx->st));
+  finalize_J(ctx, w, J, parts, active, av);
   if (grad) {
-    SweepArgs<T> a = sweep_args<T>(ctx);
-    a.active = active;
-    a.active_value = av;
-    KL(launch_adjoint<T>(a, ctx->cl, ctx->nthreads, ctx->st));
+    adjoint_sweep<T>(ctx, active, av);
     apply_VT(ctx, ctx->lam_a, w, scale, grad, active, av);
   }
 }
@@ -444,11 +545,7 @@ void gn_product_T(dd4dv_ctx* ctx, const double* p, double* Ap, const int* active
   a.gn_dx = static_cast<T*>(ctx->gn_dx);
   a.R = tl_R;
   KL(launch_tlm<T>(a, tl_cl, ctx->nthreads, ctx->st));
-  SweepArgs<T> b = sweep_args<T>(ctx);
-  b.active = active;
-  b.active_value = av;
-  b.gn_dx = static_cast<T*>(ctx->gn_dx);
-  KL(launch_adjoint<T>(b, ctx->cl, ctx->nthreads, ctx->st));
+  adjoint_sweep<T>(ctx, active, av, nullptr, static_cast<T*>(ctx->gn_dx));
   apply_VT(ctx, ctx->lam_a, p, nullptr, Ap, active, av);
 }
 
@@ -637,9 +734,8 @@ void autotune(dd4dv_ctx* ctx) {
         CK(cudaEventRecord(ev[0], ctx->st));
         forward_sweep<T>(ctx, nullptr, 0);
         CK(cudaEventRecord(ev[1], ctx->st));
-        SweepArgs<T> a = sweep_args<T>(ctx);
         CK(cudaEventRecord(ev[2], ctx->st));
-        KL(launch_adjoint<T>(a, ctx->cl, ctx->nthreads, ctx->st));
+        adjoint_sweep<T>(ctx, nullptr, 0);
         CK(cudaEventRecord(ev[3], ctx->st));
         return 0;
       });
@@ -653,6 +749,25 @@ void autotune(dd4dv_ctx* ctx) {
     CK(cudaEventElapsedTime(ta, ev[2], ev[3]));
     return true;
   };
+  // the level sweeps, with and without stored stage states (best of two each)
+  struct Best { double t = 1e300; int c = 0, nt = 0, var = 0; };
+  double lv_f[2] = {1e300, 1e300}, lv_a[2] = {1e300, 1e300};
+  if (ctx->lv_tiles && ctx->variant_f == 0 && ctx->variant_a == 0) {
+    ctx->lv_f = ctx->lv_a = true;
+    for (int use : {1, 0}) {
+      if (use && !ctx->stg) continue;
+      ctx->use_stg = use;
+      for (int rep = 0; rep < 3; ++rep) {
+        float tf = 0, ta = 0;
+        if (!run(ctx->cl, ctx->nthreads, &tf, &ta)) break;
+        if (rep == 0) continue;   // warm-up
+        lv_f[use] = std::min(lv_f[use], (double)tf);
+        lv_a[use] = std::min(lv_a[use], (double)ta);
+      }
+    }
+    ctx->use_stg = ctx->stg != nullptr;
+    ctx->lv_f = ctx->lv_a = false;
+  }
   std::vector<int> cls;
   {
     const int va = ctx->variant_a;
@@ -672,7 +787,6 @@ void autotune(dd4dv_ctx* ctx) {
   run(c0, n0, &tf0, &ta0);
   const double budget_ms = std::max(2000.0, 80.0 * (tf0 + ta0));
   double spent = 0.0;
-  struct Best { double t = 1e300; int c = 0, nt = 0, var = 0; };
   Best best_f[2], best_a[2];
   const bool have_stg = ctx->stg != nullptr;
   const int var0 = ctx->variant_f;   // the caller's choice: 1 keeps the stripe sweeps
@@ -716,10 +830,12 @@ void autotune(dd4dv_ctx* ctx) {
         }
   }
   for (auto& e : ev) cudaEventDestroy(e);
-  int use = 0;
-  if (have_stg && best_f[1].c && best_a[1].c &&
-      (!best_f[0].c || best_f[1].t + best_a[1].t < best_f[0].t + best_a[0].t))
-    use = 1;
+  // time of each stage mode with the faster kind of each sweep
+  double mode_t[2];
+  for (int u : {0, 1})
+    mode_t[u] = std::min(best_f[u].c ? best_f[u].t : 1e300, lv_f[u]) + std::min(best_a[u].c ? best_a[u].t : 1e300, lv_a[u]);
+  const int use = have_stg && mode_t[1] < 1e300 && mode_t[1] < mode_t[0] ? 1 : 0;
+  const bool use_lv_f = lv_f[use] < best_f[use].t, use_lv_a = lv_a[use] < best_a[use].t;
   if (!best_f[use].c || !best_a[use].c) {   // nothing measured: keep the starting shape
     best_f[use] = {tf0, c0, n0, var0};
     best_a[use] = {ta0, c0, n0, var0};
@@ -734,7 +850,11 @@ void autotune(dd4dv_ctx* ctx) {
   ctx->nthreads = best_a[use].nt;
   ctx->R = (ctx->max_ny + ctx->cl - 1) / ctx->cl;
   ctx->dec.cluster = ctx->cl;
-  ctx->tune_ms = best_f[use].t + best_a[use].t;
+  ctx->tune_ms = std::min(best_f[use].t, lv_f[use]) + std::min(best_a[use].t, lv_a[use]);
+  ctx->lv_f = use_lv_f;
+  ctx->lv_a = use_lv_a;
+  if (use_lv_f) ctx->variant_f = 0;   // (a cluster shape stays set for the sweeps that need one)
+  if (use_lv_a) ctx->variant_a = 0;
   sync(ctx);
   if (!use && ctx->stg && ctx->dec.ckpt_k != -2) {   // recomputing the stages won: give the memory back
     free_dec_buffer(ctx, ctx->stg);
@@ -789,6 +909,125 @@ void tune_checkpoint(dd4dv_ctx* ctx) {
   }
   if (best.k == 0 && ctx->seg) free_dec_buffer(ctx, ctx->seg);
   ctx->ckpt_ms = best.ms;
+}
+
+// Smallest number of points per level (all boxes together) from which the
+// level sweeps run.  Below it a launch per stage (about 3 us each) costs more
+// than the cluster barriers.  Measured, forward + adjoint of 32 steps, cluster
+// against level sweeps (ms):
+//   FP64: 55,000 points in 128 boxes 1.39 / 1.78; 74,000 in 8 boxes 2.00 / 1.58;
+//         88,000 in 32 boxes 2.38 / 1.98; 350,000 in 128 boxes 6.96 / 5.31
+//   FP32: 305,000 in 32 boxes 0.98 / 1.16; 350,000 in 128 boxes 1.30 / 1.27;
+//         719,000 in 256 boxes 2.52 / 1.96; 1.2 million in 128 boxes 8.6 / 3.0
+constexpr long long kLvMinPoints64 = 65000, kLvMinPoints32 = 350000;
+
+// Tiles and scratch of the level sweeps.  Leaves ctx->lv_tiles null where they
+// do not apply: too few points, boxes no wider than a thread's columns, a grid
+// whose level does not fit 32-bit offsets, or no memory for the scratch.
+template <typename T>
+void level_plan(dd4dv_ctx* ctx, const std::vector<SubDesc>& subs, const std::vector<int>& lvl_obs) {
+  constexpr int V = lv_width<T>();
+  const int nlon = ctx->m.nlon, nlat = ctx->m.nlat, n_sub = (int)subs.size();
+  long long pts = 0;
+  int maxL = 0, min_nx = 1 << 30;
+  for (const SubDesc& d : subs) {
+    pts += (long long)d.nx * d.ny;
+    maxL = std::max(maxL, d.b - d.a);
+    min_nx = std::min(min_nx, d.nx);
+  }
+  long long least = sizeof(T) == 4 ? kLvMinPoints32 : kLvMinPoints64;
+  if (const char* e = std::getenv("DD4DV_LEVEL_MIN_POINTS")) least = std::atoll(e);   // override (tests)
+  if (pts < least || maxL < 1 || min_nx <= V || 3LL * nlon * nlat >= (1LL << 31)) return;
+  auto& L = ctx->dec_allocs;
+  std::vector<int> order(n_sub);
+  for (int s = 0; s < n_sub; ++s) order[s] = s;
+  std::stable_sort(order.begin(), order.end(),
+                   [&](int x, int y) { return subs[x].b - subs[x].a > subs[y].b - subs[y].a; });
+  // thread-points per thread: more than one saves set-up where there are many CTAs all the same
+  const int iters = pts > 2000000 ? (sizeof(T) == 4 ? 4 : 2) : 1;
+  std::vector<LvTile> tiles;
+  std::vector<int> tile_off(2 * n_sub);
+  LvPlan g;
+  g.n_tile.assign(maxL, 0);
+  g.n_box.assign(maxL + 1, 0);
+  g.obs.assign(maxL + 1, 0);
+  long long elems = 0;
+  auto magic = [](int v) { return v <= 1 ? 0u : (unsigned)(0xFFFFFFFFu / (unsigned)v + 1u); };
+  for (const int s : order) {
+    const SubDesc& d = subs[s];
+    LvTile t{};
+    t.s = s;
+    t.nx = d.nx;
+    t.ny = d.ny;
+    t.nxp = d.nxp;
+    t.nq = (d.nx + V - 1) / V;
+    t.mq = magic(t.nq);
+    t.mnx = magic(d.nx);
+    t.mny = magic(d.ny);
+    t.i0 = d.i0;
+    t.j0 = d.j0;
+    t.a = d.a;
+    t.L = d.b - d.a;
+    t.flags = d.flags;
+    t.iw = (d.i0 - 1 + nlon) % nlon;
+    t.ie = (d.i0 + d.nx) % nlon;
+    t.wL = d.wL; t.wR = d.wR; t.wS = d.wS; t.wN = d.wN; t.tA = d.tA; t.tB = d.tB;
+    t.sc_lvl = d.sc_lvl;
+    t.traj_off = d.traj_off;
+    t.ptraj_off = d.ptraj_off;
+    t.stg_off = d.stg_off;
+    t.stg1_off = d.stg1_off;
+    t.ctrl_off = d.ctrl_off;
+    t.lv_off = elems;
+    elems += 3LL * d.ny * d.nxp;
+    // equal tiles of whole warps
+    const int np = t.nq * d.ny;
+    const int nt = (np + iters * kLvThreads - 1) / (iters * kLvThreads);
+    const int per = ((np + nt - 1) / nt + 31) / 32 * 32;
+    tile_off[2 * s] = (int)tiles.size() * kLvThreads;
+    tile_off[2 * s + 1] = nt * kLvThreads;
+    for (int q = 0; q < nt; ++q) {
+      t.p0 = std::min(q * per, np);
+      t.p1 = std::min((q + 1) * per, np);
+      tiles.push_back(t);
+    }
+    for (int l = 0; l < t.L; ++l) g.n_tile[l] += nt;
+    for (int l = 0; l <= t.L; ++l) {
+      ++g.n_box[l];
+      if (lvl_obs[d.obs_lvl + l] != lvl_obs[d.obs_lvl + l + 1]) g.obs[l] = 1;
+    }
+  }
+  g.tiles = (int)tiles.size();
+  // row constants, rounded once to the state precision (as load_rows of sweep.cu)
+  std::vector<T> rec(16 * (size_t)nlat);
+  for (int j = 0; j < nlat; ++j) {
+    const RowConst& rc = ctx->rows_h[j];
+    const double cn = ctx->rows_h[std::min(j + 1, nlat - 1)].c, cs = ctx->rows_h[std::max(j - 1, 0)].c;
+    fill_records(rc, cn, cs, ctx->m.dt, ctx->Bth, &rec[8 * (size_t)j], &rec[8 * (size_t)(nlat + j)]);
+  }
+  // only where the scratch fits beside what the decomposition already holds
+  size_t free_b = 0, total_b = 0;
+  CK(cudaMemGetInfo(&free_b, &total_b));
+  const size_t slots = tiles.size() * kLvThreads;
+  const size_t need = 5 * (size_t)elems * sizeof(T) + tiles.size() * sizeof(LvTile) +
+                      slots * sizeof(double) + (64u << 20);
+  if (need > free_b) return;
+  LvTile* td = dalloc<LvTile>(ctx, tiles.size(), &L);
+  ctx->lv_boxes = dalloc<int>(ctx, n_sub, &L);
+  ctx->lv_tile_off = dalloc<int>(ctx, 2 * n_sub, &L);
+  ctx->lv_rec = dalloc<T>(ctx, rec.size(), &L);
+  ctx->lv_state = dalloc<T>(ctx, 5 * (size_t)elems, &L);
+  ctx->lv_acc_m = dalloc<double>(ctx, slots, &L);
+  ctx->lv_acc_o = dalloc<double>(ctx, n_sub, &L);
+  h2d(ctx, td, tiles.data(), tiles.size() * sizeof(LvTile));
+  h2d(ctx, ctx->lv_boxes, order.data(), n_sub * sizeof(int));
+  h2d(ctx, ctx->lv_tile_off, tile_off.data(), 2 * n_sub * sizeof(int));
+  h2d(ctx, ctx->lv_rec, rec.data(), rec.size() * sizeof(T));
+  CK(cudaMemsetAsync(ctx->lv_state, 0, 5 * (size_t)elems * sizeof(T), ctx->st));
+  CK(cudaStreamSynchronize(ctx->st));   // the host tables end with this call
+  ctx->lv_tiles = td;
+  ctx->lv_elems = elems;
+  ctx->lv = std::move(g);
 }
 
 // ---------------------------------------------------------------------------
@@ -1088,6 +1327,8 @@ void build_decomposition(dd4dv_ctx* ctx, const dd4dv_decomp& d) {
     const long long wy = (long long)subs[y].nx * subs[y].ny * (subs[y].b - subs[y].a + 1);
     return wx > wy;
   });
+  ctx->lv_tiles = nullptr;
+  ctx->lv_f = ctx->lv_a = false;
   ctx->traj = dalloc<unsigned char>(ctx, ctx->traj_elems * ctx->tsize, &L);
   ctx->stg = nullptr;
   ctx->stg_elems = 0;
@@ -1186,6 +1427,11 @@ void build_decomposition(dd4dv_ctx* ctx, const dd4dv_decomp& d) {
       ctx->stg1 = dalloc<unsigned char>(ctx, used * ctx->tsize, &L);
       ctx->stg1_frac = pts > 0 ? (double)pts_in / (double)pts : 0.0;
     }
+  }
+  if (d.cluster <= 0) {
+    if (f32) level_plan<float>(ctx, subs, lvl_obs);
+    else level_plan<double>(ctx, subs, lvl_obs);
+    ctx->lv_f = ctx->lv_a = d.cluster == 0 && ctx->lv_tiles;
   }
   h2d(ctx, ctx->subs_d, subs.data(), subs.size() * sizeof(SubDesc));
   h2d(ctx, ctx->order_d, order.data(), order.size() * sizeof(int));
@@ -1534,8 +1780,7 @@ dd4dv_status dd4dv_eval_forward(dd4dv_ctx* ctx, const double* w_all, double* J_a
       using T = decltype(t);
       init_states<T>(ctx, ctx->io_c, ctx->vw, own_mask(ctx), 1);
       forward_sweep<T>(ctx, own_mask(ctx), 1);
-      KL(launch_finalize_J(ctx->subs_d, ctx->n_sub, ctx->io_c, ctx->part, ctx->cl_f, ctx->vconst,
-                           ctx->dec.lambda, ctx->dec.mu, J, pa, own_mask(ctx), 1, ctx->st));
+      finalize_J(ctx, ctx->io_c, J, pa, own_mask(ctx), 1);
       return 0;
     });
     ctx->fwd_pending = true;
@@ -1558,10 +1803,7 @@ dd4dv_status dd4dv_eval_backward(dd4dv_ctx* ctx, const double* scale, double* gr
     double* gr = device_ptrs ? grad_all : ctx->io_b;
     by_precision(ctx, [&](auto t) {
       using T = decltype(t);
-      SweepArgs<T> a = sweep_args<T>(ctx);
-      a.active = own_mask(ctx);
-      a.active_value = 1;
-      KL(launch_adjoint<T>(a, ctx->cl, ctx->nthreads, ctx->st));
+      adjoint_sweep<T>(ctx, own_mask(ctx), 1);
       apply_VT(ctx, ctx->lam_a, ctx->io_c, sc, gr, own_mask(ctx), 1);
       return 0;
     });
@@ -1628,9 +1870,7 @@ dd4dv_status dd4dv_adjoint(dd4dv_ctx* ctx, const double* w_all, const double* y_
       using T = decltype(t);
       init_states<T>(ctx, w, ctx->vw, nullptr, 0);
       forward_sweep<T>(ctx, nullptr, 0);
-      SweepArgs<T> a = sweep_args<T>(ctx);
-      a.yforce = y;
-      KL(launch_adjoint<T>(a, ctx->cl, ctx->nthreads, ctx->st));
+      adjoint_sweep<T>(ctx, nullptr, 0, y);
       apply_VT(ctx, ctx->lam_a, nullptr, nullptr, out, nullptr, 0);
       return 0;
     });
@@ -2470,11 +2710,9 @@ dd4dv_status dd4dv_profile_sweeps(dd4dv_ctx* ctx, const double* w_all, int reps,
         CK(cudaEventRecord(ev[0], ctx->st));
         forward_sweep<T>(ctx, nullptr, 0);
         CK(cudaEventRecord(ev[1], ctx->st));
-        KL(launch_finalize_J(ctx->subs_d, ctx->n_sub, ctx->io_a, ctx->part, ctx->cl_f, ctx->vconst,
-                             ctx->dec.lambda, ctx->dec.mu, ctx->io_p, nullptr, nullptr, 0, ctx->st));
-        SweepArgs<T> a = sweep_args<T>(ctx);
+        finalize_J(ctx, ctx->io_a, ctx->io_p, nullptr, nullptr, 0);
         CK(cudaEventRecord(ev[2], ctx->st));
-        KL(launch_adjoint<T>(a, ctx->cl, ctx->nthreads, ctx->st));
+        adjoint_sweep<T>(ctx, nullptr, 0);
         CK(cudaEventRecord(ev[3], ctx->st));
         apply_VT(ctx, ctx->lam_a, ctx->io_a, nullptr, ctx->io_b, nullptr, 0);
         CK(cudaEventRecord(ev[5], ctx->st));
@@ -2540,6 +2778,7 @@ dd4dv_status dd4dv_set_sweep_config(dd4dv_ctx* ctx, const int* shape) {
     ctx->cl = ca; ctx->nthreads = ta; ctx->R = Ra;
     ctx->use_stg = sg != 0;
     ctx->dec.cluster = ca;
+    ctx->lv_f = ctx->lv_a = false;   // an explicit cluster shape asks for the cluster sweeps
     ctx->drop_graphs();
     return DD4DV_OK;
   });
@@ -2582,8 +2821,8 @@ dd4dv_status dd4dv_sweep_kernels(const dd4dv_ctx* cctx, int* kinds) {
   return guard(ctx, [&] {
     require_dec(ctx);
     if (!kinds) fail(ctx, DD4DV_EINVAL, "NULL argument");
-    kinds[0] = fwd_kind_at(ctx, ctx->cl_f, ctx->nt_f);
-    kinds[1] = adj_kind_at(ctx, ctx->cl, ctx->nthreads);
+    kinds[0] = level_forward(ctx) ? 5 : fwd_kind_at(ctx, ctx->cl_f, ctx->nt_f);
+    kinds[1] = level_adjoint(ctx) ? 5 : adj_kind_at(ctx, ctx->cl, ctx->nthreads);
     return DD4DV_OK;
   });
 }

@@ -127,8 +127,11 @@ __global__ void grad_finish_kernel(const SubDesc* subs, const double* w, const d
   }
 }
 
-// J_s = 1/2 w.w + lambda J_o + mu (J_mu + overlap constant)
+// J_s = 1/2 w.w + lambda J_o + mu (J_mu + overlap constant).  J_o and J_mu
+// come per CTA of a cluster sweep (part, stride SweepArgs::cl_max = 16), or
+// after a level sweep per box (acc_o) and, doubled, per tile (acc_m).
 __global__ void finalize_J_kernel(const SubDesc* subs, const double* w, const double* part, int ncl,
+                                  const double* acc_o, const double* acc_m, const int* tile_off,
                                   const double* vconst, double lam, double mu, double* J,
                                   double* parts, const int* active, int active_value) {
   __shared__ double sh[33];
@@ -142,11 +145,21 @@ __global__ void finalize_J_kernel(const SubDesc* subs, const double* w, const do
     acc += x * x;
   }
   const double ww = block_sum(acc, sh);
+  double tiles = 0.0;
+  if (acc_m) {
+    for (int i = threadIdx.x; i < tile_off[2 * s + 1]; i += blockDim.x) tiles += acc_m[tile_off[2 * s] + i];
+    tiles = block_sum(tiles, sh);
+  }
   if (threadIdx.x == 0) {
     double Jo = 0.0, Jm = 0.0;
-    for (int r = 0; r < ncl; ++r) {
-      Jo += part[((size_t)s * 16 + r) * 2 + 0];   // stride: SweepArgs::cl_max = 16
-      Jm += part[((size_t)s * 16 + r) * 2 + 1];
+    if (acc_m) {
+      Jo = acc_o[s];
+      Jm = 0.5 * tiles;
+    } else {
+      for (int r = 0; r < ncl; ++r) {
+        Jo += part[((size_t)s * 16 + r) * 2 + 0];
+        Jm += part[((size_t)s * 16 + r) * 2 + 1];
+      }
     }
     Jm += vconst[s];
     const double Jb = 0.5 * ww;
@@ -803,8 +816,16 @@ cudaError_t launch_grad_finish(const SubDesc* subs, int n_sub, const double* w, 
 cudaError_t launch_finalize_J(const SubDesc* subs, int n_sub, const double* w, const double* part,
                               int ncl, const double* vconst, double lam, double mu, double* J,
                               double* parts, const int* active, int active_value, cudaStream_t st) {
-  finalize_J_kernel<<<n_sub, 256, 0, st>>>(subs, w, part, ncl, vconst, lam, mu, J, parts, active,
-                                           active_value);
+  finalize_J_kernel<<<n_sub, 256, 0, st>>>(subs, w, part, ncl, nullptr, nullptr, nullptr, vconst, lam, mu, J,
+                                           parts, active, active_value);
+  return cudaGetLastError();
+}
+cudaError_t launch_finalize_J_tiles(const SubDesc* subs, int n_sub, const double* w, const double* acc_o,
+                                    const double* acc_m, const int* tile_off, const double* vconst, double lam,
+                                    double mu, double* J, double* parts, const int* active, int active_value,
+                                    cudaStream_t st) {
+  finalize_J_kernel<<<n_sub, 256, 0, st>>>(subs, w, nullptr, 0, acc_o, acc_m, tile_off, vconst, lam, mu, J, parts,
+                                           active, active_value);
   return cudaGetLastError();
 }
 

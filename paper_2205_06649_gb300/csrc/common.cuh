@@ -18,6 +18,7 @@
 
 #include <cuda_runtime.h>
 #include <cstdint>
+#include <vector>
 
 namespace dd4dv {
 
@@ -117,7 +118,7 @@ struct SweepArgs {
 // threads per SM), 1024 on the FP64 path (64 registers, one CTA of 1024 or two
 // of 512 per SM).  The stripe adjoint takes up to 1024 threads (64 registers).
 template <typename T> constexpr int max_threads_forward() { return sizeof(T) == 4 ? 384 : 1024; }
-template <typename T> constexpr int min_blocks_forward() { return sizeof(T) == 4 ? 2 : 1; }
+template <typename T> constexpr int min_blocks_forward() { return sizeof(T) == 4 ? 4 : 1; }
 constexpr int kStripeAdjThreads = 1024;
 
 // ---- launchers (sweep.cu) ----
@@ -137,6 +138,65 @@ template <typename T> size_t smem_adjoint_rl(int R, int W);
 template <typename T> size_t smem_tlm(int R, int W);
 // resident clusters of the stripe adjoint sweep at cl CTAs per cluster
 template <typename T> int active_clusters_adjoint(int R, int W, int cl, int nthreads);
+
+// ---- level sweeps (level.cu) ----
+// One tile: the thread-points [p0, p1) of one box (a thread-point is V
+// neighbouring columns of a row), with everything of the box a kernel needs.
+struct LvTile {
+  int s, p0, p1;
+  int nx, ny, nxp, nq;        // nq: thread-points per row
+  unsigned mq, mnx, mny;      // multipliers for division by nq, nx, ny
+  int i0, j0, a, L, flags;
+  int iw, ie;                 // global columns of the west / east frozen ghosts
+  int wL, wR, wS, wN, tA, tB;
+  int sc_lvl;
+  long long traj_off, ptraj_off, stg_off, stg1_off, ctrl_off;
+  long long lv_off;           // one-level scratch offset (elements of T): [3][ny][nxp]
+};
+// The tiles of every box, longest window first.
+struct LvPlan {
+  int tiles = 0;
+  std::vector<int> n_tile;    // per step l: tiles of the boxes that take it (a prefix)
+  std::vector<int> n_box;     // per level l: boxes that have it (a prefix of the box list)
+  std::vector<char> obs;      // per level l: some box has observations there
+};
+template <typename T>
+struct LvArgs {
+  const LvTile* tiles;
+  const int* boxes;           // longest window first
+  const SubDesc* subs;
+  int n_tile;
+  int l;                      // step / level
+  int terms;                  // forward: accumulate the observation and overlap terms
+  int skip1;                  // first stage recomputed only where x1 is not stored
+  int mu_on;                  // mu != 0
+  T *traj, *stg, *stg1;
+  T *x1s, *x2s, *lam, *mu2, *mu1;   // one-level scratch states of every box
+  const T *tgt, *bnd, *gn_dx;
+  const T *fw, *bw;           // row constants [nlat][8] (the records of sweep.cu)
+  T dt, Bth, gBth, href;
+  T isb2[3], musb2[3];
+  int nlon, nlat;
+  double lam_w;               // weight lambda of the observation term
+  const ObsRec* obs;
+  const int* lvl_obs;
+  double* obs_force;
+  const int *sc_tgt, *sc_off, *sc_obs, *lvl_sc;
+  const double* sc_w;
+  double *acc_m, *acc_o;      // per tile and thread: twice J_mu; per box: J_o
+  const int* active;
+  int active_value;
+  double* lam_a;
+  const double* yforce;
+};
+// Columns per thread: FP32 threads take four neighbouring points (16-byte
+// accesses), FP64 threads one.
+template <typename T> __host__ __device__ constexpr int lv_width() { return sizeof(T) == 4 ? 4 : 1; }
+constexpr int kLvThreads = 128;
+template <typename T>
+cudaError_t launch_level_forward(const LvArgs<T>& a, const LvPlan& g, cudaStream_t st, long long* launches);
+template <typename T>
+cudaError_t launch_level_adjoint(const LvArgs<T>& a, const LvPlan& g, cudaStream_t st, long long* launches);
 
 // ---- auxiliary kernels (aux.cu) ----
 struct RFArgs {
@@ -171,6 +231,12 @@ cudaError_t launch_grad_finish(const SubDesc* subs, int n_sub, const double* w, 
 cudaError_t launch_finalize_J(const SubDesc* subs, int n_sub, const double* w, const double* part,
                               int cl_max, const double* vconst, double lam, double mu, double* J,
                               double* parts, const int* active, int active_value, cudaStream_t st);
+// the same after a level forward sweep: J_o per box, twice J_mu in the box's
+// tile_off[2 s + 1] slots from tile_off[2 s]
+cudaError_t launch_finalize_J_tiles(const SubDesc* subs, int n_sub, const double* w, const double* acc_o,
+                                    const double* acc_m, const int* tile_off, const double* vconst, double lam,
+                                    double mu, double* J, double* parts, const int* active, int active_value,
+                                    cudaStream_t st);
 
 template <typename T>
 struct ExchArgs {

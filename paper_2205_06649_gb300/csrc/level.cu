@@ -1,0 +1,664 @@
+// Level sweeps: the forward and adjoint sweeps of all subdomains advanced
+// together, one launch per RK3 stage, with the states in HBM / L2.
+//
+// Design (GB300, sm_103a).  The cluster sweeps (sweep.cu) keep one box in one
+// thread-block cluster for its whole window.  A box's stages are then a chain
+// of cluster barriers with a few points per thread between them, clusters pack
+// badly into GPCs, and neither the FP64 pipe (62-65 % of its rate over a sweep)
+// nor HBM (7-12 %) is busy.  Where all boxes together have enough points per
+// level, a stage of every box is one ordinary grid instead:
+//   * FP64: 24-47 FP64 instructions per point take 16 SM cycles per warp each;
+//     the 15-36 loads of a point are a tenth of that, so plain loads through L1
+//     keep the FP64 pipe fed, and every SM works until the grid's end.  Bound:
+//     the FP64 pipe (about 90 % of its rate with the overlap terms counted).
+//   * FP32: a thread takes four neighbouring columns with 16-byte loads.  Bound:
+//     latency of the loads (HBM at 45-50 % of its measured rate); groups of boxes
+//     sized for L2, strips marching north with rows kept in registers, one or
+//     two columns a thread at 1.7x the warps, and a whole step per launch with
+//     rows in shared memory all measured slower or equal.
+// A tile is a run of points of one box (flat over rows, so that every lane has
+// one); tiles are ordered longest window first, so the boxes still running at
+// step l are a prefix and the grid shrinks with them.  CTAs of 128 threads: with
+// 256 the last wave of a 175,000-point level left a fifth of the SMs idle (FP64
+// evaluation of 64 boxes 3.33 ms, with 128 3.07 ms).  Launches overlap their
+// set-up with the end of the launch before (programmatic dependent launch).
+//
+// Measured against the cluster sweeps with the launch shapes that the library
+// chooses (forward / adjoint, ms):
+//   batching workload (512 boxes, 3.9e8 points x steps), FP32: 15.8 / 30.7 ->
+//     9.6 / 17.6; FP64: 102.8 / 156.7 -> 66.6 / 93.6 (a part of it from the FP64
+//     point functions, which the level sweeps alone ran at 77 / 112 without)
+//   one 128-step window of the large workload (256 boxes), FP32: 15.4 / 29.6 -> 9.3 / 17.7
+//   differentiation workload (FP32, 16-step checkpoints): 1.68 / 4.91 -> 1.72 / 3.18
+//   medium workload (FP64, 64 boxes, 184,000 points): 1.64 / 2.31 -> 1.64 / 2.22
+//
+// The arithmetic per point is that of sweep.cu (point.cuh), so trajectories,
+// stage states and gradients are the same bit for bit; J differs by the order
+// of its partial sums.
+#include "point.cuh"
+
+namespace dd4dv {
+
+namespace {
+
+// Waits for the grids before this one (programmatic dependent launch): every
+// thread of every level kernel calls it before it reads what they wrote, also
+// where it then has nothing to do, so that a grid never ends before the ones it
+// follows.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// The CTA's tile in shared memory: one coalesced load, and no registers held
+// for the fields that only edges need.
+#define LV_TILE(t)                                                                                    \
+  __shared__ LvTile t;                                                                                \
+  if (threadIdx.x < sizeof(LvTile) / 4)                                                               \
+    reinterpret_cast<int*>(&t)[threadIdx.x] = reinterpret_cast<const int*>(a.tiles + blockIdx.x)[threadIdx.x]; \
+  __syncthreads()
+static_assert(sizeof(LvTile) % 4 == 0 && sizeof(LvTile) / 4 <= kLvThreads, "one word a thread");
+
+// V consecutive values from / to global memory (aligned to V elements).
+template <typename T, int V>
+__device__ __forceinline__ void ldv(const T* p, T* x) {
+  if constexpr (V == 4) {
+    const float4 q = *reinterpret_cast<const float4*>(p);
+    x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
+  } else if constexpr (V == 2) {
+    const float2 q = *reinterpret_cast<const float2*>(p);
+    x[0] = q.x; x[1] = q.y;
+  } else {
+    x[0] = *p;
+  }
+}
+template <typename T, int V>
+__device__ __forceinline__ void stv(T* p, const T* x) {
+  if constexpr (V == 4) *reinterpret_cast<float4*>(p) = make_float4(x[0], x[1], x[2], x[3]);
+  else if constexpr (V == 2) *reinterpret_cast<float2*>(p) = make_float2(x[0], x[1]);
+  else *p = x[0];
+}
+
+// A thread's V points (row r, columns k .. k + V - 1) of one buffer with the
+// values around them: c[v][0] west of the first, c[v][V + 1] east of the last.
+template <typename T, int V>
+struct Patch {
+  T c[3][V + 2], n[3][V], s[3][V];
+};
+
+template <typename T, int V>
+__device__ __forceinline__ void point_of(const Patch<T, V>& z, int j, Pt5<T>& p) {
+  p.h = z.c[0][j + 1]; p.u = z.c[1][j + 1]; p.v = z.c[2][j + 1];
+  p.hE = z.c[0][j + 2]; p.uE = z.c[1][j + 2]; p.vE = z.c[2][j + 2];
+  p.hW = z.c[0][j]; p.uW = z.c[1][j]; p.vW = z.c[2][j];
+  p.hN = z.n[0][j]; p.uN = z.n[1][j]; p.vN = z.n[2][j];
+  p.hS = z.s[0][j]; p.uS = z.s[1][j]; p.vS = z.s[2][j];
+}
+
+// Boundary-trajectory value at offset o of level B0, blended with half of
+// level B1 where B1 is given (as bnd_val of sweep.cu).
+template <typename T>
+__device__ __forceinline__ T frozen(const T* B0, const T* B1, int o) {
+  const T xa = B0[o];
+  return B1 ? xfma((T)0.5, xa, xmul((T)0.5, B1[o])) : xa;
+}
+
+// The patch of a state buffer Y ([3][ny][nxp]) at element offset at = r nxp + k,
+// ghosts by the box-edge rules: wall mirror (h, u, -v), periodic wrap, or the
+// frozen boundary trajectory.  A box is wider than V, so a thread has at most
+// one ghost column.
+template <typename T, int V>
+__device__ __forceinline__ void load_state_patch(const LvArgs<T>& a, const LvTile& t, const T* Y, int r, int k,
+                                                 int at, const T* B0, const T* B1, Patch<T, V>& z) {
+  const int pl = t.ny * t.nxp;
+  const bool west = k == 0, east = k + V >= t.nx, north = r == t.ny - 1, south = r == 0;
+#pragma unroll
+  for (int v = 0; v < 3; ++v) {
+    const T* y = Y + (at + v * pl);
+    ldv<T, V>(y, &z.c[v][1]);
+    if (!west) z.c[v][0] = y[-1];
+    if (!east) z.c[v][V + 1] = y[V];
+    if (!north) ldv<T, V>(y + t.nxp, z.n[v]);
+    if (!south) ldv<T, V>(y - t.nxp, z.s[v]);
+  }
+  if (west || east) {
+    const bool per = t.flags & F_PERIODIC;
+    const int pg = a.nlat * a.nlon;
+    const int o = per ? r * t.nxp + (west ? t.nx - 1 : 0) : (t.j0 + r) * a.nlon + (west ? t.iw : t.ie);
+    const T* src = (per ? Y : B0) + o;
+    const int str = per ? pl : pg;
+    T g[3];
+#pragma unroll
+    for (int v = 0; v < 3; ++v) g[v] = src[v * str];
+    if (B1 && !per) {
+#pragma unroll
+      for (int v = 0; v < 3; ++v) g[v] = xfma((T)0.5, g[v], xmul((T)0.5, B1[o + v * pg]));
+    }
+    const int je = t.nx - k + 1;   // slot of column nx
+#pragma unroll
+    for (int v = 0; v < 3; ++v) {
+      if (west) z.c[v][0] = g[v];
+#pragma unroll
+      for (int j = 2; j < V + 2; ++j)
+        if (east && j == je) z.c[v][j] = g[v];
+    }
+  }
+  if (north || south) {
+    const bool wall = t.flags & (north ? F_NWALL : F_SWALL);
+    const int pg = a.nlat * a.nlon;
+    const int row = (north ? t.j0 + t.ny : t.j0 - 1) * a.nlon;
+#pragma unroll
+    for (int j = 0; j < V; ++j) {
+      int i = t.i0 + min(k + j, t.nx - 1);
+      if (i >= a.nlon) i -= a.nlon;
+      T g[3];
+      if (wall) {
+        g[0] = z.c[0][j + 1];
+        g[1] = z.c[1][j + 1];
+        g[2] = -z.c[2][j + 1];
+      } else {
+#pragma unroll
+        for (int v = 0; v < 3; ++v) g[v] = frozen(B0, B1, row + v * pg + i);
+      }
+#pragma unroll
+      for (int v = 0; v < 3; ++v) {
+        if (north) z.n[v][j] = g[v];
+        else z.s[v][j] = g[v];
+      }
+    }
+  }
+}
+
+// The patch of an adjoint buffer M: ghosts are zero but for the periodic wrap.
+template <typename T, int V>
+__device__ __forceinline__ void load_adjoint_patch(const LvTile& t, const T* M, int r, int k, int at,
+                                                   Patch<T, V>& z) {
+  const int pl = t.ny * t.nxp;
+  const bool west = k == 0, east = k + V >= t.nx, north = r == t.ny - 1, south = r == 0;
+  const bool per = t.flags & F_PERIODIC;
+  const int je = t.nx - k + 1;
+#pragma unroll
+  for (int v = 0; v < 3; ++v) {
+    const T* y = M + (at + v * pl);
+    ldv<T, V>(y, &z.c[v][1]);
+    // periodic wrap: column -1 is nx - 1 of the row, column nx is 0
+    z.c[v][0] = west ? (per ? y[t.nx - 1] : (T)0) : y[-1];
+    const T e = east ? (per ? y[-k] : (T)0) : y[V];
+    z.c[v][V + 1] = e;
+#pragma unroll
+    for (int j = 2; j < V + 1; ++j)
+      if (east && j == je) z.c[v][j] = e;
+#pragma unroll
+    for (int j = 0; j < V; ++j) z.n[v][j] = z.s[v][j] = (T)0;
+    if (!north) ldv<T, V>(y + t.nxp, z.n[v]);
+    if (!south) ldv<T, V>(y - t.nxp, z.s[v]);
+  }
+}
+
+template <typename T>
+__device__ __forceinline__ size_t level_size(const LvTile& t) {
+  return (size_t)3 * t.ny * t.nxp;
+}
+// Where the stage states of step l live: the stage buffer, the x1-only buffer
+// of the subdomains that have one, or the one-level scratch.
+template <typename T>
+__device__ __forceinline__ T* x1_of(const LvArgs<T>& a, const LvTile& t, int l) {
+  if (a.stg) return a.stg + t.stg_off + (size_t)2 * l * level_size<T>(t);
+  if (a.stg1 && t.stg1_off >= 0) return a.stg1 + t.stg1_off + (size_t)l * level_size<T>(t);
+  return a.x1s + t.lv_off;
+}
+template <typename T>
+__device__ __forceinline__ T* x2_of(const LvArgs<T>& a, const LvTile& t, int l) {
+  if (a.stg) return a.stg + t.stg_off + (size_t)(2 * l + 1) * level_size<T>(t);
+  return a.x2s + t.lv_off;
+}
+
+__device__ __forceinline__ int lv_overlap_count(const LvTile& t, int l, int r, int k) {
+  const int cx = 1 + (k < t.wL) + (k >= t.nx - t.wR);
+  const int cy = 1 + (r < t.wS) + (r >= t.ny - t.wN);
+  const int ct = 1 + (l < t.tA) + (l > t.L - t.tB);
+  return cx * cy * ct - 1;
+}
+__device__ __forceinline__ bool lv_overlaps(const LvTile& t, int l) {
+  return (l < t.tA) || (l > t.L - t.tB) || t.wL || t.wR || t.wS || t.wN;
+}
+
+// Sum of the block's values (fixed order), on thread 0.
+__device__ __forceinline__ double lv_block_sum(double x, double* sh) {
+  sh[threadIdx.x] = x;
+  __syncthreads();
+  double s = 0.0;
+  if (threadIdx.x < 32) {
+    for (int i = threadIdx.x; i < (int)blockDim.x; i += 32) s += sh[i];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  }
+  return s;
+}
+
+// Observation misfits of one box at level l (one CTA): obs_force, and J_o
+// added to the box's accumulator.
+template <typename T>
+__device__ void lv_obs(const LvArgs<T>& a, int s, int l, double* sh) {
+  const SubDesc& d = a.subs[s];
+  const int o0 = a.lvl_obs[d.obs_lvl + l], o1 = a.lvl_obs[d.obs_lvl + l + 1];
+  if (o0 == o1) return;
+  const int nxp = d.nxp;
+  const size_t pl = (size_t)d.ny * nxp;
+  const T* X = a.traj + d.traj_off + (size_t)l * 3 * pl;
+  double Jo = 0.0;
+  for (int o = o0 + threadIdx.x; o < o1; o += blockDim.x) {
+    const ObsRec ob = a.obs[o];
+    const T* x = X + ob.var * pl + (size_t)ob.r0 * nxp;
+    const double x00 = (double)x[ob.k0];
+    const double x01 = ob.di != 0.0 ? (double)x[ob.k1] : 0.0;
+    const double x10 = ob.dj != 0.0 ? (double)x[nxp + ob.k0] : 0.0;
+    const double x11 = (ob.dj != 0.0 && ob.di != 0.0) ? (double)x[nxp + ob.k1] : 0.0;
+    a.obs_force[o] = obs_term(ob, x00, x01, x10, x11, a.lam_w, Jo);
+  }
+  Jo = lv_block_sum(Jo, sh);
+  if (threadIdx.x == 0) a.acc_o[s] += Jo;
+}
+
+// Sum of FP32 terms without the rounding of its additions (TwoSum), so that
+// the order of the points does not show in J; FP64 terms are added directly.
+template <typename T>
+struct Sum {
+  T s = (T)0, e = (T)0;
+  __device__ __forceinline__ void add(T x) {
+    if constexpr (sizeof(T) == 4) {
+      const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
+      e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b)));
+      s = t;
+    } else {
+      s += x;
+    }
+  }
+  __device__ __forceinline__ double value() const { return sizeof(T) == 4 ? (double)s + (double)e : (double)s; }
+};
+
+// c sum_v (x_v - m_v)^2 / sigma_v^2 of one point (overlap_term of sweep.cu).
+template <typename T>
+__device__ __forceinline__ void overlap_add(Sum<T>& part, int c, T x0, T x1, T x2, T m0, T m1, T m2,
+                                            const T (&isb2)[3]) {
+  const T e0 = xsub(x0, m0), e1 = xsub(x1, m1), e2 = xsub(x2, m2);
+  T sq = xmul(xmul(e0, e0), isb2[0]);
+  sq = xfma(xmul(e1, e1), isb2[1], sq);
+  sq = xfma(xmul(e2, e2), isb2[2], sq);
+  if constexpr (sizeof(T) == 4) {
+    const float p = xmul((float)c, sq);
+    part.add(p);
+    part.e = __fadd_rn(part.e, xfma((float)c, sq, -p));
+  } else {
+    part.s = xfma((T)c, sq, part.s);
+  }
+}
+
+// Twice the overlap misfit of a thread's V points at level l (the terms of
+// overlap_level of sweep.cu).
+template <typename T, int V>
+__device__ __forceinline__ void lv_overlap_part(const LvArgs<T>& a, const LvTile& t, const T* tg, int l, int r, int k,
+                                                int at, const T (*o)[V], Sum<T>& part) {
+  const int pl = t.ny * t.nxp;
+  int c[V], any = 0;
+#pragma unroll
+  for (int j = 0; j < V; ++j) {
+    c[j] = k + j < t.nx ? lv_overlap_count(t, l, r, k + j) : 0;
+    any |= c[j];
+  }
+  if (!any) return;
+  T m[3][V];
+#pragma unroll
+  for (int v = 0; v < 3; ++v) ldv<T, V>(tg + (at + v * pl), m[v]);
+#pragma unroll
+  for (int j = 0; j < V; ++j)
+    if (c[j]) overlap_add(part, c[j], o[0][j], o[1][j], o[2][j], m[0][j], m[1][j], m[2][j], a.isb2);
+}
+
+// Terms of level 0 (the initial states): starts the accumulators of J.
+template <typename T, int V>
+__global__ void __launch_bounds__(kLvThreads) lv_start_kernel(const LvArgs<T> a) {
+  LV_TILE(t);
+  grid_wait();
+  grid_release();
+  if (a.active && a.active[t.s] != a.active_value) return;
+  Sum<T> part;
+  if (lv_overlaps(t, 0)) {
+    const T* X = a.traj + t.traj_off;
+    const int pl = t.ny * t.nxp;
+    for (int p = t.p0 + threadIdx.x; p < t.p1; p += kLvThreads) {
+      const int r = mdiv(p, t.mq), k = (p - r * t.nq) * V, at = r * t.nxp + k;
+      T o[3][V];
+#pragma unroll
+      for (int v = 0; v < 3; ++v) ldv<T, V>(X + (at + v * pl), o[v]);
+      lv_overlap_part<T, V>(a, t, a.tgt + t.traj_off, 0, r, k, at, o, part);
+    }
+  }
+  a.acc_m[(size_t)blockIdx.x * kLvThreads + threadIdx.x] = part.value();
+  if (t.p0 == 0 && threadIdx.x == 0) a.acc_o[t.s] = 0.0;
+}
+
+// RK3 stage ST of step l: out = cx X + cy (Y + dt F(Y)) of every tile.  The
+// first stage's grid carries one more CTA per box of a.boxes for the
+// observations of level l; with TERMS, the third stage adds level l + 1's
+// overlap misfit.  skip1: leave the boxes out whose x1 is stored (first stage
+// recomputed for the adjoint).
+template <typename T, int V, int ST, bool TERMS>
+__global__ void __launch_bounds__(kLvThreads, 6) lv_stage_kernel(const LvArgs<T> a) {
+  constexpr bool DEV = sizeof(T) == 4;
+  __shared__ double sh[ST == 1 ? kLvThreads : 1];
+  const int l = a.l;
+  if (ST == 1 && (int)blockIdx.x >= a.n_tile) {
+    const int s = a.boxes[blockIdx.x - a.n_tile];
+    grid_wait();
+    grid_release();
+    if (a.active && a.active[s] != a.active_value) return;
+    lv_obs(a, s, l, sh);
+    return;
+  }
+  LV_TILE(t);
+  grid_wait();
+  grid_release();
+  if (a.active && a.active[t.s] != a.active_value) return;
+  if (ST == 1 && a.skip1 && t.stg1_off >= 0) return;
+  const size_t lvl = level_size<T>(t);
+  const int pl = t.ny * t.nxp;
+  const T* X = a.traj + t.traj_off + (size_t)l * lvl;
+  const T* Y = ST == 1 ? X : ST == 2 ? x1_of(a, t, l) : x2_of(a, t, l);
+  T* out = ST == 1 ? x1_of(a, t, l) : ST == 2 ? x2_of(a, t, l) : a.traj + t.traj_off + (size_t)(l + 1) * lvl;
+  const size_t G = (size_t)3 * a.nlat * a.nlon;
+  const int n = t.a + l;
+  const T* B0 = a.bnd + (size_t)(ST == 2 ? n + 1 : n) * G;
+  const T* B1 = ST == 3 ? B0 + G : nullptr;
+  const T cx = ST == 1 ? (T)0 : ST == 2 ? (T)0.75 : (T)(1.0 / 3.0);
+  const T cy = ST == 1 ? (T)1 : ST == 2 ? (T)0.25 : (T)(2.0 / 3.0);
+  const bool ovl = TERMS && lv_overlaps(t, l + 1);
+  const size_t slot = (size_t)blockIdx.x * kLvThreads + threadIdx.x;
+  double acc = 0.0;
+  if (ovl) acc = a.acc_m[slot];
+  Sum<T> part;
+  for (int p = t.p0 + threadIdx.x; p < t.p1; p += kLvThreads) {
+    const int r = mdiv(p, t.mq), k = (p - r * t.nq) * V, at = r * t.nxp + k;
+    Patch<T, V> z;
+    load_state_patch<T, V>(a, t, Y, r, k, at, B0, B1, z);
+    T x[3][V];
+    if (ST != 1) {
+#pragma unroll
+      for (int v = 0; v < 3; ++v) ldv<T, V>(X + (at + v * pl), x[v]);
+    }
+    T rc[8];
+    load_rec8(a.fw + 8 * (t.j0 + r), rc);
+    T o[3][V];
+#pragma unroll
+    for (int j = 0; j < V; ++j) {
+      Pt5<T> y;
+      point_of(z, j, y);
+      stage_math<T, DEV>(y, rc, a.dt, a.Bth, a.gBth, a.href, cx, cy, ST != 1 ? x[0][j] : (T)0,
+                         ST != 1 ? x[1][j] : (T)0, ST != 1 ? x[2][j] : (T)0, o[0][j], o[1][j], o[2][j]);
+    }
+#pragma unroll
+    for (int v = 0; v < 3; ++v) stv<T, V>(out + (at + v * pl), o[v]);
+    if (ovl) lv_overlap_part<T, V>(a, t, a.tgt + t.traj_off + (size_t)(l + 1) * lvl, l + 1, r, k, at, o, part);
+  }
+  if (ovl) a.acc_m[slot] = acc + part.value();
+}
+
+// Overlap forcing of point j: mu c (x - m) / sigma^2, or for a Gauss-Newton
+// product (m = dx) mu c dx / sigma^2 (the arithmetic of add_forcing and
+// overlap_force in sweep.cu).
+template <typename T, int V>
+__device__ __forceinline__ void overlap_force_add(const LvArgs<T>& a, int c, int j, const T (*x)[V], const T (*m)[V],
+                                                  T (*o)[V]) {
+  const T cc = (T)c;
+#pragma unroll
+  for (int v = 0; v < 3; ++v) {
+    if (a.gn_dx) o[v][j] = o[v][j] + cc * a.musb2[v] * m[v][j];
+    else o[v][j] = xfma(xmul(cc, a.musb2[v]), xsub(x[v][j], m[v][j]), o[v][j]);
+  }
+}
+
+// The forcing of one thread's V points at level l that comes before the
+// observations: external forcing, the Gauss-Newton overlap term or the overlap
+// term.
+template <typename T, int V>
+__device__ __forceinline__ void lv_force(const LvArgs<T>& a, const LvTile& t, int l, int r, int k, const T (*x)[V],
+                                         T (*o)[V]) {
+  const size_t pl = (size_t)t.ny * t.nxp, lvl = level_size<T>(t);
+  if (a.yforce) {
+    const double* y = a.yforce + t.ptraj_off + (size_t)l * 3 * t.ny * t.nx;
+#pragma unroll
+    for (int j = 0; j < V; ++j)
+      if (k + j < t.nx)
+#pragma unroll
+        for (int v = 0; v < 3; ++v) o[v][j] += (T)y[((size_t)v * t.ny + r) * t.nx + k + j];
+    return;
+  }
+  if (!a.mu_on || !lv_overlaps(t, l)) return;
+  int c[V], any = 0;
+#pragma unroll
+  for (int j = 0; j < V; ++j) {
+    c[j] = k + j < t.nx ? lv_overlap_count(t, l, r, k + j) : 0;
+    any |= c[j];
+  }
+  if (!any) return;
+  const T* q = (a.gn_dx ? a.gn_dx : a.tgt) + t.traj_off + (size_t)l * lvl + (size_t)r * t.nxp + k;
+  T m[3][V];
+#pragma unroll
+  for (int v = 0; v < 3; ++v) ldv<T, V>(q + v * pl, m[v]);
+#pragma unroll
+  for (int j = 0; j < V; ++j) {
+    if (!c[j]) continue;
+    overlap_force_add<T, V>(a, c[j], j, x, m, o);
+  }
+}
+
+// Observation forcing H^T (lambda w d) of level l at the points for which
+// mine(r, k) holds, added to the adjoint state (fixed order per target).
+template <typename T, typename F>
+__device__ __forceinline__ void lv_scatter_if(const LvArgs<T>& a, const LvTile& t, int l, T* lam, F&& mine) {
+  if (a.yforce) return;
+  const int t0 = a.lvl_sc[t.sc_lvl + l], t1 = a.lvl_sc[t.sc_lvl + l + 1];
+  if (t0 == t1) return;
+  __syncthreads();
+  const int pl = t.ny * t.nxp;
+  for (int i = t0 + threadIdx.x; i < t1; i += blockDim.x) {
+    const int g = a.sc_tgt[i];
+    const int vr = mdiv(g, t.mnx);   // v * ny + r
+    const int v = mdiv(vr, t.mny);
+    const int r = vr - v * t.ny, k = g - vr * t.nx;
+    if (!mine(r, k)) continue;
+    double acc = 0.0;
+    for (int c = a.sc_off[i]; c < a.sc_off[i + 1]; ++c) acc += a.sc_w[c] * a.obs_force[a.sc_obs[c]];
+    lam[v * pl + r * t.nxp + k] += (T)acc;
+  }
+}
+template <typename T, int V>
+__device__ __forceinline__ void lv_scatter(const LvArgs<T>& a, const LvTile& t, int l, T* lam) {
+  lv_scatter_if(a, t, l, lam, [&](int r, int k) {
+    const int p = r * t.nq + k / V;
+    return p >= t.p0 && p < t.p1;
+  });
+}
+
+// lambda(b) = forcing(b) of every tile, each box at its own last level.
+template <typename T, int V>
+__global__ void __launch_bounds__(kLvThreads) lv_lam_start_kernel(const LvArgs<T> a) {
+  LV_TILE(t);
+  grid_wait();
+  grid_release();
+  if (a.active && a.active[t.s] != a.active_value) return;
+  const size_t lvl = level_size<T>(t);
+  const int pl = t.ny * t.nxp;
+  const T* X = a.traj + t.traj_off + (size_t)t.L * lvl;
+  T* lam = a.lam + t.lv_off;
+  for (int p = t.p0 + threadIdx.x; p < t.p1; p += kLvThreads) {
+    const int r = mdiv(p, t.mq), k = (p - r * t.nq) * V, at = r * t.nxp + k;
+    T x[3][V], o[3][V];
+#pragma unroll
+    for (int v = 0; v < 3; ++v) {
+      ldv<T, V>(X + v * pl + at, x[v]);
+#pragma unroll
+      for (int j = 0; j < V; ++j) o[v][j] = (T)0;
+    }
+    lv_force<T, V>(a, t, t.L, r, k, x, o);
+#pragma unroll
+    for (int v = 0; v < 3; ++v) stv<T, V>(lam + v * pl + at, o[v]);
+  }
+  lv_scatter<T, V>(a, t, t.L, lam);
+}
+
+// Phase K of the transposed RK3 step l (rescaled stage adjoints as in
+// adj_kernel of sweep.cu):
+//   K = 1: mu2 = lambda' + dt F'(x2)^T lambda'
+//   K = 2: mu1 = mu2 + dt F'(x1)^T mu2
+//   K = 3: lambda(n) = lambda'/3 + mu2/2 + (mu1 + dt F'(x)^T mu1)/6 + forcing(n)
+template <typename T, int V, int K>
+__global__ void __launch_bounds__(kLvThreads, 4) lv_adj_kernel(const LvArgs<T> a) {
+  constexpr bool DEV = sizeof(T) == 4;
+  LV_TILE(t);
+  grid_wait();
+  grid_release();
+  if (a.active && a.active[t.s] != a.active_value) return;
+  const int l = a.l;
+  const size_t lvl = level_size<T>(t);
+  const int pl = t.ny * t.nxp;
+  const T* Z = K == 1 ? x2_of(a, t, l) : K == 2 ? x1_of(a, t, l) : a.traj + t.traj_off + (size_t)l * lvl;
+  const T* M = (K == 1 ? a.lam : K == 2 ? a.mu2 : a.mu1) + t.lv_off;
+  T* out = (K == 1 ? a.mu2 : K == 2 ? a.mu1 : a.lam) + t.lv_off;
+  const size_t G = (size_t)3 * a.nlat * a.nlon;
+  const int n = t.a + l;
+  const T* B0 = a.bnd + (size_t)(K == 2 ? n + 1 : n) * G;
+  const T* B1 = K == 1 ? B0 + G : nullptr;
+  for (int p = t.p0 + threadIdx.x; p < t.p1; p += kLvThreads) {
+    const int r = mdiv(p, t.mq), k = (p - r * t.nq) * V, at = r * t.nxp + k;
+    Patch<T, V> z, m;
+    load_state_patch<T, V>(a, t, Z, r, k, at, B0, B1, z);
+    load_adjoint_patch<T, V>(t, M, r, k, at, m);
+    T rc[8];
+    load_rec8(a.bw + 8 * (t.j0 + r), rc);
+    const int wall = (r == 0 && (t.flags & F_SWALL) ? 1 : 0) | (r == t.ny - 1 && (t.flags & F_NWALL) ? 2 : 0);
+    T o[3][V], ll[3][V], l2[3][V];
+    if (K == 3) {
+#pragma unroll
+      for (int v = 0; v < 3; ++v) {
+        ldv<T, V>(out + (at + v * pl), ll[v]);
+        ldv<T, V>(a.mu2 + t.lv_off + (at + v * pl), l2[v]);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < V; ++j) {
+      Pt5<T> zp, mp;
+      point_of(z, j, zp);
+      point_of(m, j, mp);
+      if (K == 3)
+        adj_lambda_math<T, DEV>(zp, mp, rc, a.dt, a.Bth, a.gBth, a.href, wall, ll[0][j], ll[1][j], ll[2][j],
+                                l2[0][j], l2[1][j], l2[2][j], o[0][j], o[1][j], o[2][j]);
+      else
+        adj_stage_math<T, DEV>(zp, mp, rc, a.dt, a.Bth, a.gBth, a.href, wall, o[0][j], o[1][j], o[2][j]);
+    }
+    if (K == 3) {
+      T x[3][V];
+#pragma unroll
+      for (int v = 0; v < 3; ++v)
+#pragma unroll
+        for (int j = 0; j < V; ++j) x[v][j] = z.c[v][j + 1];
+      lv_force<T, V>(a, t, l, r, k, x, o);
+    }
+#pragma unroll
+    for (int v = 0; v < 3; ++v) stv<T, V>(out + (at + v * pl), o[v]);
+  }
+  if (K == 3) lv_scatter<T, V>(a, t, l, out);
+}
+
+// lambda(a) -> packed control layout (FP64).
+template <typename T, int V>
+__global__ void __launch_bounds__(kLvThreads) lv_export_kernel(const LvArgs<T> a) {
+  LV_TILE(t);
+  grid_wait();
+  grid_release();
+  if (a.active && a.active[t.s] != a.active_value) return;
+  const size_t pl = (size_t)t.ny * t.nxp;
+  const T* lam = a.lam + t.lv_off;
+  double* out = a.lam_a + t.ctrl_off;
+  for (int p = t.p0 + threadIdx.x; p < t.p1; p += kLvThreads) {
+    const int r = mdiv(p, t.mq), k = (p - r * t.nq) * V;
+#pragma unroll
+    for (int v = 0; v < 3; ++v) {
+      T x[V];
+      ldv<T, V>(lam + v * pl + (size_t)r * t.nxp + k, x);
+#pragma unroll
+      for (int j = 0; j < V; ++j)
+        if (k + j < t.nx) out[((size_t)v * t.ny + r) * t.nx + k + j] = (double)x[j];
+    }
+  }
+}
+
+template <typename T>
+cudaError_t lv_launch(void (*kernel)(const LvArgs<T>), const LvArgs<T>& a, int blocks, cudaStream_t st) {
+  if (blocks <= 0) return cudaSuccess;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)blocks, 1, 1);
+  cfg.blockDim = dim3(kLvThreads, 1, 1);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, a);
+}
+
+}  // namespace
+
+#define LV_TRY(call)                    \
+  do {                                  \
+    cudaError_t e_ = (call);            \
+    if (e_ != cudaSuccess) return e_;   \
+    ++*launches;                        \
+  } while (0)
+
+template <typename T>
+cudaError_t launch_level_forward(const LvArgs<T>& base, const LvPlan& g, cudaStream_t st, long long* launches) {
+  constexpr int V = lv_width<T>();
+  LvArgs<T> a = base;
+  const int L = (int)g.n_tile.size();   // longest window
+  if (a.terms) LV_TRY(lv_launch<T>(lv_start_kernel<T, V>, a, g.tiles, st));
+  for (int l = 0; l <= L; ++l) {
+    a.l = l;
+    a.n_tile = l < L ? g.n_tile[l] : 0;
+    const int nob = a.terms && g.obs[l] ? g.n_box[l] : 0;
+    if (a.n_tile + nob) LV_TRY(lv_launch<T>(lv_stage_kernel<T, V, 1, false>, a, a.n_tile + nob, st));
+    if (!a.n_tile) continue;
+    LV_TRY(lv_launch<T>(lv_stage_kernel<T, V, 2, false>, a, a.n_tile, st));
+    if (a.terms) LV_TRY(lv_launch<T>(lv_stage_kernel<T, V, 3, true>, a, a.n_tile, st));
+    else LV_TRY(lv_launch<T>(lv_stage_kernel<T, V, 3, false>, a, a.n_tile, st));
+  }
+  return cudaSuccess;
+}
+
+template <typename T>
+cudaError_t launch_level_adjoint(const LvArgs<T>& base, const LvPlan& g, cudaStream_t st, long long* launches) {
+  constexpr int V = lv_width<T>();
+  LvArgs<T> a = base;
+  LV_TRY(lv_launch<T>(lv_lam_start_kernel<T, V>, a, g.tiles, st));
+  for (int l = (int)g.n_tile.size() - 1; l >= 0; --l) {
+    a.l = l;
+    a.n_tile = g.n_tile[l];
+    if (!a.stg) {   // the stage states were not stored: recompute them
+      a.skip1 = a.stg1 != nullptr;
+      LV_TRY(lv_launch<T>(lv_stage_kernel<T, V, 1, false>, a, a.n_tile, st));
+      LV_TRY(lv_launch<T>(lv_stage_kernel<T, V, 2, false>, a, a.n_tile, st));
+    }
+    LV_TRY(lv_launch<T>(lv_adj_kernel<T, V, 1>, a, a.n_tile, st));
+    LV_TRY(lv_launch<T>(lv_adj_kernel<T, V, 2>, a, a.n_tile, st));
+    LV_TRY(lv_launch<T>(lv_adj_kernel<T, V, 3>, a, a.n_tile, st));
+  }
+  LV_TRY(lv_launch<T>(lv_export_kernel<T, V>, a, g.tiles, st));
+  return cudaSuccess;
+}
+
+#define DD4DV_INST(T)                                                                                         \
+  template cudaError_t launch_level_forward<T>(const LvArgs<T>&, const LvPlan&, cudaStream_t, long long*);   \
+  template cudaError_t launch_level_adjoint<T>(const LvArgs<T>&, const LvPlan&, cudaStream_t, long long*);
+DD4DV_INST(double)
+DD4DV_INST(float)
+#undef DD4DV_INST
+
+}  // namespace dd4dv

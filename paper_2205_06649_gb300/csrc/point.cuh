@@ -1,5 +1,6 @@
 // Per-point arithmetic of the shallow-water step, its adjoint and its
-// linearisation, shared by every sweep kernel, so that all of them round alike.
+// linearisation, shared by every sweep (the shared-memory sweeps of sweep.cu and
+// the level sweeps of level.cu), so that all of them round alike.
 #pragma once
 
 #include "common.cuh"
