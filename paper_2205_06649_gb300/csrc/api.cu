@@ -42,6 +42,8 @@ struct dd4dv_ctx {
   // grid
   std::vector<RowConst> rows_h;
   RowConst* rows_d = nullptr;
+  double* grec = nullptr;     // FP64 forward records of every row (global model)
+  GlobalStepPlan gplan;
   double Bth = 0, gBth = 0;
   size_t gstate = 0;          // 3*nlat*nlon
   size_t gtraj = 0;           // (nsteps+1)*gstate
@@ -58,6 +60,13 @@ struct dd4dv_ctx {
   double rf_alpha = 0, rf_c = 1;
   double* sigma_d = nullptr;
 
+  // Turkel-Zwas calls: workspace kept between calls up to kTzKeep bytes, and the
+  // observations sorted by level on the device (made at the first dd4dv_tz_eval
+  // after dd4dv_set_observations)
+  void* tz_ws = nullptr;
+  size_t tz_ws_bytes = 0;
+  double* tz_obs = nullptr;
+  std::vector<long long> tz_off;
   std::vector<int> ob_level, ob_var;
   std::vector<double> ob_fi, ob_fj, ob_val, ob_so;
 
@@ -600,12 +609,8 @@ void reset_exchange_T(dd4dv_ctx* ctx) {
 void global_step(dd4dv_ctx* ctx, const double* x, double* nx) {
   double* s1 = ctx->gscratch;
   double* s2 = ctx->gscratch + ctx->gstate;
-  KL(launch_global_stage(x, x, s1, 0.0, 1.0, ctx->rows_d, ctx->Bth, ctx->gBth, ctx->m.dt, ctx->m.nlon,
-                         ctx->m.nlat, ctx->st));
-  KL(launch_global_stage(x, s1, s2, 0.75, 0.25, ctx->rows_d, ctx->Bth, ctx->gBth, ctx->m.dt,
-                         ctx->m.nlon, ctx->m.nlat, ctx->st));
-  KL(launch_global_stage(x, s2, nx, 1.0 / 3.0, 2.0 / 3.0, ctx->rows_d, ctx->Bth, ctx->gBth, ctx->m.dt,
-                         ctx->m.nlon, ctx->m.nlat, ctx->st));
+  CK(launch_global_step(ctx->gplan, x, s1, s2, nx, ctx->grec, ctx->m.dt * ctx->Bth, ctx->m.dt * ctx->gBth, ctx->m.nlon,
+                        ctx->m.nlat, ctx->st, &ctx->launches));
 }
 
 // Global model run x0 (device) -> out trajectory (device, FP64).
@@ -1491,6 +1496,9 @@ void build_decomposition(dd4dv_ctx* ctx, const dd4dv_decomp& d) {
 dd4dv_ctx::~dd4dv_ctx() {
   free_dec();
   cudaFree(rows_d);
+  cudaFree(grec);
+  cudaFree(tz_ws);
+  cudaFree(tz_obs);
   cudaFree(xb0);
   cudaFree(gscratch);
   cudaFree(gchunk);
@@ -1582,6 +1590,12 @@ dd4dv_status dd4dv_create(const dd4dv_model* model, void* cuda_stream, dd4dv_ctx
     ctx->gstate = 3ULL * m.nlat * m.nlon;
     ctx->gtraj = (size_t)(m.nsteps + 1) * ctx->gstate;
     ctx->rows_d = dalloc<RowConst>(ctx, m.nlat);
+    ctx->gplan = global_step_plan(m.nlon, m.nlat);
+    ctx->grec = dalloc<double>(ctx, 8 * (size_t)m.nlat);
+    std::vector<double> rec(8 * (size_t)m.nlat), back(8);
+    for (int j = 0; j < m.nlat; ++j)
+      fill_records(ctx->rows_h[j], ctx->rows_h[std::min(j + 1, m.nlat - 1)].c, ctx->rows_h[std::max(j - 1, 0)].c, m.dt,
+                   ctx->Bth, &rec[8 * (size_t)j], back.data());
     ctx->xb0 = dalloc<double>(ctx, ctx->gstate);
     ctx->gscratch = dalloc<double>(ctx, 3 * ctx->gstate);
     // chunk of global levels: at most 512 MB, at least 2 levels, at most the whole trajectory
@@ -1601,6 +1615,7 @@ dd4dv_status dd4dv_create(const dd4dv_model* model, void* cuda_stream, dd4dv_ctx
       fail(ctx, DD4DV_ENOMEM, "pinned host allocation failed");
     CK(cudaMemcpyAsync(ctx->rows_d, ctx->rows_h.data(), m.nlat * sizeof(RowConst),
                        cudaMemcpyHostToDevice, ctx->st));
+    CK(cudaMemcpyAsync(ctx->grec, rec.data(), rec.size() * sizeof(double), cudaMemcpyHostToDevice, ctx->st));
     CK(cudaMemsetAsync(ctx->err_d, 0, sizeof(int), ctx->st));
     CK(cudaStreamSynchronize(ctx->st));
     *out = ctx;
@@ -1676,6 +1691,9 @@ dd4dv_status dd4dv_set_observations(dd4dv_ctx* ctx, long long n, const int* leve
       if (!(sigma_o[k] > 0.0)) fail(ctx, DD4DV_EINVAL, "obs %lld: sigma_o must be > 0", k);
     }
     ctx->free_dec();
+    cudaFree(ctx->tz_obs);
+    ctx->tz_obs = nullptr;
+    ctx->tz_off.clear();
     ctx->ob_level.assign(level, level + n);
     ctx->ob_var.assign(var, var + n);
     ctx->ob_fi.assign(fi, fi + n);
@@ -2104,24 +2122,59 @@ TzArgs tz_args(dd4dv_ctx* ctx, int p, int q, double alpha) {
   t.slat = ctx->Bth;
   t.g = m.gravity;
   t.dt = m.dt;
+  t.rec = nullptr;
+  t.st = m.dt * t.slat;
+  t.gq = m.dt * t.slat * m.gravity / q;
   return t;
 }
 
-// Device scratch that lives for one call.
+// Device scratch of one call, cut from one block.  The context keeps a block of
+// up to kTzKeep bytes for its next call (an allocation and its release cost
+// more than a small run); a larger one lives for the call.
+constexpr size_t kTzKeep = 1ull << 30;
 struct TzBufs {
-  std::vector<void*> ptrs;
   dd4dv_ctx* ctx;
-  explicit TzBufs(dd4dv_ctx* c) : ctx(c) {}
+  unsigned char* base = nullptr;
+  size_t used = 0, bytes = 0;
+  bool kept = false;
+  TzBufs(dd4dv_ctx* c, size_t doubles) : ctx(c) {
+    bytes = doubles * sizeof(double) + 64 * 256;   // every piece starts on 256 bytes
+    kept = bytes <= kTzKeep;
+    if (kept && ctx->tz_ws_bytes >= bytes) {
+      base = static_cast<unsigned char*>(ctx->tz_ws);
+      return;
+    }
+    if (kept) {   // grow the kept block
+      cudaStreamSynchronize(ctx->st);
+      cudaFree(ctx->tz_ws);
+      ctx->tz_ws = nullptr;
+      ctx->tz_ws_bytes = 0;
+    }
+    base = dalloc<unsigned char>(ctx, bytes);
+    if (kept) {
+      ctx->tz_ws = base;
+      ctx->tz_ws_bytes = bytes;
+    }
+  }
   double* get(size_t n) {
-    double* p = dalloc<double>(ctx, n);
-    ptrs.push_back(p);
+    double* p = reinterpret_cast<double*>(base + used);
+    used += (n * sizeof(double) + 255) / 256 * 256;
+    if (used > bytes) fail(ctx, DD4DV_EINVAL, "internal error: Turkel-Zwas scratch");
     return p;
   }
   ~TzBufs() {
+    if (kept) return;
     if (ctx->st) cudaStreamSynchronize(ctx->st);
-    for (void* p : ptrs) cudaFree(p);
+    cudaFree(base);
   }
 };
+
+// The row records of the call's parameters.
+void tz_rows(dd4dv_ctx* ctx, TzArgs& t, TzBufs& b) {
+  TzRow* rec = reinterpret_cast<TzRow*>(b.get(8 * (size_t)ctx->m.nlat));
+  KL(launch_tz_rows(t, rec, ctx->st));
+  t.rec = rec;
+}
 
 void tz_step(dd4dv_ctx* ctx, const TzArgs& t, const double* x, double* s1, double* s2, double* nx) {
   KL(launch_tz_stage(t, x, x, s1, 0.0, 1.0, ctx->st));
@@ -2139,18 +2192,45 @@ void tz_run(dd4dv_ctx* ctx, const TzArgs& t, const double* x0, double* traj, dou
 // then mu2 = lam + dt F'(x2)^T lam, mu1 = mu2 + dt F'(x1)^T mu2,
 // lam(n) = lam/3 + mu2/2 + (mu1 + dt F'(x)^T mu1)/6 (the transposed SSP-RK3
 // step, as in the box sweeps).
+// force (may be null) is added to lam(n).
 void tz_adjoint_step(dd4dv_ctx* ctx, const TzArgs& t, const double* x, double* s1, double* s2, double* lam,
-                     double* mu2, double* mu1, double* g3) {
-  const size_t G = ctx->gstate;
+                     double* mu2, double* mu1, const double* force) {
   KL(launch_tz_stage(t, x, x, s1, 0.0, 1.0, ctx->st));
   KL(launch_tz_stage(t, x, s1, s2, 0.75, 0.25, ctx->st));
-  CK(cudaMemcpyAsync(mu2, lam, G * sizeof(double), cudaMemcpyDeviceToDevice, ctx->st));
-  KL(launch_tz_adj_scatter(t, s2, lam, mu2, t.dt, ctx->st));
-  CK(cudaMemcpyAsync(mu1, mu2, G * sizeof(double), cudaMemcpyDeviceToDevice, ctx->st));
-  KL(launch_tz_adj_scatter(t, s1, mu2, mu1, t.dt, ctx->st));
-  CK(cudaMemcpyAsync(g3, mu1, G * sizeof(double), cudaMemcpyDeviceToDevice, ctx->st));
-  KL(launch_tz_adj_scatter(t, x, mu1, g3, t.dt, ctx->st));
-  KL(launch_tz_lincomb(lam, lam, mu2, g3, 1.0 / 3.0, 0.5, 1.0 / 6.0, (long long)G, ctx->st));
+  KL(launch_tz_adj_stage(t, s2, lam, nullptr, nullptr, nullptr, mu2, ctx->st));
+  KL(launch_tz_adj_stage(t, s1, mu2, nullptr, nullptr, nullptr, mu1, ctx->st));
+  KL(launch_tz_adj_stage(t, x, mu1, lam, mu2, force, lam, ctx->st));
+}
+
+// The context's observations on the device, sorted by level (stable), with the
+// offsets of each level.
+void tz_observations(dd4dv_ctx* ctx) {
+  const size_t nob = ctx->has_obs ? ctx->ob_level.size() : 0;
+  const int N = ctx->m.nsteps;
+  if (!ctx->tz_off.empty()) return;
+  std::vector<size_t> ord(nob);
+  for (size_t k = 0; k < nob; ++k) ord[k] = k;
+  std::stable_sort(ord.begin(), ord.end(), [&](size_t a, size_t c) { return ctx->ob_level[a] < ctx->ob_level[c]; });
+  std::vector<double> d(4 * nob + nob);
+  int* iv = reinterpret_cast<int*>(d.data() + 4 * nob);
+  std::vector<long long> off(N + 2, 0);
+  for (size_t k = 0; k < nob; ++k) {
+    const size_t o = ord[k];
+    d[k] = ctx->ob_fi[o];
+    d[nob + k] = ctx->ob_fj[o];
+    d[2 * nob + k] = ctx->ob_val[o];
+    d[3 * nob + k] = ctx->ob_so[o];
+    iv[k] = ctx->ob_level[o];
+    iv[nob + k] = ctx->ob_var[o];
+    off[iv[k] + 1] += 1;
+  }
+  for (int n = 0; n <= N; ++n) off[n + 1] += off[n];
+  if (nob) {
+    ctx->tz_obs = dalloc<double>(ctx, d.size());
+    h2d(ctx, ctx->tz_obs, d.data(), d.size() * sizeof(double));
+    CK(cudaStreamSynchronize(ctx->st));   // the host table ends with this call
+  }
+  ctx->tz_off = std::move(off);
 }
 
 const double* tz_in(dd4dv_ctx* ctx, TzBufs& b, const double* src, size_t n, int device_ptrs) {
@@ -2167,10 +2247,11 @@ extern "C" {
 dd4dv_status dd4dv_tz_forward(dd4dv_ctx* ctx, int p, int q, double alpha, const double* x0, double* traj,
                               int device_ptrs) {
   return guard(ctx, [&] {
-    const TzArgs t = tz_args(ctx, p, q, alpha);
+    TzArgs t = tz_args(ctx, p, q, alpha);
     if (!x0 || !traj) fail(ctx, DD4DV_EINVAL, "NULL argument");
     const size_t G = ctx->gstate, T = (size_t)(ctx->m.nsteps + 1) * G;
-    TzBufs b(ctx);
+    TzBufs b(ctx, 8 * (size_t)ctx->m.nlat + 3 * G + (device_ptrs ? 0 : T));
+    tz_rows(ctx, t, b);
     const double* x = tz_in(ctx, b, x0, G, device_ptrs);
     double* out = device_ptrs ? traj : b.get(T);
     double* s = b.get(2 * G);
@@ -2184,10 +2265,11 @@ dd4dv_status dd4dv_tz_forward(dd4dv_ctx* ctx, int p, int q, double alpha, const 
 dd4dv_status dd4dv_tz_tlm(dd4dv_ctx* ctx, int p, int q, double alpha, const double* x0, const double* dx0,
                           double* dtraj, int device_ptrs) {
   return guard(ctx, [&] {
-    const TzArgs t = tz_args(ctx, p, q, alpha);
+    TzArgs t = tz_args(ctx, p, q, alpha);
     if (!x0 || !dx0 || !dtraj) fail(ctx, DD4DV_EINVAL, "NULL argument");
     const size_t G = ctx->gstate, T = (size_t)(ctx->m.nsteps + 1) * G;
-    TzBufs b(ctx);
+    TzBufs b(ctx, 8 * (size_t)ctx->m.nlat + 8 * G + (device_ptrs ? 0 : T));
+    tz_rows(ctx, t, b);
     const double* xin = tz_in(ctx, b, x0, G, device_ptrs);
     const double* dxin = tz_in(ctx, b, dx0, G, device_ptrs);
     double* dout = device_ptrs ? dtraj : b.get(T);
@@ -2215,22 +2297,21 @@ dd4dv_status dd4dv_tz_tlm(dd4dv_ctx* ctx, int p, int q, double alpha, const doub
 dd4dv_status dd4dv_tz_adjoint(dd4dv_ctx* ctx, int p, int q, double alpha, const double* x0, const double* ytraj,
                               double* dx0, int device_ptrs) {
   return guard(ctx, [&] {
-    const TzArgs t = tz_args(ctx, p, q, alpha);
+    TzArgs t = tz_args(ctx, p, q, alpha);
     if (!x0 || !ytraj || !dx0) fail(ctx, DD4DV_EINVAL, "NULL argument");
     const size_t G = ctx->gstate, T = (size_t)(ctx->m.nsteps + 1) * G;
     const int N = ctx->m.nsteps;
-    TzBufs b(ctx);
+    TzBufs b(ctx, 8 * (size_t)ctx->m.nlat + 6 * G + (device_ptrs ? 1 : 2) * T);
+    tz_rows(ctx, t, b);
     const double* xin = tz_in(ctx, b, x0, G, device_ptrs);
     const double* y = tz_in(ctx, b, ytraj, T, device_ptrs);
     double* traj = b.get(T);
-    double* w = b.get(6 * G);
-    double *s1 = w, *s2 = w + G, *lam = w + 2 * G, *mu2 = w + 3 * G, *mu1 = w + 4 * G, *g3 = w + 5 * G;
+    double* w = b.get(5 * G);
+    double *s1 = w, *s2 = w + G, *lam = w + 2 * G, *mu2 = w + 3 * G, *mu1 = w + 4 * G;
     tz_run(ctx, t, xin, traj, s1, s2);
     CK(cudaMemcpyAsync(lam, y + (size_t)N * G, G * sizeof(double), cudaMemcpyDeviceToDevice, ctx->st));
-    for (int n = N - 1; n >= 0; --n) {
-      tz_adjoint_step(ctx, t, traj + (size_t)n * G, s1, s2, lam, mu2, mu1, g3);
-      KL(launch_tz_lincomb(lam, lam, y + (size_t)n * G, nullptr, 1.0, 1.0, 0.0, (long long)G, ctx->st));
-    }
+    for (int n = N - 1; n >= 0; --n)
+      tz_adjoint_step(ctx, t, traj + (size_t)n * G, s1, s2, lam, mu2, mu1, y + (size_t)n * G);
     if (device_ptrs) CK(cudaMemcpyAsync(dx0, lam, G * sizeof(double), cudaMemcpyDeviceToDevice, ctx->st));
     else d2h(ctx, dx0, lam, G * sizeof(double));
     sync(ctx);
@@ -2241,67 +2322,41 @@ dd4dv_status dd4dv_tz_adjoint(dd4dv_ctx* ctx, int p, int q, double alpha, const 
 dd4dv_status dd4dv_tz_eval(dd4dv_ctx* ctx, int p, int q, double alpha, const double* w_in, double* J_out,
                            double* grad_out, int device_ptrs) {
   return guard(ctx, [&] {
-    const TzArgs t = tz_args(ctx, p, q, alpha);
+    TzArgs t = tz_args(ctx, p, q, alpha);
     if (!w_in || !J_out) fail(ctx, DD4DV_EINVAL, "NULL argument");
     if (!ctx->has_bg || !ctx->has_berr) fail(ctx, DD4DV_ESTATE, "set_background and set_background_error first");
     if (ctx->corr_len > 0.0) fail(ctx, DD4DV_EINVAL, "dd4dv_tz_eval takes a diagonal B (corr_len_cells = 0)");
     const size_t G = ctx->gstate, T = (size_t)(ctx->m.nsteps + 1) * G;
     const int N = ctx->m.nsteps;
     const long long plane = (long long)ctx->m.nlat * ctx->m.nlon;
-    TzBufs b(ctx);
+    const size_t nob = ctx->has_obs ? ctx->ob_level.size() : 0;
+    TzBufs b(ctx, 8 * (size_t)ctx->m.nlat + 7 * G + T + nob + 2 * kTzBlocks + 1);
+    tz_rows(ctx, t, b);
     const double* w = tz_in(ctx, b, w_in, G, device_ptrs);
     double* traj = b.get(T);
-    double* work = b.get(7 * G + 2);
+    double* work = b.get(6 * G);
     double *s1 = work, *s2 = work + G, *lam = work + 2 * G, *mu2 = work + 3 * G, *mu1 = work + 4 * G,
-           *g3 = work + 5 * G, *x0 = work + 6 * G, *Jd = work + 7 * G, *Jo = work + 7 * G + 1;
+           *x0 = work + 5 * G;
+    double* part = b.get(2 * kTzBlocks + 1);
+    double* Jd = part + 2 * kTzBlocks;
+    double* force = b.get(nob);
+    tz_observations(ctx);
+    const double* od = ctx->tz_obs;   // fi, fj, y, sigma_o, then level and var as ints
+    const int* lvd = reinterpret_cast<const int*>(od + 4 * nob);
+    const int* vrd = lvd + nob;
+    const double *fid = od, *fjd = od + nob;
+    const auto& off = ctx->tz_off;
     KL(launch_tz_scale_add(x0, ctx->xb0, w, ctx->sigma_d, plane, ctx->st));
     tz_run(ctx, t, x0, traj, s1, s2);
-    // observations sorted by level, with the offsets of each level
-    const size_t nob = ctx->has_obs ? ctx->ob_level.size() : 0;
-    std::vector<size_t> ord(nob);
-    for (size_t k = 0; k < nob; ++k) ord[k] = k;
-    std::stable_sort(ord.begin(), ord.end(), [&](size_t a, size_t c) { return ctx->ob_level[a] < ctx->ob_level[c]; });
-    std::vector<int> lv(nob), vr(nob);
-    std::vector<double> fi(nob), fj(nob), yv(nob), so(nob);
-    std::vector<long long> off(N + 2, 0);
-    for (size_t k = 0; k < nob; ++k) {
-      const size_t o = ord[k];
-      lv[k] = ctx->ob_level[o];
-      vr[k] = ctx->ob_var[o];
-      fi[k] = ctx->ob_fi[o];
-      fj[k] = ctx->ob_fj[o];
-      yv[k] = ctx->ob_val[o];
-      so[k] = ctx->ob_so[o];
-      off[lv[k] + 1] += 1;
-    }
-    for (int n = 0; n <= N; ++n) off[n + 1] += off[n];
-    const double* force = nullptr;
-    const int* lvd = nullptr;
-    const int* vrd = nullptr;
-    const double *fid = nullptr, *fjd = nullptr;
-    if (nob) {
-      double* dbl = b.get(5 * nob);
-      int* ints = reinterpret_cast<int*>(b.get(nob));   // 2 * nob ints
-      h2d(ctx, ints, lv.data(), nob * sizeof(int));
-      h2d(ctx, ints + nob, vr.data(), nob * sizeof(int));
-      h2d(ctx, dbl, fi.data(), nob * sizeof(double));
-      h2d(ctx, dbl + nob, fj.data(), nob * sizeof(double));
-      h2d(ctx, dbl + 2 * nob, yv.data(), nob * sizeof(double));
-      h2d(ctx, dbl + 3 * nob, so.data(), nob * sizeof(double));
-      lvd = ints;
-      vrd = ints + nob;
-      fid = dbl;
-      fjd = dbl + nob;
-      force = dbl + 4 * nob;
-      KL(launch_tz_obs_misfit(traj, (long long)nob, lvd, vrd, fid, fjd, dbl + 2 * nob, dbl + 3 * nob, ctx->m.nlon,
-                              ctx->m.nlat, 1.0, dbl + 4 * nob, Jo, ctx->st));
-    }
-    KL(launch_tz_finish_J(w, (long long)G, nob ? Jo : nullptr, Jd, ctx->st));
+    if (nob)
+      KL(launch_tz_obs_misfit(traj, (long long)nob, lvd, vrd, fid, fjd, od + 2 * nob, od + 3 * nob, ctx->m.nlon,
+                              ctx->m.nlat, 1.0, force, part, ctx->st));
+    KL(launch_tz_finish_J(w, (long long)G, nob > 0, part, Jd, ctx->st));
     if (grad_out) {
       CK(cudaMemsetAsync(lam, 0, G * sizeof(double), ctx->st));
       if (nob) KL(launch_tz_obs_scatter(off[N], off[N + 1], vrd, fid, fjd, force, ctx->m.nlon, ctx->m.nlat, lam, ctx->st));
       for (int n = N - 1; n >= 0; --n) {
-        tz_adjoint_step(ctx, t, traj + (size_t)n * G, s1, s2, lam, mu2, mu1, g3);
+        tz_adjoint_step(ctx, t, traj + (size_t)n * G, s1, s2, lam, mu2, mu1, nullptr);
         if (nob) KL(launch_tz_obs_scatter(off[n], off[n + 1], vrd, fid, fjd, force, ctx->m.nlon, ctx->m.nlat, lam,
                                           ctx->st));
       }

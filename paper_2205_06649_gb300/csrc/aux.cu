@@ -3,7 +3,7 @@
 // Eq. eq:cost:parallel1), the overlap exchange (Algorithm 1 "Exchange", Eq.
 // rest), the global model (Sec. 7), the observation operator H, and the
 // batched local L-BFGS (Algorithm 2/3 with L-BFGS, Remark after Alg. 5).
-#include "common.cuh"
+#include "point.cuh"
 
 #include <cfloat>
 #include <mutex>
@@ -350,45 +350,146 @@ __global__ void bnd_to_global_kernel(const T* bnd, long long n, double h_ref, lo
 
 // ---------------------------------------------------------------------------
 // Global model stage on the whole sphere: out = ca x + cb (y + dt F(y)).
-__global__ void global_stage_kernel(const double* x, const double* y, double* out, double ca,
-                                    double cb, const RowConst* rows, double Bth, double gBth,
-                                    double dt, int nlon, int nlat) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y;
-  if (i >= nlon) return;
+// Bound: the FP64 pipe, 24 instructions a point and stage (30 with x), as the
+// box sweeps (euler_pt64).  One thread per point, flat over rows so that every
+// lane has one; set-up overlaps the stage before (programmatic dependent
+// launch).  Small grids take global_step_kernel instead.
+constexpr int kGlobalThreads = 128;
+__global__ void __launch_bounds__(kGlobalThreads) global_stage_kernel(const double* x, const double* y, double* out,
+                                                                      double ca, double cb, const double* rec,
+                                                                      double dtB, double dtgB, int nlon, int nlat) {
+  const unsigned idx = blockIdx.x * kGlobalThreads + threadIdx.x;
+  const unsigned P = (unsigned)nlat * nlon;
+  const int j = (int)(idx / (unsigned)nlon), i = (int)(idx - (unsigned)j * nlon);
+  grid_wait();
+  grid_release();
+  if (idx >= P) return;
+  const size_t o = idx;
+  const size_t oE = i + 1 < nlon ? o + 1 : o + 1 - nlon, oW = i > 0 ? o - 1 : o + nlon - 1;
+  const bool top = j + 1 == nlat, bot = j == 0;
+  const size_t oN = top ? o : o + nlon, oS = bot ? o : o - nlon;
+  Pt5<double> z;
+  const double *H = y, *U = y + P, *V = y + 2 * (size_t)P;
+  z.h = H[o]; z.u = U[o]; z.v = V[o];
+  z.hE = H[oE]; z.uE = U[oE]; z.vE = V[oE];
+  z.hW = H[oW]; z.uW = U[oW]; z.vW = V[oW];
+  z.hN = H[oN]; z.uN = U[oN]; z.vN = top ? -z.v : V[oN];
+  z.hS = H[oS]; z.uS = U[oS]; z.vS = bot ? -z.v : V[oS];
+  double rc[8];
+  load_rec8(rec + 8 * j, rc);
+  double x0 = 0.0, x1 = 0.0, x2 = 0.0;
+  if (ca != 0.0) {
+    x0 = x[o];
+    x1 = x[o + P];
+    x2 = x[o + 2 * (size_t)P];
+  }
+  double o0, o1, o2;
+  stage_math<double, false>(z, rc, 0.0, dtB, dtgB, 0.0, ca, cb, x0, x1, x2, o0, o1, o2);
+  out[o] = o0;
+  out[o + P] = o1;
+  out[o + 2 * (size_t)P] = o2;
+}
+
+// A whole RK3 step of the global model per launch, for grids whose stages are
+// short: a stage of 512 x 256 points keeps the FP64 pipe busy for 6.3 us of its
+// 12.5, the rest is launch, load latency and drain.  A CTA owns a tile of
+// tx x ty points, loads it with three halo points a side, and forms the first
+// stage on the tile and two halo points, the second on one, all in shared
+// memory; rows beyond a wall are the mirror (h, u, -v) of the wall row at every
+// stage.  The recomputed halos cost 15-25 % more FP64 work.  Same values as the
+// stage kernel bit for bit.  Per step, one launch per stage of the kernel with
+// the old arithmetic -> this one: 32 x 16 points 14.9 -> 5.6 us, 128 x 64 16.9 ->
+// 5.7, 256 x 128 18.6 -> 11.5, 512 x 256 39.0 -> 30.0 (stage kernel above: 40).
+constexpr int kStepThreads = 384;
+struct StepTile {
+  int tx, ty;
+};
+__host__ __device__ inline size_t step_smem(int tx, int ty) {
+  return 3 * sizeof(double) * ((size_t)(tx + 6) * (ty + 6) + (size_t)(tx + 4) * (ty + 4) + (size_t)(tx + 2) * (ty + 2));
+}
+extern __shared__ __align__(16) double step_sm[];
+
+__global__ void __launch_bounds__(kStepThreads) global_step_kernel(const double* x, double* nx, const double* rec,
+                                                                   double dtB, double dtgB, int nlon, int nlat,
+                                                                   StepTile tile) {
+  const int tx = tile.tx, ty = tile.ty;
+  const int i0 = blockIdx.x * tx, j0 = blockIdx.y * ty;
+  const int cx = min(tx, nlon - i0), cy = min(ty, nlat - j0);   // own points
   const size_t P = (size_t)nlat * nlon;
-  const double* H = y;
-  const double* U = y + P;
-  const double* V = y + 2 * P;
-  const int iE = (i + 1) % nlon, iW = (i - 1 + nlon) % nlon;
-  const size_t o = (size_t)j * nlon + i;
-  const RowConst rc = rows[j];
-  const double h = H[o], u = U[o], v = V[o];
-  const double hE = H[(size_t)j * nlon + iE], hW = H[(size_t)j * nlon + iW];
-  const double uE = U[(size_t)j * nlon + iE], uW = U[(size_t)j * nlon + iW];
-  const double vE = V[(size_t)j * nlon + iE], vW = V[(size_t)j * nlon + iW];
-  double hN, uN, vN, cN, hS, uS, vS, cS;
-  if (j + 1 < nlat) {
-    const size_t q = (size_t)(j + 1) * nlon + i;
-    hN = H[q]; uN = U[q]; vN = V[q]; cN = rows[j + 1].c;
-  } else {
-    hN = h; uN = u; vN = -v; cN = rc.c;
-  }
-  if (j > 0) {
-    const size_t q = (size_t)(j - 1) * nlon + i;
-    hS = H[q]; uS = U[q]; vS = V[q]; cS = rows[j - 1].c;
-  } else {
-    hS = h; uS = u; vS = -v; cS = rc.c;
-  }
-  const double fu = rc.f + rc.tau * u;
-  const double Fu = -rc.A * u * (uE - uW) - Bth * v * (uN - uS) + fu * v - rc.gA * (hE - hW);
-  const double Fv = -rc.A * u * (vE - vW) - Bth * v * (vN - vS) - fu * u - gBth * (hN - hS);
-  const double Fh = -rc.A * (hE * uE - hW * uW) - rc.BinvC * (hN * vN * cN - hS * vS * cS);
-  const double F[3] = {Fh, Fu, Fv};
-  for (int c = 0; c < 3; ++c) {
-    const size_t q = (size_t)c * P + o;
-    out[q] = (ca == 0.0 ? 0.0 : ca * x[q]) + cb * (y[q] + dt * F[c]);
-  }
+  // planes of the tile with 3, 2 and 1 halo points; row pitch tx + 2 halo
+  double* X = step_sm;
+  double* A = X + 3 * (tx + 6) * (ty + 6);
+  double* B = A + 3 * (tx + 4) * (ty + 4);
+  grid_wait();
+  grid_release();
+  // f(r, c, v) for the points of the tile grown by h, rows inside the grid
+  auto points = [&](int h, auto&& f) {
+    const int w = cx + 2 * h, n = w * (cy + 2 * h);
+    for (int p = threadIdx.x; p < n; p += kStepThreads) {
+      const int q = p / w, r = q - h, c = p - q * w - h;
+      if (j0 + r >= 0 && j0 + r < nlat) f(r, c);
+    }
+  };
+  // writes a point of a plane set with halo h, and the mirror rows of the walls
+  auto put = [&](double* Z, int h, int r, int c, double a, double b, double d) {
+    const int w = tx + 2 * h, pl = w * (ty + 2 * h), o = (r + h) * w + c + h;
+    Z[o] = a;
+    Z[o + pl] = b;
+    Z[o + 2 * pl] = d;
+    if (j0 + r == 0 && r > -h) {
+      Z[o - w] = a;
+      Z[o - w + pl] = b;
+      Z[o - w + 2 * pl] = -d;
+    }
+    if (j0 + r == nlat - 1 && r + 1 < cy + h) {
+      Z[o + w] = a;
+      Z[o + w + pl] = b;
+      Z[o + w + 2 * pl] = -d;
+    }
+  };
+  // one stage at point (r, c) from plane set Y with halo h
+  auto stage = [&](const double* Y, int h, int r, int c, double ca, double cb, double& a, double& b, double& d) {
+    const int w = tx + 2 * h, pl = w * (ty + 2 * h), o = (r + h) * w + c + h;
+    Pt5<double> z;
+    z.h = Y[o]; z.u = Y[o + pl]; z.v = Y[o + 2 * pl];
+    z.hE = Y[o + 1]; z.uE = Y[o + 1 + pl]; z.vE = Y[o + 1 + 2 * pl];
+    z.hW = Y[o - 1]; z.uW = Y[o - 1 + pl]; z.vW = Y[o - 1 + 2 * pl];
+    z.hN = Y[o + w]; z.uN = Y[o + w + pl]; z.vN = Y[o + w + 2 * pl];
+    z.hS = Y[o - w]; z.uS = Y[o - w + pl]; z.vS = Y[o - w + 2 * pl];
+    const int xw = tx + 6, xp = xw * (ty + 6), xo = (r + 3) * xw + c + 3;
+    double rc[8];
+    load_rec8(rec + 8 * (j0 + r), rc);
+    const bool x3 = ca != 0.0;
+    stage_math<double, false>(z, rc, 0.0, dtB, dtgB, 0.0, ca, cb, x3 ? X[xo] : 0.0, x3 ? X[xo + xp] : 0.0,
+                              x3 ? X[xo + 2 * xp] : 0.0, a, b, d);
+  };
+  points(3, [&](int r, int c) {
+    int i = (i0 + c) % nlon;
+    if (i < 0) i += nlon;
+    const double* q = x + (size_t)(j0 + r) * nlon + i;
+    put(X, 3, r, c, q[0], q[P], q[2 * P]);
+  });
+  __syncthreads();
+  points(2, [&](int r, int c) {
+    double a, b, d;
+    stage(X, 3, r, c, 0.0, 1.0, a, b, d);
+    put(A, 2, r, c, a, b, d);
+  });
+  __syncthreads();
+  points(1, [&](int r, int c) {
+    double a, b, d;
+    stage(A, 2, r, c, 0.75, 0.25, a, b, d);
+    put(B, 1, r, c, a, b, d);
+  });
+  __syncthreads();
+  points(0, [&](int r, int c) {
+    double a, b, d;
+    stage(B, 1, r, c, 1.0 / 3.0, 2.0 / 3.0, a, b, d);
+    double* q = nx + (size_t)(j0 + r) * nlon + i0 + c;
+    q[0] = a;
+    q[P] = b;
+    q[2 * P] = d;
+  });
 }
 
 // H: bilinear interpolation in index space (lon periodic), corners in the
@@ -882,12 +983,58 @@ cudaError_t launch_restrict_level(const SubDesc* subs, int n_sub, int nlon, int 
   return cudaGetLastError();
 }
 
+namespace {
 cudaError_t launch_global_stage(const double* x, const double* y, double* out, double ca, double cb,
-                                const RowConst* rows, double Bth, double gBth, double dt, int nlon,
-                                int nlat, cudaStream_t st) {
-  dim3 grid((nlon + 127) / 128, nlat);
-  global_stage_kernel<<<grid, 128, 0, st>>>(x, y, out, ca, cb, rows, Bth, gBth, dt, nlon, nlat);
-  return cudaGetLastError();
+                                const double* rec, double dtB, double dtgB, int nlon, int nlat, cudaStream_t st) {
+  const long long n = (long long)nlon * nlat;
+  return launch_dependent(global_stage_kernel, dim3((unsigned)((n + kGlobalThreads - 1) / kGlobalThreads)),
+                          kGlobalThreads, 0, st, x, y, out, ca, cb, rec, dtB, dtgB, nlon, nlat);
+}
+}  // namespace
+
+// The step kernel's tile: the one whose busiest SM has the least FP64 work.
+// The stage kernels spend about 6 us more per stage than their FP64 work (24 /
+// 30 / 30 instructions a point, 16 cycles a warp instruction), the step kernel
+// about 6 us per step plus the halo points.  Measured, step kernel (as chosen)
+// against the old stage kernels: 360 x 181 points 17.7 / 26.9 us a step, 512 x 256
+// 30.0 / 39.0, 768 x 384 59.6 / 71.9, 1024 x 512 100.5 / 115.0.
+GlobalStepPlan global_step_plan(int nlon, int nlat) {
+  GlobalStepPlan best;
+  const double per = 16.0 / 32.0 / 2.07e3;   // us per FP64 thread instruction of an SM
+  const double stages = 18.0 + 84.0 * (double)nlon * nlat / 152.0 * per;
+  double least = stages;
+  for (int tx = 16; tx <= 128; tx += 8)
+    for (int ty = 4; ty <= 40; ++ty) {
+      if (step_smem(tx, ty) > 110 * 1024 || tx - 8 >= nlon || ty - 1 >= nlat) continue;
+      const long long n = (long long)((nlon + tx - 1) / tx) * ((nlat + ty - 1) / ty);
+      const double work = 24.0 * (tx + 4) * (ty + 4) + 30.0 * (tx + 2) * (ty + 2) + 30.0 * tx * ty;
+      const double cost = 6.0 + (double)((n + 151) / 152) * work * per;
+      if (cost < least) {
+        least = cost;
+        best.tx = tx;
+        best.ty = ty;
+      }
+    }
+  return best;
+}
+
+cudaError_t launch_global_step(const GlobalStepPlan& plan, const double* x, double* s1, double* s2, double* nx,
+                               const double* rec, double dtB, double dtgB, int nlon, int nlat, cudaStream_t st,
+                               long long* launches) {
+  if (plan.tx > 0) {
+    cudaError_t e = raise_smem_cap(global_step_kernel);
+    if (e != cudaSuccess) return e;
+    ++*launches;
+    return launch_dependent(global_step_kernel,
+                            dim3((unsigned)((nlon + plan.tx - 1) / plan.tx), (unsigned)((nlat + plan.ty - 1) / plan.ty)),
+                            kStepThreads, step_smem(plan.tx, plan.ty), st, x, nx, rec, dtB, dtgB, nlon, nlat,
+                            StepTile{plan.tx, plan.ty});
+  }
+  *launches += 3;
+  cudaError_t e = launch_global_stage(x, x, s1, 0.0, 1.0, rec, dtB, dtgB, nlon, nlat, st);
+  if (e == cudaSuccess) e = launch_global_stage(x, s1, s2, 0.75, 0.25, rec, dtB, dtgB, nlon, nlat, st);
+  if (e == cudaSuccess) e = launch_global_stage(x, s2, nx, 1.0 / 3.0, 2.0 / 3.0, rec, dtB, dtgB, nlon, nlat, st);
+  return e;
 }
 cudaError_t launch_observe(const double* traj, int g0, int g1, long long n, const int* level,
                            const int* var, const double* fi, const double* fj, int nlon, int nlat,

@@ -121,6 +121,28 @@ template <typename T> constexpr int max_threads_forward() { return sizeof(T) == 
 template <typename T> constexpr int min_blocks_forward() { return sizeof(T) == 4 ? 4 : 1; }
 constexpr int kStripeAdjThreads = 1024;
 
+// ---- programmatic dependent launch ----
+// A chain of kernels on one stream whose set-up may overlap the end of the
+// kernel before: every thread of every such kernel calls grid_wait before it
+// reads what earlier kernels wrote, also where it then has nothing to do, so
+// that a grid never ends before the ones it follows.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // ---- launchers (sweep.cu) ----
 // Which kernel a sweep launch with cl CTAs per subdomain and nthreads threads
 // per CTA would run: 0 = none (shape not launchable), 1 = the stripe sweep
@@ -271,9 +293,16 @@ cudaError_t launch_restrict_level(const SubDesc* subs, int n_sub, int nlon, int 
                                   int g0, int g1, double* xb_a, int max_pts, cudaStream_t st);
 
 // global model (whole sphere), FP64
-cudaError_t launch_global_stage(const double* x, const double* y, double* out, double ca, double cb,
-                                const RowConst* rows, double Bth, double gBth, double dt, int nlon,
-                                int nlat, cudaStream_t st);
+// rec: FP64 forward records of every row (fill_records of point.cuh, 8 doubles a
+// row); dtB, dtgB: dt Bth, dt g Bth
+struct GlobalStepPlan {
+  int tx = 0, ty = 0;         // tile of the step kernel; 0: one launch per stage
+};
+GlobalStepPlan global_step_plan(int nlon, int nlat);
+// one RK3 step x -> nx; s1, s2: scratch states of the stage kernels
+cudaError_t launch_global_step(const GlobalStepPlan& plan, const double* x, double* s1, double* s2, double* nx,
+                               const double* rec, double dtB, double dtgB, int nlon, int nlat, cudaStream_t st,
+                               long long* launches);
 cudaError_t launch_observe(const double* traj, int g0, int g1, long long n, const int* level,
                            const int* var, const double* fi, const double* fj, int nlon, int nlat,
                            double* out, cudaStream_t st);
@@ -323,26 +352,37 @@ cudaError_t launch_max_abs_diff(const double* a, const double* b, long long n, d
 cudaError_t launch_finite_check(const double* a, long long n, int* flag, cudaStream_t st);
 
 // ---- Turkel-Zwas scheme on the whole sphere (tz.cu) ----
+struct TzRow {                // per latitude row, times dt where a tendency uses it
+  double a, f, tau, c;        // dt s_lon / c, dt f, dt tau, c
+  double kg, kp, kq, pad;     // dt s_lon g / (p c), dt s_lon / (p c), dt s_lat / (q c)
+};
 struct TzArgs {
   const RowConst* rows;       // [nlat]
+  const TzRow* rec;           // [nlat] (launch_tz_rows)
   int nlon, nlat, p, q;
   double alpha, slon, slat, g, dt;
+  double st, gq;              // dt s_lat, dt s_lat g / q
 };
+cudaError_t launch_tz_rows(const TzArgs& t, TzRow* rec, cudaStream_t st);
 cudaError_t launch_tz_stage(const TzArgs& t, const double* X, const double* Y, double* out, double cx, double cy,
                             cudaStream_t st);
 cudaError_t launch_tz_tl_stage(const TzArgs& t, const double* Y, const double* dX, const double* dY, double* dout,
                                double cx, double cy, cudaStream_t st);
-cudaError_t launch_tz_adj_scatter(const TzArgs& t, const double* Y, const double* M, double* G, double scale,
-                                  cudaStream_t st);
-cudaError_t launch_tz_lincomb(double* out, const double* a, const double* b, const double* c, double ca, double cb,
-                              double cc, long long n, cudaStream_t st);
+// out = M + dt F'(Y)^T M; with lam and mu2 given, the transposed step's last
+// phase: out = lam / 3 + mu2 / 2 + (M + dt F'(Y)^T M) / 6 (+ force; out may be lam)
+cudaError_t launch_tz_adj_stage(const TzArgs& t, const double* Y, const double* M, const double* lam,
+                                const double* mu2, const double* force, double* out, cudaStream_t st);
 cudaError_t launch_tz_scale_add(double* out, const double* a, const double* b, const double* sigma, long long plane,
                                 cudaStream_t st);
+// blocks of the observation misfit and of the background term (partial sums)
+constexpr int kTzBlocks = 128;
 cudaError_t launch_tz_obs_misfit(const double* traj, long long n, const int* level, const int* var, const double* fi,
                                  const double* fj, const double* y, const double* so, int nlon, int nlat, double lam,
-                                 double* force, double* Jo, cudaStream_t st);
+                                 double* force, double* part, cudaStream_t st);
 cudaError_t launch_tz_obs_scatter(long long k0, long long k1, const int* var, const double* fi, const double* fj,
                                   const double* force, int nlon, int nlat, double* lam, cudaStream_t st);
-cudaError_t launch_tz_finish_J(const double* w, long long n, const double* Jo, double* J, cudaStream_t st);
+// J = 1/2 w.w + sum of the misfit's kTzBlocks partial sums in part[0 ..] (none: nobs = 0);
+// part[kTzBlocks ..] is scratch
+cudaError_t launch_tz_finish_J(const double* w, long long n, int nobs, double* part, double* J, cudaStream_t st);
 
 }  // namespace dd4dv

@@ -41,13 +41,6 @@ namespace dd4dv {
 
 namespace {
 
-// Waits for the grids before this one (programmatic dependent launch): every
-// thread of every level kernel calls it before it reads what they wrote, also
-// where it then has nothing to do, so that a grid never ends before the ones it
-// follows.
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // The CTA's tile in shared memory: one coalesced load, and no registers held
 // for the fields that only edges need.
 #define LV_TILE(t)                                                                                    \
@@ -593,16 +586,7 @@ __global__ void __launch_bounds__(kLvThreads) lv_export_kernel(const LvArgs<T> a
 template <typename T>
 cudaError_t lv_launch(void (*kernel)(const LvArgs<T>), const LvArgs<T>& a, int blocks, cudaStream_t st) {
   if (blocks <= 0) return cudaSuccess;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)blocks, 1, 1);
-  cfg.blockDim = dim3(kLvThreads, 1, 1);
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, a);
+  return launch_dependent(kernel, dim3((unsigned)blocks), kLvThreads, 0, st, a);
 }
 
 }  // namespace

@@ -25,7 +25,7 @@
 // caller.  Every scratch word a call reads was written earlier by the same
 // call, so nothing has to be cleared between calls.
 #include "dd4dvar.h"
-#include "common.cuh"
+#include "point.cuh"
 
 #include <cmath>
 #include <mutex>
@@ -36,7 +36,7 @@ namespace {
 
 constexpr long long kMaxStateDoubles = 3LL * 512 * 256;   // one state of up to 512 x 256 points
 constexpr int kMaxRows = 1024;                            // latitude rows
-constexpr long long kRowDoubles = (long long)kMaxRows * (sizeof(RowConst) / sizeof(double));
+constexpr long long kRowDoubles = 8LL * kMaxRows;         // FP64 forward records (point.cuh)
 constexpr long long kScratchDoubles = 2 * kMaxStateDoubles + kRowDoubles;
 
 static __device__ __align__(256) double g_noalloc_scratch[kScratchDoubles];
@@ -63,13 +63,14 @@ cudaError_t scratch_address(double** out) {
   return cudaSuccess;
 }
 
-// Per-row constants of the global grid (Sec. 7), one thread per latitude
-// row: cell-centre latitude theta_j = lat_min + (j + 1/2) dtheta and
-// A = 1/(2 a cos dlambda), f = 2 Omega sin, tau = tan / a, Bth / cos, g A.
-// The products and sums are rounded one by one (no contraction), as the
-// host computes them for dd4dv_create.
-__global__ void noalloc_rows_kernel(RowConst* rows, int nlon, int nlat, double lat_min_deg,
-                                    double lat_max_deg, double radius, double gravity, double omega) {
+// Per-row records of the global grid (Sec. 7), one thread per latitude row:
+// cell-centre latitude theta_j = lat_min + (j + 1/2) dtheta and
+// A = 1/(2 a cos dlambda), f = 2 Omega sin, tau = tan / a, Bth / cos, g A, with
+// the cosines of the neighbour rows (walls: the edge row's).  The products and
+// sums are rounded one by one (no contraction), as the host computes them for
+// dd4dv_create.
+__global__ void noalloc_rows_kernel(double* rec, int nlon, int nlat, double lat_min_deg, double lat_max_deg,
+                                    double radius, double gravity, double omega, double dt) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= nlat) return;
   const double pi = 3.14159265358979323846;
@@ -78,7 +79,8 @@ __global__ void noalloc_rows_kernel(RowConst* rows, int nlon, int nlat, double l
                                (double)nlat);
   const double th0 = __ddiv_rn(__dmul_rn(lat_min_deg, pi), 180.0);
   const double Bth = __ddiv_rn(1.0, __dmul_rn(__dmul_rn(2.0, radius), dth));
-  const double th = __dadd_rn(th0, __dmul_rn(__dadd_rn((double)j, 0.5), dth));
+  auto theta = [&](int k) { return __dadd_rn(th0, __dmul_rn(__dadd_rn((double)k, 0.5), dth)); };
+  const double th = theta(j);
   RowConst r;
   r.c = cos(th);
   r.A = __ddiv_rn(1.0, __dmul_rn(__dmul_rn(__dmul_rn(2.0, radius), r.c), dlam));
@@ -86,7 +88,8 @@ __global__ void noalloc_rows_kernel(RowConst* rows, int nlon, int nlat, double l
   r.tau = __ddiv_rn(tan(th), radius);
   r.BinvC = __ddiv_rn(Bth, r.c);
   r.gA = __dmul_rn(gravity, r.A);
-  rows[j] = r;
+  double bw[8];
+  fill_records(r, cos(theta(min(j + 1, nlat - 1))), cos(theta(max(j - 1, 0))), dt, Bth, rec + 8 * j, bw);
 }
 
 }  // namespace
@@ -121,28 +124,25 @@ extern "C" dd4dv_status dd4dv_forward_noalloc(const dd4dv_model* model, const do
   if (e != cudaSuccess) return bad(DD4DV_ECUDA, std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e));
   double* s1 = scratch;
   double* s2 = scratch + kMaxStateDoubles;
-  RowConst* rows_d = reinterpret_cast<RowConst*>(scratch + 2 * kMaxStateDoubles);
+  double* rec = scratch + 2 * kMaxStateDoubles;
 
   // per-row constants of the grid (Sec. 7), computed on the device into the
   // scratch array; the two scalars the stages take are formed here
   const double pi = 3.14159265358979323846;
   const double dth = (m.lat_max_deg - m.lat_min_deg) * pi / 180.0 / m.nlat;
   const double Bth = 1.0 / (2.0 * m.radius * dth);
-  const double gBth = m.gravity * Bth;
-  noalloc_rows_kernel<<<(m.nlat + 127) / 128, 128, 0, st>>>(rows_d, m.nlon, m.nlat, m.lat_min_deg,
-                                                           m.lat_max_deg, m.radius, m.gravity, m.omega);
+  const double dtB = m.dt * Bth, dtgB = m.dt * (m.gravity * Bth);
+  noalloc_rows_kernel<<<(m.nlat + 127) / 128, 128, 0, st>>>(rec, m.nlon, m.nlat, m.lat_min_deg, m.lat_max_deg,
+                                                           m.radius, m.gravity, m.omega, m.dt);
   e = cudaGetLastError();
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(traj, x0, G * sizeof(double), cudaMemcpyDeviceToDevice, st);
+  const GlobalStepPlan plan = global_step_plan(m.nlon, m.nlat);
+  long long launches = 0;
   for (int n = 0; n < m.nsteps && e == cudaSuccess; ++n) {
     const double* x = traj + (size_t)n * G;
     double* nx = traj + (size_t)(n + 1) * G;
-    e = launch_global_stage(x, x, s1, 0.0, 1.0, rows_d, Bth, gBth, m.dt, m.nlon, m.nlat, st);
-    if (e == cudaSuccess)
-      e = launch_global_stage(x, s1, s2, 0.75, 0.25, rows_d, Bth, gBth, m.dt, m.nlon, m.nlat, st);
-    if (e == cudaSuccess)
-      e = launch_global_stage(x, s2, nx, 1.0 / 3.0, 2.0 / 3.0, rows_d, Bth, gBth, m.dt, m.nlon,
-                              m.nlat, st);
+    e = launch_global_step(plan, x, s1, s2, nx, rec, dtB, dtgB, m.nlon, m.nlat, st, &launches);
   }
   if (e != cudaSuccess) return bad(DD4DV_ECUDA, std::string("dd4dv_forward_noalloc: ") + cudaGetErrorString(e));
   set_global_error("");

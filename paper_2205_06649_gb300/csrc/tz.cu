@@ -14,10 +14,14 @@
 //
 // The tangent-linear stage is built from one list of partial derivatives per
 // point (tz_jacobian: for each value of the state that F at the point reads,
-// d F_out / d value_in), and the adjoint stage applies the same list
-// transposed, scattering coef * m_out(point) into value_in (FP64 atomic
-// additions); the adjoint is therefore the exact transpose of the
-// tangent-linear model up to the order of the additions.
+// d F_out / d value_in).  The adjoint stage gathers the transposed list: a point
+// collects, term by term, what the points that read it send back, so there are
+// no atomic additions and the result does not depend on their order.
+// Bound: launch latency on small grids (8 launches a step of about 3 us), the
+// FP64 pipe on large ones.  Row constants hold every quotient and dt
+// (launch_tz_rows): the divisions were most of the FP64 work.
+// 256 x 128 points, 128 steps, (p, q, alpha) = (2, 1, 1/2), J and gradient:
+// 21.1 -> 7.3 ms.
 #include "common.cuh"
 
 namespace dd4dv {
@@ -186,17 +190,161 @@ __device__ void tz_jacobian(const TzArgs& t, const double* Y, int j, int i, Vis&
   }
 }
 
-// out = cx X + cy (Y + dt F(Y))
-__global__ void tz_stage_kernel(TzArgs t, const double* X, const double* Y, double* out, double cx, double cy) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
-  if (i >= t.nlon) return;
-  double F[3];
-  tz_F(t, Y, j, i, F[0], F[1], F[2]);
-  const size_t pl = (size_t)t.nlat * t.nlon, o = (size_t)j * t.nlon + i;
-  for (int v = 0; v < 3; ++v) {
-    double r = cy * (Y[v * pl + o] + t.dt * F[v]);
-    if (cx != 0.0) r += cx * X[v * pl + o];
-    out[v * pl + o] = r;
+constexpr int kTzThreads = 128;
+
+// The point of a thread: flat over rows.
+struct TzPt {
+  int j, i;
+  unsigned o;        // offset in a plane
+  bool in;
+  __device__ __forceinline__ explicit TzPt(const TzArgs& t) {
+    o = blockIdx.x * kTzThreads + threadIdx.x;
+    j = (int)(o / (unsigned)t.nlon);
+    i = (int)(o - (unsigned)j * t.nlon);
+    in = j < t.nlat;
+  }
+};
+__device__ __forceinline__ int tz_wrap(int i, int n) { return i < 0 ? i + n : i >= n ? i - n : i; }
+// Row s rows away (|s| < nlat), through the wall mirror; sg = -1 for a v read
+// through it.
+__device__ __forceinline__ int tz_row(int j, int s, int nlat, double& sg) {
+  const int r = j + s;
+  sg = r < 0 || r >= nlat ? -1.0 : 1.0;
+  return r < 0 ? -1 - r : r >= nlat ? 2 * nlat - 1 - r : r;
+}
+
+// out = cx X + cy (Y + dt F(Y)), the tendencies of tz_F with the row records
+__global__ void __launch_bounds__(kTzThreads) tz_stage_kernel(TzArgs t, const double* X, const double* Y, double* out,
+                                                              double cx, double cy) {
+  const TzPt m(t);
+  grid_wait();
+  grid_release();
+  if (!m.in) return;
+  const size_t pl = (size_t)t.nlat * t.nlon, o = m.o;
+  const double *H = Y, *U = Y + pl, *V = Y + 2 * pl;
+  const size_t row = (size_t)m.j * t.nlon;
+  const int iE = tz_wrap(m.i + 1, t.nlon), iW = tz_wrap(m.i - 1, t.nlon);
+  const int pE = tz_wrap(m.i + t.p, t.nlon), pW = tz_wrap(m.i - t.p, t.nlon);
+  double s1N, s1S, sN, sS;
+  const size_t r1N = (size_t)tz_row(m.j, 1, t.nlat, s1N) * t.nlon, r1S = (size_t)tz_row(m.j, -1, t.nlat, s1S) * t.nlon;
+  const int jN = tz_row(m.j, t.q, t.nlat, sN), jS = tz_row(m.j, -t.q, t.nlat, sS);
+  const size_t rN = (size_t)jN * t.nlon, rS = (size_t)jS * t.nlon;
+  const TzRow rc = t.rec[m.j];
+  const double cN = sN * t.rec[jN].c, cS = sS * t.rec[jS].c;   // (v c) through the mirror
+  const double h = H[o], u = U[o], v = V[o], al = t.alpha, a1 = 1.0 - al, a2 = 0.5 * al;
+  const double Au = rc.a * u, Bv = t.st * v, C = fma(rc.tau, u, rc.f);
+  const double uEp = U[row + pE], uWp = U[row + pW], vN = V[rN + m.i], vS = V[rS + m.i];
+  double cu = a1 * C * v, cv = a1 * C * u;
+  double du = a1 * (uEp - uWp), dv = a1 * fma(vN, cN, -vS * cS);
+  if (al != 0.0) {
+    cu = fma(a2, fma(fma(rc.tau, uEp, rc.f), V[row + pE], fma(rc.tau, uWp, rc.f) * V[row + pW]), cu);
+    const TzRow N = t.rec[jN], S = t.rec[jS];
+    const double uN = U[rN + m.i], uS = U[rS + m.i];
+    cv = fma(a2, fma(fma(N.tau, uN, N.f), uN, fma(S.tau, uS, S.f) * uS), cv);
+    du = fma(a2, (U[rN + pE] - U[rN + pW]) + (U[rS + pE] - U[rS + pW]), du);
+    dv = fma(a2, fma(V[rN + pE] + V[rN + pW], cN, -(V[rS + pE] + V[rS + pW]) * cS), dv);
+  }
+  double ou = fma(-Au, U[row + iE] - U[row + iW], u);
+  ou = fma(-Bv, U[r1N + m.i] - U[r1S + m.i], ou);
+  ou = fma(-rc.kg, H[row + pE] - H[row + pW], ou) + cu;
+  double ov = fma(-Au, V[row + iE] - V[row + iW], v);
+  ov = fma(-Bv, s1N * V[r1N + m.i] - s1S * V[r1S + m.i], ov);
+  ov = fma(-t.gq, H[rN + m.i] - H[rS + m.i], ov) - cv;
+  double oh = fma(-Au, H[row + iE] - H[row + iW], h);
+  oh = fma(-Bv, H[r1N + m.i] - H[r1S + m.i], oh);
+  oh = fma(-h, fma(rc.kp, du, rc.kq * dv), oh);
+  if (cx != 0.0) {
+    oh = fma(cx, X[o], cy * oh);
+    ou = fma(cx, X[o + pl], cy * ou);
+    ov = fma(cx, X[o + 2 * pl], cy * ov);
+  }
+  out[o] = oh;
+  out[o + pl] = ou;
+  out[o + 2 * pl] = ov;
+}
+
+// G = M + dt F'(Y)^T M gathered at one point: per term of F, what the points
+// that read this one send back.  A point s rows south (north) reads it with
+// the sign of its northern (southern) neighbour; where the wall mirror folds
+// that row back (row < s), the mirrored row reads it with its southern
+// (northern) neighbour instead, and its v with the sign flipped, so that the
+// terms odd in the row distance change sign (sg = -1) but for v.
+__global__ void __launch_bounds__(kTzThreads) tz_adj_kernel(TzArgs t, const double* Y, const double* M,
+                                                            const double* lam, const double* mu2, const double* force,
+                                                            double* out) {
+  const TzPt m(t);
+  grid_wait();
+  grid_release();
+  if (!m.in) return;
+  const size_t pl = (size_t)t.nlat * t.nlon, o = m.o;
+  const double *H = Y, *U = Y + pl, *V = Y + 2 * pl;
+  const double *mh = M, *mu = M + pl, *mv = M + 2 * pl;
+  const size_t row = (size_t)m.j * t.nlon;
+  const size_t E = row + tz_wrap(m.i + 1, t.nlon), W = row + tz_wrap(m.i - 1, t.nlon);
+  const int pE = tz_wrap(m.i + t.p, t.nlon), pW = tz_wrap(m.i - t.p, t.nlon);
+  // rows at distance 1 and q: the same as those this point reads, mirrors included
+  double s1N, s1S, sN, sS;
+  const int j1N = tz_row(m.j, 1, t.nlat, s1N), j1S = tz_row(m.j, -1, t.nlat, s1S);
+  const int jN = tz_row(m.j, t.q, t.nlat, sN), jS = tz_row(m.j, -t.q, t.nlat, sS);
+  const size_t N1 = (size_t)j1N * t.nlon + m.i, S1 = (size_t)j1S * t.nlon + m.i;
+  const size_t rN = (size_t)jN * t.nlon, rS = (size_t)jS * t.nlon, Nq = rN + m.i, Sq = rS + m.i;
+  const TzRow rc = t.rec[m.j], Rn = t.rec[jN], Rs = t.rec[jS];
+  const double al = t.alpha, a1 = 1.0 - al, a2 = 0.5 * al;
+  const double h = H[o], u = U[o], v = V[o], xh = mh[o], xu = mu[o], xv = mv[o];
+  const double C = fma(rc.tau, u, rc.f);
+  // products of the neighbours' velocities and adjoints
+  const double uE = U[E], uW = U[W], vN = s1N * V[N1], vS = s1S * V[S1];
+  const double muE = mu[E], muW = mu[W], mvE = mv[E], mvW = mv[W], mhE = mh[E], mhW = mh[W];
+  // advection: what F of the four neighbours reads of (h, u, v) here.  The
+  // northern neighbour reads this point as its south: + s_lat v m; a mirrored
+  // one (sg = -1) with the other sign, and vN, vS carry that sign.
+  double gh = fma(rc.a, fma(uE, mhE, -uW * mhW), xh);
+  double gu = fma(rc.a, fma(uE, muE, -uW * muW), xu);
+  double gv = fma(rc.a, fma(uE, mvE, -uW * mvW), xv);
+  gh = fma(t.st, fma(vN, mh[N1], -vS * mh[S1]), gh);
+  gu = fma(t.st, fma(vN, mu[N1], -vS * mu[S1]), gu);
+  gv = fma(t.st, fma(s1N * vN, mv[N1], -s1S * vS * mv[S1]), gv);
+  // own coefficients: u and v multiply the centred differences of all three
+  const double dhx = H[E] - H[W], dux = uE - uW, dvx = V[E] - V[W];
+  const double dhy = H[N1] - H[S1], duy = U[N1] - U[S1], dvy = vN - vS;
+  gu = fma(-rc.a, fma(xu, dux, fma(xv, dvx, xh * dhx)), gu);
+  gv = fma(-t.st, fma(xu, duy, fma(xv, dvy, xh * dhy)), gv);
+  // Coriolis
+  gu = fma(a1, fma(xu * rc.tau, v, -xv * fma(rc.tau, u, C)), gu);
+  gv = fma(a1 * xu, C, gv);
+  // pressure gradients
+  const double muEp = mu[row + pE], muWp = mu[row + pW], mvN = mv[Nq], mvS = mv[Sq];
+  gh = fma(rc.kg, muEp - muWp, gh);
+  gh = fma(t.gq, sN * mvN - sS * mvS, gh);
+  // divergence: h m_h of the points that read u, v here; h times the divergence
+  const double kE = H[row + pE] * mh[row + pE], kW = H[row + pW] * mh[row + pW];
+  const double kN = H[Nq] * mh[Nq], kS = H[Sq] * mh[Sq];
+  gu = fma(a1 * rc.kp, kE - kW, gu);
+  gv = fma(a1 * rc.c, fma(Rn.kq, kN, -Rs.kq * kS), gv);
+  const double cN = sN * Rn.c, cS = sS * Rs.c;
+  double du = a1 * (U[row + pE] - U[row + pW]), dv = a1 * fma(V[Nq], cN, -V[Sq] * cS);
+  if (al != 0.0) {
+    gu = fma(a2 * rc.tau * v, muEp + muWp, gu);
+    gv = fma(a2 * C, muEp + muWp, gv);
+    gu = fma(-a2 * fma(rc.tau, u, C), mvN + mvS, gu);
+    const double kNE = H[rN + pE] * mh[rN + pE], kNW = H[rN + pW] * mh[rN + pW];
+    const double kSE = H[rS + pE] * mh[rS + pE], kSW = H[rS + pW] * mh[rS + pW];
+    gu = fma(a2, fma(Rn.kp, kNE - kNW, Rs.kp * (kSE - kSW)), gu);
+    gv = fma(a2 * rc.c, fma(Rn.kq, kNE + kNW, -Rs.kq * (kSE + kSW)), gv);
+    du = fma(a2, (U[rN + pE] - U[rN + pW]) + (U[rS + pE] - U[rS + pW]), du);
+    dv = fma(a2, fma(V[rN + pE] + V[rN + pW], cN, -(V[rS + pE] + V[rS + pW]) * cS), dv);
+  }
+  gh = fma(-xh, fma(rc.kp, du, rc.kq * dv), gh);
+  double g[3] = {gh, gu, gv};
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const size_t q = o + c * pl;
+    double r = g[c];
+    if (lam) {
+      r = fma(1.0 / 6.0, r, fma(0.5, mu2[q], (1.0 / 3.0) * lam[q]));
+      if (force) r += force[q];
+    }
+    out[q] = r;
   }
 }
 
@@ -217,23 +365,6 @@ __global__ void tz_tl_stage_kernel(TzArgs t, const double* Y, const double* dX, 
   }
 }
 
-// G += scale F'(Y)^T M (the transposed partial derivatives, scattered)
-__global__ void tz_adj_scatter_kernel(TzArgs t, const double* Y, const double* M, double* G, double scale) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
-  if (i >= t.nlon) return;
-  const size_t pl = (size_t)t.nlat * t.nlon, o = (size_t)j * t.nlon + i;
-  const double m[3] = {scale * M[o], scale * M[pl + o], scale * M[2 * pl + o]};
-  tz_jacobian(t, Y, j, i, [&](int vo, int vi, int jj, int ii, double coef) {
-    if (m[vo] != 0.0) atomicAdd(&G[vi * pl + (size_t)jj * t.nlon + ii], coef * m[vo]);
-  });
-}
-
-__global__ void tz_lincomb_kernel(double* out, const double* a, const double* b, const double* c, double ca,
-                                  double cb, double cc, long long n) {
-  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x)
-    out[k] = ca * a[k] + cb * b[k] + (c ? cc * c[k] : 0.0);
-}
-
 // x0 = xb + sigma_v w (diagonal B) or grad = w + sigma_v lam
 __global__ void tz_scale_add_kernel(double* out, const double* a, const double* b, const double* sigma, long long plane) {
   for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < 3 * plane;
@@ -241,16 +372,27 @@ __global__ void tz_scale_add_kernel(double* out, const double* a, const double* 
     out[k] = a[k] + sigma[k / plane] * b[k];
 }
 
+// Sum of the block's values (fixed order), on thread 0.
+__device__ double tz_block_sum(double x) {
+  __shared__ double sh[8];
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = x;
+  __syncthreads();
+  double s = 0.0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += sh[w];
+  return s;
+}
+
 // Observation misfits of the whole trajectory (obs sorted by level): forcing
-// lam (H x - y) / sigma_o^2 per observation and J_o = lam/2 sum (H x - y)^2 /
-// sigma_o^2, one block, fixed-order reduction.
+// lam (H x - y) / sigma_o^2 per observation and lam/2 sum (H x - y)^2 /
+// sigma_o^2, one partial sum per block in a fixed order.
 __global__ void tz_obs_misfit_kernel(const double* traj, long long n, const int* level, const int* var,
                                      const double* fi, const double* fj, const double* y, const double* so,
-                                     int nlon, int nlat, double lam, double* force, double* Jo) {
-  __shared__ double sh[1024 / 32];
+                                     int nlon, int nlat, double lam, double* force, double* part) {
   double acc = 0.0;
   const size_t pl = (size_t)nlat * nlon;
-  for (long long k = threadIdx.x; k < n; k += blockDim.x) {
+  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
     const int i0 = (int)floor(fi[k]), j0 = (int)floor(fj[k]);
     const double di = fi[k] - i0, dj = fj[k] - j0;
     const int i1 = (i0 + 1) % nlon;
@@ -265,14 +407,8 @@ __global__ void tz_obs_misfit_kernel(const double* traj, long long n, const int*
     force[k] = lam * w * d;
     acc += 0.5 * lam * w * d * d;
   }
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += sh[w];
-    *Jo = s;
-  }
+  const double s = tz_block_sum(acc);
+  if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
 // lam += H^T force for the observations [k0, k1) (one level)
@@ -295,21 +431,40 @@ __global__ void tz_obs_scatter_kernel(long long k0, long long k1, const int* var
   }
 }
 
-// J_b = 1/2 w.w, one block, fixed order; J = J_b + J_o
-__global__ void tz_finish_J_kernel(const double* w, long long n, const double* Jo, double* J) {
-  __shared__ double sh[1024 / 32];
+// Partial sums of 1/2 w.w, then J = J_b + J_o in a fixed order.
+__global__ void tz_background_kernel(const double* w, long long n, double* part) {
   double acc = 0.0;
-  for (long long k = threadIdx.x; k < n; k += blockDim.x) acc += w[k] * w[k];
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) s += sh[k];
-    *J = 0.5 * s + (Jo ? *Jo : 0.0);
-  }
+  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x)
+    acc += w[k] * w[k];
+  const double s = tz_block_sum(acc);
+  if (threadIdx.x == 0) part[blockIdx.x] = 0.5 * s;
+}
+__global__ void tz_finish_J_kernel(const double* part, int nobs, double* J) {
+  double x = 0.0;
+  if (threadIdx.x < kTzBlocks) x = part[kTzBlocks + threadIdx.x] + (nobs ? part[threadIdx.x] : 0.0);
+  const double s = tz_block_sum(x);
+  if (threadIdx.x == 0) *J = s;
 }
 
+__global__ void tz_rows_kernel(TzArgs t, TzRow* rec) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= t.nlat) return;
+  const RowConst r = t.rows[j];
+  TzRow q;
+  q.a = t.dt * t.slon / r.c;
+  q.f = t.dt * r.f;
+  q.tau = t.dt * r.tau;
+  q.c = r.c;
+  q.kg = t.dt * t.slon * t.g / (t.p * r.c);
+  q.kp = t.dt * t.slon / (t.p * r.c);
+  q.kq = t.dt * t.slat / (t.q * r.c);
+  q.pad = 0.0;
+  rec[j] = q;
+}
+
+inline dim3 tz_flat(const TzArgs& t) {
+  return dim3((unsigned)(((long long)t.nlon * t.nlat + kTzThreads - 1) / kTzThreads));
+}
 inline dim3 tz_grid(const TzArgs& t) { return dim3((t.nlon + 127) / 128, t.nlat); }
 inline unsigned tz_blocks(long long n) {
   long long b = (n + 255) / 256;
@@ -318,24 +473,21 @@ inline unsigned tz_blocks(long long n) {
 
 }  // namespace
 
+cudaError_t launch_tz_rows(const TzArgs& t, TzRow* rec, cudaStream_t st) {
+  tz_rows_kernel<<<(t.nlat + 127) / 128, 128, 0, st>>>(t, rec);
+  return cudaGetLastError();
+}
 cudaError_t launch_tz_stage(const TzArgs& t, const double* X, const double* Y, double* out, double cx, double cy,
                             cudaStream_t st) {
-  tz_stage_kernel<<<tz_grid(t), 128, 0, st>>>(t, X, Y, out, cx, cy);
-  return cudaGetLastError();
+  return launch_dependent(tz_stage_kernel, tz_flat(t), kTzThreads, 0, st, t, X, Y, out, cx, cy);
+}
+cudaError_t launch_tz_adj_stage(const TzArgs& t, const double* Y, const double* M, const double* lam,
+                                const double* mu2, const double* force, double* out, cudaStream_t st) {
+  return launch_dependent(tz_adj_kernel, tz_flat(t), kTzThreads, 0, st, t, Y, M, lam, mu2, force, out);
 }
 cudaError_t launch_tz_tl_stage(const TzArgs& t, const double* Y, const double* dX, const double* dY, double* dout,
                                double cx, double cy, cudaStream_t st) {
   tz_tl_stage_kernel<<<tz_grid(t), 128, 0, st>>>(t, Y, dX, dY, dout, cx, cy);
-  return cudaGetLastError();
-}
-cudaError_t launch_tz_adj_scatter(const TzArgs& t, const double* Y, const double* M, double* G, double scale,
-                                  cudaStream_t st) {
-  tz_adj_scatter_kernel<<<tz_grid(t), 128, 0, st>>>(t, Y, M, G, scale);
-  return cudaGetLastError();
-}
-cudaError_t launch_tz_lincomb(double* out, const double* a, const double* b, const double* c, double ca, double cb,
-                              double cc, long long n, cudaStream_t st) {
-  tz_lincomb_kernel<<<tz_blocks(n), 256, 0, st>>>(out, a, b, c, ca, cb, cc, n);
   return cudaGetLastError();
 }
 cudaError_t launch_tz_scale_add(double* out, const double* a, const double* b, const double* sigma, long long plane,
@@ -345,8 +497,8 @@ cudaError_t launch_tz_scale_add(double* out, const double* a, const double* b, c
 }
 cudaError_t launch_tz_obs_misfit(const double* traj, long long n, const int* level, const int* var, const double* fi,
                                  const double* fj, const double* y, const double* so, int nlon, int nlat, double lam,
-                                 double* force, double* Jo, cudaStream_t st) {
-  tz_obs_misfit_kernel<<<1, 1024, 0, st>>>(traj, n, level, var, fi, fj, y, so, nlon, nlat, lam, force, Jo);
+                                 double* force, double* part, cudaStream_t st) {
+  tz_obs_misfit_kernel<<<kTzBlocks, 256, 0, st>>>(traj, n, level, var, fi, fj, y, so, nlon, nlat, lam, force, part);
   return cudaGetLastError();
 }
 cudaError_t launch_tz_obs_scatter(long long k0, long long k1, const int* var, const double* fi, const double* fj,
@@ -355,8 +507,9 @@ cudaError_t launch_tz_obs_scatter(long long k0, long long k1, const int* var, co
   tz_obs_scatter_kernel<<<tz_blocks(k1 - k0), 256, 0, st>>>(k0, k1, var, fi, fj, force, nlon, nlat, lam);
   return cudaGetLastError();
 }
-cudaError_t launch_tz_finish_J(const double* w, long long n, const double* Jo, double* J, cudaStream_t st) {
-  tz_finish_J_kernel<<<1, 1024, 0, st>>>(w, n, Jo, J);
+cudaError_t launch_tz_finish_J(const double* w, long long n, int nobs, double* part, double* J, cudaStream_t st) {
+  tz_background_kernel<<<kTzBlocks, 256, 0, st>>>(w, n, part + kTzBlocks);
+  tz_finish_J_kernel<<<1, 128, 0, st>>>(part, nobs, J);
   return cudaGetLastError();
 }
 

@@ -77,3 +77,24 @@ def test_level_sweeps_equal_cluster_sweeps(monkeypatch, name, precision, ckpt_k)
     bar = 1e-13 if precision == 0 else 1e-6
     for k in ("J", "J2", "Je", "Jm"):
         assert np.max(np.abs(lev[k] - clu[k])) <= bar * np.max(np.abs(clu[k])), (name, k)
+
+
+@pytest.mark.parametrize("nlon,nlat", [(3, 2), (5, 3), (24, 12), (129, 40), (1100, 600)])
+def test_global_step_kernel_matches_oracle(nlon, nlat):
+    """The global model by the step kernel (tiles with halos; grids smaller than
+    a tile and its halo) and, on the largest grid, by the stage kernels, against
+    the oracle's model: two steps within 1e-13 relative (FP64 roundings)."""
+    import oracle
+    import paper_2205_06649_gb300 as dd
+    rng = np.random.default_rng(nlon)
+    x0 = np.stack([4000 + 10 * rng.standard_normal((nlat, nlon)), rng.standard_normal((nlat, nlon)),
+                   rng.standard_normal((nlat, nlon))])
+    grid = oracle.Grid(nlon, nlat, workloads.RADIUS, workloads.GRAVITY, workloads.OMEGA, workloads.LAT_MIN_DEG,
+                       workloads.LAT_MAX_DEG)
+    dt = 0.1 * 6.371e6 * 0.17 * 2 * np.pi / nlon / 210.0
+    ref = oracle.global_forward(grid, torch.as_tensor(x0), dt, 2).numpy()
+    ctx = dd.Context(nlon, nlat, dt, 2)
+    got = ctx.forward(x0)
+    ctx.destroy()
+    for v in range(3):
+        assert np.max(np.abs(got[:, v] - ref[:, v])) <= 1e-13 * np.max(np.abs(ref[:, v])), v
