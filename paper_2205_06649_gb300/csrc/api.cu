@@ -42,7 +42,7 @@ struct dd4dv_ctx {
   // grid
   std::vector<RowConst> rows_h;
   RowConst* rows_d = nullptr;
-  double* grec = nullptr;     // FP64 forward records of every row (global model)
+  double* grec = nullptr;     // records of every row (global model runs)
   GlobalStepPlan gplan;
   double Bth = 0, gBth = 0;
   size_t gstate = 0;          // 3*nlat*nlon
@@ -282,10 +282,12 @@ SweepArgs<T> sweep_args(dd4dv_ctx* ctx) {
   for (int v = 0; v < 3; ++v) a.isb2[v] = 1.0 / (ctx->sigma_b[v] * ctx->sigma_b[v]);
   a.lam = ctx->dec.lambda;
   a.mu = ctx->dec.mu;
-  const double scale = sizeof(T) == 8 ? a.dt : 1.0;   // the FP64 point functions take dt Bth and dt g Bth
+  const double scale = sizeof(T) == 8 ? a.dt : 1.0;   // adjoint_pt64 takes dt Bth and dt g Bth
   a.dt_s = (T)a.dt;
-  a.Bth_s = (T)(scale * a.Bth);
-  a.gBth_s = (T)(scale * a.gBth);
+  a.Bth_s = (T)a.Bth;
+  a.gBth_s = (T)a.gBth;
+  a.Bth_a = (T)(scale * a.Bth);
+  a.gBth_a = (T)(scale * a.gBth);
   a.href_s = (T)a.h_ref;
   for (int v = 0; v < 3; ++v) {
     a.isb2_s[v] = (T)a.isb2[v];
@@ -403,8 +405,10 @@ LvArgs<T> level_args(dd4dv_ctx* ctx, const int* active, int av) {
   a.bw = a.fw + 8 * (size_t)ctx->m.nlat;
   const double scale = sizeof(T) == 8 ? ctx->m.dt : 1.0;   // as in sweep_args
   a.dt = (T)ctx->m.dt;
-  a.Bth = (T)(scale * ctx->Bth);
-  a.gBth = (T)(scale * ctx->gBth);
+  a.Bth = (T)ctx->Bth;
+  a.gBth = (T)ctx->gBth;
+  a.Bth_a = (T)(scale * ctx->Bth);
+  a.gBth_a = (T)(scale * ctx->gBth);
   a.href = (T)(sizeof(T) == 4 ? ctx->m.h_ref : 0.0);
   for (int v = 0; v < 3; ++v) {
     const double isb2 = 1.0 / (ctx->sigma_b[v] * ctx->sigma_b[v]);
@@ -624,15 +628,16 @@ void global_run(dd4dv_ctx* ctx, const double* x0, double* out) {
 // levels are produced in the chunk buffer, gchunk_lv at a time, and handed to
 // sink(g0, g1, levels) (levels g0..g1, level-major FP64) in order.  The last
 // level of a chunk is the first of the next.
-template <typename Sink>
-void global_run_chunked(dd4dv_ctx* ctx, const double* x0, Sink&& sink) {
+// step(ctx, x, nx) advances one level.
+template <typename Step, typename Sink>
+void global_run_chunked(dd4dv_ctx* ctx, const double* x0, Step&& step, Sink&& sink) {
   const size_t G = ctx->gstate;
   const int K = ctx->gchunk_lv - 1;
   double* c = ctx->gchunk;
   CK(cudaMemcpyAsync(c, x0, G * sizeof(double), cudaMemcpyDeviceToDevice, ctx->st));
   for (int g0 = 0;;) {
     const int g1 = std::min(g0 + K, ctx->m.nsteps);
-    for (int n = g0; n < g1; ++n) global_step(ctx, c + (size_t)(n - g0) * G, c + (size_t)(n - g0 + 1) * G);
+    for (int n = g0; n < g1; ++n) step(ctx, c + (size_t)(n - g0) * G, c + (size_t)(n - g0 + 1) * G);
     sink(g0, g1, c);
     if (g1 >= ctx->m.nsteps) break;
     CK(cudaMemcpyAsync(c, c + (size_t)(g1 - g0) * G, G * sizeof(double), cudaMemcpyDeviceToDevice, ctx->st));
@@ -640,11 +645,27 @@ void global_run_chunked(dd4dv_ctx* ctx, const double* x0, Sink&& sink) {
   }
 }
 
+// One step of the background forecast.  Its levels become the boundary
+// trajectory and the targets, on the FP32 path rounded to FP32, where another
+// last bit here and there flips an FP32 value; so it keeps one order of
+// operations, that of the results on record, in a kernel of its own.
+void background_step(dd4dv_ctx* ctx, const double* x, double* nx) {
+  double* s1 = ctx->gscratch;
+  double* s2 = ctx->gscratch + ctx->gstate;
+  auto stage = [&](const double* y, double* out, double ca, double cb) {
+    KL(launch_background_stage(x, y, out, ca, cb, ctx->rows_d, ctx->Bth, ctx->gBth, ctx->m.dt, ctx->m.nlon,
+                               ctx->m.nlat, ctx->st));
+  };
+  stage(x, s1, 0.0, 1.0);
+  stage(s1, s2, 0.75, 0.25);
+  stage(s2, nx, 1.0 / 3.0, 2.0 / 3.0);
+}
+
 template <typename T>
 void background_pass(dd4dv_ctx* ctx, bool xb_a) {
   const size_t G = ctx->gstate;
   const int nlon = ctx->m.nlon, nlat = ctx->m.nlat;
-  global_run_chunked(ctx, ctx->xb0, [&](int g0, int g1, const double* lv) {
+  global_run_chunked(ctx, ctx->xb0, background_step, [&](int g0, int g1, const double* lv) {
     const long long n = (long long)(g1 - g0 + 1) * G;
     KL(launch_bnd_from_global<T>(lv, n, h_ref_of(ctx), nlon, nlat, static_cast<T*>(ctx->bnd) + (size_t)g0 * G,
                                  ctx->st));
@@ -1592,10 +1613,10 @@ dd4dv_status dd4dv_create(const dd4dv_model* model, void* cuda_stream, dd4dv_ctx
     ctx->rows_d = dalloc<RowConst>(ctx, m.nlat);
     ctx->gplan = global_step_plan(m.nlon, m.nlat);
     ctx->grec = dalloc<double>(ctx, 8 * (size_t)m.nlat);
-    std::vector<double> rec(8 * (size_t)m.nlat), back(8);
+    std::vector<double> rec(8 * (size_t)m.nlat);
     for (int j = 0; j < m.nlat; ++j)
-      fill_records(ctx->rows_h[j], ctx->rows_h[std::min(j + 1, m.nlat - 1)].c, ctx->rows_h[std::max(j - 1, 0)].c, m.dt,
-                   ctx->Bth, &rec[8 * (size_t)j], back.data());
+      fill_global_record(ctx->rows_h[j], ctx->rows_h[std::min(j + 1, m.nlat - 1)].c, ctx->rows_h[std::max(j - 1, 0)].c,
+                         m.dt, ctx->Bth, &rec[8 * (size_t)j]);
     ctx->xb0 = dalloc<double>(ctx, ctx->gstate);
     ctx->gscratch = dalloc<double>(ctx, 3 * ctx->gstate);
     // chunk of global levels: at most 512 MB, at least 2 levels, at most the whole trajectory
@@ -2031,7 +2052,7 @@ dd4dv_status dd4dv_forward(dd4dv_ctx* ctx, const double* x0, double* traj, int d
     const size_t G = ctx->gstate;
     double* in = ctx->gscratch + 2 * G;
     h2d(ctx, in, x0, G * sizeof(double));
-    global_run_chunked(ctx, in, [&](int g0, int g1, const double* lv) {
+    global_run_chunked(ctx, in, global_step, [&](int g0, int g1, const double* lv) {
       d2h(ctx, traj + (size_t)g0 * G, lv, (size_t)(g1 - g0 + 1) * G * sizeof(double));
     });
     sync(ctx);

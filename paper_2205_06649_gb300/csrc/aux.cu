@@ -349,12 +349,65 @@ __global__ void bnd_to_global_kernel(const T* bnd, long long n, double h_ref, lo
 }
 
 // ---------------------------------------------------------------------------
+// Stage of the background forecast on the whole sphere: out = ca x + cb (y + dt
+// F(y)).  (It runs at set_decomposition, and at a reset that has no copy.)
+__global__ void background_stage_kernel(const double* x, const double* y, double* out, double ca,
+                                    double cb, const RowConst* rows, double Bth, double gBth,
+                                    double dt, int nlon, int nlat) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = blockIdx.y;
+  if (i >= nlon) return;
+  const size_t P = (size_t)nlat * nlon;
+  const double* H = y;
+  const double* U = y + P;
+  const double* V = y + 2 * P;
+  const int iE = (i + 1) % nlon, iW = (i - 1 + nlon) % nlon;
+  const size_t o = (size_t)j * nlon + i;
+  const RowConst rc = rows[j];
+  const double h = H[o], u = U[o], v = V[o];
+  const double hE = H[(size_t)j * nlon + iE], hW = H[(size_t)j * nlon + iW];
+  const double uE = U[(size_t)j * nlon + iE], uW = U[(size_t)j * nlon + iW];
+  const double vE = V[(size_t)j * nlon + iE], vW = V[(size_t)j * nlon + iW];
+  double hN, uN, vN, cN, hS, uS, vS, cS;
+  if (j + 1 < nlat) {
+    const size_t q = (size_t)(j + 1) * nlon + i;
+    hN = H[q]; uN = U[q]; vN = V[q]; cN = rows[j + 1].c;
+  } else {
+    hN = h; uN = u; vN = -v; cN = rc.c;
+  }
+  if (j > 0) {
+    const size_t q = (size_t)(j - 1) * nlon + i;
+    hS = H[q]; uS = U[q]; vS = V[q]; cS = rows[j - 1].c;
+  } else {
+    hS = h; uS = u; vS = -v; cS = rc.c;
+  }
+  const double fu = rc.f + rc.tau * u;
+  const double Fu = -rc.A * u * (uE - uW) - Bth * v * (uN - uS) + fu * v - rc.gA * (hE - hW);
+  const double Fv = -rc.A * u * (vE - vW) - Bth * v * (vN - vS) - fu * u - gBth * (hN - hS);
+  const double Fh = -rc.A * (hE * uE - hW * uW) - rc.BinvC * (hN * vN * cN - hS * vS * cS);
+  const double F[3] = {Fh, Fu, Fv};
+  for (int c = 0; c < 3; ++c) {
+    const size_t q = (size_t)c * P + o;
+    out[q] = (ca == 0.0 ? 0.0 : ca * x[q]) + cb * (y[q] + dt * F[c]);
+  }
+}
+
 // Global model stage on the whole sphere: out = ca x + cb (y + dt F(y)).
 // Bound: the FP64 pipe, 24 instructions a point and stage (30 with x), as the
 // box sweeps (euler_pt64).  One thread per point, flat over rows so that every
 // lane has one; set-up overlaps the stage before (programmatic dependent
 // launch).  Small grids take global_step_kernel instead.
 constexpr int kGlobalThreads = 128;
+__device__ __forceinline__ void global_pt(const Pt5<double>& z, const double (&rc)[8], double dtB, double dtgB,
+                                          double ca, double cb, double x0, double x1, double x2, double& o0,
+                                          double& o1, double& o2) {
+  euler_pt64(z, rc, dtB, dtgB, o0, o1, o2);
+  if (ca != 0.0) {
+    o0 = xfma(ca, x0, xmul(cb, o0));
+    o1 = xfma(ca, x1, xmul(cb, o1));
+    o2 = xfma(ca, x2, xmul(cb, o2));
+  }
+}
 __global__ void __launch_bounds__(kGlobalThreads) global_stage_kernel(const double* x, const double* y, double* out,
                                                                       double ca, double cb, const double* rec,
                                                                       double dtB, double dtgB, int nlon, int nlat) {
@@ -384,7 +437,7 @@ __global__ void __launch_bounds__(kGlobalThreads) global_stage_kernel(const doub
     x2 = x[o + 2 * (size_t)P];
   }
   double o0, o1, o2;
-  stage_math<double, false>(z, rc, 0.0, dtB, dtgB, 0.0, ca, cb, x0, x1, x2, o0, o1, o2);
+  global_pt(z, rc, dtB, dtgB, ca, cb, x0, x1, x2, o0, o1, o2);
   out[o] = o0;
   out[o + P] = o1;
   out[o + 2 * (size_t)P] = o2;
@@ -460,8 +513,7 @@ __global__ void __launch_bounds__(kStepThreads) global_step_kernel(const double*
     double rc[8];
     load_rec8(rec + 8 * (j0 + r), rc);
     const bool x3 = ca != 0.0;
-    stage_math<double, false>(z, rc, 0.0, dtB, dtgB, 0.0, ca, cb, x3 ? X[xo] : 0.0, x3 ? X[xo + xp] : 0.0,
-                              x3 ? X[xo + 2 * xp] : 0.0, a, b, d);
+    global_pt(z, rc, dtB, dtgB, ca, cb, x3 ? X[xo] : 0.0, x3 ? X[xo + xp] : 0.0, x3 ? X[xo + 2 * xp] : 0.0, a, b, d);
   };
   points(3, [&](int r, int c) {
     int i = (i0 + c) % nlon;
@@ -980,6 +1032,14 @@ cudaError_t launch_restrict_level(const SubDesc* subs, int n_sub, int nlon, int 
                                   int g0, int g1, double* xb_a, int max_pts, cudaStream_t st) {
   dim3 grid(blocks_for(max_pts, 256, 64), n_sub);
   restrict_level_kernel<<<grid, 256, 0, st>>>(subs, nlon, nlat, glob, g0, g1, xb_a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_background_stage(const double* x, const double* y, double* out, double ca, double cb,
+                                    const RowConst* rows, double Bth, double gBth, double dt, int nlon, int nlat,
+                                    cudaStream_t st) {
+  dim3 grid((nlon + 127) / 128, nlat);
+  background_stage_kernel<<<grid, 128, 0, st>>>(x, y, out, ca, cb, rows, Bth, gBth, dt, nlon, nlat);
   return cudaGetLastError();
 }
 

@@ -80,6 +80,7 @@ struct SweepArgs {
   // the same constants rounded once to the state precision on the host, so
   // that the FP32 sweeps run no FP64 conversion per stage or level
   T dt_s, Bth_s, gBth_s, href_s;
+  T Bth_a, gBth_a;            // for the adjoint point functions (FP64: times dt)
   T isb2_s[3], musb2_s[3];    // 1 / sigma_b^2 and mu / sigma_b^2
   const ObsRec* obs;          // per-subdomain, per-level sorted
   const int* lvl_obs;         // obs ranges per (subdomain, level)
@@ -197,6 +198,7 @@ struct LvArgs {
   const T *tgt, *bnd, *gn_dx;
   const T *fw, *bw;           // row constants [nlat][8] (the records of sweep.cu)
   T dt, Bth, gBth, href;
+  T Bth_a, gBth_a;            // for the adjoint point functions (FP64: times dt)
   T isb2[3], musb2[3];
   int nlon, nlat;
   double lam_w;               // weight lambda of the observation term
@@ -293,8 +295,13 @@ cudaError_t launch_restrict_level(const SubDesc* subs, int n_sub, int nlon, int 
                                   int g0, int g1, double* xb_a, int max_pts, cudaStream_t st);
 
 // global model (whole sphere), FP64
-// rec: FP64 forward records of every row (fill_records of point.cuh, 8 doubles a
-// row); dtB, dtgB: dt Bth, dt g Bth
+// One stage, out = ca x + cb (y + dt F(y)), with the arithmetic of the
+// background forecast (see background_pass).
+cudaError_t launch_background_stage(const double* x, const double* y, double* out, double ca, double cb,
+                                    const RowConst* rows, double Bth, double gBth, double dt, int nlon, int nlat,
+                                    cudaStream_t st);
+// Model runs.  rec: records of every row (fill_global_record of point.cuh, 8
+// doubles a row); dtB, dtgB: dt Bth, dt g Bth.
 struct GlobalStepPlan {
   int tx = 0, ty = 0;         // tile of the step kernel; 0: one launch per stage
 };

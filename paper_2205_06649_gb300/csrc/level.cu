@@ -7,7 +7,7 @@
 // badly into GPCs, and neither the FP64 pipe (62-65 % of its rate over a sweep)
 // nor HBM (7-12 %) is busy.  Where all boxes together have enough points per
 // level, a stage of every box is one ordinary grid instead:
-//   * FP64: 24-47 FP64 instructions per point take 16 SM cycles per warp each;
+//   * FP64: 28-47 FP64 instructions per point take 16 SM cycles per warp each;
 //     the 15-36 loads of a point are a tenth of that, so plain loads through L1
 //     keep the FP64 pipe fed, and every SM works until the grid's end.  Bound:
 //     the FP64 pipe (about 90 % of its rate with the overlap terms counted).
@@ -541,10 +541,10 @@ __global__ void __launch_bounds__(kLvThreads, 4) lv_adj_kernel(const LvArgs<T> a
       point_of(z, j, zp);
       point_of(m, j, mp);
       if (K == 3)
-        adj_lambda_math<T, DEV>(zp, mp, rc, a.dt, a.Bth, a.gBth, a.href, wall, ll[0][j], ll[1][j], ll[2][j],
+        adj_lambda_math<T, DEV>(zp, mp, rc, a.dt, a.Bth_a, a.gBth_a, a.href, wall, ll[0][j], ll[1][j], ll[2][j],
                                 l2[0][j], l2[1][j], l2[2][j], o[0][j], o[1][j], o[2][j]);
       else
-        adj_stage_math<T, DEV>(zp, mp, rc, a.dt, a.Bth, a.gBth, a.href, wall, o[0][j], o[1][j], o[2][j]);
+        adj_stage_math<T, DEV>(zp, mp, rc, a.dt, a.Bth_a, a.gBth_a, a.href, wall, o[0][j], o[1][j], o[2][j]);
     }
     if (K == 3) {
       T x[3][V];

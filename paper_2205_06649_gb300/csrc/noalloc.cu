@@ -36,7 +36,7 @@ namespace {
 
 constexpr long long kMaxStateDoubles = 3LL * 512 * 256;   // one state of up to 512 x 256 points
 constexpr int kMaxRows = 1024;                            // latitude rows
-constexpr long long kRowDoubles = 8LL * kMaxRows;         // FP64 forward records (point.cuh)
+constexpr long long kRowDoubles = 8LL * kMaxRows;         // records of the global model (point.cuh)
 constexpr long long kScratchDoubles = 2 * kMaxStateDoubles + kRowDoubles;
 
 static __device__ __align__(256) double g_noalloc_scratch[kScratchDoubles];
@@ -88,8 +88,7 @@ __global__ void noalloc_rows_kernel(double* rec, int nlon, int nlat, double lat_
   r.tau = __ddiv_rn(tan(th), radius);
   r.BinvC = __ddiv_rn(Bth, r.c);
   r.gA = __dmul_rn(gravity, r.A);
-  double bw[8];
-  fill_records(r, cos(theta(min(j + 1, nlat - 1))), cos(theta(max(j - 1, 0))), dt, Bth, rec + 8 * j, bw);
+  fill_global_record(r, cos(theta(min(j + 1, nlat - 1))), cos(theta(max(j - 1, 0))), dt, Bth, rec + 8 * j);
 }
 
 }  // namespace

@@ -125,32 +125,7 @@ __device__ __forceinline__ void rhs_adj_pt(const Pt5<T>& z, const Pt5<T>& m, T A
   }
 }
 
-// d + dt F'(Z) d at one point (FP64 records, see euler_pt64).
-__device__ __forceinline__ void tangent_pt64(const Pt5<double>& z, const Pt5<double>& d, const double (&rc)[8],
-                                             double Bth, double gBth, double& oh, double& ou, double& ov) {
-  const double u = z.u, v = z.v, du = d.u, dv = d.v;
-  const double fu = __fma_rn(rc[2], u, rc[1]), Au = rc[0] * u, Bv = Bth * v, Ad = rc[0] * du, Bd = Bth * dv;
-  const double td = rc[2] * du;
-  ou = __fma_rn(-rc[3], d.hE - d.hW, d.u);
-  ou = __fma_rn(-Ad, z.uE - z.uW, ou);
-  ou = __fma_rn(-Au, d.uE - d.uW, ou);
-  ou = __fma_rn(-Bd, z.uN - z.uS, ou);
-  ou = __fma_rn(-Bv, d.uN - d.uS, ou);
-  ou = __fma_rn(fu, dv, ou);
-  ou = __fma_rn(td, v, ou);
-  ov = __fma_rn(-gBth, d.hN - d.hS, d.v);
-  ov = __fma_rn(-Ad, z.vE - z.vW, ov);
-  ov = __fma_rn(-Au, d.vE - d.vW, ov);
-  ov = __fma_rn(-Bd, z.vN - z.vS, ov);
-  ov = __fma_rn(-Bv, d.vN - d.vS, ov);
-  ov = __fma_rn(-fu, du, ov);
-  ov = __fma_rn(-td, u, ov);
-  oh = __fma_rn(-rc[0], __fma_rn(d.hE, z.uE, z.hE * d.uE) - __fma_rn(d.hW, z.uW, z.hW * d.uW), d.h);
-  oh = __fma_rn(-rc[4], __fma_rn(d.hN, z.vN, z.hN * d.vN), oh);
-  oh = __fma_rn(rc[5], __fma_rn(d.hS, z.vS, z.hS * d.vS), oh);
-}
-
-// Tangent-linear tendencies dF = F'(Z) dZ at one point (FP32 records).
+// Tangent-linear tendencies dF = F'(Z) dZ at one point.
 template <typename T, bool DEV>
 __device__ __forceinline__ void rhs_tl_pt(const Pt5<T>& z, const Pt5<T>& d, T A, T f, T tau, T BinvC, T gA,
                                           T cN, T cS, T Bth, T gBth, T href, T& dFh, T& dFu, T& dFv) {
@@ -204,41 +179,47 @@ __device__ __forceinline__ T overlap_term(T part, int c, T x0, T x1, T x2, T t0,
   return xfma((T)c, sq, part);
 }
 
-// FP64 forms.  The FP64 pipe issues one warp instruction in 16 cycles per SM
-// and bounds every FP64 sweep, so the point functions are written for the
-// fewest FP64 instructions: the row records and Bth, g Bth hold dt times the
-// constant, the cos ratios of the neighbour rows are folded into one constant
-// each, and every term is one fused multiply-add into the value that it
-// changes.  A stage takes 24 (first) or 30 instructions instead of 28 or 34, a
-// stage adjoint 38 instead of 45, lambda(n) 47 instead of 54.  Measured on the
-// medium workload (64 boxes of 72 x 36..40 points, clusters of 4 x 192
-// threads): forward 1.86 -> 1.64 ms, adjoint 2.67 -> 2.32 ms.
-// Records (per row j, N = row j + 1, S = row j - 1, walls mirrored):
-//   fw: dt A, dt f, dt tau, dt g A, dt Bth cN / c, dt Bth cS / c
-//   bw: dt A, dt f, dt tau, dt g A, dt Bth c / cN, dt Bth c / cS, 2 dt tau
-__host__ __device__ inline void fill_records(const RowConst& r, double cN, double cS, double dt, double Bth,
-                                             double* fw, double* bw) {
-  const double f[8] = {dt * r.A, dt * r.f, dt * r.tau, dt * r.gA, dt * Bth * cN / r.c, dt * Bth * cS / r.c, 0.0, 0.0};
-  const double b[8] = {dt * r.A, dt * r.f, dt * r.tau, dt * r.gA, dt * Bth * r.c / cN, dt * Bth * r.c / cS,
-                       2.0 * dt * r.tau, 0.0};
-  for (int q = 0; q < 8; ++q) {
-    fw[q] = f[q];
-    bw[q] = b[q];
-  }
-}
-// FP32: the constants themselves, rounded once.
-//   fw: A, f, tau, Bth / c, g A, cN, cS, 0;  bw: A, f, tau, g A, Bth c, 1 / cN, 1 / cS, 2 tau
-__host__ __device__ inline void fill_records(const RowConst& r, double cN, double cS, double, double Bth, float* fw,
-                                             float* bw) {
+// Row records of the sweeps (per row j, N = row j + 1, S = row j - 1, walls
+// mirrored):
+//   fw (both precisions): A, f, tau, Bth / c, g A, cN, cS, 0
+//   bw FP32: A, f, tau, g A, Bth c, 1 / cN, 1 / cS, 2 tau
+//   bw FP64: dt A, dt f, dt tau, dt g A, dt Bth c / cN, dt Bth c / cS, 2 dt tau, 0
+template <typename T>
+__host__ __device__ inline void fill_records(const RowConst& r, double cN, double cS, double dt, double Bth, T* fw,
+                                             T* bw) {
   const double f[8] = {r.A, r.f, r.tau, r.BinvC, r.gA, cN, cS, 0.0};
-  const double b[8] = {r.A, r.f, r.tau, r.gA, Bth * r.c, 1.0 / cN, 1.0 / cS, 2.0 * r.tau};
+  const double b32[8] = {r.A, r.f, r.tau, r.gA, Bth * r.c, 1.0 / cN, 1.0 / cS, 2.0 * r.tau};
+  const double b64[8] = {dt * r.A, dt * r.f, dt * r.tau, dt * r.gA, dt * Bth * r.c / cN, dt * Bth * r.c / cS,
+                         2.0 * dt * r.tau, 0.0};
   for (int q = 0; q < 8; ++q) {
-    fw[q] = (float)f[q];
-    bw[q] = (float)b[q];
+    fw[q] = (T)f[q];
+    bw[q] = (T)(sizeof(T) == 8 ? b64[q] : b32[q]);
   }
 }
 
-// Y + dt F(Y) at one point.
+// FP64 forms for the fewest FP64 instructions.  The FP64 pipe issues one warp
+// instruction in 16 cycles per SM and bounds every FP64 sweep.  The records
+// (and Bth, g Bth) hold dt times the constant, the cos ratios of the neighbour
+// rows are folded into one constant each, and every term is one fused
+// multiply-add into the value that it changes: a stage adjoint takes 38
+// instructions instead of 45, lambda(n) 47 instead of 54 (medium workload, 64
+// boxes of 72 x 36..40 points in clusters of 4 x 192 threads: adjoint 2.67 ->
+// 2.32 ms).  The box model's forward stages keep the order of rhs_pt: their
+// rounding of h, some 1e-13 of a misfit, is what an analysis amplifies, and a
+// second order of roundings would show in it at 1e-10.
+
+// Y + dt F(Y) at one point (global model runs): 24 instructions, from rec =
+// dt A, dt f, dt tau, dt g A, dt Bth cN / c, dt Bth cS / c and dt Bth, dt g Bth.
+__host__ __device__ inline void fill_global_record(const RowConst& r, double cN, double cS, double dt, double Bth,
+                                                   double* rec) {
+  rec[0] = dt * r.A;
+  rec[1] = dt * r.f;
+  rec[2] = dt * r.tau;
+  rec[3] = dt * r.gA;
+  rec[4] = dt * Bth * cN / r.c;
+  rec[5] = dt * Bth * cS / r.c;
+  rec[6] = rec[7] = 0.0;
+}
 __device__ __forceinline__ void euler_pt64(const Pt5<double>& y, const double (&rc)[8], double Bth, double gBth,
                                            double& oh, double& ou, double& ov) {
   const double fu = xfma(rc[2], y.u, rc[1]), Au = xmul(rc[0], y.u), Bv = xmul(Bth, y.v);
@@ -295,15 +276,11 @@ __device__ __forceinline__ void adjoint_pt64(const Pt5<double>& z, const Pt5<dou
 template <typename T, bool DEV>
 __device__ __forceinline__ void stage_math(const Pt5<T>& y, const T (&rc)[8], T dt, T Bth, T gBth, T href, T cx,
                                            T cy, T xh, T xu, T xv, T& o0, T& o1, T& o2) {
-  if constexpr (sizeof(T) == 8) {
-    euler_pt64(y, rc, Bth, gBth, o0, o1, o2);
-  } else {
-    T Fh, Fu, Fv;
-    rhs_pt<T, DEV>(y, rc[0], rc[1], rc[2], rc[3], rc[4], rc[5], rc[6], Bth, gBth, href, Fh, Fu, Fv);
-    o0 = xfma(dt, Fh, y.h);
-    o1 = xfma(dt, Fu, y.u);
-    o2 = xfma(dt, Fv, y.v);
-  }
+  T Fh, Fu, Fv;
+  rhs_pt<T, DEV>(y, rc[0], rc[1], rc[2], rc[3], rc[4], rc[5], rc[6], Bth, gBth, href, Fh, Fu, Fv);
+  o0 = xfma(dt, Fh, y.h);
+  o1 = xfma(dt, Fu, y.u);
+  o2 = xfma(dt, Fv, y.v);
   if (cy != (T)1) {
     o0 = xmul(cy, o0);
     o1 = xmul(cy, o1);

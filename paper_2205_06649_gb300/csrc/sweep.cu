@@ -1164,7 +1164,7 @@ __global__ void __launch_bounds__(kStripeAdjThreads, 1) adj_kernel(SweepArgs<T> 
   // Gauss-Newton products, which take no targets)
   const bool pre_tg = g.tgb && a.mu != 0.0 && !a.gn_dx && !a.yforce;
   for (int i = threadIdx.x; i < g.BUF; i += blockDim.x) Lp[i] = (T)0;
-  const T dt = a.dt_s, Bth = a.Bth_s, gBth = a.gBth_s, href = a.href_s;
+  const T dt = a.dt_s, Bth = a.Bth_a, gBth = a.gBth_a, href = a.href_s;
   const int wall_s = (g.flags & F_SWALL) ? 1 : 0;
   const int wall_n = (g.flags & F_NWALL) ? 2 : 0;
   const size_t lvl_sz = (size_t)3 * g.ny * g.d.nxp;
@@ -1400,16 +1400,10 @@ __device__ void stage_tl(const SweepArgs<T>& a, const Geo<T>& g, const RowSmem<T
     Pt5<T> z, d;
     load5(Y, o, g.P, Lay<T>::CS, g.RS, z);
     load5(DY, o, g.P, Lay<T>::CS, g.RS, d);
-    T xh, xu, xv;
-    ld3(DX, o, g.P, xh, xu, xv);
-    if constexpr (!DEV) {
-      T dh, du, dv;
-      tangent_pt64(z, d, rc, Bth, gBth, dh, du, dv);
-      st3(dout, o, g.P, cx * xh + cy * dh, cx * xu + cy * du, cx * xv + cy * dv);
-      continue;
-    }
     T Fh, Fu, Fv;
     rhs_tl_pt<T, DEV>(z, d, rc[0], rc[1], rc[2], rc[3], rc[4], rc[5], rc[6], Bth, gBth, href, Fh, Fu, Fv);
+    T xh, xu, xv;
+    ld3(DX, o, g.P, xh, xu, xv);
     st3(dout, o, g.P, cx * xh + cy * (d.h + dt * Fh), cx * xu + cy * (d.u + dt * Fu),
         cx * xv + cy * (d.v + dt * Fv));
   }
@@ -2085,7 +2079,7 @@ __global__ void __launch_bounds__(kDeepThreads, 1) adj_deep_kernel(SweepArgs<flo
   cp_async_commit();
   const size_t pl = (size_t)g.ny * g.d.nxp;
   const size_t lvl = 3 * pl;
-  const float dt = a.dt_s, Bth = a.Bth_s, gBth = a.gBth_s, href = a.href_s;
+  const float dt = a.dt_s, Bth = a.Bth_a, gBth = a.gBth_a, href = a.href_s;
   // lambda(b) = forcing(b) on own rows
   load_rows_async2(g, X, a.traj + g.d.traj_off + (size_t)g.L * lvl, 0, g.Rn - 1);
   cp_async_commit();
