@@ -119,7 +119,7 @@ struct SweepArgs {
 // threads per SM), 1024 on the FP64 path (64 registers, one CTA of 1024 or two
 // of 512 per SM).  The stripe adjoint takes up to 1024 threads (64 registers).
 template <typename T> constexpr int max_threads_forward() { return sizeof(T) == 4 ? 384 : 1024; }
-template <typename T> constexpr int min_blocks_forward() { return sizeof(T) == 4 ? 4 : 1; }
+template <typename T> constexpr int min_blocks_forward() { return sizeof(T) == 4 ? 2 : 1; }
 constexpr int kStripeAdjThreads = 1024;
 
 // ---- programmatic dependent launch ----
