@@ -145,6 +145,7 @@ struct dd4dv_ctx {
   LvPlan lv;
   LvTile* lv_tiles = nullptr;
   int *lv_boxes = nullptr, *lv_tile_off = nullptr;
+  long long* lv_box_off = nullptr;
   void *lv_rec = nullptr, *lv_state = nullptr;
   double *lv_acc_m = nullptr, *lv_acc_o = nullptr;
   long long lv_elems = 0;     // elements of one level of every box
@@ -388,6 +389,8 @@ LvArgs<T> level_args(dd4dv_ctx* ctx, const int* active, int av) {
   LvArgs<T> a{};
   a.tiles = ctx->lv_tiles;
   a.boxes = ctx->lv_boxes;
+  a.box_off = ctx->lv_box_off;
+  a.err = ctx->err_d;
   a.subs = ctx->subs_d;
   a.mu_on = ctx->dec.mu != 0.0;
   a.traj = static_cast<T*>(ctx->traj);
@@ -947,23 +950,35 @@ void tune_checkpoint(dd4dv_ctx* ctx) {
 //         719,000 in 256 boxes 2.52 / 1.96; 1.2 million in 128 boxes 8.6 / 3.0
 constexpr long long kLvMinPoints64 = 65000, kLvMinPoints32 = 350000;
 
+// The pipelined FP32 adjoint kernels run where every box is at most kRingMaxNx
+// wide (a tile of 224 thread-points has three rows or more) and each of two
+// CTAs per SM has kRingMinTiles tiles or more: with fewer, the ring's start and
+// the uneven last tiles cost more than the waits for memory.  Measured, plain
+// against pipelined adjoint of 32 steps (ms): boxes of 72 x 72 points, 2.5 tiles
+// a CTA 1.10 / 1.13, 5 2.00 / 1.80, 10 4.29 / 3.32; of 136 x 72, 2.5 0.94 / 1.03,
+// 5 1.78 / 1.72, 10 3.97 / 3.02; of 32 x 28, 6.7 3.01 / 2.75.
+constexpr int kRingMaxNx = kRingPoints / 3 * 4, kRingMinTiles = 4;
+
 // Tiles and scratch of the level sweeps.  Leaves ctx->lv_tiles null where they
-// do not apply: too few points, boxes no wider than a thread's columns, a grid
+// do not apply: too few points, boxes no wider than a thread's columns or of a
+// single row (a thread has one ghost row at most), a grid
 // whose level does not fit 32-bit offsets, or no memory for the scratch.
 template <typename T>
 void level_plan(dd4dv_ctx* ctx, const std::vector<SubDesc>& subs, const std::vector<int>& lvl_obs) {
   constexpr int V = lv_width<T>();
   const int nlon = ctx->m.nlon, nlat = ctx->m.nlat, n_sub = (int)subs.size();
   long long pts = 0;
-  int maxL = 0, min_nx = 1 << 30;
+  int maxL = 0, min_nx = 1 << 30, max_nx = 0, min_ny = 1 << 30;
   for (const SubDesc& d : subs) {
     pts += (long long)d.nx * d.ny;
     maxL = std::max(maxL, d.b - d.a);
     min_nx = std::min(min_nx, d.nx);
+    max_nx = std::max(max_nx, d.nx);
+    min_ny = std::min(min_ny, d.ny);
   }
   long long least = sizeof(T) == 4 ? kLvMinPoints32 : kLvMinPoints64;
   if (const char* e = std::getenv("DD4DV_LEVEL_MIN_POINTS")) least = std::atoll(e);   // override (tests)
-  if (pts < least || maxL < 1 || min_nx <= V || 3LL * nlon * nlat >= (1LL << 31)) return;
+  if (pts < least || maxL < 1 || min_nx <= V || min_ny < 2 || 3LL * nlon * nlat >= (1LL << 31)) return;
   auto& L = ctx->dec_allocs;
   std::vector<int> order(n_sub);
   for (int s = 0; s < n_sub; ++s) order[s] = s;
@@ -971,10 +986,12 @@ void level_plan(dd4dv_ctx* ctx, const std::vector<SubDesc>& subs, const std::vec
                    [&](int x, int y) { return subs[x].b - subs[x].a > subs[y].b - subs[y].a; });
   // thread-points per thread: more than one saves set-up where there are many CTAs all the same
   const int iters = pts > 2000000 ? (sizeof(T) == 4 ? 4 : 2) : 1;
-  std::vector<LvTile> tiles;
+  std::vector<LvTile> tiles, ring_tiles;
   std::vector<int> tile_off(2 * n_sub);
+  std::vector<long long> box_off(n_sub);
   LvPlan g;
   g.n_tile.assign(maxL, 0);
+  g.n_ring.assign(maxL, 0);
   g.n_box.assign(maxL + 1, 0);
   g.obs.assign(maxL + 1, 0);
   long long elems = 0;
@@ -1004,7 +1021,7 @@ void level_plan(dd4dv_ctx* ctx, const std::vector<SubDesc>& subs, const std::vec
     t.stg_off = d.stg_off;
     t.stg1_off = d.stg1_off;
     t.ctrl_off = d.ctrl_off;
-    t.lv_off = elems;
+    t.lv_off = box_off[s] = elems;
     elems += 3LL * d.ny * d.nxp;
     // equal tiles of whole warps
     const int np = t.nq * d.ny;
@@ -1018,12 +1035,53 @@ void level_plan(dd4dv_ctx* ctx, const std::vector<SubDesc>& subs, const std::vec
       tiles.push_back(t);
     }
     for (int l = 0; l < t.L; ++l) g.n_tile[l] += nt;
+    if (max_nx <= kRingMaxNx) {   // equal tiles of whole rows, a thread-point per computing thread
+      int m = (d.ny + kRingPoints / t.nq - 1) / (kRingPoints / t.nq);
+      const int R = (d.ny + m - 1) / m;
+      m = (d.ny + R - 1) / R;
+      for (int q = 0; q < m; ++q) {
+        t.p0 = q * R * t.nq;
+        t.p1 = std::min((q + 1) * R * t.nq, np);
+        ring_tiles.push_back(t);
+      }
+      for (int l = 0; l < t.L; ++l) g.n_ring[l] += m;
+      // states with a ghost row on either side, states without, row constants
+      // and ghost columns, second level of blended ghosts (Slot of level.cu)
+      const int full = 3 * (R + 2) * d.nxp, own = 3 * R * d.nxp, cols = (6 * R + 3) / 4 * 4, rc = 8 * R;
+      const int need[3] = {2 * full + 2 * cols + rc + 6 * d.nxp, 2 * full + cols + rc, 2 * full + 2 * own + cols + rc};
+      for (int q = 0; q < 3; ++q) g.ring[q].slot_floats = std::max(g.ring[q].slot_floats, need[q]);
+    }
     for (int l = 0; l <= t.L; ++l) {
       ++g.n_box[l];
       if (lvl_obs[d.obs_lvl + l] != lvl_obs[d.obs_lvl + l + 1]) g.obs[l] = 1;
     }
   }
   g.tiles = (int)tiles.size();
+  // Pipelined adjoint kernels: as many resident CTAs as the registers allow,
+  // with two slots or more (up to four) in the shared memory that each has.
+  if (sizeof(T) == 4 && !ring_tiles.empty()) {
+    int sms = 0, dev = 0;
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    long long ring_min = kRingMinTiles;
+    if (const char* e = std::getenv("DD4DV_RING_MIN_TILES")) ring_min = std::atoll(e);   // override (tests)
+    for (int q = 0; q < 3 && g.n_ring[0] >= ring_min * 2 * sms; ++q) {
+      LvRing& r = g.ring[q];
+      r.own_floats = q == 2 ? 12 * kRingPoints : 0;
+      for (int c = 2; c > 0 && !r.slots; --c) {
+        const int bytes = 228 * 1024 / c - 1024 - 1536;   // less the system's and the static part
+        const int fit = (bytes / 4 - r.own_floats) / r.slot_floats;
+        if (fit >= 2) {
+          r.slots = std::min(fit, 4);
+          r.ctas = c * sms;
+        }
+      }
+    }
+    for (const LvRing& r : g.ring)
+      if (!r.slots) ring_tiles.clear();
+    if (ring_tiles.empty())
+      for (LvRing& r : g.ring) r = LvRing{};
+  }
   // row constants, rounded once to the state precision (as load_rows of sweep.cu)
   std::vector<T> rec(16 * (size_t)nlat);
   for (int j = 0; j < nlat; ++j) {
@@ -1035,19 +1093,26 @@ void level_plan(dd4dv_ctx* ctx, const std::vector<SubDesc>& subs, const std::vec
   size_t free_b = 0, total_b = 0;
   CK(cudaMemGetInfo(&free_b, &total_b));
   const size_t slots = tiles.size() * kLvThreads;
-  const size_t need = 5 * (size_t)elems * sizeof(T) + tiles.size() * sizeof(LvTile) +
+  const size_t need = 5 * (size_t)elems * sizeof(T) + (tiles.size() + ring_tiles.size()) * sizeof(LvTile) +
                       slots * sizeof(double) + (64u << 20);
   if (need > free_b) return;
   LvTile* td = dalloc<LvTile>(ctx, tiles.size(), &L);
   ctx->lv_boxes = dalloc<int>(ctx, n_sub, &L);
   ctx->lv_tile_off = dalloc<int>(ctx, 2 * n_sub, &L);
+  ctx->lv_box_off = dalloc<long long>(ctx, n_sub, &L);
   ctx->lv_rec = dalloc<T>(ctx, rec.size(), &L);
   ctx->lv_state = dalloc<T>(ctx, 5 * (size_t)elems, &L);
   ctx->lv_acc_m = dalloc<double>(ctx, slots, &L);
   ctx->lv_acc_o = dalloc<double>(ctx, n_sub, &L);
   h2d(ctx, td, tiles.data(), tiles.size() * sizeof(LvTile));
+  if (!ring_tiles.empty()) {
+    LvTile* rd = dalloc<LvTile>(ctx, ring_tiles.size(), &L);
+    h2d(ctx, rd, ring_tiles.data(), ring_tiles.size() * sizeof(LvTile));
+    g.ring_tiles = rd;
+  }
   h2d(ctx, ctx->lv_boxes, order.data(), n_sub * sizeof(int));
   h2d(ctx, ctx->lv_tile_off, tile_off.data(), 2 * n_sub * sizeof(int));
+  h2d(ctx, ctx->lv_box_off, box_off.data(), n_sub * sizeof(long long));
   h2d(ctx, ctx->lv_rec, rec.data(), rec.size() * sizeof(T));
   CK(cudaMemsetAsync(ctx->lv_state, 0, 5 * (size_t)elems * sizeof(T), ctx->st));
   CK(cudaStreamSynchronize(ctx->st));   // the host tables end with this call

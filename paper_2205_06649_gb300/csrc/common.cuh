@@ -176,9 +176,17 @@ struct LvTile {
   long long traj_off, ptraj_off, stg_off, stg1_off, ctrl_off;
   long long lv_off;           // one-level scratch offset (elements of T): [3][ny][nxp]
 };
+// A pipelined kernel's CTAs (at most), slots, floats per slot and before the
+// slots; slots = 0: the plain kernel runs.
+struct LvRing {
+  int ctas = 0, slots = 0, slot_floats = 0, own_floats = 0;
+};
 // The tiles of every box, longest window first.
 struct LvPlan {
   int tiles = 0;
+  LvRing ring[3];                       // adjoint phases 1, 2, 3
+  const LvTile* ring_tiles = nullptr;   // their tiles: whole rows
+  std::vector<int> n_ring;              // as n_tile
   std::vector<int> n_tile;    // per step l: tiles of the boxes that take it (a prefix)
   std::vector<int> n_box;     // per level l: boxes that have it (a prefix of the box list)
   std::vector<char> obs;      // per level l: some box has observations there
@@ -187,8 +195,11 @@ template <typename T>
 struct LvArgs {
   const LvTile* tiles;
   const int* boxes;           // longest window first
+  const long long* box_off;   // lv_off of every box
   const SubDesc* subs;
   int n_tile;
+  int n_cta, slots, slot_floats;   // pipelined kernels: CTAs, ring
+  int* err;                   // device error word (0 = ok)
   int l;                      // step / level
   int terms;                  // forward: accumulate the observation and overlap terms
   int skip1;                  // first stage recomputed only where x1 is not stored
@@ -217,6 +228,8 @@ struct LvArgs {
 // accesses), FP64 threads one.
 template <typename T> __host__ __device__ constexpr int lv_width() { return sizeof(T) == 4 ? 4 : 1; }
 constexpr int kLvThreads = 128;
+constexpr int kRingThreads = 256;   // pipelined kernels: a thread-point for each of the
+constexpr int kRingPoints = 224;    // first 224 threads, the last warp copies
 template <typename T>
 cudaError_t launch_level_forward(const LvArgs<T>& a, const LvPlan& g, cudaStream_t st, long long* launches);
 template <typename T>

@@ -12,10 +12,12 @@
 //     keep the FP64 pipe fed, and every SM works until the grid's end.  Bound:
 //     the FP64 pipe (about 90 % of its rate with the overlap terms counted).
 //   * FP32: a thread takes four neighbouring columns with 16-byte loads.  Bound:
-//     latency of the loads (HBM at 45-50 % of its measured rate); groups of boxes
-//     sized for L2, strips marching north with rows kept in registers, one or
-//     two columns a thread at 1.7x the warps, and a whole step per launch with
-//     rows in shared memory all measured slower or equal.
+//     latency of the loads (forward HBM at 55 % of its measured rate); groups of
+//     boxes sized for L2, strips marching north with rows kept in registers, one
+//     or two columns a thread at 1.7x the warps, and a whole step per launch with
+//     rows in shared memory (11.9 / 17.9 ms for 9.6 / 17.6 of the batching
+//     workload: 1.7x the instructions) all measured slower or equal.  The adjoint
+//     of many tiles runs pipelined (lv_ring_adj_kernel).
 // A tile is a run of points of one box (flat over rows, so that every lane has
 // one); tiles are ordered longest window first, so the boxes still running at
 // step l are a prefix and the grid shrinks with them.  CTAs of 128 threads: with
@@ -26,16 +28,19 @@
 // Measured against the cluster sweeps with the launch shapes that the library
 // chooses (forward / adjoint, ms):
 //   batching workload (512 boxes, 3.9e8 points x steps), FP32: 15.8 / 30.7 ->
-//     9.6 / 17.6; FP64: 102.8 / 156.7 -> 66.6 / 93.6 (a part of it from the FP64
-//     point functions, which the level sweeps alone ran at 77 / 112 without)
-//   one 128-step window of the large workload (256 boxes), FP32: 15.4 / 29.6 -> 9.3 / 17.7
+//     9.6 / 13.5; FP64: 102.8 / 156.7 -> 76.0 / 92.5 (a part of it from the FP64
+//     adjoint's point function, without which the level sweeps took 77 / 112)
+//   one 128-step window of the large workload (256 boxes), FP32: 15.4 / 29.6 -> 9.3 / 13.9
 //   differentiation workload (FP32, 16-step checkpoints): 1.68 / 4.91 -> 1.72 / 3.18
-//   medium workload (FP64, 64 boxes, 184,000 points): 1.64 / 2.31 -> 1.64 / 2.22
+//   medium workload (FP64, 64 boxes, 184,000 points): 1.82 / 2.31 -> 1.82 / 2.16
 //
 // The arithmetic per point is that of sweep.cu (point.cuh), so trajectories,
 // stage states and gradients are the same bit for bit; J differs by the order
 // of its partial sums.
 #include "point.cuh"
+
+#include <algorithm>
+#include <cstdint>
 
 namespace dd4dv {
 
@@ -583,10 +588,466 @@ __global__ void __launch_bounds__(kLvThreads) lv_export_kernel(const LvArgs<T> a
   }
 }
 
+// ---- pipelined adjoint phases (FP32) ----
+// lv_adj_kernel holds its 30 loads in registers, a few at a time, and waits for
+// each batch (120 registers, 16 warps an SM, 7.9 of 12.5 cycles an instruction
+// spent waiting for memory, HBM at 30-39 % of its rate).  Here CTAs stay and
+// take tile after tile of whole rows (one thread-point for each of 224
+// threads), and a warp of its own copies the states of the tiles ahead into a
+// ring of slots in shared memory: bulk copies for the rows and their constants,
+// 4-byte copies for the ghosts, one barrier a slot, no barrier between the
+// computing warps.  What is in flight no longer depends on the registers.
+// Bound: instruction issue (45-48 % of the slots, 560 instructions for a warp's
+// 128 points) and the wait for a slot.  Phases 1, 2, 3 of 2.9 million points:
+// 40.6, 39.5, 63.8 -> 30.7, 27.4, 57.3 us; adjoint sweep of the batching
+// workload 17.6 -> 13.5 ms, of a 128-step window of the large workload 17.7 ->
+// 13.9 ms.  With the copies made by a computing warp and a CTA barrier a tile
+// the same sweep took 16.7 ms; the row constants read through L1 (small beside
+// the slots) cost another 3 %.  The forward stages, which hold half as much in
+// registers, gained nothing from it (9.6 -> 12.3 ms) and stay plain.
+constexpr int kRingWait = 1 << 20;   // polls before a copy counts as lost
+constexpr int kDescs = 8;            // tile descriptors in shared memory
+constexpr int kRingSlots = 4;        // at most
+
+__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void ring_copy(void* dst, const void* src, int bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   smem_addr(dst)),
+               "l"(src), "r"(bytes), "r"(smem_addr(bar))
+               : "memory");
+}
+__device__ __forceinline__ void copy4(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ bool ring_wait(uint64_t* bar, unsigned parity) {
+  for (int i = 0; i < kRingWait; ++i) {
+    unsigned ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.b32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_addr(bar)), "r"(parity)
+        : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+
+// A slot: NF states with a ghost row on either side, NO states without, with
+// BL (ghosts blended from two boundary levels) the second level's rows beyond
+// the box, the rows' constants, and the ghost columns [level][side][v][row].
+template <int NF, int NO, bool BL>
+struct Slot {
+  float* base;
+  int R, nxp;
+  __device__ __forceinline__ int full() const { return (R + 2) * nxp; }   // plane of a state with ghost rows
+  __device__ __forceinline__ int own() const { return R * nxp; }
+  __device__ __forceinline__ float* state(int i) const {
+    return base + (i < NF ? 3 * i * full() : 3 * NF * full() + 3 * (i - NF) * own());
+  }
+  __device__ __forceinline__ float* rows2() const { return base + 3 * NF * full() + 3 * NO * own(); }
+  __device__ __forceinline__ float* rec() const { return rows2() + (BL ? 6 * nxp : 0); }   // row constants
+  __device__ __forceinline__ float* cols() const { return rec() + 8 * R; }
+};
+template <int NF, int NO, bool BL>
+__device__ __forceinline__ Slot<NF, NO, BL> slot_of(const LvTile& t, float* base) {
+  return Slot<NF, NO, BL>{base, mdiv(t.p1 - t.p0, t.mq), t.nxp};
+}
+
+// Starts the copies of tile t (one warp): src(i) is state i, B0 (B1 = B0 + G
+// with BL) the boundary level of the first state's ghosts.
+template <int NF, int NO, bool BL, typename S>
+__device__ __forceinline__ void ring_issue(const LvArgs<float>& a, const LvTile& t, float* base, uint64_t* bar,
+                                           bool skip, const float* rec, const float* B0, S&& src) {
+  const int lane = threadIdx.x & 31;
+  const Slot<NF, NO, BL> sl = slot_of<NF, NO, BL>(t, base);
+  const int r0 = mdiv(t.p0, t.mq), r1 = r0 + sl.R, ra = max(r0 - 1, 0), rb = min(r1 + 1, t.ny);
+  const int bf = (rb - ra) * t.nxp * 4, bo = sl.R * t.nxp * 4, pl = t.ny * t.nxp;
+  if (lane == 0) {
+    const int tx = skip ? 0 : 3 * (NF * bf + NO * bo) + 32 * sl.R;
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(tx) : "memory");
+  }
+  __syncwarp();
+  if (!skip) {
+    if (lane < 3 * (NF + NO)) {
+      const int i = lane / 3, v = lane - 3 * i;
+      const float* s = src(i) + v * pl;
+      if (i < NF) ring_copy(sl.state(i) + v * sl.full() + (ra - r0 + 1) * t.nxp, s + ra * t.nxp, bf, bar);
+      else ring_copy(sl.state(i) + v * sl.own(), s + r0 * t.nxp, bo, bar);
+    } else if (lane == 31) {
+      ring_copy(sl.rec(), rec + 8 * (t.j0 + r0), 32 * sl.R, bar);
+    }
+    const int pg = a.nlat * a.nlon, G = 3 * pg;
+    if (!(t.flags & F_PERIODIC)) {
+      float* g = sl.cols();
+      for (int r = lane; r < sl.R; r += 32) {
+        const float* b = B0 + (t.j0 + r0 + r) * a.nlon;
+#pragma unroll
+        for (int v = 0; v < 3; ++v) {
+          copy4(g + v * sl.R + r, b + v * pg + t.iw);
+          copy4(g + (3 + v) * sl.R + r, b + v * pg + t.ie);
+          if (BL) {
+            copy4(g + (6 + v) * sl.R + r, b + G + v * pg + t.iw);
+            copy4(g + (9 + v) * sl.R + r, b + G + v * pg + t.ie);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {   // rows beyond the box
+      if (side ? r1 < t.ny : r0 > 0) continue;
+      if (t.flags & (side ? F_NWALL : F_SWALL)) continue;
+      const float* b = B0 + (t.j0 + (side ? t.ny : -1)) * a.nlon;
+      float* d = sl.state(0) + (side ? sl.R + 1 : 0) * t.nxp;
+      for (int k = lane; k < t.nx; k += 32) {
+        int i = t.i0 + k;
+        if (i >= a.nlon) i -= a.nlon;
+#pragma unroll
+        for (int v = 0; v < 3; ++v) {
+          copy4(d + v * sl.full() + k, b + v * pg + i);
+          if (BL) copy4(sl.rows2() + (3 * side + v) * t.nxp + k, b + G + v * pg + i);
+        }
+      }
+    }
+  }
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_addr(bar)) : "memory");
+}
+
+// The patch of the state in slot sl, ghosts as in load_state_patch.
+template <int NF, int NO, bool BL>
+__device__ __forceinline__ void ring_state(const LvTile& t, const Slot<NF, NO, BL>& sl, int rr, int r, int k,
+                                           Patch<float, 4>& z) {
+  const bool west = k == 0, east = k + 4 >= t.nx, north = r == t.ny - 1, south = r == 0;
+  const bool per = t.flags & F_PERIODIC;
+  const float* y = sl.state(0) + (rr + 1) * t.nxp + k;
+  const float *w = y - 1, *e = y + 4;
+  int sw = sl.full(), se = sw;
+  if (west) {
+    w = per ? y + t.nx - 1 : sl.cols() + rr;
+    sw = per ? sw : sl.R;
+  }
+  if (east) {
+    e = per ? y - k : sl.cols() + 3 * sl.R + rr;
+    se = per ? se : sl.R;
+  }
+#pragma unroll
+  for (int v = 0; v < 3; ++v) {
+    ldv<float, 4>(y + v * sl.full(), &z.c[v][1]);
+    z.c[v][0] = w[v * sw];
+    z.c[v][5] = e[v * se];
+    ldv<float, 4>(y + v * sl.full() + t.nxp, z.n[v]);
+    ldv<float, 4>(y + v * sl.full() - t.nxp, z.s[v]);
+  }
+  if (BL && !per && (west || east)) {
+    const float* g = sl.cols() + (west ? 6 : 9) * sl.R + rr;
+#pragma unroll
+    for (int v = 0; v < 3; ++v) {
+      const float b = xfma(0.5f, west ? z.c[v][0] : z.c[v][5], xmul(0.5f, g[v * sl.R]));
+      if (west) z.c[v][0] = b;
+      else z.c[v][5] = b;
+    }
+  }
+  if (east) {   // column nx inside the four columns
+    const int je = t.nx - k + 1;
+#pragma unroll
+    for (int v = 0; v < 3; ++v)
+#pragma unroll
+      for (int j = 2; j < 5; ++j)
+        if (j == je) z.c[v][j] = z.c[v][5];
+  }
+  if (north || south) {
+    const bool wall = t.flags & (north ? F_NWALL : F_SWALL);
+#pragma unroll
+    for (int v = 0; v < 3; ++v) {
+      float g[4];
+      if (BL && !wall) ldv<float, 4>(sl.rows2() + (north ? 3 + v : v) * t.nxp + k, g);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        float x = north ? z.n[v][j] : z.s[v][j];
+        if (wall) x = v == 2 ? -z.c[v][j + 1] : z.c[v][j + 1];
+        else if (BL) x = xfma(0.5f, x, xmul(0.5f, g[j]));
+        if (north) z.n[v][j] = x;
+        else z.s[v][j] = x;
+      }
+    }
+  }
+}
+// The patch of the adjoint state in slot sl, ghosts as in load_adjoint_patch.
+template <int NF, int NO, bool BL>
+__device__ __forceinline__ void ring_adjoint(const LvTile& t, const Slot<NF, NO, BL>& sl, int rr, int r, int k,
+                                             Patch<float, 4>& z) {
+  const bool west = k == 0, east = k + 4 >= t.nx, north = r == t.ny - 1, south = r == 0;
+  const bool per = t.flags & F_PERIODIC;
+  const float* y = sl.state(1) + (rr + 1) * t.nxp + k;
+  const float* w = west ? y + t.nx - 1 : y - 1;
+  const float* e = east ? y - k : y + 4;
+  const int je = t.nx - k + 1;
+#pragma unroll
+  for (int v = 0; v < 3; ++v) {
+    const int o = v * sl.full();
+    ldv<float, 4>(y + o, &z.c[v][1]);
+    const float we = w[o], ee = e[o];
+    z.c[v][0] = west && !per ? 0.f : we;
+    const float x = east && !per ? 0.f : ee;
+    z.c[v][5] = x;
+#pragma unroll
+    for (int j = 2; j < 5; ++j)
+      if (east && j == je) z.c[v][j] = x;
+    ldv<float, 4>(y + o + t.nxp, z.n[v]);
+    ldv<float, 4>(y + o - t.nxp, z.s[v]);
+  }
+  if (north || south) {
+#pragma unroll
+    for (int v = 0; v < 3; ++v)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (north) z.n[v][j] = 0.f;
+        if (south) z.s[v][j] = 0.f;
+      }
+  }
+}
+
+// The CTA's tiles b, b + n_cta, ...  The last warp copies: issue(t, slot base, barrier) starts a tile's copies.
+// The others compute, each at its own pace: body(t, slot base, next, wait), which calls wait() before it
+// reads the slot; next is the CTA's next tile or null.
+template <typename I, typename B>
+__device__ __forceinline__ void ring_run(const LvArgs<float>& a, float* smem, I&& issue, B&& body) {
+  __shared__ __align__(16) LvTile desc[kDescs];
+  __shared__ uint64_t full[kRingSlots], empty[kRingSlots];
+  static_assert(sizeof(LvTile) % 16 == 0, "copied in 16-byte pieces");
+  constexpr int kWords = sizeof(LvTile) / 4, kAhead = 3;   // descriptors ahead of the tile whose copies start
+  static_assert(kDescs >= kRingSlots + kAhead + 1, "a descriptor stays until its tile is done");
+  const int n = (a.n_tile - (int)blockIdx.x + a.n_cta - 1) / a.n_cta, S = a.slots;
+  auto tile = [&](int j) { return (int)blockIdx.x + j * a.n_cta; };
+  for (int i = threadIdx.x; i < min(kAhead, n) * kWords; i += kRingThreads)
+    reinterpret_cast<int*>(desc)[i] = reinterpret_cast<const int*>(a.tiles + tile(i / kWords))[i % kWords];
+  if (threadIdx.x < S) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 33;" ::"r"(smem_addr(full + threadIdx.x)) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(empty + threadIdx.x)),
+                 "r"(kRingPoints / 32)
+                 : "memory");
+  }
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  asm volatile("fence.proxy.async;" ::: "memory");
+  __syncthreads();
+  grid_wait();
+  grid_release();
+  if (threadIdx.x >= kRingPoints) {
+    const int lane = threadIdx.x & 31;
+    asm volatile("fence.proxy.async;" ::: "memory");   // earlier grids' stores, before the bulk copies read them
+    int j = 0;
+    for (; j < n; ++j) {
+      const int slot = j % S;
+      if (j >= S && !ring_wait(empty + slot, (unsigned)(j / S - 1) & 1u)) break;
+      // one copy group a tile, with descriptor j + kAhead in it: all but the newest are
+      // complete, so descriptors up to j + 1 are there before full[slot] can be
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+      __syncwarp();
+      if (j + kAhead < n && lane < (int)sizeof(LvTile) / 16)
+        copy16(reinterpret_cast<char*>(desc + (j + kAhead) % kDescs) + 16 * lane,
+               reinterpret_cast<const char*>(a.tiles + tile(j + kAhead)) + 16 * lane);
+      issue(desc[j % kDescs], smem + (size_t)slot * a.slot_floats, full + slot);
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (j < n) {   // a wait ran out: report, wait for the copies that were started
+      if (lane == 0) atomicExch(a.err, 3);
+      for (int q = max(j - S, 0); q < j; ++q) ring_wait(full + q % S, (unsigned)(q / S) & 1u);
+    }
+    return;
+  }
+  int slot = 0;
+  unsigned parity = 0;
+  for (int j = 0; j < n; ++j) {
+    bool ok = true;
+    body(desc[j % kDescs], smem + (size_t)slot * a.slot_floats, j + 1 < n ? desc + (j + 1) % kDescs : nullptr,
+         [&]() { return ok = ring_wait(full + slot, parity); });
+    if (!ok) {
+      atomicExch(a.err, 3);
+      return;
+    }
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0)
+      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(empty + slot)) : "memory");
+    if (++slot == S) {
+      slot = 0;
+      parity ^= 1u;
+    }
+  }
+}
+
+// Whether one of the columns k .. k + 3 can be in an overlap.
+__device__ __forceinline__ bool over_any(const LvTile& t, int l, int r, int k) {
+  return l < t.tA || l > t.L - t.tB || r < t.wS || r >= t.ny - t.wN || k < t.wL || k + 4 > t.nx - t.wR;
+}
+// A thread's overlap counts and values (targets, or the tangent-linear run of a
+// Gauss-Newton product).
+struct Over {
+  int c[4], any;
+  float m[3][4];
+};
+// A thread's overlap values of the next tile, copied to 48 bytes of its own
+// while it works on this one (see lv_force).
+__device__ __forceinline__ void over_prefetch(const LvTile& t, const float* q, int l, float* own) {
+  const int p = t.p0 + threadIdx.x;
+  if (p < t.p1 && lv_overlaps(t, l)) {
+    const int r = mdiv(p, t.mq), k = (p - r * t.nq) * 4, pl = t.ny * t.nxp;
+    if (!over_any(t, l, r, k)) return;
+    asm volatile("cp.async.wait_all;" ::: "memory");   // (values of a tile that was left out)
+#pragma unroll
+    for (int v = 0; v < 3; ++v) copy16(own + v * 4 * kRingPoints, q + (r * t.nxp + k + v * pl));
+  }
+}
+__device__ __forceinline__ void over_take(const LvTile& t, int l, int r, int k, const float* own, Over& ov) {
+  ov.any = 0;
+  if (!over_any(t, l, r, k)) return;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    ov.c[j] = k + j < t.nx ? lv_overlap_count(t, l, r, k + j) : 0;
+    ov.any |= ov.c[j];
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+#pragma unroll
+  for (int v = 0; v < 3; ++v) ldv<float, 4>(own + v * 4 * kRingPoints, ov.m[v]);
+}
+
+// lv_adj_kernel, pipelined.
+template <int K>
+__global__ void __launch_bounds__(kRingThreads, 2) lv_ring_adj_kernel(const LvArgs<float> a) {
+  constexpr int NO = K == 3 ? 2 : 0;
+  constexpr bool BL = K == 1;
+  const int l = a.l;
+  const size_t G = (size_t)3 * a.nlat * a.nlon;
+  auto skip = [&](const LvTile& t) { return a.active && a.active[t.s] != a.active_value; };
+  float* const dst = K == 1 ? a.mu2 : K == 2 ? a.mu1 : a.lam;
+  extern __shared__ __align__(16) float ring_smem[];
+  float* own = ring_smem + threadIdx.x * 4;   // K = 3: the thread's overlap values, before the slots
+  float* slots = ring_smem + (K == 3 ? 12 * kRingPoints : 0);
+  const bool over = K == 3 && !a.yforce && a.mu_on;
+  auto target = [&](const LvTile& t) {
+    return (a.gn_dx ? a.gn_dx : a.tgt) + t.traj_off + (size_t)l * level_size<float>(t);
+  };
+  bool first = true;
+  ring_run(
+      a, slots,
+      [&](const LvTile& t, float* base, uint64_t* bar) {
+        const float* Z = K == 1   ? x2_of(a, t, l)
+                         : K == 2 ? x1_of(a, t, l)
+                                  : a.traj + t.traj_off + (size_t)l * level_size<float>(t);
+        const float* M = (K == 1 ? a.lam : K == 2 ? a.mu2 : a.mu1) + t.lv_off;
+        ring_issue<2, NO, BL>(a, t, base, bar, skip(t), a.bw, a.bnd + (size_t)(t.a + l + (K == 2)) * G, [&](int i) {
+          return i == 0 ? Z : i == 1 ? M : i == 2 ? a.lam + t.lv_off : a.mu2 + t.lv_off;
+        });
+      },
+      [&](const LvTile& t, float* base, const LvTile* next, auto&& wait) {
+        const int pl = t.ny * t.nxp, p = t.p0 + threadIdx.x;
+        const int r = mdiv(p, t.mq), k = (p - r * t.nq) * 4, at = r * t.nxp + k, rr = r - mdiv(t.p0, t.mq);
+        const bool mine = p < t.p1 && !skip(t);
+        if (over && first) over_prefetch(t, target(t), l, own);
+        first = false;
+        if (!wait()) return;
+        if (mine) {
+          const Slot<2, NO, BL> sl = slot_of<2, NO, BL>(t, base);
+          float rc[8];
+          load_rec8(sl.rec() + 8 * rr, rc);
+          const int wall = (r == 0 && (t.flags & F_SWALL) ? 1 : 0) | (r == t.ny - 1 && (t.flags & F_NWALL) ? 2 : 0);
+          Patch<float, 4> z, m;
+          ring_state(t, sl, rr, r, k, z);
+          ring_adjoint(t, sl, rr, r, k, m);
+          float o[3][4], ll[3][4], l2[3][4];
+          if (K == 3) {
+#pragma unroll
+            for (int v = 0; v < 3; ++v) {
+              ldv<float, 4>(sl.state(2) + v * sl.own() + rr * t.nxp + k, ll[v]);
+              ldv<float, 4>(sl.state(3) + v * sl.own() + rr * t.nxp + k, l2[v]);
+            }
+          }
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            Pt5<float> zp, mp;
+            point_of(z, j, zp);
+            point_of(m, j, mp);
+            if (K == 3)
+              adj_lambda_math<float, true>(zp, mp, rc, a.dt, a.Bth_a, a.gBth_a, a.href, wall, ll[0][j], ll[1][j],
+                                           ll[2][j], l2[0][j], l2[1][j], l2[2][j], o[0][j], o[1][j], o[2][j]);
+            else
+              adj_stage_math<float, true>(zp, mp, rc, a.dt, a.Bth_a, a.gBth_a, a.href, wall, o[0][j], o[1][j],
+                                          o[2][j]);
+          }
+          if (K == 3 && (a.yforce || (over && lv_overlaps(t, l)))) {
+            float x[3][4];
+#pragma unroll
+            for (int v = 0; v < 3; ++v)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) x[v][j] = z.c[v][j + 1];
+            if (over) {
+              Over ov;
+              over_take(t, l, r, k, own, ov);
+              if (ov.any)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                  if (ov.c[j]) overlap_force_add<float, 4>(a, ov.c[j], j, x, ov.m, o);
+            } else {
+              lv_force<float, 4>(a, t, l, r, k, x, o);   // external forcing
+            }
+          }
+          float* out = dst + t.lv_off + at;
+#pragma unroll
+          for (int v = 0; v < 3; ++v) stv<float, 4>(out + v * pl, o[v]);
+        }
+        if (over && next) over_prefetch(*next, target(*next), l, own);
+      });
+}
+
+// Observation forcing of level l, a CTA per box that goes on beyond it (after
+// the pipelined phase 3; lv_lam_start_kernel adds a box's last level).
+__global__ void __launch_bounds__(kRingThreads) lv_scatter_kernel(const LvArgs<float> a) {
+  const int s = a.boxes[blockIdx.x];
+  grid_wait();
+  grid_release();
+  if (a.active && a.active[s] != a.active_value) return;
+  const SubDesc& d = a.subs[s];
+  const int t0 = a.lvl_sc[d.sc_lvl + a.l], t1 = a.lvl_sc[d.sc_lvl + a.l + 1];
+  float* lam = a.lam + a.box_off[s];
+  for (int i = t0 + threadIdx.x; i < t1; i += blockDim.x) {
+    const int g = a.sc_tgt[i], vr = g / d.nx, k = g - vr * d.nx;   // vr = v ny + r
+    double acc = 0.0;
+    for (int c = a.sc_off[i]; c < a.sc_off[i + 1]; ++c) acc += a.sc_w[c] * a.obs_force[a.sc_obs[c]];
+    lam[(size_t)vr * d.nxp + k] += (float)acc;
+  }
+}
+
 template <typename T>
 cudaError_t lv_launch(void (*kernel)(const LvArgs<T>), const LvArgs<T>& a, int blocks, cudaStream_t st) {
   if (blocks <= 0) return cudaSuccess;
   return launch_dependent(kernel, dim3((unsigned)blocks), kLvThreads, 0, st, a);
+}
+
+// Adjoint phase q + 1: the plain kernel, or the pipelined one where the plan
+// has rings.
+template <typename T>
+cudaError_t lv_phase(void (*plain)(const LvArgs<T>), void (*ring)(const LvArgs<float>), const LvArgs<T>& base,
+                     const LvPlan& g, int q, cudaStream_t st) {
+  if constexpr (sizeof(T) == 4) {
+    const LvRing& rg = g.ring[q];
+    if (rg.slots) {
+      LvArgs<T> a = base;
+      a.tiles = g.ring_tiles;
+      a.n_tile = g.n_ring[a.l];
+      a.n_cta = std::min(a.n_tile, rg.ctas);
+      a.slots = rg.slots;
+      a.slot_floats = rg.slot_floats;
+      const size_t smem = ((size_t)rg.slots * rg.slot_floats + rg.own_floats) * sizeof(float);
+      cudaError_t e = cudaFuncSetAttribute(ring, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+      return launch_dependent(ring, dim3((unsigned)a.n_cta), kRingThreads, smem, st, a);
+    }
+  }
+  return lv_launch<T>(plain, base, base.n_tile, st);
 }
 
 }  // namespace
@@ -630,9 +1091,12 @@ cudaError_t launch_level_adjoint(const LvArgs<T>& base, const LvPlan& g, cudaStr
       LV_TRY(lv_launch<T>(lv_stage_kernel<T, V, 1, false>, a, a.n_tile, st));
       LV_TRY(lv_launch<T>(lv_stage_kernel<T, V, 2, false>, a, a.n_tile, st));
     }
-    LV_TRY(lv_launch<T>(lv_adj_kernel<T, V, 1>, a, a.n_tile, st));
-    LV_TRY(lv_launch<T>(lv_adj_kernel<T, V, 2>, a, a.n_tile, st));
-    LV_TRY(lv_launch<T>(lv_adj_kernel<T, V, 3>, a, a.n_tile, st));
+    LV_TRY(lv_phase<T>(lv_adj_kernel<T, V, 1>, lv_ring_adj_kernel<1>, a, g, 0, st));
+    LV_TRY(lv_phase<T>(lv_adj_kernel<T, V, 2>, lv_ring_adj_kernel<2>, a, g, 1, st));
+    LV_TRY(lv_phase<T>(lv_adj_kernel<T, V, 3>, lv_ring_adj_kernel<3>, a, g, 2, st));
+    if constexpr (sizeof(T) == 4)
+      if (g.ring[2].slots && g.obs[l] && !a.yforce)
+        LV_TRY(launch_dependent(lv_scatter_kernel, dim3((unsigned)g.n_box[l + 1]), kRingThreads, 0, st, a));
   }
   LV_TRY(lv_launch<T>(lv_export_kernel<T, V>, a, g.tiles, st));
   return cudaSuccess;

@@ -4,7 +4,8 @@ and adjoint runs bit for bit, J up to the order of its partial sums (FP64: a
 few roundings of at most 1e5 terms, 1e-13; FP32 state: the cluster sweeps add a
 thread's FP32 terms in FP32, 1e-6 as between launch shapes), with boxes that
 are periodic, at walls, one tile or several, of widths that are and are not
-multiples of a thread's columns, and windows of different lengths."""
+multiples of a thread's columns, and windows of different lengths; the FP32
+adjoint also by the pipelined kernels (one and several tiles per CTA)."""
 import numpy as np
 import pytest
 import torch
@@ -19,6 +20,7 @@ CASES = {
     "periodic": dict(nlon=61, nlat=38, nsteps=23, P1=1, P2=2, Q=2, o_lat=2, o_t=2),   # odd width, wrap in lon
     "one box": dict(nlon=33, nlat=14, nsteps=9, P1=1, P2=1, Q=1),
     "walls": dict(nlon=24, nlat=12, nsteps=9, P1=3, P2=1, Q=2, o_lon=2, o_t=1),       # both walls in every box
+    "many rows": dict(nlon=384, nlat=160, nsteps=12, P1=4, P2=2, Q=4, o_lon=4, o_lat=4),   # several tiles per CTA
     "wide": dict(nlon=300, nlat=48, nsteps=6, P1=2, P2=2, Q=1, o_lon=3, o_lat=3),     # several tiles per box
 }
 
@@ -32,13 +34,15 @@ def _built():
 
 
 @pytest.mark.parametrize("name", list(CASES))
-@pytest.mark.parametrize("precision,ckpt_k", [(0, 0), (0, -1), (0, -3), (1, 0), (1, 4)])
-def test_level_sweeps_equal_cluster_sweeps(monkeypatch, name, precision, ckpt_k):
+@pytest.mark.parametrize("precision,ckpt_k,pipelined",
+                         [(0, 0, 0), (0, -1, 0), (0, -3, 0), (1, 0, 0), (1, 4, 0), (1, 0, 1), (1, 4, 1)])
+def test_level_sweeps_equal_cluster_sweeps(monkeypatch, name, precision, ckpt_k, pipelined):
     import paper_2205_06649_gb300 as dd
     over = dict(obs_count=400, obs_every=2, corr_len=1.5)
     wl = (workloads.preset("ragged") if name == "ragged" else tiny_workload(**{**over, **CASES[name]}))
     inp = workloads.generate(wl)
     monkeypatch.setenv("DD4DV_LEVEL_MIN_POINTS", "1")
+    monkeypatch.setenv("DD4DV_RING_MIN_TILES", "0" if pipelined else str(1 << 40))
     ctx = dd.Context(wl.nlon, wl.nlat, inp["dt"], wl.nsteps, precision=precision)
     ctx.set_background(inp["x_b0"])
     ctx.set_background_error(wl.sigma_b, wl.corr_len, wl.rf_passes)
