@@ -948,7 +948,11 @@ void tune_checkpoint(dd4dv_ctx* ctx) {
 //         88,000 in 32 boxes 2.38 / 1.98; 350,000 in 128 boxes 6.96 / 5.31
 //   FP32: 305,000 in 32 boxes 0.98 / 1.16; 350,000 in 128 boxes 1.30 / 1.27;
 //         719,000 in 256 boxes 2.52 / 1.96; 1.2 million in 128 boxes 8.6 / 3.0
+// Small boxes in FP64 pack one or more to an SM with few barriers and stay with
+// the cluster sweeps whatever their number: 20 x 18 points, 256 boxes 2.01 / 2.29
+// (28 x 24: 3.23 / 3.39, 48 x 24: 4.54 / 4.72; 512 boxes 9.18 / 9.03).
 constexpr long long kLvMinPoints64 = 65000, kLvMinPoints32 = 350000;
+constexpr int kLvMinBox64 = 700;
 
 // The pipelined FP32 adjoint kernels run where every box is at most kRingMaxNx
 // wide (a tile of 224 thread-points has three rows or more) and each of two
@@ -976,7 +980,7 @@ void level_plan(dd4dv_ctx* ctx, const std::vector<SubDesc>& subs, const std::vec
     max_nx = std::max(max_nx, d.nx);
     min_ny = std::min(min_ny, d.ny);
   }
-  long long least = sizeof(T) == 4 ? kLvMinPoints32 : kLvMinPoints64;
+  long long least = sizeof(T) == 4 ? kLvMinPoints32 : std::max<long long>(kLvMinPoints64, (long long)kLvMinBox64 * n_sub);
   if (const char* e = std::getenv("DD4DV_LEVEL_MIN_POINTS")) least = std::atoll(e);   // override (tests)
   if (pts < least || maxL < 1 || min_nx <= V || min_ny < 2 || 3LL * nlon * nlat >= (1LL << 31)) return;
   auto& L = ctx->dec_allocs;
