@@ -384,6 +384,10 @@ bool level_adjoint(const dd4dv_ctx* ctx) {
   return ctx->lv_a && ctx->variant_a == 0 && (ctx->ckpt == 0 || level_forward(ctx));
 }
 
+// Whether a Gauss-Newton product's tangent-linear sweep runs as a level sweep
+// (FP64, about the levels that a level forward sweep stores).
+bool tangent_level(const dd4dv_ctx* ctx) { return ctx->m.precision == 0 && level_forward(ctx); }
+
 template <typename T>
 LvArgs<T> level_args(dd4dv_ctx* ctx, const int* active, int av) {
   LvArgs<T> a{};
@@ -554,13 +558,20 @@ void gn_product_T(dd4dv_ctx* ctx, const double* p, double* Ap, const int* active
   int tl_cl = 0, tl_R = 0;
   tlm_shape(ctx, &tl_cl, &tl_R);
   apply_V(ctx, p, ctx->io_c, active, av);
-  SweepArgs<T> a = sweep_args<T>(ctx);
-  a.active = active;
-  a.active_value = av;
-  a.dx0 = ctx->io_c;
-  a.gn_dx = static_cast<T*>(ctx->gn_dx);
-  a.R = tl_R;
-  KL(launch_tlm<T>(a, tl_cl, ctx->nthreads, ctx->st));
+  if (tangent_level(ctx)) {
+    LvArgs<double> a = level_args<double>(ctx, active, av);
+    a.dx = static_cast<double*>(ctx->gn_dx);
+    a.dx0 = ctx->io_c;
+    CK(launch_level_tangent(a, ctx->lv, ctx->st, &ctx->launches));
+  } else {
+    SweepArgs<T> a = sweep_args<T>(ctx);
+    a.active = active;
+    a.active_value = av;
+    a.dx0 = ctx->io_c;
+    a.gn_dx = static_cast<T*>(ctx->gn_dx);
+    a.R = tl_R;
+    KL(launch_tlm<T>(a, tl_cl, ctx->nthreads, ctx->st));
+  }
   adjoint_sweep<T>(ctx, active, av, nullptr, static_cast<T*>(ctx->gn_dx));
   apply_VT(ctx, ctx->lam_a, p, nullptr, Ap, active, av);
 }

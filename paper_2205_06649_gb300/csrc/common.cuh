@@ -223,6 +223,8 @@ struct LvArgs {
   int active_value;
   double* lam_a;
   const double* yforce;
+  T* dx;                      // tangent-linear sweep: dx (trajectory layout), and
+  const double* dx0;          // dx(a), packed control layout
 };
 // Columns per thread: FP32 threads take four neighbouring points (16-byte
 // accesses), FP64 threads one.
@@ -234,6 +236,9 @@ template <typename T>
 cudaError_t launch_level_forward(const LvArgs<T>& a, const LvPlan& g, cudaStream_t st, long long* launches);
 template <typename T>
 cudaError_t launch_level_adjoint(const LvArgs<T>& a, const LvPlan& g, cudaStream_t st, long long* launches);
+
+// tangent-linear sweep of a Gauss-Newton product (a.dx, obs_force from a.dx0)
+cudaError_t launch_level_tangent(const LvArgs<double>& a, const LvPlan& g, cudaStream_t st, long long* launches);
 
 // ---- auxiliary kernels (aux.cu) ----
 struct RFArgs {

@@ -565,6 +565,101 @@ __global__ void __launch_bounds__(kLvThreads, 4) lv_adj_kernel(const LvArgs<T> a
   if (K == 3) lv_scatter<T, V>(a, t, l, out);
 }
 
+// ---- tangent-linear sweep of a Gauss-Newton product ----
+// About the trajectory (and the stage states, where they are stored) of the
+// last forward sweep: dx of every level to a.dx, the linear observations of
+// every level to obs_force.  FP64 only: the FP32 sweep (tlm_kernel of sweep.cu)
+// leaves the contraction of its arithmetic to the compiler, and its FP32
+// roundings show in a product.  Bound: the FP64 pipe (some 55 instructions a
+// point and stage).  Medium workload (64 boxes): 3.1 ms by clusters, 2.5 here (a
+// product 7.55 -> 6.95 ms).
+__device__ __forceinline__ void lv_obs_lin(const LvArgs<double>& a, int s, int l) {
+  const SubDesc& d = a.subs[s];
+  const int o0 = a.lvl_obs[d.obs_lvl + l], o1 = a.lvl_obs[d.obs_lvl + l + 1];
+  const size_t pl = (size_t)d.ny * d.nxp;
+  const double* X = a.dx + d.traj_off + (size_t)l * 3 * pl;
+  for (int o = o0 + threadIdx.x; o < o1; o += blockDim.x) {
+    const ObsRec ob = a.obs[o];
+    const double* x = X + ob.var * pl + (size_t)ob.r0 * d.nxp;
+    const double wj0 = 1.0 - ob.dj, wi0 = 1.0 - ob.di;
+    double acc = (wj0 * wi0) * x[ob.k0];
+    if (ob.di != 0.0) acc += (wj0 * ob.di) * x[ob.k1];
+    if (ob.dj != 0.0) {
+      acc += (ob.dj * wi0) * x[d.nxp + ob.k0];
+      if (ob.di != 0.0) acc += (ob.dj * ob.di) * x[d.nxp + ob.k1];
+    }
+    a.obs_force[o] = a.lam_w * ob.w * acc;
+  }
+}
+__global__ void __launch_bounds__(kLvThreads) lv_tl_start_kernel(const LvArgs<double> a) {
+  LV_TILE(t);
+  grid_wait();
+  grid_release();
+  if (a.active && a.active[t.s] != a.active_value) return;
+  const int pl = t.ny * t.nxp;
+  const double* src = a.dx0 + t.ctrl_off;
+  double* D = a.dx + t.traj_off;
+  for (int p = t.p0 + threadIdx.x; p < t.p1; p += kLvThreads) {
+    const int r = mdiv(p, t.mq), k = p - r * t.nq, at = r * t.nxp + k;
+#pragma unroll
+    for (int v = 0; v < 3; ++v) D[at + v * pl] = src[((size_t)v * t.ny + r) * t.nx + k];
+  }
+}
+// Stage ST of step l: out = cx dX + cy (dY + dt F'(Y) dY).  The first stage's
+// grid carries the observations of level l as lv_stage_kernel does.
+template <int ST>
+__global__ void __launch_bounds__(kLvThreads, 4) lv_tl_kernel(const LvArgs<double> a) {
+  const int l = a.l;
+  if (ST == 1 && (int)blockIdx.x >= a.n_tile) {
+    const int s = a.boxes[blockIdx.x - a.n_tile];
+    grid_wait();
+    grid_release();
+    if (a.active && a.active[s] != a.active_value) return;
+    lv_obs_lin(a, s, l);
+    return;
+  }
+  LV_TILE(t);
+  grid_wait();
+  grid_release();
+  if (a.active && a.active[t.s] != a.active_value) return;
+  const size_t lvl = level_size<double>(t);
+  const int pl = t.ny * t.nxp;
+  const double* Y = ST == 1 ? a.traj + t.traj_off + (size_t)l * lvl : ST == 2 ? x1_of(a, t, l) : x2_of(a, t, l);
+  const double* DX = a.dx + t.traj_off + (size_t)l * lvl;
+  const double* DY = ST == 1 ? DX : (ST == 2 ? a.mu2 : a.mu1) + t.lv_off;
+  double* out = ST == 3 ? a.dx + t.traj_off + (size_t)(l + 1) * lvl : (ST == 1 ? a.mu2 : a.mu1) + t.lv_off;
+  const size_t G = (size_t)3 * a.nlat * a.nlon;
+  const int n = t.a + l;
+  const double* B0 = a.bnd + (size_t)(ST == 2 ? n + 1 : n) * G;
+  const double* B1 = ST == 3 ? B0 + G : nullptr;
+  const double cx = ST == 1 ? 0.0 : ST == 2 ? 0.75 : 1.0 / 3.0, cy = ST == 1 ? 1.0 : ST == 2 ? 0.25 : 2.0 / 3.0;
+  for (int p = t.p0 + threadIdx.x; p < t.p1; p += kLvThreads) {
+    const int r = mdiv(p, t.mq), k = p - r * t.nq, at = r * t.nxp + k;
+    Patch<double, 1> z, d;
+    load_state_patch<double, 1>(a, t, Y, r, k, at, B0, B1, z);
+    load_adjoint_patch<double, 1>(t, DY, r, k, at, d);   // ghosts zero or periodic ...
+    double rc[8];
+    load_rec8(a.fw + 8 * (t.j0 + r), rc);
+    double x[3];
+#pragma unroll
+    for (int v = 0; v < 3; ++v) {
+      x[v] = ST == 1 ? 0.0 : DX[at + v * pl];
+      const double m = v == 2 ? -d.c[v][1] : d.c[v][1];   // ... but mirrored at walls
+      if (r == 0 && (t.flags & F_SWALL)) d.s[v][0] = m;
+      if (r == t.ny - 1 && (t.flags & F_NWALL)) d.n[v][0] = m;
+    }
+    Pt5<double> zp, dp;
+    point_of(z, 0, zp);
+    point_of(d, 0, dp);
+    double Fh, Fu, Fv;
+    rhs_tl_pt<double, false>(zp, dp, rc[0], rc[1], rc[2], rc[3], rc[4], rc[5], rc[6], a.Bth, a.gBth, a.href, Fh, Fu,
+                             Fv);
+    out[at] = cx * x[0] + cy * (dp.h + a.dt * Fh);
+    out[at + pl] = cx * x[1] + cy * (dp.u + a.dt * Fu);
+    out[at + 2 * pl] = cx * x[2] + cy * (dp.v + a.dt * Fv);
+  }
+}
+
 // lambda(a) -> packed control layout (FP64).
 template <typename T, int V>
 __global__ void __launch_bounds__(kLvThreads) lv_export_kernel(const LvArgs<T> a) {
@@ -1099,6 +1194,27 @@ cudaError_t launch_level_adjoint(const LvArgs<T>& base, const LvPlan& g, cudaStr
         LV_TRY(launch_dependent(lv_scatter_kernel, dim3((unsigned)g.n_box[l + 1]), kRingThreads, 0, st, a));
   }
   LV_TRY(lv_launch<T>(lv_export_kernel<T, V>, a, g.tiles, st));
+  return cudaSuccess;
+}
+
+cudaError_t launch_level_tangent(const LvArgs<double>& base, const LvPlan& g, cudaStream_t st, long long* launches) {
+  LvArgs<double> a = base;
+  const int L = (int)g.n_tile.size();
+  a.skip1 = a.stg1 != nullptr;
+  LV_TRY(lv_launch<double>(lv_tl_start_kernel, a, g.tiles, st));
+  for (int l = 0; l <= L; ++l) {
+    a.l = l;
+    a.n_tile = l < L ? g.n_tile[l] : 0;
+    const int nob = g.obs[l] ? g.n_box[l] : 0;
+    if (a.n_tile + nob) LV_TRY(lv_launch<double>(lv_tl_kernel<1>, a, a.n_tile + nob, st));
+    if (!a.n_tile) continue;
+    if (!a.stg) {   // the stage states were not stored: recompute them
+      LV_TRY(lv_launch<double>(lv_stage_kernel<double, 1, 1, false>, a, a.n_tile, st));
+      LV_TRY(lv_launch<double>(lv_stage_kernel<double, 1, 2, false>, a, a.n_tile, st));
+    }
+    LV_TRY(lv_launch<double>(lv_tl_kernel<2>, a, a.n_tile, st));
+    LV_TRY(lv_launch<double>(lv_tl_kernel<3>, a, a.n_tile, st));
+  }
   return cudaSuccess;
 }
 
