@@ -958,11 +958,11 @@ void tune_checkpoint(dd4dv_ctx* ctx) {
 //   FP64: 55,000 points in 128 boxes 1.39 / 1.78; 74,000 in 8 boxes 2.00 / 1.58;
 //         88,000 in 32 boxes 2.38 / 1.98; 350,000 in 128 boxes 6.96 / 5.31
 //   FP32: 305,000 in 32 boxes 0.98 / 1.16; 350,000 in 128 boxes 1.30 / 1.27;
-//         719,000 in 256 boxes 2.52 / 1.96; 1.2 million in 128 boxes 8.6 / 3.0
+//         442,000 in 512 boxes 3.61 / 1.50; 719,000 in 256 boxes 2.52 / 1.96; 1.2 million in 128 boxes 8.6 / 3.0
 // Small boxes in FP64 pack one or more to an SM with few barriers and stay with
 // the cluster sweeps whatever their number: 20 x 18 points, 256 boxes 2.01 / 2.29
 // (28 x 24: 3.23 / 3.39, 48 x 24: 4.54 / 4.72; 512 boxes 9.18 / 9.03).
-constexpr long long kLvMinPoints64 = 65000, kLvMinPoints32 = 350000;
+constexpr long long kLvMinPoints64 = 65000, kLvMinPoints32 = 400000;
 constexpr int kLvMinBox64 = 700;
 
 // The pipelined FP32 adjoint kernels run where every box is at most kRingMaxNx
