@@ -627,8 +627,8 @@ void reset_exchange_T(dd4dv_ctx* ctx) {
 void global_step(dd4dv_ctx* ctx, const double* x, double* nx) {
   double* s1 = ctx->gscratch;
   double* s2 = ctx->gscratch + ctx->gstate;
-  CK(launch_global_step(ctx->gplan, x, s1, s2, nx, ctx->grec, ctx->m.dt * ctx->Bth, ctx->m.dt * ctx->gBth, ctx->m.nlon,
-                        ctx->m.nlat, ctx->st, &ctx->launches));
+  CK(launch_global_step(ctx->gplan, x, s1, s2, nx, ctx->grec, ctx->m.dt, ctx->Bth, ctx->gBth, ctx->m.nlon, ctx->m.nlat,
+                        ctx->st, &ctx->launches));
 }
 
 // Global model run x0 (device) -> out trajectory (device, FP64).
@@ -642,16 +642,15 @@ void global_run(dd4dv_ctx* ctx, const double* x0, double* out) {
 // levels are produced in the chunk buffer, gchunk_lv at a time, and handed to
 // sink(g0, g1, levels) (levels g0..g1, level-major FP64) in order.  The last
 // level of a chunk is the first of the next.
-// step(ctx, x, nx) advances one level.
-template <typename Step, typename Sink>
-void global_run_chunked(dd4dv_ctx* ctx, const double* x0, Step&& step, Sink&& sink) {
+template <typename Sink>
+void global_run_chunked(dd4dv_ctx* ctx, const double* x0, Sink&& sink) {
   const size_t G = ctx->gstate;
   const int K = ctx->gchunk_lv - 1;
   double* c = ctx->gchunk;
   CK(cudaMemcpyAsync(c, x0, G * sizeof(double), cudaMemcpyDeviceToDevice, ctx->st));
   for (int g0 = 0;;) {
     const int g1 = std::min(g0 + K, ctx->m.nsteps);
-    for (int n = g0; n < g1; ++n) step(ctx, c + (size_t)(n - g0) * G, c + (size_t)(n - g0 + 1) * G);
+    for (int n = g0; n < g1; ++n) global_step(ctx, c + (size_t)(n - g0) * G, c + (size_t)(n - g0 + 1) * G);
     sink(g0, g1, c);
     if (g1 >= ctx->m.nsteps) break;
     CK(cudaMemcpyAsync(c, c + (size_t)(g1 - g0) * G, G * sizeof(double), cudaMemcpyDeviceToDevice, ctx->st));
@@ -659,27 +658,11 @@ void global_run_chunked(dd4dv_ctx* ctx, const double* x0, Step&& step, Sink&& si
   }
 }
 
-// One step of the background forecast.  Its levels become the boundary
-// trajectory and the targets, on the FP32 path rounded to FP32, where another
-// last bit here and there flips an FP32 value; so it keeps one order of
-// operations, that of the results on record, in a kernel of its own.
-void background_step(dd4dv_ctx* ctx, const double* x, double* nx) {
-  double* s1 = ctx->gscratch;
-  double* s2 = ctx->gscratch + ctx->gstate;
-  auto stage = [&](const double* y, double* out, double ca, double cb) {
-    KL(launch_background_stage(x, y, out, ca, cb, ctx->rows_d, ctx->Bth, ctx->gBth, ctx->m.dt, ctx->m.nlon,
-                               ctx->m.nlat, ctx->st));
-  };
-  stage(x, s1, 0.0, 1.0);
-  stage(s1, s2, 0.75, 0.25);
-  stage(s2, nx, 1.0 / 3.0, 2.0 / 3.0);
-}
-
 template <typename T>
 void background_pass(dd4dv_ctx* ctx, bool xb_a) {
   const size_t G = ctx->gstate;
   const int nlon = ctx->m.nlon, nlat = ctx->m.nlat;
-  global_run_chunked(ctx, ctx->xb0, background_step, [&](int g0, int g1, const double* lv) {
+  global_run_chunked(ctx, ctx->xb0, [&](int g0, int g1, const double* lv) {
     const long long n = (long long)(g1 - g0 + 1) * G;
     KL(launch_bnd_from_global<T>(lv, n, h_ref_of(ctx), nlon, nlat, static_cast<T*>(ctx->bnd) + (size_t)g0 * G,
                                  ctx->st));
@@ -1696,7 +1679,7 @@ dd4dv_status dd4dv_create(const dd4dv_model* model, void* cuda_stream, dd4dv_ctx
     std::vector<double> rec(8 * (size_t)m.nlat);
     for (int j = 0; j < m.nlat; ++j)
       fill_global_record(ctx->rows_h[j], ctx->rows_h[std::min(j + 1, m.nlat - 1)].c, ctx->rows_h[std::max(j - 1, 0)].c,
-                         m.dt, ctx->Bth, &rec[8 * (size_t)j]);
+                         &rec[8 * (size_t)j]);
     ctx->xb0 = dalloc<double>(ctx, ctx->gstate);
     ctx->gscratch = dalloc<double>(ctx, 3 * ctx->gstate);
     // chunk of global levels: at most 512 MB, at least 2 levels, at most the whole trajectory
@@ -2132,7 +2115,7 @@ dd4dv_status dd4dv_forward(dd4dv_ctx* ctx, const double* x0, double* traj, int d
     const size_t G = ctx->gstate;
     double* in = ctx->gscratch + 2 * G;
     h2d(ctx, in, x0, G * sizeof(double));
-    global_run_chunked(ctx, in, global_step, [&](int g0, int g1, const double* lv) {
+    global_run_chunked(ctx, in, [&](int g0, int g1, const double* lv) {
       d2h(ctx, traj + (size_t)g0 * G, lv, (size_t)(g1 - g0 + 1) * G * sizeof(double));
     });
     sync(ctx);

@@ -349,68 +349,16 @@ __global__ void bnd_to_global_kernel(const T* bnd, long long n, double h_ref, lo
 }
 
 // ---------------------------------------------------------------------------
-// Stage of the background forecast on the whole sphere: out = ca x + cb (y + dt
-// F(y)).  (It runs at set_decomposition, and at a reset that has no copy.)
-__global__ void background_stage_kernel(const double* x, const double* y, double* out, double ca,
-                                    double cb, const RowConst* rows, double Bth, double gBth,
-                                    double dt, int nlon, int nlat) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y;
-  if (i >= nlon) return;
-  const size_t P = (size_t)nlat * nlon;
-  const double* H = y;
-  const double* U = y + P;
-  const double* V = y + 2 * P;
-  const int iE = (i + 1) % nlon, iW = (i - 1 + nlon) % nlon;
-  const size_t o = (size_t)j * nlon + i;
-  const RowConst rc = rows[j];
-  const double h = H[o], u = U[o], v = V[o];
-  const double hE = H[(size_t)j * nlon + iE], hW = H[(size_t)j * nlon + iW];
-  const double uE = U[(size_t)j * nlon + iE], uW = U[(size_t)j * nlon + iW];
-  const double vE = V[(size_t)j * nlon + iE], vW = V[(size_t)j * nlon + iW];
-  double hN, uN, vN, cN, hS, uS, vS, cS;
-  if (j + 1 < nlat) {
-    const size_t q = (size_t)(j + 1) * nlon + i;
-    hN = H[q]; uN = U[q]; vN = V[q]; cN = rows[j + 1].c;
-  } else {
-    hN = h; uN = u; vN = -v; cN = rc.c;
-  }
-  if (j > 0) {
-    const size_t q = (size_t)(j - 1) * nlon + i;
-    hS = H[q]; uS = U[q]; vS = V[q]; cS = rows[j - 1].c;
-  } else {
-    hS = h; uS = u; vS = -v; cS = rc.c;
-  }
-  const double fu = rc.f + rc.tau * u;
-  const double Fu = -rc.A * u * (uE - uW) - Bth * v * (uN - uS) + fu * v - rc.gA * (hE - hW);
-  const double Fv = -rc.A * u * (vE - vW) - Bth * v * (vN - vS) - fu * u - gBth * (hN - hS);
-  const double Fh = -rc.A * (hE * uE - hW * uW) - rc.BinvC * (hN * vN * cN - hS * vS * cS);
-  const double F[3] = {Fh, Fu, Fv};
-  for (int c = 0; c < 3; ++c) {
-    const size_t q = (size_t)c * P + o;
-    out[q] = (ca == 0.0 ? 0.0 : ca * x[q]) + cb * (y[q] + dt * F[c]);
-  }
-}
-
 // Global model stage on the whole sphere: out = ca x + cb (y + dt F(y)).
-// Bound: the FP64 pipe, 24 instructions a point and stage (30 with x), as the
-// box sweeps (euler_pt64).  One thread per point, flat over rows so that every
-// lane has one; set-up overlaps the stage before (programmatic dependent
-// launch).  Small grids take global_step_kernel instead.
+// Bound: the FP64 pipe, 28 instructions a point and stage (34 with x, global_pt).
+// One thread per point, flat over rows so that every lane has one; set-up overlaps
+// the stage before (programmatic dependent launch).  Small grids take
+// global_step_kernel instead.
 constexpr int kGlobalThreads = 128;
-__device__ __forceinline__ void global_pt(const Pt5<double>& z, const double (&rc)[8], double dtB, double dtgB,
-                                          double ca, double cb, double x0, double x1, double x2, double& o0,
-                                          double& o1, double& o2) {
-  euler_pt64(z, rc, dtB, dtgB, o0, o1, o2);
-  if (ca != 0.0) {
-    o0 = xfma(ca, x0, xmul(cb, o0));
-    o1 = xfma(ca, x1, xmul(cb, o1));
-    o2 = xfma(ca, x2, xmul(cb, o2));
-  }
-}
 __global__ void __launch_bounds__(kGlobalThreads) global_stage_kernel(const double* x, const double* y, double* out,
                                                                       double ca, double cb, const double* rec,
-                                                                      double dtB, double dtgB, int nlon, int nlat) {
+                                                                      double dt, double Bth, double gBth, int nlon,
+                                                                      int nlat) {
   const unsigned idx = blockIdx.x * kGlobalThreads + threadIdx.x;
   const unsigned P = (unsigned)nlat * nlon;
   const int j = (int)(idx / (unsigned)nlon), i = (int)(idx - (unsigned)j * nlon);
@@ -437,22 +385,22 @@ __global__ void __launch_bounds__(kGlobalThreads) global_stage_kernel(const doub
     x2 = x[o + 2 * (size_t)P];
   }
   double o0, o1, o2;
-  global_pt(z, rc, dtB, dtgB, ca, cb, x0, x1, x2, o0, o1, o2);
+  global_pt(z, rc, dt, Bth, gBth, ca, cb, x0, x1, x2, o0, o1, o2);
   out[o] = o0;
   out[o + P] = o1;
   out[o + 2 * (size_t)P] = o2;
 }
 
 // A whole RK3 step of the global model per launch, for grids whose stages are
-// short: a stage of 512 x 256 points keeps the FP64 pipe busy for 6.3 us of its
-// 12.5, the rest is launch, load latency and drain.  A CTA owns a tile of
+// short beside their launch, load latency and drain.  A CTA owns a tile of
 // tx x ty points, loads it with three halo points a side, and forms the first
 // stage on the tile and two halo points, the second on one, all in shared
 // memory; rows beyond a wall are the mirror (h, u, -v) of the wall row at every
-// stage.  The recomputed halos cost 15-25 % more FP64 work.  Same values as the
-// stage kernel bit for bit.  Per step, one launch per stage of the kernel with
-// the old arithmetic -> this one: 32 x 16 points 14.9 -> 5.6 us, 128 x 64 16.9 ->
-// 5.7, 256 x 128 18.6 -> 11.5, 512 x 256 39.0 -> 30.0 (stage kernel above: 40).
+// stage.  The recomputed halos cost 17 % more FP64 work at 512 x 256 points, 35 % at
+// 256 x 128 and 68 % up to 128 x 64 (tiles of 16 x 4).  Same values as the stage
+// kernel bit for bit.  Per step, three plain stage launches with the same
+// arithmetic -> this kernel: 32 x 16 points 12.5 -> 6.0 us, 128 x 64 16.5 -> 6.1,
+// 256 x 128 18.6 -> 12.7, 512 x 256 39.0 -> 33.6.
 constexpr int kStepThreads = 384;
 struct StepTile {
   int tx, ty;
@@ -463,8 +411,8 @@ __host__ __device__ inline size_t step_smem(int tx, int ty) {
 extern __shared__ __align__(16) double step_sm[];
 
 __global__ void __launch_bounds__(kStepThreads) global_step_kernel(const double* x, double* nx, const double* rec,
-                                                                   double dtB, double dtgB, int nlon, int nlat,
-                                                                   StepTile tile) {
+                                                                   double dt, double Bth, double gBth, int nlon,
+                                                                   int nlat, StepTile tile) {
   const int tx = tile.tx, ty = tile.ty;
   const int i0 = blockIdx.x * tx, j0 = blockIdx.y * ty;
   const int cx = min(tx, nlon - i0), cy = min(ty, nlat - j0);   // own points
@@ -513,7 +461,8 @@ __global__ void __launch_bounds__(kStepThreads) global_step_kernel(const double*
     double rc[8];
     load_rec8(rec + 8 * (j0 + r), rc);
     const bool x3 = ca != 0.0;
-    global_pt(z, rc, dtB, dtgB, ca, cb, x3 ? X[xo] : 0.0, x3 ? X[xo + xp] : 0.0, x3 ? X[xo + 2 * xp] : 0.0, a, b, d);
+    global_pt(z, rc, dt, Bth, gBth, ca, cb, x3 ? X[xo] : 0.0, x3 ? X[xo + xp] : 0.0, x3 ? X[xo + 2 * xp] : 0.0, a, b,
+              d);
   };
   points(3, [&](int r, int c) {
     int i = (i0 + c) % nlon;
@@ -1035,39 +984,32 @@ cudaError_t launch_restrict_level(const SubDesc* subs, int n_sub, int nlon, int 
   return cudaGetLastError();
 }
 
-cudaError_t launch_background_stage(const double* x, const double* y, double* out, double ca, double cb,
-                                    const RowConst* rows, double Bth, double gBth, double dt, int nlon, int nlat,
-                                    cudaStream_t st) {
-  dim3 grid((nlon + 127) / 128, nlat);
-  background_stage_kernel<<<grid, 128, 0, st>>>(x, y, out, ca, cb, rows, Bth, gBth, dt, nlon, nlat);
-  return cudaGetLastError();
-}
-
 namespace {
 cudaError_t launch_global_stage(const double* x, const double* y, double* out, double ca, double cb,
-                                const double* rec, double dtB, double dtgB, int nlon, int nlat, cudaStream_t st) {
+                                const double* rec, double dt, double Bth, double gBth, int nlon, int nlat,
+                                cudaStream_t st) {
   const long long n = (long long)nlon * nlat;
   return launch_dependent(global_stage_kernel, dim3((unsigned)((n + kGlobalThreads - 1) / kGlobalThreads)),
-                          kGlobalThreads, 0, st, x, y, out, ca, cb, rec, dtB, dtgB, nlon, nlat);
+                          kGlobalThreads, 0, st, x, y, out, ca, cb, rec, dt, Bth, gBth, nlon, nlat);
 }
 }  // namespace
 
-// The step kernel's tile: the one whose busiest SM has the least FP64 work.
-// The stage kernels spend about 6 us more per stage than their FP64 work (24 /
-// 30 / 30 instructions a point, 16 cycles a warp instruction), the step kernel
-// about 6 us per step plus the halo points.  Measured, step kernel (as chosen)
-// against the old stage kernels: 360 x 181 points 17.7 / 26.9 us a step, 512 x 256
-// 30.0 / 39.0, 768 x 384 59.6 / 71.9, 1024 x 512 100.5 / 115.0.
+// The step kernel's tile: the one whose busiest SM has the least FP64 work (28 /
+// 34 / 34 instructions a point, 16 cycles a warp instruction of an SM).  The step
+// kernel takes about 6 us a step beside that, the stage kernels 13.  Measured, step
+// kernel against stage kernels (us a step): 32 x 16 points 6.0 / 7.0, 128 x 64
+// 6.1 / 8.0, 256 x 128 12.7 / 11.4, 360 x 181 19.8 / 18.7, 512 x 256 33.6 / 41.5; from
+// 768 x 384 (67.6 / 63.7) and 1024 x 512 (114.3 / 105.3) the stage kernels run.
 GlobalStepPlan global_step_plan(int nlon, int nlat) {
   GlobalStepPlan best;
   const double per = 16.0 / 32.0 / 2.07e3;   // us per FP64 thread instruction of an SM
-  const double stages = 18.0 + 84.0 * (double)nlon * nlat / 152.0 * per;
+  const double stages = 13.0 + 96.0 * (double)nlon * nlat / 152.0 * per;
   double least = stages;
   for (int tx = 16; tx <= 128; tx += 8)
     for (int ty = 4; ty <= 40; ++ty) {
       if (step_smem(tx, ty) > 110 * 1024 || tx - 8 >= nlon || ty - 1 >= nlat) continue;
       const long long n = (long long)((nlon + tx - 1) / tx) * ((nlat + ty - 1) / ty);
-      const double work = 24.0 * (tx + 4) * (ty + 4) + 30.0 * (tx + 2) * (ty + 2) + 30.0 * tx * ty;
+      const double work = 28.0 * (tx + 4) * (ty + 4) + 34.0 * (tx + 2) * (ty + 2) + 34.0 * tx * ty;
       const double cost = 6.0 + (double)((n + 151) / 152) * work * per;
       if (cost < least) {
         least = cost;
@@ -1079,21 +1021,21 @@ GlobalStepPlan global_step_plan(int nlon, int nlat) {
 }
 
 cudaError_t launch_global_step(const GlobalStepPlan& plan, const double* x, double* s1, double* s2, double* nx,
-                               const double* rec, double dtB, double dtgB, int nlon, int nlat, cudaStream_t st,
-                               long long* launches) {
+                               const double* rec, double dt, double Bth, double gBth, int nlon, int nlat,
+                               cudaStream_t st, long long* launches) {
   if (plan.tx > 0) {
     cudaError_t e = raise_smem_cap(global_step_kernel);
     if (e != cudaSuccess) return e;
     ++*launches;
     return launch_dependent(global_step_kernel,
                             dim3((unsigned)((nlon + plan.tx - 1) / plan.tx), (unsigned)((nlat + plan.ty - 1) / plan.ty)),
-                            kStepThreads, step_smem(plan.tx, plan.ty), st, x, nx, rec, dtB, dtgB, nlon, nlat,
+                            kStepThreads, step_smem(plan.tx, plan.ty), st, x, nx, rec, dt, Bth, gBth, nlon, nlat,
                             StepTile{plan.tx, plan.ty});
   }
   *launches += 3;
-  cudaError_t e = launch_global_stage(x, x, s1, 0.0, 1.0, rec, dtB, dtgB, nlon, nlat, st);
-  if (e == cudaSuccess) e = launch_global_stage(x, s1, s2, 0.75, 0.25, rec, dtB, dtgB, nlon, nlat, st);
-  if (e == cudaSuccess) e = launch_global_stage(x, s2, nx, 1.0 / 3.0, 2.0 / 3.0, rec, dtB, dtgB, nlon, nlat, st);
+  cudaError_t e = launch_global_stage(x, x, s1, 0.0, 1.0, rec, dt, Bth, gBth, nlon, nlat, st);
+  if (e == cudaSuccess) e = launch_global_stage(x, s1, s2, 0.75, 0.25, rec, dt, Bth, gBth, nlon, nlat, st);
+  if (e == cudaSuccess) e = launch_global_stage(x, s2, nx, 1.0 / 3.0, 2.0 / 3.0, rec, dt, Bth, gBth, nlon, nlat, st);
   return e;
 }
 cudaError_t launch_observe(const double* traj, int g0, int g1, long long n, const int* level,

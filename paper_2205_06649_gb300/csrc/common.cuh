@@ -313,21 +313,15 @@ cudaError_t launch_restrict_level(const SubDesc* subs, int n_sub, int nlon, int 
                                   int g0, int g1, double* xb_a, int max_pts, cudaStream_t st);
 
 // global model (whole sphere), FP64
-// One stage, out = ca x + cb (y + dt F(y)), with the arithmetic of the
-// background forecast (see background_pass).
-cudaError_t launch_background_stage(const double* x, const double* y, double* out, double ca, double cb,
-                                    const RowConst* rows, double Bth, double gBth, double dt, int nlon, int nlat,
-                                    cudaStream_t st);
-// Model runs.  rec: records of every row (fill_global_record of point.cuh, 8
-// doubles a row); dtB, dtgB: dt Bth, dt g Bth.
+// rec: records of every row (fill_global_record of point.cuh, 8 doubles a row)
 struct GlobalStepPlan {
   int tx = 0, ty = 0;         // tile of the step kernel; 0: one launch per stage
 };
 GlobalStepPlan global_step_plan(int nlon, int nlat);
 // one RK3 step x -> nx; s1, s2: scratch states of the stage kernels
 cudaError_t launch_global_step(const GlobalStepPlan& plan, const double* x, double* s1, double* s2, double* nx,
-                               const double* rec, double dtB, double dtgB, int nlon, int nlat, cudaStream_t st,
-                               long long* launches);
+                               const double* rec, double dt, double Bth, double gBth, int nlon, int nlat,
+                               cudaStream_t st, long long* launches);
 cudaError_t launch_observe(const double* traj, int g0, int g1, long long n, const int* level,
                            const int* var, const double* fi, const double* fj, int nlon, int nlat,
                            double* out, cudaStream_t st);

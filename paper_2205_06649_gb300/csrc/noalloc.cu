@@ -70,7 +70,7 @@ cudaError_t scratch_address(double** out) {
 // sums are rounded one by one (no contraction), as the host computes them for
 // dd4dv_create.
 __global__ void noalloc_rows_kernel(double* rec, int nlon, int nlat, double lat_min_deg, double lat_max_deg,
-                                    double radius, double gravity, double omega, double dt) {
+                                    double radius, double gravity, double omega) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= nlat) return;
   const double pi = 3.14159265358979323846;
@@ -88,7 +88,7 @@ __global__ void noalloc_rows_kernel(double* rec, int nlon, int nlat, double lat_
   r.tau = __ddiv_rn(tan(th), radius);
   r.BinvC = __ddiv_rn(Bth, r.c);
   r.gA = __dmul_rn(gravity, r.A);
-  fill_global_record(r, cos(theta(min(j + 1, nlat - 1))), cos(theta(max(j - 1, 0))), dt, Bth, rec + 8 * j);
+  fill_global_record(r, cos(theta(min(j + 1, nlat - 1))), cos(theta(max(j - 1, 0))), rec + 8 * j);
 }
 
 }  // namespace
@@ -130,9 +130,9 @@ extern "C" dd4dv_status dd4dv_forward_noalloc(const dd4dv_model* model, const do
   const double pi = 3.14159265358979323846;
   const double dth = (m.lat_max_deg - m.lat_min_deg) * pi / 180.0 / m.nlat;
   const double Bth = 1.0 / (2.0 * m.radius * dth);
-  const double dtB = m.dt * Bth, dtgB = m.dt * (m.gravity * Bth);
+  const double gBth = m.gravity * Bth;
   noalloc_rows_kernel<<<(m.nlat + 127) / 128, 128, 0, st>>>(rec, m.nlon, m.nlat, m.lat_min_deg, m.lat_max_deg,
-                                                           m.radius, m.gravity, m.omega, m.dt);
+                                                           m.radius, m.gravity, m.omega);
   e = cudaGetLastError();
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(traj, x0, G * sizeof(double), cudaMemcpyDeviceToDevice, st);
@@ -141,7 +141,7 @@ extern "C" dd4dv_status dd4dv_forward_noalloc(const dd4dv_model* model, const do
   for (int n = 0; n < m.nsteps && e == cudaSuccess; ++n) {
     const double* x = traj + (size_t)n * G;
     double* nx = traj + (size_t)(n + 1) * G;
-    e = launch_global_step(plan, x, s1, s2, nx, rec, dtB, dtgB, m.nlon, m.nlat, st, &launches);
+    e = launch_global_step(plan, x, s1, s2, nx, rec, m.dt, Bth, gBth, m.nlon, m.nlat, st, &launches);
   }
   if (e != cudaSuccess) return bad(DD4DV_ECUDA, std::string("dd4dv_forward_noalloc: ") + cudaGetErrorString(e));
   set_global_error("");

@@ -197,44 +197,55 @@ __host__ __device__ inline void fill_records(const RowConst& r, double cN, doubl
   }
 }
 
-// FP64 forms for the fewest FP64 instructions.  The FP64 pipe issues one warp
+// One RK3 stage of the global model at one point, out = ca X + cb (Y + dt F(Y))
+// from rec = A, f, tau, g A, Bth / c, cN, cS.  28 FP64 instructions (34 with X).
+// Forecasts and model runs share it, so that a run from the background is the
+// library's own background trajectory.  The tendencies are summed before they
+// meet the state: h is some 4000 m, and with one fused operation a term into it
+// (24 instructions) its roundings were 1.0-1.25x larger.
+__host__ __device__ inline void fill_global_record(const RowConst& r, double cN, double cS, double* rec) {
+  rec[0] = r.A;
+  rec[1] = r.f;
+  rec[2] = r.tau;
+  rec[3] = r.gA;
+  rec[4] = r.BinvC;
+  rec[5] = cN;
+  rec[6] = cS;
+  rec[7] = 0.0;
+}
+__device__ __forceinline__ void global_pt(const Pt5<double>& y, const double (&rc)[8], double dt, double Bth,
+                                          double gBth, double ca, double cb, double x0, double x1, double x2,
+                                          double& oh, double& ou, double& ov) {
+  const double fu = xfma(rc[2], y.u, rc[1]), Au = xmul(rc[0], y.u), Bv = xmul(Bth, y.v);
+  double Fu = xfma(-Au, xsub(y.uE, y.uW), -xmul(Bv, xsub(y.uN, y.uS)));
+  Fu = xfma(fu, y.v, Fu);
+  Fu = xfma(-rc[3], xsub(y.hE, y.hW), Fu);
+  double Fv = xfma(-Au, xsub(y.vE, y.vW), -xmul(Bv, xsub(y.vN, y.vS)));
+  Fv = xfma(-fu, y.u, Fv);
+  Fv = xfma(-gBth, xsub(y.hN, y.hS), Fv);
+  const double fx = xfma(y.hE, y.uE, -xmul(y.hW, y.uW));
+  const double fy = xfma(xmul(y.hN, y.vN), rc[5], -xmul(xmul(y.hS, y.vS), rc[6]));
+  const double Fh = xfma(-rc[0], fx, -xmul(rc[4], fy));
+  oh = xfma(dt, Fh, y.h);
+  ou = xfma(dt, Fu, y.u);
+  ov = xfma(dt, Fv, y.v);
+  if (ca != 0.0) {
+    oh = xfma(ca, x0, xmul(cb, oh));
+    ou = xfma(ca, x1, xmul(cb, ou));
+    ov = xfma(ca, x2, xmul(cb, ov));
+  }
+}
+
+// The FP64 adjoint in its form of fewest FP64 instructions.  The FP64 pipe issues one warp
 // instruction in 16 cycles per SM and bounds every FP64 sweep.  The records
 // (and Bth, g Bth) hold dt times the constant, the cos ratios of the neighbour
 // rows are folded into one constant each, and every term is one fused
 // multiply-add into the value that it changes: a stage adjoint takes 38
 // instructions instead of 45, lambda(n) 47 instead of 54 (medium workload, 64
 // boxes of 72 x 36..40 points in clusters of 4 x 192 threads: adjoint 2.67 ->
-// 2.32 ms).  The box model's forward stages keep the order of rhs_pt: their
+// 2.32 ms).  The forward stages keep the order of rhs_pt and global_pt: their
 // rounding of h, some 1e-13 of a misfit, is what an analysis amplifies, and a
 // second order of roundings would show in it at 1e-10.
-
-// Y + dt F(Y) at one point (global model runs): 24 instructions, from rec =
-// dt A, dt f, dt tau, dt g A, dt Bth cN / c, dt Bth cS / c and dt Bth, dt g Bth.
-__host__ __device__ inline void fill_global_record(const RowConst& r, double cN, double cS, double dt, double Bth,
-                                                   double* rec) {
-  rec[0] = dt * r.A;
-  rec[1] = dt * r.f;
-  rec[2] = dt * r.tau;
-  rec[3] = dt * r.gA;
-  rec[4] = dt * Bth * cN / r.c;
-  rec[5] = dt * Bth * cS / r.c;
-  rec[6] = rec[7] = 0.0;
-}
-__device__ __forceinline__ void euler_pt64(const Pt5<double>& y, const double (&rc)[8], double Bth, double gBth,
-                                           double& oh, double& ou, double& ov) {
-  const double fu = xfma(rc[2], y.u, rc[1]), Au = xmul(rc[0], y.u), Bv = xmul(Bth, y.v);
-  ou = xfma(-rc[3], xsub(y.hE, y.hW), y.u);
-  ou = xfma(-Au, xsub(y.uE, y.uW), ou);
-  ou = xfma(-Bv, xsub(y.uN, y.uS), ou);
-  ou = xfma(fu, y.v, ou);
-  ov = xfma(-gBth, xsub(y.hN, y.hS), y.v);
-  ov = xfma(-Au, xsub(y.vE, y.vW), ov);
-  ov = xfma(-Bv, xsub(y.vN, y.vS), ov);
-  ov = xfma(-fu, y.u, ov);
-  oh = xfma(-rc[0], xfma(y.hE, y.uE, -xmul(y.hW, y.uW)), y.h);
-  oh = xfma(-rc[4], xmul(y.hN, y.vN), oh);
-  oh = xfma(rc[5], xmul(y.hS, y.vS), oh);
-}
 // M + dt F'(Z)^T M at one point (the terms of rhs_adj_pt).
 __device__ __forceinline__ void adjoint_pt64(const Pt5<double>& z, const Pt5<double>& m, const double (&rc)[8],
                                              double Bth, double gBth, int wall, double& oh, double& ou, double& ov) {
