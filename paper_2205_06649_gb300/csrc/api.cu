@@ -2207,8 +2207,7 @@ TzArgs tz_args(dd4dv_ctx* ctx, int p, int q, double alpha) {
   t.g = m.gravity;
   t.dt = m.dt;
   t.rec = nullptr;
-  t.st = m.dt * t.slat;
-  t.gq = m.dt * t.slat * m.gravity / q;
+  t.gq = t.slat * m.gravity / q;
   return t;
 }
 

@@ -371,16 +371,16 @@ cudaError_t launch_max_abs_diff(const double* a, const double* b, long long n, d
 cudaError_t launch_finite_check(const double* a, long long n, int* flag, cudaStream_t st);
 
 // ---- Turkel-Zwas scheme on the whole sphere (tz.cu) ----
-struct TzRow {                // per latitude row, times dt where a tendency uses it
-  double a, f, tau, c;        // dt s_lon / c, dt f, dt tau, c
-  double kg, kp, kq, pad;     // dt s_lon g / (p c), dt s_lon / (p c), dt s_lat / (q c)
+struct TzRow {                // per latitude row
+  double a, f, tau, c;        // s_lon / c, f, tau, c
+  double kg, kp, kq, pad;     // s_lon g / (p c), s_lon / (p c), s_lat / (q c)
 };
 struct TzArgs {
   const RowConst* rows;       // [nlat]
   const TzRow* rec;           // [nlat] (launch_tz_rows)
   int nlon, nlat, p, q;
   double alpha, slon, slat, g, dt;
-  double st, gq;              // dt s_lat, dt s_lat g / q
+  double gq;                  // s_lat g / q
 };
 cudaError_t launch_tz_rows(const TzArgs& t, TzRow* rec, cudaStream_t st);
 cudaError_t launch_tz_stage(const TzArgs& t, const double* X, const double* Y, double* out, double cx, double cy,

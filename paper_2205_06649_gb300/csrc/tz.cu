@@ -18,10 +18,17 @@
 // collects, term by term, what the points that read it send back, so there are
 // no atomic additions and the result does not depend on their order.
 // Bound: launch latency on small grids (8 launches a step of about 3 us), the
-// FP64 pipe on large ones.  Row constants hold every quotient and dt
-// (launch_tz_rows): the divisions were most of the FP64 work.
-// 256 x 128 points, 128 steps, (p, q, alpha) = (2, 1, 1/2), J and gradient:
-// 21.1 -> 7.3 ms.
+// FP64 pipe on large ones.  Row constants hold every quotient (launch_tz_rows):
+// the divisions were most of the FP64 work.  256 x 128 points, 128 steps,
+// (p, q, alpha) = (2, 1, 1/2), J and gradient: 21.1 -> 7.6 ms.
+//
+// Roundings: h is some 4000 m and every operation on it rounds by up to 2e-13 m,
+// in the combination (1/3) X + (2/3) Y to one side, so that a run drifts by its
+// order of operations.  The order here (tendencies summed and multiplied by dt
+// first, (1/3) X rounded by itself) is that of the plain stage: with dt in the row
+// constants, one operation a term into the state and (2/3) Y rounded by itself,
+// 2 % faster, gradients of 54- to 172-step runs were up to 2.3 times further from
+// a plain 64-bit evaluation (236 x 98 points, 172 steps: 2.0e-12 against 8.6e-13).
 #include "common.cuh"
 
 namespace dd4dv {
@@ -232,7 +239,7 @@ __global__ void __launch_bounds__(kTzThreads) tz_stage_kernel(TzArgs t, const do
   const TzRow rc = t.rec[m.j];
   const double cN = sN * t.rec[jN].c, cS = sS * t.rec[jS].c;   // (v c) through the mirror
   const double h = H[o], u = U[o], v = V[o], al = t.alpha, a1 = 1.0 - al, a2 = 0.5 * al;
-  const double Au = rc.a * u, Bv = t.st * v, C = fma(rc.tau, u, rc.f);
+  const double Au = rc.a * u, Bv = t.slat * v, C = fma(rc.tau, u, rc.f);
   const double uEp = U[row + pE], uWp = U[row + pW], vN = V[rN + m.i], vS = V[rS + m.i];
   double cu = a1 * C * v, cv = a1 * C * u;
   double du = a1 * (uEp - uWp), dv = a1 * fma(vN, cN, -vS * cS);
@@ -244,19 +251,19 @@ __global__ void __launch_bounds__(kTzThreads) tz_stage_kernel(TzArgs t, const do
     du = fma(a2, (U[rN + pE] - U[rN + pW]) + (U[rS + pE] - U[rS + pW]), du);
     dv = fma(a2, fma(V[rN + pE] + V[rN + pW], cN, -(V[rS + pE] + V[rS + pW]) * cS), dv);
   }
-  double ou = fma(-Au, U[row + iE] - U[row + iW], u);
-  ou = fma(-Bv, U[r1N + m.i] - U[r1S + m.i], ou);
-  ou = fma(-rc.kg, H[row + pE] - H[row + pW], ou) + cu;
-  double ov = fma(-Au, V[row + iE] - V[row + iW], v);
-  ov = fma(-Bv, s1N * V[r1N + m.i] - s1S * V[r1S + m.i], ov);
-  ov = fma(-t.gq, H[rN + m.i] - H[rS + m.i], ov) - cv;
-  double oh = fma(-Au, H[row + iE] - H[row + iW], h);
-  oh = fma(-Bv, H[r1N + m.i] - H[r1S + m.i], oh);
-  oh = fma(-h, fma(rc.kp, du, rc.kq * dv), oh);
+  double Fu = fma(Au, U[row + iE] - U[row + iW], Bv * (U[r1N + m.i] - U[r1S + m.i]));
+  Fu = cu - fma(rc.kg, H[row + pE] - H[row + pW], Fu);
+  double Fv = fma(Au, V[row + iE] - V[row + iW], Bv * (s1N * V[r1N + m.i] - s1S * V[r1S + m.i]));
+  Fv = -cv - fma(t.gq, H[rN + m.i] - H[rS + m.i], Fv);
+  double Fh = fma(Au, H[row + iE] - H[row + iW], Bv * (H[r1N + m.i] - H[r1S + m.i]));
+  Fh = -fma(h, fma(rc.kp, du, rc.kq * dv), Fh);
+  // One rounding of the size of h a stage, not one a term, and (1/3) X rounded by
+  // itself: see the head of the file.
+  double oh = fma(t.dt, Fh, h), ou = fma(t.dt, Fu, u), ov = fma(t.dt, Fv, v);
   if (cx != 0.0) {
-    oh = fma(cx, X[o], cy * oh);
-    ou = fma(cx, X[o + pl], cy * ou);
-    ov = fma(cx, X[o + 2 * pl], cy * ov);
+    oh = fma(cy, oh, __dmul_rn(cx, X[o]));
+    ou = fma(cy, ou, __dmul_rn(cx, X[o + pl]));
+    ov = fma(cy, ov, __dmul_rn(cx, X[o + 2 * pl]));
   }
   out[o] = oh;
   out[o + pl] = ou;
@@ -298,17 +305,17 @@ __global__ void __launch_bounds__(kTzThreads) tz_adj_kernel(TzArgs t, const doub
   // advection: what F of the four neighbours reads of (h, u, v) here.  The
   // northern neighbour reads this point as its south: + s_lat v m; a mirrored
   // one (sg = -1) with the other sign, and vN, vS carry that sign.
-  double gh = fma(rc.a, fma(uE, mhE, -uW * mhW), xh);
-  double gu = fma(rc.a, fma(uE, muE, -uW * muW), xu);
-  double gv = fma(rc.a, fma(uE, mvE, -uW * mvW), xv);
-  gh = fma(t.st, fma(vN, mh[N1], -vS * mh[S1]), gh);
-  gu = fma(t.st, fma(vN, mu[N1], -vS * mu[S1]), gu);
-  gv = fma(t.st, fma(s1N * vN, mv[N1], -s1S * vS * mv[S1]), gv);
+  double gh = rc.a * fma(uE, mhE, -uW * mhW);
+  double gu = rc.a * fma(uE, muE, -uW * muW);
+  double gv = rc.a * fma(uE, mvE, -uW * mvW);
+  gh = fma(t.slat, fma(vN, mh[N1], -vS * mh[S1]), gh);
+  gu = fma(t.slat, fma(vN, mu[N1], -vS * mu[S1]), gu);
+  gv = fma(t.slat, fma(s1N * vN, mv[N1], -s1S * vS * mv[S1]), gv);
   // own coefficients: u and v multiply the centred differences of all three
   const double dhx = H[E] - H[W], dux = uE - uW, dvx = V[E] - V[W];
   const double dhy = H[N1] - H[S1], duy = U[N1] - U[S1], dvy = vN - vS;
   gu = fma(-rc.a, fma(xu, dux, fma(xv, dvx, xh * dhx)), gu);
-  gv = fma(-t.st, fma(xu, duy, fma(xv, dvy, xh * dhy)), gv);
+  gv = fma(-t.slat, fma(xu, duy, fma(xv, dvy, xh * dhy)), gv);
   // Coriolis
   gu = fma(a1, fma(xu * rc.tau, v, -xv * fma(rc.tau, u, C)), gu);
   gv = fma(a1 * xu, C, gv);
@@ -335,7 +342,7 @@ __global__ void __launch_bounds__(kTzThreads) tz_adj_kernel(TzArgs t, const doub
     dv = fma(a2, fma(V[rN + pE] + V[rN + pW], cN, -(V[rS + pE] + V[rS + pW]) * cS), dv);
   }
   gh = fma(-xh, fma(rc.kp, du, rc.kq * dv), gh);
-  double g[3] = {gh, gu, gv};
+  double g[3] = {fma(t.dt, gh, xh), fma(t.dt, gu, xu), fma(t.dt, gv, xv)};
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const size_t q = o + c * pl;
@@ -451,13 +458,13 @@ __global__ void tz_rows_kernel(TzArgs t, TzRow* rec) {
   if (j >= t.nlat) return;
   const RowConst r = t.rows[j];
   TzRow q;
-  q.a = t.dt * t.slon / r.c;
-  q.f = t.dt * r.f;
-  q.tau = t.dt * r.tau;
+  q.a = t.slon / r.c;
+  q.f = r.f;
+  q.tau = r.tau;
   q.c = r.c;
-  q.kg = t.dt * t.slon * t.g / (t.p * r.c);
-  q.kp = t.dt * t.slon / (t.p * r.c);
-  q.kq = t.dt * t.slat / (t.q * r.c);
+  q.kg = t.slon * t.g / (t.p * r.c);
+  q.kp = t.slon / (t.p * r.c);
+  q.kq = t.slat / (t.q * r.c);
   q.pad = 0.0;
   rec[j] = q;
 }

@@ -34,3 +34,32 @@ def test_forward_run_is_the_background_trajectory(nlon, nlat, P1, P2):
     run, back = ctx.forward(inp["x_b0"]), ctx.boundary_trajectory()
     ctx.destroy()
     assert np.array_equal(run, back)
+
+
+def test_turkel_zwas_run_drifts_like_the_plain_step():
+    """Every operation on h rounds by up to half an ulp (2.3e-13 m), in the RK3
+    combination 1/3 X + 2/3 Y to one side, so that the mean of h drifts by the
+    order of its operations.  The run's order rounds 1/3 X first and fuses 2/3 Y;
+    the oracle's divides and adds.  Their drifts per step, from the same
+    combinations of random values, differ by 5e-14 m; fusing 1/3 X instead would
+    leave no difference, so half of it is the bar."""
+    import oracle
+    import paper_2205_06649_gb300 as dd
+    nlon, nlat, nsteps = 96, 48, 120
+    wl = workloads.preset("small", nlon=nlon, nlat=nlat, nsteps=nsteps)
+    inp = workloads.generate(wl)
+    ctx = dd.Context(nlon, nlat, inp["dt"], nsteps)
+    run = ctx.tz_forward(3, 1, 0.0, inp["x_t0"])[-1, 0]
+    ctx.destroy()
+    grid = oracle.Grid(nlon, nlat, workloads.RADIUS, workloads.GRAVITY, workloads.OMEGA, workloads.LAT_MIN_DEG,
+                       workloads.LAT_MAX_DEG)
+    ref = oracle.tz_forward(grid, torch.as_tensor(inp["x_t0"]), inp["dt"], nsteps, 3, 1, 0.0).numpy()[-1, 0]
+    rng = np.random.default_rng(0)
+    X = 4000.0 + 30.0 * rng.standard_normal(200000)
+    Y = X + 0.01 * rng.standard_normal(X.size)
+    L = np.longdouble
+    fused = (L(2.0 / 3.0) * Y.astype(L) + ((1.0 / 3.0) * X).astype(L)).astype(np.float64)
+    want = np.mean(fused - (X / 3.0 + (2.0 / 3.0) * Y))
+    got = np.mean(run - ref) / nsteps
+    assert -6e-14 < want < -4e-14
+    assert abs(got - want) <= 0.5 * abs(want), (got, want)
