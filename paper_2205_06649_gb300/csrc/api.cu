@@ -142,6 +142,7 @@ struct dd4dv_ctx {
   // level sweeps (level.cu): tiles and scratch states; lv_f / lv_a: the forward
   // / adjoint sweeps run them (else the cluster sweeps)
   bool lv_f = false, lv_a = false;
+  bool all_levels = false;    // the last forward sweep stored every level
   LvPlan lv;
   LvTile* lv_tiles = nullptr;
   int *lv_boxes = nullptr, *lv_tile_off = nullptr;
@@ -380,7 +381,9 @@ void apply_VT(dd4dv_ctx* ctx, const double* y, const double* w, const double* sc
 bool level_forward(const dd4dv_ctx* ctx) { return ctx->lv_f && ctx->variant_f == 0; }
 bool level_adjoint(const dd4dv_ctx* ctx) {
   // the level adjoint reads every level: under checkpoints only the level
-  // forward has stored them (it always stores every level)
+  // forward stores them (it always stores every level).  A forward sweep that
+  // ran before another variant was set may not have: adjoint_sweep looks at
+  // all_levels too.
   return ctx->lv_a && ctx->variant_a == 0 && (ctx->ckpt == 0 || level_forward(ctx));
 }
 
@@ -445,6 +448,7 @@ LvArgs<T> level_args(dd4dv_ctx* ctx, const int* active, int av) {
 // evaluations checkpoint, and leaves the terms of J out.
 template <typename T>
 void forward_sweep(dd4dv_ctx* ctx, const int* active, int av, bool full = false) {
+  ctx->all_levels = full || ctx->ckpt == 0 || level_forward(ctx);
   if (level_forward(ctx)) {
     LvArgs<T> a = level_args<T>(ctx, active, av);
     a.terms = !full;
@@ -480,7 +484,7 @@ void finalize_J(dd4dv_ctx* ctx, const double* w, double* J, double* parts, const
 // product by the tangent-linear run in gn_dx.
 template <typename T>
 void adjoint_sweep(dd4dv_ctx* ctx, const int* active, int av, const double* yforce = nullptr, T* gn_dx = nullptr) {
-  if (level_adjoint(ctx)) {
+  if (level_adjoint(ctx) && ctx->all_levels) {
     LvArgs<T> a = level_args<T>(ctx, active, av);
     a.yforce = yforce;
     a.gn_dx = gn_dx;

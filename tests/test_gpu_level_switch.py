@@ -1,0 +1,72 @@
+"""What may change between, and around, the calls that run level sweeps: kernel
+variants, masks, streams of other contexts, memory."""
+import numpy as np
+import pytest
+import torch
+
+import workloads
+from _helpers import tiny_workload
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    import __graft_entry__ as g
+    g.build()
+
+
+@pytest.fixture
+def level_context(monkeypatch):
+    """make(precision, ckpt_k, cluster, env, **workload): a context whose boxes
+    are advanced by level sweeps whatever their number of points."""
+    made = []
+
+    def make(precision=0, ckpt_k=0, cluster=0, env=None, **kw):
+        import paper_2205_06649_gb300 as dd
+        wl = tiny_workload(**{**dict(obs_count=400, obs_every=2, corr_len=1.5), **kw})
+        inp = workloads.generate(wl)
+        for k, v in {"DD4DV_LEVEL_MIN_POINTS": 1, **(env or {})}.items():
+            monkeypatch.setenv(k, str(v))
+        ctx = dd.Context(wl.nlon, wl.nlat, inp["dt"], wl.nsteps, precision=precision)
+        made.append(ctx)
+        ctx.set_background(inp["x_b0"])
+        ctx.set_background_error(wl.sigma_b, wl.corr_len, wl.rf_passes)
+        so = np.asarray(wl.sigma_o)[inp["obs_var"]]
+        y = np.where(inp["obs_var"] == 0, workloads.H_REF, 0.0) + so * inp["obs_noise"]
+        ctx.set_observations(inp["obs_level"], inp["obs_var"], inp["obs_fi"], inp["obs_fj"], y, so)
+        ctx.set_decomposition(wl.P1, wl.P2, wl.Q, wl.o_lon, wl.o_lat, wl.o_t, inp["lon_cuts"], inp["lat_cuts"],
+                              inp["t_cuts"], cluster=cluster, ckpt_k=ckpt_k)
+        return ctx
+
+    yield make
+    for ctx in made:
+        ctx.destroy()
+
+
+def controls(ctx, seed=17):
+    return 0.3 * np.random.default_rng(seed).standard_normal(ctx.ctrl_total)
+
+
+RAGGED = dict(nlon=70, nlat=38, nsteps=30, P1=3, P2=2, Q=2, o_lon=3, o_lat=3, o_t=3, uneven=True)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_backward_after_a_variant_change_reads_what_was_stored(level_context, precision):
+    """Under checkpoints the cluster forward stores every fourth level only; a
+    backward pass that follows a return to the level sweeps must recompute the
+    others, not read them as if they were there."""
+    ctx = level_context(precision, ckpt_k=4, **RAGGED)
+    assert ctx.sweep_kernels() == {"forward": 5, "adjoint": 5}
+    w = controls(ctx)
+    _, ref = ctx.eval(w)
+    ctx.eval(0.0 * w)   # other levels in the trajectory buffer
+    ctx.set_sweep_variant(1, 1)
+    ctx.eval_forward(w)
+    ctx.set_sweep_variant(0, 0)
+    assert np.array_equal(ctx.eval_backward(), ref)
+    ctx.eval_forward(w)   # and the other way: a level forward, a cluster adjoint
+    ctx.set_sweep_variant(1, 1)
+    assert np.array_equal(ctx.eval_backward(), ref)
