@@ -452,7 +452,9 @@ dd4dv_status dd4dv_stage1_stored(const dd4dv_ctx* ctx, int* n_subs, double* pt_s
  * partial sums, and give way to the cluster sweeps when a variant other than 0
  * or a launch shape (dd4dv_set_sweep_config) is set.  The environment variable
  * DD4DV_LEVEL_MIN_POINTS, read by dd4dv_set_decomposition, replaces the number
- * of points from which they are chosen.
+ * of points from which they are chosen; DD4DV_RING_MIN_TILES the number of tiles
+ * per CTA from which the FP32 adjoint runs pipelined, and DD4DV_RING_MAX_CTAS
+ * bounds the CTAs of a pipelined launch (all three for tests).
  * forward: 0 = level sweep where chosen, else deep-halo sweep wherever it
  * applies (default), 1 = stripe sweep only, 2 = the two-buffer stripe forward where it applies (else as
  * 1).  adjoint: 0 and 1 as for the forward (the stripe adjoint takes its

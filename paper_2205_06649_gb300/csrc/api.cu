@@ -1067,6 +1067,8 @@ void level_plan(dd4dv_ctx* ctx, const std::vector<SubDesc>& subs, const std::vec
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     long long ring_min = kRingMinTiles;
     if (const char* e = std::getenv("DD4DV_RING_MIN_TILES")) ring_min = std::atoll(e);   // override (tests)
+    int most = 1 << 30;
+    if (const char* e = std::getenv("DD4DV_RING_MAX_CTAS")) most = std::max(1, std::atoi(e));   // override (tests)
     for (int q = 0; q < 3 && g.n_ring[0] >= ring_min * 2 * sms; ++q) {
       LvRing& r = g.ring[q];
       r.own_floats = q == 2 ? 12 * kRingPoints : 0;
@@ -1075,7 +1077,7 @@ void level_plan(dd4dv_ctx* ctx, const std::vector<SubDesc>& subs, const std::vec
         const int fit = (bytes / 4 - r.own_floats) / r.slot_floats;
         if (fit >= 2) {
           r.slots = std::min(fit, 4);
-          r.ctas = c * sms;
+          r.ctas = std::min(c * sms, most);
         }
       }
     }

@@ -949,10 +949,11 @@ __device__ __forceinline__ void ring_run(const LvArgs<float>& a, float* smem, I&
       asm volatile("cp.async.commit_group;" ::: "memory");
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
-    if (j < n) {   // a wait ran out: report, wait for the copies that were started
-      if (lane == 0) atomicExch(a.err, 3);
-      for (int q = max(j - S, 0); q < j; ++q) ring_wait(full + q % S, (unsigned)(q / S) & 1u);
-    }
+    if (j < n && lane == 0) atomicExch(a.err, 3);   // a wait ran out
+    // The copies of the last tiles end before this warp does, also where a
+    // computing warp has given up on them: none may reach the shared memory of
+    // the CTA that comes next.  (The copying warp has nothing else to do by then.)
+    for (int q = max(j - S, 0); q < j; ++q) ring_wait(full + q % S, (unsigned)(q / S) & 1u);
     return;
   }
   int slot = 0;
@@ -963,7 +964,7 @@ __device__ __forceinline__ void ring_run(const LvArgs<float>& a, float* smem, I&
          [&]() { return ok = ring_wait(full + slot, parity); });
     if (!ok) {
       atomicExch(a.err, 3);
-      return;
+      break;
     }
     __syncwarp();
     if ((threadIdx.x & 31) == 0)
@@ -973,6 +974,9 @@ __device__ __forceinline__ void ring_run(const LvArgs<float>& a, float* smem, I&
       parity ^= 1u;
     }
   }
+  // overlap values prefetched for a tile that was left out, or given up, may
+  // still be on their way
+  asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 // Whether one of the columns k .. k + 3 can be in an overlap.

@@ -70,3 +70,36 @@ def test_backward_after_a_variant_change_reads_what_was_stored(level_context, pr
     ctx.eval_forward(w)   # and the other way: a level forward, a cluster adjoint
     ctx.set_sweep_variant(1, 1)
     assert np.array_equal(ctx.eval_backward(), ref)
+
+
+RING = {
+    "ragged": RAGGED,
+    "many rows": dict(nlon=384, nlat=160, nsteps=12, P1=4, P2=2, Q=4, o_lon=4, o_lat=4),
+    "wide": dict(nlon=560, nlat=90, nsteps=6, P1=2, P2=2, Q=2, o_lon=4, o_lat=3),     # boxes 288 wide, rows in threes
+    "walls": dict(nlon=52, nlat=64, nsteps=9, P1=2, P2=1, Q=3, o_lon=3, o_t=1),
+    "one box": dict(nlon=33, nlat=100, nsteps=9, P1=1, P2=1, Q=1),                    # periodic
+}
+
+
+@pytest.mark.parametrize("name", list(RING))
+@pytest.mark.parametrize("ctas", [1, 3, 8])
+def test_pipelined_adjoint_in_its_steady_state(level_context, name, ctas):
+    """The pipelined adjoint with so few CTAs that each takes many tiles: slots
+    and descriptors come round again, masked boxes are passed over (the last
+    ones too), gradients stay bit for bit those of the plain phases."""
+    out, kernels = [], []
+    for env in (dict(DD4DV_RING_MIN_TILES=0, DD4DV_RING_MAX_CTAS=ctas), dict(DD4DV_RING_MIN_TILES=1 << 40)):
+        ctx = level_context(1, env=env, **RING[name])
+        w, rng = controls(ctx), np.random.default_rng(3)
+        p, force = rng.standard_normal(ctx.ctrl_total), rng.standard_normal(ctx.traj_total)
+        ctx.exchange(0.5 * w)
+        k0 = ctx.launch_count()
+        r = [ctx.eval(w)[1], ctx.gn_hessvec(w, p), ctx.adjoint(w, force)]
+        kernels.append(ctx.launch_count() - k0)
+        for m in ((np.arange(ctx.n_sub) % 3 == 0), np.arange(ctx.n_sub) < (ctx.n_sub + 1) // 2):
+            ctx.set_owned(m.astype(np.int32))
+            r.append(ctx.eval(w)[1])
+        out.append(r)
+    assert kernels[0] != kernels[1]   # (the pipelined form adds the observations in a kernel of their own)
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
