@@ -52,10 +52,12 @@ typedef enum {
   DD4DV_ENOMEM = -2,       /* device or pinned host allocation failed      */
   DD4DV_ECUDA = -3,        /* CUDA runtime error (message has the details) */
   DD4DV_ESTATE = -4,       /* call made before its prerequisites           */
-  DD4DV_ETIMEOUT = -5,     /* reserved, never returned: no kernel of this
-                              library spin-waits (the sweeps synchronise
-                              only through hardware cluster barriers), so
-                              there is no bounded wait that could run out  */
+  DD4DV_ETIMEOUT = -5,     /* a bounded device wait ran out: a copy of the
+                              pipelined FP32 adjoint did not arrive.  The
+                              gradients of that sweep are NaN; the context
+                              stays usable.  A call with device pointers
+                              does not synchronise, so the next call on the
+                              context returns it instead                    */
   DD4DV_ENONFINITE = -6,   /* NaN or Inf in an input                       */
   DD4DV_NOTCONV = 1        /* warning: stopping test not met, outputs valid */
 } dd4dv_status;
@@ -452,9 +454,10 @@ dd4dv_status dd4dv_stage1_stored(const dd4dv_ctx* ctx, int* n_subs, double* pt_s
  * partial sums, and give way to the cluster sweeps when a variant other than 0
  * or a launch shape (dd4dv_set_sweep_config) is set.  The environment variable
  * DD4DV_LEVEL_MIN_POINTS, read by dd4dv_set_decomposition, replaces the number
- * of points from which they are chosen; DD4DV_RING_MIN_TILES the number of tiles
- * per CTA from which the FP32 adjoint runs pipelined, and DD4DV_RING_MAX_CTAS
- * bounds the CTAs of a pipelined launch (all three for tests).
+ * of points from which they are chosen.  Three more are for tests:
+ * DD4DV_RING_MIN_TILES replaces the number of tiles per CTA from which the FP32
+ * adjoint runs pipelined, DD4DV_RING_MAX_CTAS bounds the CTAs of a pipelined
+ * launch, and with DD4DV_RING_EXPIRE set its waits run out at once.
  * forward: 0 = level sweep where chosen, else deep-halo sweep wherever it
  * applies (default), 1 = stripe sweep only, 2 = the two-buffer stripe forward where it applies (else as
  * 1).  adjoint: 0 and 1 as for the forward (the stripe adjoint takes its

@@ -127,6 +127,7 @@ struct dd4dv_ctx {
   double* scal_d = nullptr;
   double* scal_h = nullptr;   // pinned
   int* err_d = nullptr;
+  int* late_h = nullptr;      // pinned, written by the device: a lost copy (see ring_lost in level.cu)
   int vblocks = 8;
   bool fwd_pending = false;
   LbState* lbst_h = nullptr;  // pinned
@@ -182,11 +183,15 @@ namespace {
   throw Fail{st};
 }
 
+void sync(dd4dv_ctx* ctx);
+
 template <typename F>
 dd4dv_status guard(dd4dv_ctx* ctx, F&& f) {
   if (!ctx) return DD4DV_EINVAL;
   ctx->err.clear();
   try {
+    // a copy lost since the last synchronisation, by a call with device pointers
+    if (ctx->late_h && *(volatile int*)ctx->late_h) sync(ctx);
     return f();
   } catch (const Fail& e) {
     return e.st;
@@ -218,6 +223,11 @@ void sync(dd4dv_ctx* ctx) {
   CK(cudaMemcpy(&h, ctx->err_d, sizeof(int), cudaMemcpyDeviceToHost));
   if (h) {
     CK(cudaMemset(ctx->err_d, 0, sizeof(int)));
+    if (h == kErrLostCopy) {
+      *ctx->late_h = 0;
+      fail(ctx, DD4DV_ETIMEOUT, "adjoint sweep: a copy did not reach shared memory within the wait limit; the "
+                                "gradients of that sweep are NaN");
+    }
     fail(ctx, DD4DV_EINVAL, "device kernel rejected its launch configuration (code %d)", h);
   }
 }
@@ -398,6 +408,7 @@ LvArgs<T> level_args(dd4dv_ctx* ctx, const int* active, int av) {
   a.boxes = ctx->lv_boxes;
   a.box_off = ctx->lv_box_off;
   a.err = ctx->err_d;
+  a.late = ctx->late_h;
   a.subs = ctx->subs_d;
   a.mu_on = ctx->dec.mu != 0.0;
   a.traj = static_cast<T*>(ctx->traj);
@@ -1067,6 +1078,7 @@ void level_plan(dd4dv_ctx* ctx, const std::vector<SubDesc>& subs, const std::vec
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     long long ring_min = kRingMinTiles;
     if (const char* e = std::getenv("DD4DV_RING_MIN_TILES")) ring_min = std::atoll(e);   // override (tests)
+    g.ring_expire = std::getenv("DD4DV_RING_EXPIRE") != nullptr;   // (tests)
     int most = 1 << 30;
     if (const char* e = std::getenv("DD4DV_RING_MAX_CTAS")) most = std::max(1, std::atoi(e));   // override (tests)
     for (int q = 0; q < 3 && g.n_ring[0] >= ring_min * 2 * sms; ++q) {
@@ -1597,6 +1609,7 @@ dd4dv_ctx::~dd4dv_ctx() {
   cudaFree(scal_d);
   cudaFree(err_d);
   cudaFreeHost(counter_h);
+  cudaFreeHost(late_h);
   cudaFreeHost(phase_h);
   cudaFreeHost(scal_h);
   cudaFree(ptraj_io);
@@ -1701,8 +1714,10 @@ dd4dv_status dd4dv_create(const dd4dv_model* model, void* cuda_stream, dd4dv_ctx
     ctx->scal_d = dalloc<double>(ctx, 8);
     ctx->err_d = dalloc<int>(ctx, 1);
     if (cudaMallocHost(&ctx->counter_h, 4 * sizeof(int)) != cudaSuccess ||
-        cudaMallocHost(&ctx->scal_h, 8 * sizeof(double)) != cudaSuccess)
+        cudaMallocHost(&ctx->scal_h, 8 * sizeof(double)) != cudaSuccess ||
+        cudaMallocHost(&ctx->late_h, sizeof(int)) != cudaSuccess)
       fail(ctx, DD4DV_ENOMEM, "pinned host allocation failed");
+    *ctx->late_h = 0;
     CK(cudaMemcpyAsync(ctx->rows_d, ctx->rows_h.data(), m.nlat * sizeof(RowConst),
                        cudaMemcpyHostToDevice, ctx->st));
     CK(cudaMemcpyAsync(ctx->grec, rec.data(), rec.size() * sizeof(double), cudaMemcpyHostToDevice, ctx->st));

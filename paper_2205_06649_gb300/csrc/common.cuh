@@ -162,6 +162,10 @@ template <typename T> size_t smem_tlm(int R, int W);
 // resident clusters of the stripe adjoint sweep at cl CTAs per cluster
 template <typename T> int active_clusters_adjoint(int R, int W, int cl, int nthreads);
 
+// Device error words: 1 and 2, a cluster sweep rejected its launch (sweep.cu); 3, a
+// wait of a pipelined level kernel ran out (level.cu).
+constexpr int kErrLostCopy = 3;
+
 // ---- level sweeps (level.cu) ----
 // One tile: the thread-points [p0, p1) of one box (a thread-point is V
 // neighbouring columns of a row), with everything of the box a kernel needs.
@@ -186,6 +190,7 @@ struct LvPlan {
   int tiles = 0;
   LvRing ring[3];                       // adjoint phases 1, 2, 3
   const LvTile* ring_tiles = nullptr;   // their tiles: whole rows
+  bool ring_expire = false;             // their waits run out at once (a test of what follows)
   std::vector<int> n_ring;              // as n_tile
   std::vector<int> n_tile;    // per step l: tiles of the boxes that take it (a prefix)
   std::vector<int> n_box;     // per level l: boxes that have it (a prefix of the box list)
@@ -200,6 +205,7 @@ struct LvArgs {
   int n_tile;
   int n_cta, slots, slot_floats;   // pipelined kernels: CTAs, ring
   int* err;                   // device error word (0 = ok)
+  int* late;                  // the same for lost copies in host memory: read without a synchronisation
   int l;                      // step / level
   int terms;                  // forward: accumulate the observation and overlap terms
   int skip1;                  // first stage recomputed only where x1 is not stored

@@ -660,13 +660,15 @@ __global__ void __launch_bounds__(kLvThreads, 4) lv_tl_kernel(const LvArgs<doubl
   }
 }
 
-// lambda(a) -> packed control layout (FP64).
+// lambda(a) -> packed control layout (FP64); NaN where a pipelined phase of this
+// sweep lost a copy, so that no caller takes the gradient for one.
 template <typename T, int V>
 __global__ void __launch_bounds__(kLvThreads) lv_export_kernel(const LvArgs<T> a) {
   LV_TILE(t);
   grid_wait();
   grid_release();
   if (a.active && a.active[t.s] != a.active_value) return;
+  const bool lost = sizeof(T) == 4 && *a.err == kErrLostCopy;
   const size_t pl = (size_t)t.ny * t.nxp;
   const T* lam = a.lam + t.lv_off;
   double* out = a.lam_a + t.ctrl_off;
@@ -678,7 +680,7 @@ __global__ void __launch_bounds__(kLvThreads) lv_export_kernel(const LvArgs<T> a
       ldv<T, V>(lam + v * pl + (size_t)r * t.nxp + k, x);
 #pragma unroll
       for (int j = 0; j < V; ++j)
-        if (k + j < t.nx) out[((size_t)v * t.ny + r) * t.nx + k + j] = (double)x[j];
+        if (k + j < t.nx) out[((size_t)v * t.ny + r) * t.nx + k + j] = lost ? __longlong_as_double(-1LL) : (double)x[j];
     }
   }
 }
@@ -717,8 +719,9 @@ __device__ __forceinline__ void copy4(void* dst, const void* src) {
 __device__ __forceinline__ void copy16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
 }
+template <int POLLS>
 __device__ __forceinline__ bool ring_wait(uint64_t* bar, unsigned parity) {
-  for (int i = 0; i < kRingWait; ++i) {
+  for (int i = 0; i < POLLS; ++i) {
     unsigned ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
@@ -730,6 +733,14 @@ __device__ __forceinline__ bool ring_wait(uint64_t* bar, unsigned parity) {
     if (ok) return true;
   }
   return false;
+}
+
+// A copy did not arrive in time: the result is not valid.  The export kernel then
+// writes NaN for it, and the host reports it.
+__device__ __noinline__ void ring_lost(int* err, int* late) {
+  atomicExch(err, kErrLostCopy);
+  *(volatile int*)late = kErrLostCopy;
+  __threadfence_system();
 }
 
 // A slot: NF states with a ghost row on either side, NO states without, with
@@ -909,7 +920,8 @@ __device__ __forceinline__ void ring_adjoint(const LvTile& t, const Slot<NF, NO,
 // The CTA's tiles b, b + n_cta, ...  The last warp copies: issue(t, slot base, barrier) starts a tile's copies.
 // The others compute, each at its own pace: body(t, slot base, next, wait), which calls wait() before it
 // reads the slot; next is the CTA's next tile or null.
-template <typename I, typename B>
+// POLLS: kRingWait, or 0 in the kernels that a test of the waits runs.
+template <int POLLS, typename I, typename B>
 __device__ __forceinline__ void ring_run(const LvArgs<float>& a, float* smem, I&& issue, B&& body) {
   __shared__ __align__(16) LvTile desc[kDescs];
   __shared__ uint64_t full[kRingSlots], empty[kRingSlots];
@@ -937,7 +949,7 @@ __device__ __forceinline__ void ring_run(const LvArgs<float>& a, float* smem, I&
     int j = 0;
     for (; j < n; ++j) {
       const int slot = j % S;
-      if (j >= S && !ring_wait(empty + slot, (unsigned)(j / S - 1) & 1u)) break;
+      if (j >= S && !ring_wait<POLLS>(empty + slot, (unsigned)(j / S - 1) & 1u)) break;
       // one copy group a tile, with descriptor j + kAhead in it: all but the newest are
       // complete, so descriptors up to j + 1 are there before full[slot] can be
       asm volatile("cp.async.wait_group 1;" ::: "memory");
@@ -949,11 +961,11 @@ __device__ __forceinline__ void ring_run(const LvArgs<float>& a, float* smem, I&
       asm volatile("cp.async.commit_group;" ::: "memory");
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
-    if (j < n && lane == 0) atomicExch(a.err, 3);   // a wait ran out
+    if (j < n && lane == 0) ring_lost(a.err, a.late);   // a wait ran out
     // The copies of the last tiles end before this warp does, also where a
     // computing warp has given up on them: none may reach the shared memory of
     // the CTA that comes next.  (The copying warp has nothing else to do by then.)
-    for (int q = max(j - S, 0); q < j; ++q) ring_wait(full + q % S, (unsigned)(q / S) & 1u);
+    for (int q = max(j - S, 0); q < j; ++q) ring_wait<kRingWait>(full + q % S, (unsigned)(q / S) & 1u);
     return;
   }
   int slot = 0;
@@ -961,9 +973,9 @@ __device__ __forceinline__ void ring_run(const LvArgs<float>& a, float* smem, I&
   for (int j = 0; j < n; ++j) {
     bool ok = true;
     body(desc[j % kDescs], smem + (size_t)slot * a.slot_floats, j + 1 < n ? desc + (j + 1) % kDescs : nullptr,
-         [&]() { return ok = ring_wait(full + slot, parity); });
+         [&]() { return ok = ring_wait<POLLS>(full + slot, parity); });
     if (!ok) {
-      atomicExch(a.err, 3);
+      ring_lost(a.err, a.late);
       break;
     }
     __syncwarp();
@@ -1015,7 +1027,7 @@ __device__ __forceinline__ void over_take(const LvTile& t, int l, int r, int k, 
 }
 
 // lv_adj_kernel, pipelined.
-template <int K>
+template <int K, int POLLS>
 __global__ void __launch_bounds__(kRingThreads, 2) lv_ring_adj_kernel(const LvArgs<float> a) {
   constexpr int NO = K == 3 ? 2 : 0;
   constexpr bool BL = K == 1;
@@ -1031,7 +1043,7 @@ __global__ void __launch_bounds__(kRingThreads, 2) lv_ring_adj_kernel(const LvAr
     return (a.gn_dx ? a.gn_dx : a.tgt) + t.traj_off + (size_t)l * level_size<float>(t);
   };
   bool first = true;
-  ring_run(
+  ring_run<POLLS>(
       a, slots,
       [&](const LvTile& t, float* base, uint64_t* bar) {
         const float* Z = K == 1   ? x2_of(a, t, l)
@@ -1126,14 +1138,14 @@ cudaError_t lv_launch(void (*kernel)(const LvArgs<T>), const LvArgs<T>& a, int b
   return launch_dependent(kernel, dim3((unsigned)blocks), kLvThreads, 0, st, a);
 }
 
-// Adjoint phase q + 1: the plain kernel, or the pipelined one where the plan
+// Adjoint phase K: the plain kernel, or the pipelined one where the plan
 // has rings.
-template <typename T>
-cudaError_t lv_phase(void (*plain)(const LvArgs<T>), void (*ring)(const LvArgs<float>), const LvArgs<T>& base,
-                     const LvPlan& g, int q, cudaStream_t st) {
+template <typename T, int K>
+cudaError_t lv_phase(const LvArgs<T>& base, const LvPlan& g, cudaStream_t st) {
   if constexpr (sizeof(T) == 4) {
-    const LvRing& rg = g.ring[q];
+    const LvRing& rg = g.ring[K - 1];
     if (rg.slots) {
+      auto ring = g.ring_expire ? lv_ring_adj_kernel<K, 0> : lv_ring_adj_kernel<K, kRingWait>;
       LvArgs<T> a = base;
       a.tiles = g.ring_tiles;
       a.n_tile = g.n_ring[a.l];
@@ -1146,7 +1158,7 @@ cudaError_t lv_phase(void (*plain)(const LvArgs<T>), void (*ring)(const LvArgs<f
       return launch_dependent(ring, dim3((unsigned)a.n_cta), kRingThreads, smem, st, a);
     }
   }
-  return lv_launch<T>(plain, base, base.n_tile, st);
+  return lv_launch<T>(lv_adj_kernel<T, lv_width<T>(), K>, base, base.n_tile, st);
 }
 
 }  // namespace
@@ -1190,9 +1202,9 @@ cudaError_t launch_level_adjoint(const LvArgs<T>& base, const LvPlan& g, cudaStr
       LV_TRY(lv_launch<T>(lv_stage_kernel<T, V, 1, false>, a, a.n_tile, st));
       LV_TRY(lv_launch<T>(lv_stage_kernel<T, V, 2, false>, a, a.n_tile, st));
     }
-    LV_TRY(lv_phase<T>(lv_adj_kernel<T, V, 1>, lv_ring_adj_kernel<1>, a, g, 0, st));
-    LV_TRY(lv_phase<T>(lv_adj_kernel<T, V, 2>, lv_ring_adj_kernel<2>, a, g, 1, st));
-    LV_TRY(lv_phase<T>(lv_adj_kernel<T, V, 3>, lv_ring_adj_kernel<3>, a, g, 2, st));
+    LV_TRY((lv_phase<T, 1>(a, g, st)));
+    LV_TRY((lv_phase<T, 2>(a, g, st)));
+    LV_TRY((lv_phase<T, 3>(a, g, st)));
     if constexpr (sizeof(T) == 4)
       if (g.ring[2].slots && g.obs[l] && !a.yforce)
         LV_TRY(launch_dependent(lv_scatter_kernel, dim3((unsigned)g.n_box[l + 1]), kRingThreads, 0, st, a));

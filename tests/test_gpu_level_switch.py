@@ -103,3 +103,26 @@ def test_pipelined_adjoint_in_its_steady_state(level_context, name, ctas):
     assert kernels[0] != kernels[1]   # (the pipelined form adds the observations in a kernel of their own)
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+def test_lost_copy_is_reported_and_never_returned_as_a_gradient(level_context, monkeypatch):
+    """A wait of the pipelined adjoint that runs out (here: at once, no polls)
+    gives DD4DV_ETIMEOUT; a call with device pointers does not synchronise, so
+    its gradient is NaN and the next call reports it.  The context stays usable."""
+    import paper_2205_06649_gb300 as dd
+    many = RING["many rows"]
+    ref = level_context(1, env=dict(DD4DV_RING_MIN_TILES=1 << 40), **many)
+    w = controls(ref)
+    J, g = ref.eval(w)
+    ctx = level_context(1, env=dict(DD4DV_RING_MIN_TILES=0, DD4DV_RING_MAX_CTAS=8, DD4DV_RING_EXPIRE=1), **many)
+    monkeypatch.delenv("DD4DV_RING_EXPIRE")
+    with pytest.raises(dd.DD4DVError, match="ETIMEOUT.*did not reach"):
+        ctx.eval(w)
+    wd = torch.as_tensor(w, device="cuda")
+    Jd, gd = ctx.eval(wd)
+    torch.cuda.synchronize()
+    assert np.array_equal(Jd.cpu().numpy(), J) and torch.isnan(gd).any()
+    with pytest.raises(dd.DD4DVError, match="ETIMEOUT"):
+        ctx.eval(wd)
+    ctx.set_sweep_variant(1, 1)
+    assert np.array_equal(ctx.eval(w)[1], g)
