@@ -6,9 +6,6 @@
 #include "point.cuh"
 
 #include <cfloat>
-#include <mutex>
-#include <set>
-#include <utility>
 
 namespace dd4dv {
 
@@ -827,25 +824,6 @@ __global__ void vgrad_kernel(const SubDesc* subs, const double* w, const double*
     const double gv = (w ? w[o + i] : 0.0) + (double)pl[r * pitch + k];
     grad[o + i] = scale ? sc * gv : gv;
   }
-}
-
-// Raises a kernel's dynamic shared-memory cap to the 227 KB opt-in maximum,
-// once per (kernel, device): the attribute belongs to the device current at
-// the call, so a context on another device sets it again.
-template <typename K>
-cudaError_t raise_smem_cap(K kernel) {
-  static std::mutex mu;
-  static std::set<std::pair<const void*, int>> done;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  std::lock_guard<std::mutex> lock(mu);
-  const std::pair<const void*, int> key{reinterpret_cast<const void*>(kernel), dev};
-  if (done.count(key)) return cudaSuccess;
-  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-  if (e != cudaSuccess) return e;
-  done.insert(key);
-  return cudaSuccess;
 }
 
 inline unsigned blocks_for(long long n, int t, int cap = 152 * 16) {

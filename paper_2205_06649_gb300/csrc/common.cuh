@@ -18,6 +18,9 @@
 
 #include <cuda_runtime.h>
 #include <cstdint>
+#include <mutex>
+#include <set>
+#include <utility>
 #include <vector>
 
 namespace dd4dv {
@@ -142,6 +145,30 @@ cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+// Raises a kernel's dynamic shared-memory cap to the 227 KB opt-in maximum less
+// its static part, once per (kernel, device) and never down again: the attribute
+// belongs to the process, and another thread may be about to launch the kernel
+// with more than this caller needs.  (It is set on the device current at the
+// call, so a context on another device sets it again.)
+template <typename K>
+cudaError_t raise_smem_cap(K kernel) {
+  static std::mutex mu;
+  static std::set<std::pair<const void*, int>> done;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(mu);
+  const std::pair<const void*, int> key{reinterpret_cast<const void*>(kernel), dev};
+  if (done.count(key)) return cudaSuccess;
+  cudaFuncAttributes fa;
+  e = cudaFuncGetAttributes(&fa, kernel);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448 - (int)fa.sharedSizeBytes);
+  if (e != cudaSuccess) return e;
+  done.insert(key);
+  return cudaSuccess;
 }
 
 // ---- launchers (sweep.cu) ----

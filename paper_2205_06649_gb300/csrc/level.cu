@@ -1153,7 +1153,7 @@ cudaError_t lv_phase(const LvArgs<T>& base, const LvPlan& g, cudaStream_t st) {
       a.slots = rg.slots;
       a.slot_floats = rg.slot_floats;
       const size_t smem = ((size_t)rg.slots * rg.slot_floats + rg.own_floats) * sizeof(float);
-      cudaError_t e = cudaFuncSetAttribute(ring, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaError_t e = raise_smem_cap(ring);
       if (e != cudaSuccess) return e;
       return launch_dependent(ring, dim3((unsigned)a.n_cta), kRingThreads, smem, st, a);
     }

@@ -126,3 +126,31 @@ def test_lost_copy_is_reported_and_never_returned_as_a_gradient(level_context, m
         ctx.eval(wd)
     ctx.set_sweep_variant(1, 1)
     assert np.array_equal(ctx.eval(w)[1], g)
+
+
+def test_pipelined_adjoints_of_two_contexts_on_two_threads(level_context):
+    """Two contexts whose pipelined launches ask for different amounts of shared
+    memory, each on its own thread: neither may lower the limit that the other is
+    about to launch with."""
+    import threading
+    env = dict(DD4DV_RING_MIN_TILES=0)
+    pair = [level_context(1, env=env, nlon=33, nlat=14, nsteps=40, P1=1, P2=1, Q=1),
+            level_context(1, env=env, nlon=384, nlat=160, nsteps=40, P1=4, P2=2, Q=1, o_lon=4, o_lat=4)]
+    w = [controls(c) for c in pair]
+    ref = [c.eval(v)[1] for c, v in zip(pair, w)]
+    wrong = []
+
+    def work(k):
+        try:
+            for _ in range(60):
+                if not np.array_equal(pair[k].eval(w[k])[1], ref[k]):
+                    wrong.append((k, "gradient"))
+        except Exception as e:   # noqa: BLE001 (shown below)
+            wrong.append((k, str(e)))
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in (0, 1)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong
