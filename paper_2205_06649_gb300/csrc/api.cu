@@ -5,6 +5,7 @@
 // builds index tables and enqueues work.
 #include "dd4dvar.h"
 #include "point.cuh"
+#include "tuning.h"
 
 #include <algorithm>
 #include <cmath>
@@ -788,8 +789,8 @@ void autotune(dd4dv_ctx* ctx) {
     return true;
   };
   // the level sweeps, with and without stored stage states (best of two each)
-  struct Best { double t = 1e300; int c = 0, nt = 0, var = 0; };
-  double lv_f[2] = {1e300, 1e300}, lv_a[2] = {1e300, 1e300};
+  struct Best { double t = kNotTimed; int c = 0, nt = 0, var = 0; };
+  SweepTimes times[2];
   if (ctx->lv_tiles && ctx->variant_f == 0 && ctx->variant_a == 0) {
     ctx->lv_f = ctx->lv_a = true;
     for (int use : {1, 0}) {
@@ -799,8 +800,8 @@ void autotune(dd4dv_ctx* ctx) {
         float tf = 0, ta = 0;
         if (!run(ctx->cl, ctx->nthreads, &tf, &ta)) break;
         if (rep == 0) continue;   // warm-up
-        lv_f[use] = std::min(lv_f[use], (double)tf);
-        lv_a[use] = std::min(lv_a[use], (double)ta);
+        times[use].level_f = std::min(times[use].level_f, (double)tf);
+        times[use].level_a = std::min(times[use].level_a, (double)ta);
       }
     }
     ctx->use_stg = ctx->stg != nullptr;
@@ -868,12 +869,12 @@ void autotune(dd4dv_ctx* ctx) {
         }
   }
   for (auto& e : ev) cudaEventDestroy(e);
-  // time of each stage mode with the faster kind of each sweep
-  double mode_t[2];
-  for (int u : {0, 1})
-    mode_t[u] = std::min(best_f[u].c ? best_f[u].t : 1e300, lv_f[u]) + std::min(best_a[u].c ? best_a[u].t : 1e300, lv_a[u]);
-  const int use = have_stg && mode_t[1] < 1e300 && mode_t[1] < mode_t[0] ? 1 : 0;
-  const bool use_lv_f = lv_f[use] < best_f[use].t, use_lv_a = lv_a[use] < best_a[use].t;
+  for (int u : {0, 1}) {
+    times[u].cluster_f = best_f[u].t;
+    times[u].cluster_a = best_a[u].t;
+  }
+  const SweepChoice pick = choose_sweeps(times, have_stg, ctx->ckpt > 0);
+  const int use = pick.stored;
   if (!best_f[use].c || !best_a[use].c) {   // nothing measured: keep the starting shape
     best_f[use] = {tf0, c0, n0, var0};
     best_a[use] = {ta0, c0, n0, var0};
@@ -888,11 +889,11 @@ void autotune(dd4dv_ctx* ctx) {
   ctx->nthreads = best_a[use].nt;
   ctx->R = (ctx->max_ny + ctx->cl - 1) / ctx->cl;
   ctx->dec.cluster = ctx->cl;
-  ctx->tune_ms = std::min(best_f[use].t, lv_f[use]) + std::min(best_a[use].t, lv_a[use]);
-  ctx->lv_f = use_lv_f;
-  ctx->lv_a = use_lv_a;
-  if (use_lv_f) ctx->variant_f = 0;   // (a cluster shape stays set for the sweeps that need one)
-  if (use_lv_a) ctx->variant_a = 0;
+  ctx->tune_ms = pick.ms < kNotTimed ? pick.ms : best_f[use].t + best_a[use].t;
+  ctx->lv_f = pick.level_f;
+  ctx->lv_a = pick.level_a;
+  if (ctx->lv_f) ctx->variant_f = 0;   // (a cluster shape stays set for the sweeps that need one)
+  if (ctx->lv_a) ctx->variant_a = 0;
   sync(ctx);
   if (!use && ctx->stg && ctx->dec.ckpt_k != -2) {   // recomputing the stages won: give the memory back
     free_dec_buffer(ctx, ctx->stg);

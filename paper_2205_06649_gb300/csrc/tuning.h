@@ -1,0 +1,35 @@
+// What the autotuner concludes from its timings.  Plain C++, no CUDA: the rules
+// can be tested by themselves.
+#pragma once
+
+namespace dd4dv {
+
+constexpr double kNotTimed = 1e300;
+
+// The fastest forward and adjoint sweep of each kind (ms) with one stage mode.
+struct SweepTimes {
+  double cluster_f = kNotTimed, cluster_a = kNotTimed, level_f = kNotTimed, level_a = kNotTimed;
+};
+struct SweepChoice {
+  int stored = 0;                         // stage states stored (1) or recomputed (0)
+  bool level_f = false, level_a = false;
+  double ms = 2 * kNotTimed;
+};
+
+// The fastest pair of sweeps that can run together.  t[0]: stages recomputed,
+// t[1]: stored (only where have_stored).  Under checkpoints the cluster forward
+// stores some levels only, and the level adjoint, which reads every level, follows
+// a level forward or does not run.
+inline SweepChoice choose_sweeps(const SweepTimes (&t)[2], bool have_stored, bool checkpoints) {
+  SweepChoice best;
+  for (int u = 0; u <= (have_stored ? 1 : 0); ++u)
+    for (int k = 0; k < 4; ++k) {
+      const bool lf = k & 1, la = k & 2;
+      if (checkpoints && la && !lf) continue;
+      const double ms = (lf ? t[u].level_f : t[u].cluster_f) + (la ? t[u].level_a : t[u].cluster_a);
+      if (ms < best.ms) best = {u, lf, la, ms};
+    }
+  return best;
+}
+
+}  // namespace dd4dv
