@@ -121,9 +121,9 @@ typedef struct {
  * recompute the stage states alone, with the same results);
  * -2 = choose by timing: after the launch shapes are set (or autotuned), one
  * evaluation is timed with stored stage states (when their buffer fits),
- * with recomputed stages and with checkpoints every 8, 16 and 32 levels, the
- * fastest is kept and the unused buffers are freed (dd4dv_checkpoint_interval
- * reports the choice).
+ * with recomputed stages and with checkpoints every 8, 16 and 32 levels (not
+ * where level sweeps run, which ignore an interval), the fastest is kept and the
+ * unused buffers are freed (dd4dv_checkpoint_interval reports the choice).
  */
 typedef struct {
   int P1, P2, Q;

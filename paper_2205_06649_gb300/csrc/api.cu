@@ -901,12 +901,9 @@ void autotune(dd4dv_ctx* ctx) {
   }
 }
 
-// Checkpoint intervals the library tries for ckpt_k = -2.
-constexpr int kTunedCkpt[3] = {8, 16, 32};
-
 // ckpt_k = -2: time one forward + adjoint evaluation (w = 0, CUDA events,
 // best of two) with stored stage states (when their buffer exists), with the
-// stages recomputed, and with k-step checkpoints for k in kTunedCkpt, at the
+// stages recomputed, and with the k-step checkpoints of checkpoint_candidates, at the
 // current launch shapes; keep the fastest and free the buffers it does not
 // use.  Results do not depend on the choice.
 void tune_checkpoint(dd4dv_ctx* ctx) {
@@ -936,7 +933,9 @@ void tune_checkpoint(dd4dv_ctx* ctx) {
   std::vector<Cand> c;
   if (ctx->stg) c.push_back({0, true, time_eval(0, true)});
   c.push_back({0, false, time_eval(0, false)});
-  for (int k : kTunedCkpt) c.push_back({k, false, time_eval(k, false)});
+  ctx->ckpt = 0;
+  for (int k : checkpoint_candidates(level_forward(ctx), level_adjoint(ctx)))
+    c.push_back({k, false, time_eval(k, false)});
   for (auto& e : ev) cudaEventDestroy(e);
   const Cand best = *std::min_element(c.begin(), c.end(), [](const Cand& a, const Cand& b) { return a.ms < b.ms; });
   ctx->ckpt = best.k;

@@ -2,6 +2,8 @@
 // can be tested by themselves.
 #pragma once
 
+#include <vector>
+
 namespace dd4dv {
 
 constexpr double kNotTimed = 1e300;
@@ -30,6 +32,16 @@ inline SweepChoice choose_sweeps(const SweepTimes (&t)[2], bool have_stored, boo
       if (ms < best.ms) best = {u, lf, la, ms};
     }
   return best;
+}
+
+// Checkpoint intervals worth timing for ckpt_k = -2.  Level sweeps store every
+// level whatever the interval, and recompute the stage states alone: every
+// interval would time the same kernels, and noise would choose one and keep its
+// segment buffers.
+constexpr int kTunedCkpt[3] = {8, 16, 32};
+inline std::vector<int> checkpoint_candidates(bool level_f, bool level_a) {
+  if (level_f && level_a) return {};
+  return {kTunedCkpt, kTunedCkpt + 3};
 }
 
 }  // namespace dd4dv

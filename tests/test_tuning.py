@@ -14,6 +14,10 @@ PROGRAM = r"""
 #include <cstring>
 using namespace dd4dv;
 int main(int argc, char** argv) {
+  if (!std::strcmp(argv[1], "ckpt")) {
+    for (int k : checkpoint_candidates(std::atoi(argv[2]), std::atoi(argv[3]))) std::printf("%d ", k);
+    return 0;
+  }
   SweepTimes t[2];
   double* f[8] = {&t[0].cluster_f, &t[0].cluster_a, &t[0].level_f, &t[0].level_a,
                   &t[1].cluster_f, &t[1].cluster_a, &t[1].level_f, &t[1].level_a};
@@ -51,3 +55,9 @@ def run(tmp_path_factory):
 ])
 def test_choose_sweeps(run, stored, ckpt, ms, want):
     assert run("sweeps", stored, ckpt, *ms.split()) == want
+
+
+def test_no_checkpoint_interval_is_timed_where_none_has_an_effect(run):
+    assert run("ckpt", 1, 1) == ""
+    for f, a in ((0, 0), (1, 0), (0, 1)):
+        assert run("ckpt", f, a).split() == ["8", "16", "32"]
