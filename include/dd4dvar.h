@@ -454,8 +454,9 @@ dd4dv_status dd4dv_stage1_stored(const dd4dv_ctx* ctx, int* n_subs, double* pt_s
  * partial sums, and give way to the cluster sweeps when a variant other than 0
  * or a launch shape (dd4dv_set_sweep_config) is set.  The environment variable
  * DD4DV_LEVEL_MIN_POINTS, read by dd4dv_set_decomposition, replaces the number
- * of points from which they are chosen.  Three more are for tests:
- * DD4DV_RING_MIN_TILES replaces the number of tiles per CTA from which the FP32
+ * of points from which they are chosen.  Four more are for tests:
+ * DD4DV_LEVEL_ROUNDS replaces the points (FP32: groups of four) that a thread takes,
+ * DD4DV_RING_MIN_TILES the number of tiles per CTA from which the FP32
  * adjoint runs pipelined, DD4DV_RING_MAX_CTAS bounds the CTAs of a pipelined
  * launch, and with DD4DV_RING_EXPIRE set its waits run out at once.
  * forward: 0 = level sweep where chosen, else deep-halo sweep wherever it

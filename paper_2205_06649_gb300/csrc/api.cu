@@ -145,9 +145,18 @@ struct dd4dv_ctx {
   // / adjoint sweeps run them (else the cluster sweeps)
   bool lv_f = false, lv_a = false;
   bool all_levels = false;    // the last forward sweep stored every level
-  LvPlan lv;
-  LvTile* lv_tiles = nullptr;
-  int *lv_boxes = nullptr, *lv_tile_off = nullptr;
+  // lists of boxes and their tiles: all of them, and the owned ones alone (where
+  // some are not: the masked evaluations then launch no CTA for the others)
+  struct LvSet {
+    LvPlan plan;
+    LvTile *tiles = nullptr, *ring_tiles = nullptr, *fine_tiles = nullptr;
+    int *boxes = nullptr, *tile_off = nullptr;
+  } lv, lv_own;
+  bool lv_own_on = false;
+  std::vector<LvTile> lv_tiles_h, lv_ring_h;
+  std::vector<int> lv_order_h;
+  long long lv_ring_least = 0;   // tiles from which the adjoint runs pipelined
+  int lv_rounds = 1;          // rounds of a tile
   long long* lv_box_off = nullptr;
   void *lv_rec = nullptr, *lv_state = nullptr;
   double *lv_acc_m = nullptr, *lv_acc_o = nullptr;
@@ -402,11 +411,16 @@ bool level_adjoint(const dd4dv_ctx* ctx) {
 // (FP64, about the levels that a level forward sweep stores).
 bool tangent_level(const dd4dv_ctx* ctx) { return ctx->m.precision == 0 && level_forward(ctx); }
 
+// The boxes that a level sweep with this mask can have to advance.
+const dd4dv_ctx::LvSet& level_set(const dd4dv_ctx* ctx, const int* active) {
+  return active && ctx->lv_own_on ? ctx->lv_own : ctx->lv;
+}
+
 template <typename T>
 LvArgs<T> level_args(dd4dv_ctx* ctx, const int* active, int av) {
   LvArgs<T> a{};
-  a.tiles = ctx->lv_tiles;
-  a.boxes = ctx->lv_boxes;
+  a.tiles = level_set(ctx, active).tiles;
+  a.boxes = level_set(ctx, active).boxes;
   a.box_off = ctx->lv_box_off;
   a.err = ctx->err_d;
   a.late = ctx->late_h;
@@ -465,7 +479,7 @@ void forward_sweep(dd4dv_ctx* ctx, const int* active, int av, bool full = false)
     LvArgs<T> a = level_args<T>(ctx, active, av);
     a.terms = !full;
     if (full) a.stg = a.stg1 = nullptr;
-    CK(launch_level_forward<T>(a, ctx->lv, ctx->st, &ctx->launches));
+    CK(launch_level_forward<T>(a, level_set(ctx, active).plan, ctx->st, &ctx->launches));
     return;
   }
   SweepArgs<T> a = sweep_args<T>(ctx);
@@ -484,8 +498,9 @@ void forward_sweep(dd4dv_ctx* ctx, const int* active, int av, bool full = false)
 // J (and parts) from the terms that the last forward sweep left.
 void finalize_J(dd4dv_ctx* ctx, const double* w, double* J, double* parts, const int* active, int av) {
   if (level_forward(ctx))
-    KL(launch_finalize_J_tiles(ctx->subs_d, ctx->n_sub, w, ctx->lv_acc_o, ctx->lv_acc_m, ctx->lv_tile_off,
-                               ctx->vconst, ctx->dec.lambda, ctx->dec.mu, J, parts, active, av, ctx->st));
+    KL(launch_finalize_J_tiles(ctx->subs_d, ctx->n_sub, w, ctx->lv_acc_o, ctx->lv_acc_m,
+                               level_set(ctx, active).tile_off, ctx->vconst, ctx->dec.lambda, ctx->dec.mu, J, parts,
+                               active, av, ctx->st));
   else
     KL(launch_finalize_J(ctx->subs_d, ctx->n_sub, w, ctx->part, ctx->cl_f, ctx->vconst, ctx->dec.lambda,
                          ctx->dec.mu, J, parts, active, av, ctx->st));
@@ -500,7 +515,7 @@ void adjoint_sweep(dd4dv_ctx* ctx, const int* active, int av, const double* yfor
     LvArgs<T> a = level_args<T>(ctx, active, av);
     a.yforce = yforce;
     a.gn_dx = gn_dx;
-    CK(launch_level_adjoint<T>(a, ctx->lv, ctx->st, &ctx->launches));
+    CK(launch_level_adjoint<T>(a, level_set(ctx, active).plan, ctx->st, &ctx->launches));
     return;
   }
   SweepArgs<T> a = sweep_args<T>(ctx);
@@ -578,7 +593,7 @@ void gn_product_T(dd4dv_ctx* ctx, const double* p, double* Ap, const int* active
     LvArgs<double> a = level_args<double>(ctx, active, av);
     a.dx = static_cast<double*>(ctx->gn_dx);
     a.dx0 = ctx->io_c;
-    CK(launch_level_tangent(a, ctx->lv, ctx->st, &ctx->launches));
+    CK(launch_level_tangent(a, level_set(ctx, active).plan, ctx->st, &ctx->launches));
   } else {
     SweepArgs<T> a = sweep_args<T>(ctx);
     a.active = active;
@@ -791,7 +806,7 @@ void autotune(dd4dv_ctx* ctx) {
   // the level sweeps, with and without stored stage states (best of two each)
   struct Best { double t = kNotTimed; int c = 0, nt = 0, var = 0; };
   SweepTimes times[2];
-  if (ctx->lv_tiles && ctx->variant_f == 0 && ctx->variant_a == 0) {
+  if (ctx->lv.tiles && ctx->variant_f == 0 && ctx->variant_a == 0) {
     ctx->lv_f = ctx->lv_a = true;
     for (int use : {1, 0}) {
       if (use && !ctx->stg) continue;
@@ -972,7 +987,63 @@ constexpr int kLvMinBox64 = 700;
 // 5 1.78 / 1.72, 10 3.97 / 3.02; of 32 x 28, 6.7 3.01 / 2.75.
 constexpr int kRingMaxNx = kRingPoints / 3 * 4, kRingMinTiles = 4;
 
-// Tiles and scratch of the level sweeps.  Leaves ctx->lv_tiles null where they
+// A thread takes several thread-points (rounds) where there are many CTAs all the
+// same.  Measured, FP32 forward of 4.9 million points with 1, 2 and 4 rounds 11.2, 10.1
+// and 9.7 ms (2.9 million: 10.9, 10.0, 9.4; the pipelined adjoint has tiles of its own);
+// FP64 adjoint with 1 and 2 rounds 96.1 and 93.8 ms, forward 76.2 and 76.0.
+template <typename T>
+int level_rounds(long long pts) {
+  return pts > 2000000 ? (sizeof(T) == 4 ? 4 : 2) : 1;
+}
+
+// Equal tiles of whole warps of t's box, `rounds` thread-points a thread.
+void split_box(LvTile t, int rounds, std::vector<LvTile>& out) {
+  const int np = t.nq * t.ny;
+  const int nt = (np + rounds * kLvThreads - 1) / (rounds * kLvThreads);
+  const int per = ((np + nt - 1) / nt + 31) / 32 * 32;
+  for (int q = 0; q < nt; ++q) {
+    t.p0 = std::min(q * per, np);
+    t.p1 = std::min((q + 1) * per, np);
+    out.push_back(t);
+  }
+}
+
+// Counts of a list of tiles (longest window first): tiles, pipelined tiles and
+// boxes per step or level, and each box's accumulator slots (tile_off).
+void count_tiles(LvPlan& g, const std::vector<LvTile>& tiles, const std::vector<LvTile>& ring_tiles, int maxL,
+                 int n_sub, std::vector<int>* tile_off) {
+  g.tiles = (int)tiles.size();
+  g.n_tile.assign(maxL, 0);
+  g.n_ring.assign(maxL, 0);
+  g.n_box.assign(maxL + 1, 0);
+  tile_off->assign(2 * n_sub, 0);
+  for (size_t i = 0; i < tiles.size(); ++i) {
+    const LvTile& t = tiles[i];
+    for (int l = 0; l < t.L; ++l) ++g.n_tile[l];
+    int* slots = &(*tile_off)[2 * t.s];
+    if (t.p0 == 0) {   // a box's first tile
+      slots[0] = (int)i * kLvThreads;
+      for (int l = 0; l <= t.L; ++l) ++g.n_box[l];
+    }
+    slots[1] += kLvThreads;
+  }
+  for (const LvTile& t : ring_tiles)
+    for (int l = 0; l < t.L; ++l) ++g.n_ring[l];
+}
+
+// Moves a list to the device (set's buffers) and into set.
+void upload_set(dd4dv_ctx* ctx, dd4dv_ctx::LvSet& set, LvPlan& g, const std::vector<LvTile>& tiles,
+                const std::vector<LvTile>& ring_tiles, const std::vector<int>& order,
+                const std::vector<int>& tile_off) {
+  if (!tiles.empty()) h2d(ctx, set.tiles, tiles.data(), tiles.size() * sizeof(LvTile));
+  if (!ring_tiles.empty()) h2d(ctx, set.ring_tiles, ring_tiles.data(), ring_tiles.size() * sizeof(LvTile));
+  if (!order.empty()) h2d(ctx, set.boxes, order.data(), order.size() * sizeof(int));
+  h2d(ctx, set.tile_off, tile_off.data(), tile_off.size() * sizeof(int));
+  g.ring_tiles = set.ring_tiles;
+  set.plan = std::move(g);
+}
+
+// Tiles and scratch of the level sweeps.  Leaves ctx->lv.tiles null where they
 // do not apply: too few points, boxes no wider than a thread's columns or of a
 // single row (a thread has one ghost row at most), a grid
 // whose level does not fit 32-bit offsets, or no memory for the scratch.
@@ -997,15 +1068,11 @@ void level_plan(dd4dv_ctx* ctx, const std::vector<SubDesc>& subs, const std::vec
   for (int s = 0; s < n_sub; ++s) order[s] = s;
   std::stable_sort(order.begin(), order.end(),
                    [&](int x, int y) { return subs[x].b - subs[x].a > subs[y].b - subs[y].a; });
-  // thread-points per thread: more than one saves set-up where there are many CTAs all the same
-  const int iters = pts > 2000000 ? (sizeof(T) == 4 ? 4 : 2) : 1;
+  ctx->lv_rounds = level_rounds<T>(pts);
+  if (const char* e = std::getenv("DD4DV_LEVEL_ROUNDS")) ctx->lv_rounds = std::max(1, std::atoi(e));   // override (tests)
   std::vector<LvTile> tiles, ring_tiles;
-  std::vector<int> tile_off(2 * n_sub);
   std::vector<long long> box_off(n_sub);
   LvPlan g;
-  g.n_tile.assign(maxL, 0);
-  g.n_ring.assign(maxL, 0);
-  g.n_box.assign(maxL + 1, 0);
   g.obs.assign(maxL + 1, 0);
   long long elems = 0;
   auto magic = [](int v) { return v <= 1 ? 0u : (unsigned)(0xFFFFFFFFu / (unsigned)v + 1u); };
@@ -1036,40 +1103,27 @@ void level_plan(dd4dv_ctx* ctx, const std::vector<SubDesc>& subs, const std::vec
     t.ctrl_off = d.ctrl_off;
     t.lv_off = box_off[s] = elems;
     elems += 3LL * d.ny * d.nxp;
-    // equal tiles of whole warps
-    const int np = t.nq * d.ny;
-    const int nt = (np + iters * kLvThreads - 1) / (iters * kLvThreads);
-    const int per = ((np + nt - 1) / nt + 31) / 32 * 32;
-    tile_off[2 * s] = (int)tiles.size() * kLvThreads;
-    tile_off[2 * s + 1] = nt * kLvThreads;
-    for (int q = 0; q < nt; ++q) {
-      t.p0 = std::min(q * per, np);
-      t.p1 = std::min((q + 1) * per, np);
-      tiles.push_back(t);
-    }
-    for (int l = 0; l < t.L; ++l) g.n_tile[l] += nt;
+    split_box(t, ctx->lv_rounds, tiles);
     if (max_nx <= kRingMaxNx) {   // equal tiles of whole rows, a thread-point per computing thread
       int m = (d.ny + kRingPoints / t.nq - 1) / (kRingPoints / t.nq);
       const int R = (d.ny + m - 1) / m;
       m = (d.ny + R - 1) / R;
       for (int q = 0; q < m; ++q) {
         t.p0 = q * R * t.nq;
-        t.p1 = std::min((q + 1) * R * t.nq, np);
+        t.p1 = std::min((q + 1) * R * t.nq, t.nq * d.ny);
         ring_tiles.push_back(t);
       }
-      for (int l = 0; l < t.L; ++l) g.n_ring[l] += m;
       // states with a ghost row on either side, states without, row constants
       // and ghost columns, second level of blended ghosts (Slot of level.cu)
       const int full = 3 * (R + 2) * d.nxp, own = 3 * R * d.nxp, cols = (6 * R + 3) / 4 * 4, rc = 8 * R;
       const int need[3] = {2 * full + 2 * cols + rc + 6 * d.nxp, 2 * full + cols + rc, 2 * full + 2 * own + cols + rc};
       for (int q = 0; q < 3; ++q) g.ring[q].slot_floats = std::max(g.ring[q].slot_floats, need[q]);
     }
-    for (int l = 0; l <= t.L; ++l) {
-      ++g.n_box[l];
+    for (int l = 0; l <= t.L; ++l)
       if (lvl_obs[d.obs_lvl + l] != lvl_obs[d.obs_lvl + l + 1]) g.obs[l] = 1;
-    }
   }
-  g.tiles = (int)tiles.size();
+  std::vector<int> tile_off;
+  count_tiles(g, tiles, ring_tiles, maxL, n_sub, &tile_off);
   // Pipelined adjoint kernels: as many resident CTAs as the registers allow,
   // with two slots or more (up to four) in the shared memory that each has.
   if (sizeof(T) == 4 && !ring_tiles.empty()) {
@@ -1081,7 +1135,8 @@ void level_plan(dd4dv_ctx* ctx, const std::vector<SubDesc>& subs, const std::vec
     g.ring_expire = std::getenv("DD4DV_RING_EXPIRE") != nullptr;   // (tests)
     int most = 1 << 30;
     if (const char* e = std::getenv("DD4DV_RING_MAX_CTAS")) most = std::max(1, std::atoi(e));   // override (tests)
-    for (int q = 0; q < 3 && g.n_ring[0] >= ring_min * 2 * sms; ++q) {
+    ctx->lv_ring_least = ring_min * 2 * sms;
+    for (int q = 0; q < 3 && g.n_ring[0] >= ctx->lv_ring_least; ++q) {
       LvRing& r = g.ring[q];
       r.own_floats = q == 2 ? 12 * kRingPoints : 0;
       for (int c = 2; c > 0 && !r.slots; --c) {
@@ -1112,29 +1167,101 @@ void level_plan(dd4dv_ctx* ctx, const std::vector<SubDesc>& subs, const std::vec
   const size_t need = 5 * (size_t)elems * sizeof(T) + (tiles.size() + ring_tiles.size()) * sizeof(LvTile) +
                       slots * sizeof(double) + (64u << 20);
   if (need > free_b) return;
-  LvTile* td = dalloc<LvTile>(ctx, tiles.size(), &L);
-  ctx->lv_boxes = dalloc<int>(ctx, n_sub, &L);
-  ctx->lv_tile_off = dalloc<int>(ctx, 2 * n_sub, &L);
+  dd4dv_ctx::LvSet set;
+  set.tiles = dalloc<LvTile>(ctx, tiles.size(), &L);
+  set.boxes = dalloc<int>(ctx, n_sub, &L);
+  set.tile_off = dalloc<int>(ctx, 2 * n_sub, &L);
   ctx->lv_box_off = dalloc<long long>(ctx, n_sub, &L);
   ctx->lv_rec = dalloc<T>(ctx, rec.size(), &L);
   ctx->lv_state = dalloc<T>(ctx, 5 * (size_t)elems, &L);
   ctx->lv_acc_m = dalloc<double>(ctx, slots, &L);
   ctx->lv_acc_o = dalloc<double>(ctx, n_sub, &L);
-  h2d(ctx, td, tiles.data(), tiles.size() * sizeof(LvTile));
-  if (!ring_tiles.empty()) {
-    LvTile* rd = dalloc<LvTile>(ctx, ring_tiles.size(), &L);
-    h2d(ctx, rd, ring_tiles.data(), ring_tiles.size() * sizeof(LvTile));
-    g.ring_tiles = rd;
-  }
-  h2d(ctx, ctx->lv_boxes, order.data(), n_sub * sizeof(int));
-  h2d(ctx, ctx->lv_tile_off, tile_off.data(), 2 * n_sub * sizeof(int));
+  if (!ring_tiles.empty()) set.ring_tiles = dalloc<LvTile>(ctx, ring_tiles.size(), &L);
+  upload_set(ctx, set, g, tiles, ring_tiles, order, tile_off);
   h2d(ctx, ctx->lv_box_off, box_off.data(), n_sub * sizeof(long long));
   h2d(ctx, ctx->lv_rec, rec.data(), rec.size() * sizeof(T));
   CK(cudaMemsetAsync(ctx->lv_state, 0, 5 * (size_t)elems * sizeof(T), ctx->st));
   CK(cudaStreamSynchronize(ctx->st));   // the host tables end with this call
-  ctx->lv_tiles = td;
   ctx->lv_elems = elems;
-  ctx->lv = std::move(g);
+  ctx->lv = std::move(set);
+  ctx->lv_tiles_h = std::move(tiles);
+  ctx->lv_ring_h = std::move(ring_tiles);
+  ctx->lv_order_h = std::move(order);
+}
+
+// The list of the owned boxes, after dd4dv_set_owned.  A rank that owns a share of
+// the boxes would else launch the CTAs of all of them for every stage.  Per box the
+// tiles stay as they are, so J keeps the order of its sums: a sharded run makes the
+// line-search decisions of a run that owns everything.  Where the lists find no
+// memory, the masks on the full list do the same work.  A share whose points ask for
+// one round takes tiles of one round in the kernels that add nothing up.
+// Evaluations, ms, of 1/4, 1/8, 1/16 and 1/32 of the boxes, masks on the full list /
+// these lists / cluster sweeps: FP64, 512 boxes 50.6, 28.9, 18.6, 13.8 / 45.7, 23.8,
+// 12.9, 8.2 / 60.6, 31.6, 16.4, 10.0; FP32, 512 boxes 10.3, 8.0, 6.8, 6.3 / 7.7, 4.9, 3.4,
+// 3.0 / 12.0, 7.0, 4.4, 2.9; FP32, 256 boxes 10.6, 8.6, 7.7, 7.6 / 8.5, 6.2, 4.6, 4.2 /
+// 11.7, 7.4, 4.3, 4.4; FP32 with 16-step checkpoints, 128 boxes 2.6, 2.9, 2.4, 2.1 / 2.7,
+// 2.5, 2.1, 1.8 / 2.4, 2.2, 1.8, 1.8.
+void own_level_set(dd4dv_ctx* ctx) {
+  ctx->lv_own_on = false;
+  if (!ctx->lv.tiles || ctx->owned_all) return;
+  dd4dv_ctx::LvSet& o = ctx->lv_own;
+  auto& L = ctx->dec_allocs;
+  const int n_sub = ctx->n_sub;
+  if (!o.tiles) {
+    dd4dv_ctx::LvSet n;
+    try {
+      n.tiles = dalloc<LvTile>(ctx, ctx->lv_tiles_h.size(), &L);
+      n.boxes = dalloc<int>(ctx, n_sub, &L);
+      n.tile_off = dalloc<int>(ctx, 2 * n_sub, &L);
+      if (!ctx->lv_ring_h.empty()) n.ring_tiles = dalloc<LvTile>(ctx, ctx->lv_ring_h.size(), &L);
+      if (ctx->lv_rounds > 1) {
+        std::vector<LvTile> all;
+        for (const LvTile& t : ctx->lv_tiles_h)
+          if (t.p0 == 0) split_box(t, 1, all);
+        n.fine_tiles = dalloc<LvTile>(ctx, all.size(), &L);
+      }
+    } catch (const Fail&) {
+      ctx->err.clear();
+      return;   // (what was allocated goes with the decomposition)
+    }
+    o = n;
+  }
+  std::vector<LvTile> tiles, ring_tiles, fine;
+  std::vector<int> order, tile_off;
+  int maxL = 0;
+  long long pts = 0;
+  auto owned = [&](int s) { return ctx->owned_h[s] != 0; };
+  for (const LvTile& t : ctx->lv_tiles_h) {
+    if (!owned(t.s)) continue;
+    tiles.push_back(t);
+    if (t.p0) continue;   // once per box:
+    maxL = std::max(maxL, t.L);
+    pts += (long long)t.nx * t.ny;
+    if (o.fine_tiles) split_box(t, 1, fine);
+  }
+  for (const LvTile& t : ctx->lv_ring_h)
+    if (owned(t.s)) ring_tiles.push_back(t);
+  for (int s : ctx->lv_order_h)
+    if (owned(s)) order.push_back(s);
+  LvPlan g = ctx->lv.plan;
+  g.obs.resize(maxL + 1);
+  count_tiles(g, tiles, ring_tiles, maxL, n_sub, &tile_off);
+  if (ring_tiles.empty() || g.n_ring[0] < ctx->lv_ring_least) {
+    ring_tiles.clear();
+    for (LvRing& r : g.ring) r = LvRing{};
+  }
+  const bool one_round = o.fine_tiles && level_rounds<double>(pts) == 1;
+  if (one_round) {
+    g.fine = (int)fine.size();
+    g.n_fine.assign(maxL, 0);
+    for (const LvTile& t : fine)
+      for (int l = 0; l < t.L; ++l) ++g.n_fine[l];
+    if (!fine.empty()) h2d(ctx, o.fine_tiles, fine.data(), fine.size() * sizeof(LvTile));
+    g.fine_tiles = o.fine_tiles;
+  }
+  upload_set(ctx, o, g, tiles, ring_tiles, order, tile_off);
+  CK(cudaStreamSynchronize(ctx->st));   // the host tables end with this call
+  ctx->lv_own_on = true;
 }
 
 // ---------------------------------------------------------------------------
@@ -1434,8 +1561,8 @@ void build_decomposition(dd4dv_ctx* ctx, const dd4dv_decomp& d) {
     const long long wy = (long long)subs[y].nx * subs[y].ny * (subs[y].b - subs[y].a + 1);
     return wx > wy;
   });
-  ctx->lv_tiles = nullptr;
-  ctx->lv_f = ctx->lv_a = false;
+  ctx->lv = ctx->lv_own = {};
+  ctx->lv_own_on = ctx->lv_f = ctx->lv_a = false;
   ctx->traj = dalloc<unsigned char>(ctx, ctx->traj_elems * ctx->tsize, &L);
   ctx->stg = nullptr;
   ctx->stg_elems = 0;
@@ -1538,7 +1665,7 @@ void build_decomposition(dd4dv_ctx* ctx, const dd4dv_decomp& d) {
   if (d.cluster <= 0) {
     if (f32) level_plan<float>(ctx, subs, lvl_obs);
     else level_plan<double>(ctx, subs, lvl_obs);
-    ctx->lv_f = ctx->lv_a = d.cluster == 0 && ctx->lv_tiles;
+    ctx->lv_f = ctx->lv_a = d.cluster == 0 && ctx->lv.tiles;
   }
   h2d(ctx, ctx->subs_d, subs.data(), subs.size() * sizeof(SubDesc));
   h2d(ctx, ctx->order_d, order.data(), order.size() * sizeof(int));
@@ -2738,6 +2865,10 @@ dd4dv_status dd4dv_set_owned(dd4dv_ctx* ctx, const int* owned) {
     ctx->owned_h = m;
     ctx->owned_all = std::all_of(m.begin(), m.end(), [](int v) { return v == 1; });
     ctx->fwd_pending = false;
+    if (ctx->lv.tiles) {
+      ctx->drop_graphs();   // (their level sweeps hold the list of the mask before)
+      own_level_set(ctx);
+    }
     return DD4DV_OK;
   });
 }

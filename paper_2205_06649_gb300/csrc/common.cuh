@@ -219,6 +219,10 @@ struct LvPlan {
   const LvTile* ring_tiles = nullptr;   // their tiles: whole rows
   bool ring_expire = false;             // their waits run out at once (a test of what follows)
   std::vector<int> n_ring;              // as n_tile
+  // tiles of one round, for the kernels that add nothing up (null: the same tiles)
+  const LvTile* fine_tiles = nullptr;
+  int fine = 0;
+  std::vector<int> n_fine;
   std::vector<int> n_tile;    // per step l: tiles of the boxes that take it (a prefix)
   std::vector<int> n_box;     // per level l: boxes that have it (a prefix of the box list)
   std::vector<char> obs;      // per level l: some box has observations there

@@ -1170,6 +1170,18 @@ cudaError_t lv_phase(const LvArgs<T>& base, const LvPlan& g, cudaStream_t st) {
     ++*launches;                        \
   } while (0)
 
+// The list of a launch: the tiles that keep the order of J's sums, or those of one
+// round where the plan has some.  Returns the number of all its tiles.
+template <typename T>
+int lv_list(LvArgs<T>& a, const LvArgs<T>& base, const LvPlan& g, int l, bool sums) {
+  const bool fine = !sums && g.fine_tiles;
+  const auto& n = fine ? g.n_fine : g.n_tile;
+  a.l = l;
+  a.tiles = fine ? g.fine_tiles : base.tiles;
+  a.n_tile = l < (int)n.size() ? n[l] : 0;
+  return fine ? g.fine : g.tiles;
+}
+
 template <typename T>
 cudaError_t launch_level_forward(const LvArgs<T>& base, const LvPlan& g, cudaStream_t st, long long* launches) {
   constexpr int V = lv_width<T>();
@@ -1177,12 +1189,12 @@ cudaError_t launch_level_forward(const LvArgs<T>& base, const LvPlan& g, cudaStr
   const int L = (int)g.n_tile.size();   // longest window
   if (a.terms) LV_TRY(lv_launch<T>(lv_start_kernel<T, V>, a, g.tiles, st));
   for (int l = 0; l <= L; ++l) {
-    a.l = l;
-    a.n_tile = l < L ? g.n_tile[l] : 0;
+    lv_list(a, base, g, l, false);
     const int nob = a.terms && g.obs[l] ? g.n_box[l] : 0;
     if (a.n_tile + nob) LV_TRY(lv_launch<T>(lv_stage_kernel<T, V, 1, false>, a, a.n_tile + nob, st));
     if (!a.n_tile) continue;
     LV_TRY(lv_launch<T>(lv_stage_kernel<T, V, 2, false>, a, a.n_tile, st));
+    lv_list(a, base, g, l, a.terms);
     if (a.terms) LV_TRY(lv_launch<T>(lv_stage_kernel<T, V, 3, true>, a, a.n_tile, st));
     else LV_TRY(lv_launch<T>(lv_stage_kernel<T, V, 3, false>, a, a.n_tile, st));
   }
@@ -1193,10 +1205,10 @@ template <typename T>
 cudaError_t launch_level_adjoint(const LvArgs<T>& base, const LvPlan& g, cudaStream_t st, long long* launches) {
   constexpr int V = lv_width<T>();
   LvArgs<T> a = base;
-  LV_TRY(lv_launch<T>(lv_lam_start_kernel<T, V>, a, g.tiles, st));
+  const int all = lv_list(a, base, g, 0, false);
+  LV_TRY(lv_launch<T>(lv_lam_start_kernel<T, V>, a, all, st));
   for (int l = (int)g.n_tile.size() - 1; l >= 0; --l) {
-    a.l = l;
-    a.n_tile = g.n_tile[l];
+    lv_list(a, base, g, l, false);
     if (!a.stg) {   // the stage states were not stored: recompute them
       a.skip1 = a.stg1 != nullptr;
       LV_TRY(lv_launch<T>(lv_stage_kernel<T, V, 1, false>, a, a.n_tile, st));
@@ -1209,7 +1221,7 @@ cudaError_t launch_level_adjoint(const LvArgs<T>& base, const LvPlan& g, cudaStr
       if (g.ring[2].slots && g.obs[l] && !a.yforce)
         LV_TRY(launch_dependent(lv_scatter_kernel, dim3((unsigned)g.n_box[l + 1]), kRingThreads, 0, st, a));
   }
-  LV_TRY(lv_launch<T>(lv_export_kernel<T, V>, a, g.tiles, st));
+  LV_TRY(lv_launch<T>(lv_export_kernel<T, V>, a, all, st));
   return cudaSuccess;
 }
 
@@ -1217,10 +1229,10 @@ cudaError_t launch_level_tangent(const LvArgs<double>& base, const LvPlan& g, cu
   LvArgs<double> a = base;
   const int L = (int)g.n_tile.size();
   a.skip1 = a.stg1 != nullptr;
-  LV_TRY(lv_launch<double>(lv_tl_start_kernel, a, g.tiles, st));
+  const int all = lv_list(a, base, g, 0, false);
+  LV_TRY(lv_launch<double>(lv_tl_start_kernel, a, all, st));
   for (int l = 0; l <= L; ++l) {
-    a.l = l;
-    a.n_tile = l < L ? g.n_tile[l] : 0;
+    lv_list(a, base, g, l, false);
     const int nob = g.obs[l] ? g.n_box[l] : 0;
     if (a.n_tile + nob) LV_TRY(lv_launch<double>(lv_tl_kernel<1>, a, a.n_tile + nob, st));
     if (!a.n_tile) continue;

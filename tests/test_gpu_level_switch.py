@@ -154,3 +154,63 @@ def test_pipelined_adjoints_of_two_contexts_on_two_threads(level_context):
     for t in threads:
         t.join()
     assert not wrong
+
+
+@pytest.mark.parametrize("precision,ckpt_k", [(0, 0), (0, -1), (1, 0)])
+def test_tiles_of_several_rounds(level_context, precision, ckpt_k):
+    """Tiles in which a thread takes several points (decompositions of more than
+    2 million points): states and gradients to the last bit as with one round, J
+    up to the order of its sums (1e-13 of FP64 terms, as between sweep kinds)."""
+    out = []
+    for rounds in (1, 2, 4):
+        ctx = level_context(precision, ckpt_k, env=dict(DD4DV_LEVEL_ROUNDS=rounds, DD4DV_RING_MIN_TILES=1 << 40), **RAGGED)
+        w = controls(ctx)
+        ctx.exchange(0.5 * w)
+        J, g = ctx.eval(w)
+        out.append((J, g, ctx.trajectories(w), ctx.gn_hessvec(w, 0.1 * w)))
+    for J, *rest in out[1:]:
+        assert np.max(np.abs(J - out[0][0])) <= 1e-13 * np.max(np.abs(J))
+        for a, b in zip(rest, out[0][1:]):
+            assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("precision,ring,rounds", [(0, 0, 1), (0, 0, 2), (1, 0, 1), (1, 0, 4), (1, 1, 4)])
+def test_owned_boxes_alone_give_what_all_of_them_give(level_context, precision, ring, rounds):
+    """Evaluations and local solves of a share of the boxes launch those boxes
+    alone: J, gradients and solved controls to the last bit as with all boxes
+    owned, whatever the share (windows of one length only, one box, none)."""
+    import paper_2205_06649_gb300 as dd
+    env = dict(DD4DV_RING_MIN_TILES=0 if ring else 1 << 40, DD4DV_LEVEL_ROUNDS=rounds)
+    kw = dict(env=env, nlon=96, nlat=60, nsteps=31, P1=3, P2=2, Q=3, o_lon=3, o_lat=3, o_t=3, uneven=True)
+    ctx = level_context(precision, **kw)
+    w = controls(ctx)
+    b, off = np.asarray(ctx.boxes), np.asarray(ctx.offsets)
+    n = ctx.n_sub
+    J, g = ctx.eval(w)
+    masks = [np.arange(n) % 2 == 1, b[:, 5] - b[:, 4] == (b[:, 5] - b[:, 4]).min(), np.arange(n) == n - 1,
+             np.arange(n) < n // 3, np.zeros(n, dtype=bool)]
+    for m in masks:
+        ctx.set_owned(m.astype(np.int32))
+        Jm, gm = ctx.eval(w)
+        Jf = ctx.eval_forward(w)
+        gb = ctx.eval_backward()
+        for s in np.nonzero(m)[0]:
+            c = slice(off[s], off[s + 1])
+            assert Jm[s] == J[s] and Jf[s] == J[s], s
+            assert np.array_equal(gm[c], g[c]) and np.array_equal(gb[c], g[c]), s
+    ctx.set_owned(None)
+    J2, g2 = ctx.eval(w)
+    assert np.array_equal(J2, J) and np.array_equal(g2, g)
+    # an outer iteration in three shares against one of all boxes
+    solver = dd.solver_defaults(max_local_iters=6, max_outer=1, eps_outer=0.0)
+    whole = level_context(precision, **kw)
+    whole.outer_step(solver)
+    got = np.zeros(ctx.ctrl_total)
+    for k in range(3):
+        ctx.set_owned((np.arange(n) % 3 == k).astype(np.int32))
+        ctx.set_controls(0.0 * got)
+        ctx.local_solve(solver)
+        x = ctx.get_controls()
+        for s in range(k, n, 3):
+            got[off[s]:off[s + 1]] = x[off[s]:off[s + 1]]
+    assert np.array_equal(got, whole.get_controls()) and got.any()
