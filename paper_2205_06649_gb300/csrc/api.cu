@@ -214,11 +214,28 @@ dd4dv_status guard(dd4dv_ctx* ctx, F&& f) {
   }
 }
 
+// Memory kept only because it makes calls faster, given up when another
+// allocation needs it: the Turkel-Zwas block.  Returns whether there was any.
+bool release_spare(dd4dv_ctx* ctx) {
+  if (ctx->tz_ws) {
+    cudaStreamSynchronize(ctx->st);
+    cudaFree(ctx->tz_ws);
+    ctx->tz_ws = nullptr;
+    ctx->tz_ws_bytes = 0;
+    return true;
+  }
+  return false;
+}
+
 template <typename T>
 T* dalloc(dd4dv_ctx* ctx, size_t n, std::vector<void*>* list = nullptr) {
   void* p = nullptr;
   if (n == 0) n = 1;
   cudaError_t e = cudaMalloc(&p, n * sizeof(T));
+  while (e == cudaErrorMemoryAllocation && release_spare(ctx)) {
+    cudaGetLastError();
+    e = cudaMalloc(&p, n * sizeof(T));
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     fail(ctx, DD4DV_ENOMEM, "cudaMalloc(%zu bytes): %s", n * sizeof(T), cudaGetErrorString(e));
@@ -2561,6 +2578,7 @@ dd4dv_status dd4dv_tz_eval(dd4dv_ctx* ctx, int p, int q, double alpha, const dou
     const int N = ctx->m.nsteps;
     const long long plane = (long long)ctx->m.nlat * ctx->m.nlon;
     const size_t nob = ctx->has_obs ? ctx->ob_level.size() : 0;
+    tz_observations(ctx);   // (before the scratch, which an allocation may ask back)
     TzBufs b(ctx, 8 * (size_t)ctx->m.nlat + 7 * G + T + nob + 2 * kTzBlocks + 1);
     tz_rows(ctx, t, b);
     const double* w = tz_in(ctx, b, w_in, G, device_ptrs);
@@ -2571,7 +2589,6 @@ dd4dv_status dd4dv_tz_eval(dd4dv_ctx* ctx, int p, int q, double alpha, const dou
     double* part = b.get(2 * kTzBlocks + 1);
     double* Jd = part + 2 * kTzBlocks;
     double* force = b.get(nob);
-    tz_observations(ctx);
     const double* od = ctx->tz_obs;   // fi, fj, y, sigma_o, then level and var as ints
     const int* lvd = reinterpret_cast<const int*>(od + 4 * nob);
     const int* vrd = lvd + nob;

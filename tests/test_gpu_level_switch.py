@@ -214,3 +214,56 @@ def test_owned_boxes_alone_give_what_all_of_them_give(level_context, precision, 
         for s in range(k, n, 3):
             got[off[s]:off[s + 1]] = x[off[s]:off[s + 1]]
     assert np.array_equal(got, whole.get_controls()) and got.any()
+
+
+# ---- memory ----
+
+GRID = dict(nlon=512, nlat=256, nsteps=10, P1=6, P2=4, Q=1, o_lon=4, o_lat=4, corr_len=0.0)   # 190,000 points a level
+
+
+class Hog:
+    """Holds all device memory but `leave` bytes."""
+
+    def __init__(self, leave):
+        torch.cuda.empty_cache()
+        free, _ = torch.cuda.mem_get_info()
+        self.t = torch.empty(max(0, free - int(leave)), dtype=torch.uint8, device="cuda")
+
+    def __enter__(self):
+        return self
+
+    def __exit__(self, *_):
+        del self.t
+        torch.cuda.empty_cache()
+
+
+def test_kept_turkel_zwas_block_is_given_back(level_context):
+    """The block that Turkel-Zwas calls keep (here 75 MB) goes when another
+    allocation needs it, and comes back with the next such call."""
+    import paper_2205_06649_gb300 as dd
+    kw = dict(nlon=256, nlat=128, nsteps=90, P1=4, P2=4, Q=1, o_lon=4, o_lat=4, o_t=0, corr_len=0.0, obs_count=100)
+    wl = tiny_workload(**kw)
+    inp = workloads.generate(wl)
+    ctx = dd.Context(wl.nlon, wl.nlat, inp["dt"], wl.nsteps)
+    try:
+        ctx.set_background(inp["x_b0"])
+        ctx.set_background_error(wl.sigma_b, 0.0, 4)
+        so = np.asarray(wl.sigma_o)[inp["obs_var"]]
+        ctx.set_observations(inp["obs_level"], inp["obs_var"], inp["obs_fi"], inp["obs_fj"], 0.0 * so, so)
+        v = 0.1 * np.random.default_rng(1).standard_normal(3 * wl.nlon * wl.nlat)
+        J, g = ctx.tz_eval(2, 1, 0.5, v)
+        dec = (wl.P1, wl.P2, wl.Q, wl.o_lon, wl.o_lat, wl.o_t, inp["lon_cuts"], inp["lat_cuts"], inp["t_cuts"])
+        ctx.set_decomposition(*dec, ckpt_k=-1, cluster=4)   # (loads its kernels)
+        b = np.asarray(ctx.boxes)
+        copies = 8 * 3 * (wl.nsteps + 1) * (int(np.sum(b[:, 3] * ((b[:, 1] + 3) // 4 * 4))) + wl.nlon * wl.nlat)
+        ctx.set_background(inp["x_b0"])                     # frees the decomposition
+        free = torch.cuda.mem_get_info()[0]
+        ctx.set_decomposition(*dec, ckpt_k=-1, cluster=4)
+        used = free - torch.cuda.mem_get_info()[0] - copies   # without the copies for a reset, which are optional
+        ctx.set_background(inp["x_b0"])
+        with Hog(used - 40 * 2**20):
+            ctx.set_decomposition(*dec, ckpt_k=-1, cluster=4)
+        J2, g2 = ctx.tz_eval(2, 1, 0.5, v)
+        assert J2 == J and np.max(np.abs(g2 - g)) <= 1e-12 * np.max(np.abs(g))
+    finally:
+        ctx.destroy()
