@@ -161,6 +161,8 @@ struct dd4dv_ctx {
   void *lv_rec = nullptr, *lv_state = nullptr;
   double *lv_acc_m = nullptr, *lv_acc_o = nullptr;
   long long lv_elems = 0;     // elements of one level of every box
+  std::vector<void*> lv_allocs;   // the level sweeps' buffers
+  void free_level();
   std::vector<void*> dec_allocs;
 
   ~dd4dv_ctx();
@@ -227,12 +229,13 @@ bool release_spare(dd4dv_ctx* ctx) {
   return false;
 }
 
+// spare = false: fails rather than have release_spare free anything.
 template <typename T>
-T* dalloc(dd4dv_ctx* ctx, size_t n, std::vector<void*>* list = nullptr) {
+T* dalloc(dd4dv_ctx* ctx, size_t n, std::vector<void*>* list = nullptr, bool spare = true) {
   void* p = nullptr;
   if (n == 0) n = 1;
   cudaError_t e = cudaMalloc(&p, n * sizeof(T));
-  while (e == cudaErrorMemoryAllocation && release_spare(ctx)) {
+  while (e == cudaErrorMemoryAllocation && spare && release_spare(ctx)) {
     cudaGetLastError();
     e = cudaMalloc(&p, n * sizeof(T));
   }
@@ -1060,10 +1063,15 @@ void upload_set(dd4dv_ctx* ctx, dd4dv_ctx::LvSet& set, LvPlan& g, const std::vec
   set.plan = std::move(g);
 }
 
-// Tiles and scratch of the level sweeps.  Leaves ctx->lv.tiles null where they
+// What optional buffers leave free: 4 GB + 5 % of the device.
+double memory_reserve(size_t total_b) { return 4.0 * (1ull << 30) + 0.05 * (double)total_b; }
+
+// Tiles and scratch of the level sweeps (level_upload moves the tiles to the device
+// once the stage buffers are known).  Leaves ctx->lv.tiles null where they
 // do not apply: too few points, boxes no wider than a thread's columns or of a
 // single row (a thread has one ghost row at most), a grid
-// whose level does not fit 32-bit offsets, or no memory for the scratch.
+// whose level does not fit 32-bit offsets, or no memory for the scratch beside the
+// reserve.
 template <typename T>
 void level_plan(dd4dv_ctx* ctx, const std::vector<SubDesc>& subs, const std::vector<int>& lvl_obs) {
   constexpr int V = lv_width<T>();
@@ -1080,7 +1088,7 @@ void level_plan(dd4dv_ctx* ctx, const std::vector<SubDesc>& subs, const std::vec
   long long least = sizeof(T) == 4 ? kLvMinPoints32 : std::max<long long>(kLvMinPoints64, (long long)kLvMinBox64 * n_sub);
   if (const char* e = std::getenv("DD4DV_LEVEL_MIN_POINTS")) least = std::atoll(e);   // override (tests)
   if (pts < least || maxL < 1 || min_nx <= V || min_ny < 2 || 3LL * nlon * nlat >= (1LL << 31)) return;
-  auto& L = ctx->dec_allocs;
+  auto& L = ctx->lv_allocs;
   std::vector<int> order(n_sub);
   for (int s = 0; s < n_sub; ++s) order[s] = s;
   std::stable_sort(order.begin(), order.end(),
@@ -1177,33 +1185,49 @@ void level_plan(dd4dv_ctx* ctx, const std::vector<SubDesc>& subs, const std::vec
     const double cn = ctx->rows_h[std::min(j + 1, nlat - 1)].c, cs = ctx->rows_h[std::max(j - 1, 0)].c;
     fill_records(rc, cn, cs, ctx->m.dt, ctx->Bth, &rec[8 * (size_t)j], &rec[8 * (size_t)(nlat + j)]);
   }
-  // only where the scratch fits beside what the decomposition already holds
   size_t free_b = 0, total_b = 0;
   CK(cudaMemGetInfo(&free_b, &total_b));
   const size_t slots = tiles.size() * kLvThreads;
-  const size_t need = 5 * (size_t)elems * sizeof(T) + (tiles.size() + ring_tiles.size()) * sizeof(LvTile) +
-                      slots * sizeof(double) + (64u << 20);
-  if (need > free_b) return;
+  const double need = 5.0 * (double)elems * sizeof(T) + (double)(tiles.size() + ring_tiles.size()) * sizeof(LvTile) +
+                      (double)slots * sizeof(double);
+  if (need + memory_reserve(total_b) > (double)free_b) return;
   dd4dv_ctx::LvSet set;
-  set.tiles = dalloc<LvTile>(ctx, tiles.size(), &L);
-  set.boxes = dalloc<int>(ctx, n_sub, &L);
-  set.tile_off = dalloc<int>(ctx, 2 * n_sub, &L);
-  ctx->lv_box_off = dalloc<long long>(ctx, n_sub, &L);
-  ctx->lv_rec = dalloc<T>(ctx, rec.size(), &L);
-  ctx->lv_state = dalloc<T>(ctx, 5 * (size_t)elems, &L);
-  ctx->lv_acc_m = dalloc<double>(ctx, slots, &L);
-  ctx->lv_acc_o = dalloc<double>(ctx, n_sub, &L);
-  if (!ring_tiles.empty()) set.ring_tiles = dalloc<LvTile>(ctx, ring_tiles.size(), &L);
-  upload_set(ctx, set, g, tiles, ring_tiles, order, tile_off);
+  try {
+    set.tiles = dalloc<LvTile>(ctx, tiles.size(), &L, false);
+    set.boxes = dalloc<int>(ctx, n_sub, &L, false);
+    set.tile_off = dalloc<int>(ctx, 2 * n_sub, &L, false);
+    if (!ring_tiles.empty()) set.ring_tiles = dalloc<LvTile>(ctx, ring_tiles.size(), &L, false);
+    ctx->lv_box_off = dalloc<long long>(ctx, n_sub, &L, false);
+    ctx->lv_rec = dalloc<T>(ctx, rec.size(), &L, false);
+    ctx->lv_state = dalloc<T>(ctx, 5 * (size_t)elems, &L, false);
+    ctx->lv_acc_m = dalloc<double>(ctx, slots, &L, false);
+    ctx->lv_acc_o = dalloc<double>(ctx, n_sub, &L, false);
+  } catch (const Fail&) {
+    ctx->err.clear();
+    ctx->free_level();
+    return;
+  }
   h2d(ctx, ctx->lv_box_off, box_off.data(), n_sub * sizeof(long long));
   h2d(ctx, ctx->lv_rec, rec.data(), rec.size() * sizeof(T));
   CK(cudaMemsetAsync(ctx->lv_state, 0, 5 * (size_t)elems * sizeof(T), ctx->st));
   CK(cudaStreamSynchronize(ctx->st));   // the host tables end with this call
   ctx->lv_elems = elems;
-  ctx->lv = std::move(set);
+  ctx->lv = set;
+  ctx->lv.plan = std::move(g);
   ctx->lv_tiles_h = std::move(tiles);
   ctx->lv_ring_h = std::move(ring_tiles);
   ctx->lv_order_h = std::move(order);
+}
+
+void level_upload(dd4dv_ctx* ctx, const std::vector<SubDesc>& subs) {
+  if (!ctx->lv.tiles) return;
+  for (auto* list : {&ctx->lv_tiles_h, &ctx->lv_ring_h})
+    for (LvTile& t : *list) t.stg1_off = subs[t.s].stg1_off;
+  LvPlan g = std::move(ctx->lv.plan);
+  std::vector<int> tile_off;
+  count_tiles(g, ctx->lv_tiles_h, ctx->lv_ring_h, (int)g.n_tile.size(), ctx->n_sub, &tile_off);
+  upload_set(ctx, ctx->lv, g, ctx->lv_tiles_h, ctx->lv_ring_h, ctx->lv_order_h, tile_off);
+  CK(cudaStreamSynchronize(ctx->st));   // tile_off ends with this call
 }
 
 // The list of the owned boxes, after dd4dv_set_owned.  A rank that owns a share of
@@ -1222,20 +1246,20 @@ void own_level_set(dd4dv_ctx* ctx) {
   ctx->lv_own_on = false;
   if (!ctx->lv.tiles || ctx->owned_all) return;
   dd4dv_ctx::LvSet& o = ctx->lv_own;
-  auto& L = ctx->dec_allocs;
+  auto& L = ctx->lv_allocs;
   const int n_sub = ctx->n_sub;
   if (!o.tiles) {
     dd4dv_ctx::LvSet n;
     try {
-      n.tiles = dalloc<LvTile>(ctx, ctx->lv_tiles_h.size(), &L);
-      n.boxes = dalloc<int>(ctx, n_sub, &L);
-      n.tile_off = dalloc<int>(ctx, 2 * n_sub, &L);
-      if (!ctx->lv_ring_h.empty()) n.ring_tiles = dalloc<LvTile>(ctx, ctx->lv_ring_h.size(), &L);
+      n.tiles = dalloc<LvTile>(ctx, ctx->lv_tiles_h.size(), &L, false);
+      n.boxes = dalloc<int>(ctx, n_sub, &L, false);
+      n.tile_off = dalloc<int>(ctx, 2 * n_sub, &L, false);
+      if (!ctx->lv_ring_h.empty()) n.ring_tiles = dalloc<LvTile>(ctx, ctx->lv_ring_h.size(), &L, false);
       if (ctx->lv_rounds > 1) {
         std::vector<LvTile> all;
         for (const LvTile& t : ctx->lv_tiles_h)
           if (t.p0 == 0) split_box(t, 1, all);
-        n.fine_tiles = dalloc<LvTile>(ctx, all.size(), &L);
+        n.fine_tiles = dalloc<LvTile>(ctx, all.size(), &L, false);
       }
     } catch (const Fail&) {
       ctx->err.clear();
@@ -1578,8 +1602,6 @@ void build_decomposition(dd4dv_ctx* ctx, const dd4dv_decomp& d) {
     const long long wy = (long long)subs[y].nx * subs[y].ny * (subs[y].b - subs[y].a + 1);
     return wx > wy;
   });
-  ctx->lv = ctx->lv_own = {};
-  ctx->lv_own_on = ctx->lv_f = ctx->lv_a = false;
   ctx->traj = dalloc<unsigned char>(ctx, ctx->traj_elems * ctx->tsize, &L);
   ctx->stg = nullptr;
   ctx->stg_elems = 0;
@@ -1635,6 +1657,12 @@ void build_decomposition(dd4dv_ctx* ctx, const dd4dv_decomp& d) {
   ctx->lon_cov_d = dalloc<int>(ctx, lon_cov.size(), &L);
   ctx->lat_cov_d = dalloc<int>(ctx, lat_cov.size(), &L);
   ctx->t_cov_d = dalloc<int>(ctx, t_cov.size(), &L);
+  // The level sweeps' scratch, a few levels, before the stage states, which take
+  // what is left.
+  if (d.cluster <= 0) {
+    if (f32) level_plan<float>(ctx, subs, lvl_obs);
+    else level_plan<double>(ctx, subs, lvl_obs);
+  }
   // Stored stage states (ckpt_k = 0) are twice the trajectory: allocate them
   // last, and only if they leave a reserve of 4 GB + 5 % of the device free;
   // otherwise the adjoint recomputes the stages.
@@ -1642,7 +1670,7 @@ void build_decomposition(dd4dv_ctx* ctx, const dd4dv_decomp& d) {
     size_t free_b = 0, total_b = 0;
     CK(cudaMemGetInfo(&free_b, &total_b));
     const double need = (double)std::max<long long>(1, stgl) * ctx->tsize;
-    const double reserve = 4.0 * (1ull << 30) + 0.05 * (double)total_b;
+    const double reserve = memory_reserve(total_b);
     if (need + reserve <= (double)free_b) {
       ctx->stg_elems = stgl;
       ctx->stg = dalloc<unsigned char>(ctx, std::max<long long>(1, stgl) * ctx->tsize, &L);
@@ -1661,7 +1689,7 @@ void build_decomposition(dd4dv_ctx* ctx, const dd4dv_decomp& d) {
   if (!f32 && !ctx->stg && (d.ckpt_k == 0 || d.ckpt_k == -3)) {
     size_t free_b = 0, total_b = 0;
     CK(cudaMemGetInfo(&free_b, &total_b));
-    const double reserve = 4.0 * (1ull << 30) + 0.05 * (double)total_b;
+    const double reserve = memory_reserve(total_b);
     const double budget = ((double)free_b - reserve) / (double)ctx->tsize;
     long long used = 0, pts_in = 0;
     for (int idx : order) {
@@ -1679,11 +1707,8 @@ void build_decomposition(dd4dv_ctx* ctx, const dd4dv_decomp& d) {
       ctx->stg1_frac = pts > 0 ? (double)pts_in / (double)pts : 0.0;
     }
   }
-  if (d.cluster <= 0) {
-    if (f32) level_plan<float>(ctx, subs, lvl_obs);
-    else level_plan<double>(ctx, subs, lvl_obs);
-    ctx->lv_f = ctx->lv_a = d.cluster == 0 && ctx->lv.tiles;
-  }
+  level_upload(ctx, subs);
+  ctx->lv_f = ctx->lv_a = d.cluster == 0 && ctx->lv.tiles;
   h2d(ctx, ctx->subs_d, subs.data(), subs.size() * sizeof(SubDesc));
   h2d(ctx, ctx->order_d, order.data(), order.size() * sizeof(int));
   {
@@ -1722,7 +1747,7 @@ void build_decomposition(dd4dv_ctx* ctx, const dd4dv_decomp& d) {
     size_t free_b = 0, total_b = 0;
     CK(cudaMemGetInfo(&free_b, &total_b));
     const double need = (double)(ctx->gtraj + ctx->traj_elems) * ctx->tsize;
-    if (need + 4.0 * (1ull << 30) + 0.05 * (double)total_b <= (double)free_b) {
+    if (need + memory_reserve(total_b) <= (double)free_b) {
       ctx->bnd0 = dalloc<unsigned char>(ctx, ctx->gtraj * ctx->tsize, &L);
       ctx->tgt0 = dalloc<unsigned char>(ctx, ctx->traj_elems * ctx->tsize, &L);
       CK(cudaMemcpyAsync(ctx->bnd0, ctx->bnd, ctx->gtraj * ctx->tsize, cudaMemcpyDeviceToDevice, ctx->st));
@@ -1769,11 +1794,25 @@ void dd4dv_ctx::drop_graphs() {
   og.valid = false;
 }
 
+// Gives the level sweeps' memory back; cluster sweeps run from here on.
+void dd4dv_ctx::free_level() {
+  if (st) cudaStreamSynchronize(st);
+  drop_graphs();
+  for (void* p : lv_allocs) cudaFree(p);
+  lv_allocs.clear();
+  lv = lv_own = {};
+  lv_own_on = lv_f = lv_a = false;
+  lv_tiles_h = {};
+  lv_ring_h = {};
+  lv_order_h = {};
+}
+
 void dd4dv_ctx::free_dec() {
   if (st) cudaStreamSynchronize(st);
   drop_graphs();
   cudaFreeHost(lbst_h);
   lbst_h = nullptr;
+  free_level();
   for (void* p : dec_allocs) cudaFree(p);
   dec_allocs.clear();
   cudaFreeHost(phase_h);

@@ -237,6 +237,20 @@ class Hog:
         torch.cuda.empty_cache()
 
 
+def test_level_scratch_leaves_the_reserve(level_context):
+    """With less free memory than the reserve of the optional buffers (4 GB + 5 %
+    of the device) the level sweeps' scratch is left out: what the context
+    allocates later has to find its memory."""
+    ref = level_context(0, **GRID)
+    assert ref.sweep_kernels() == {"forward": 5, "adjoint": 5}
+    w = controls(ref)
+    g = ref.eval(w)[1]
+    with Hog(4 * 2**30 + 0.05 * torch.cuda.mem_get_info()[1] - 256 * 2**20):
+        ctx = level_context(0, ckpt_k=-1, **GRID)
+        assert 5 not in ctx.sweep_kernels().values()
+        assert np.array_equal(ctx.eval(w)[1], g)
+
+
 def test_kept_turkel_zwas_block_is_given_back(level_context):
     """The block that Turkel-Zwas calls keep (here 75 MB) goes when another
     allocation needs it, and comes back with the next such call."""
