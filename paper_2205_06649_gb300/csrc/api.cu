@@ -930,6 +930,7 @@ void autotune(dd4dv_ctx* ctx) {
   if (ctx->lv_f) ctx->variant_f = 0;   // (a cluster shape stays set for the sweeps that need one)
   if (ctx->lv_a) ctx->variant_a = 0;
   sync(ctx);
+  if (!ctx->lv_f && !ctx->lv_a) ctx->free_level();
   if (!use && ctx->stg && ctx->dec.ckpt_k != -2) {   // recomputing the stages won: give the memory back
     free_dec_buffer(ctx, ctx->stg);
     ctx->stg_elems = 0;
@@ -3124,8 +3125,8 @@ dd4dv_status dd4dv_set_sweep_config(dd4dv_ctx* ctx, const int* shape) {
     ctx->cl = ca; ctx->nthreads = ta; ctx->R = Ra;
     ctx->use_stg = sg != 0;
     ctx->dec.cluster = ca;
-    ctx->lv_f = ctx->lv_a = false;   // an explicit cluster shape asks for the cluster sweeps
     ctx->drop_graphs();
+    ctx->free_level();   // an explicit cluster shape asks for the cluster sweeps
     return DD4DV_OK;
   });
 }

@@ -251,6 +251,14 @@ def test_level_scratch_leaves_the_reserve(level_context):
         assert np.array_equal(ctx.eval(w)[1], g)
 
 
+def test_launch_shapes_give_the_level_scratch_back(level_context):
+    ctx = level_context(0, **GRID)
+    cfg = ctx.sweep_config()
+    free = torch.cuda.mem_get_info()[0]
+    ctx.set_sweep_config(cfg["forward"], cfg["adjoint"], cfg["stored_stages"])
+    assert torch.cuda.mem_get_info()[0] - free >= 16 * 2**20
+
+
 def test_kept_turkel_zwas_block_is_given_back(level_context):
     """The block that Turkel-Zwas calls keep (here 75 MB) goes when another
     allocation needs it, and comes back with the next such call."""
