@@ -217,7 +217,8 @@ dd4dv_status guard(dd4dv_ctx* ctx, F&& f) {
 }
 
 // Memory kept only because it makes calls faster, given up when another
-// allocation needs it: the Turkel-Zwas block.  Returns whether there was any.
+// allocation needs it: the Turkel-Zwas block, then the level sweeps' buffers (the
+// cluster sweeps run on).  Returns whether there was any.
 bool release_spare(dd4dv_ctx* ctx) {
   if (ctx->tz_ws) {
     cudaStreamSynchronize(ctx->st);
@@ -226,7 +227,9 @@ bool release_spare(dd4dv_ctx* ctx) {
     ctx->tz_ws_bytes = 0;
     return true;
   }
-  return false;
+  if (!ctx->lv.tiles) return false;
+  ctx->free_level();
+  return true;
 }
 
 // spare = false: fails rather than have release_spare free anything.

@@ -251,6 +251,28 @@ def test_level_scratch_leaves_the_reserve(level_context):
         assert np.array_equal(ctx.eval(w)[1], g)
 
 
+def test_lazily_made_buffers_find_the_memory_of_the_level_scratch(level_context):
+    """A Gauss-Newton product needs a trajectory more.  Where only the level
+    sweeps' scratch (here five levels of ten) stands in its way, that goes and the
+    cluster sweeps run."""
+    kw = {**GRID, "nsteps": 3}
+    ref = level_context(0, **kw)
+    w, p = controls(ref), controls(ref, 5)
+    h = ref.gn_hessvec(w, p)
+    ctx = level_context(0, **kw)
+    b = np.asarray(ctx.boxes)
+    level = 3 * 8 * int(np.sum(b[:, 3] * ((b[:, 1] + 3) // 4 * 4)))
+    need = 4 * level + 4 * 8 * ctx.ctrl_total   # four levels of dx and four control vectors
+    assert 5 * level > 16 * 2**20
+    with Hog(need - 2.5 * level):
+        assert ctx.sweep_kernels() == {"forward": 5, "adjoint": 5}
+        got = ctx.gn_hessvec(w, p)
+        assert 5 not in ctx.sweep_kernels().values()
+    assert np.max(np.abs(got - h)) <= 1e-12 * np.max(np.abs(h))
+    _, g = ref.eval(w)
+    assert np.array_equal(ctx.eval(w)[1], g)
+
+
 def test_launch_shapes_give_the_level_scratch_back(level_context):
     ctx = level_context(0, **GRID)
     cfg = ctx.sweep_config()
