@@ -1104,7 +1104,6 @@ void level_plan(dd4dv_ctx* ctx, const std::vector<SubDesc>& subs, const std::vec
   LvPlan g;
   g.obs.assign(maxL + 1, 0);
   long long elems = 0;
-  auto magic = [](int v) { return v <= 1 ? 0u : (unsigned)(0xFFFFFFFFu / (unsigned)v + 1u); };
   for (const int s : order) {
     const SubDesc& d = subs[s];
     LvTile t{};
@@ -1113,9 +1112,10 @@ void level_plan(dd4dv_ctx* ctx, const std::vector<SubDesc>& subs, const std::vec
     t.ny = d.ny;
     t.nxp = d.nxp;
     t.nq = (d.nx + V - 1) / V;
-    t.mq = magic(t.nq);
-    t.mnx = magic(d.nx);
-    t.mny = magic(d.ny);
+    if (!level_box_fits(d.nx, d.ny, d.nxp, t.nq)) return;
+    t.mq = magic_of(t.nq);
+    t.mnx = magic_of(d.nx);
+    t.mny = magic_of(d.ny);
     t.i0 = d.i0;
     t.j0 = d.j0;
     t.a = d.a;

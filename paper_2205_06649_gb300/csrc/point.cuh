@@ -7,13 +7,15 @@
 
 namespace dd4dv {
 
-// Division by a per-CTA constant d >= 1 through a precomputed multiplier
+// Division by a constant d >= 1 of a CTA or tile through a precomputed multiplier
 // m = ceil(2^32 / d) (m = 0 encodes d = 1): floor(a / d) = floor(a m / 2^32)
 // exactly whenever a * d < 2^32.  (With m = (2^32 + e) / d, 0 <= e < d, the
 // product is a / d + a e / (d 2^32); the extra term is below 1 / d, the gap
-// from a / d up to the next integer, when a e < 2^32.)  Every dividend here is
-// an index into a CTA's shared-memory stripe, below 2^20, and every divisor
-// is a row length or a row count: a * d stays below 2^31.
+// from a / d up to the next integer, when a e < 2^32.)  In the cluster sweeps a
+// dividend is an index into a CTA's shared-memory stripe, below 2^20, and a divisor
+// a row length or a row count; the level sweeps divide indices of a whole box, up
+// to three planes of it, and level_box_fits (tuning.h) holds their products below
+// 2^32.
 __host__ __device__ __forceinline__ unsigned magic_of(int d) {
   return d <= 1 ? 0u : (unsigned)(0xFFFFFFFFu / (unsigned)d + 1u);
 }

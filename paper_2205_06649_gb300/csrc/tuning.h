@@ -1,5 +1,6 @@
-// What the autotuner concludes from its timings.  Plain C++, no CUDA: the rules
-// can be tested by themselves.
+// What the autotuner concludes from its timings, and which boxes the level sweeps'
+// index arithmetic holds for.  Plain C++, no CUDA: the rules can be tested by
+// themselves.
 #pragma once
 
 #include <vector>
@@ -42,6 +43,16 @@ constexpr int kTunedCkpt[3] = {8, 16, 32};
 inline std::vector<int> checkpoint_candidates(bool level_f, bool level_a) {
   if (level_f && level_a) return {};
   return {kTunedCkpt, kTunedCkpt + 3};
+}
+
+// Whether the level sweeps' 32-bit index arithmetic is exact for a box of nx x ny
+// points, rows padded to nxp, nq thread-points a row: a quotient a / d through
+// magic_of(d) needs a d < 2^32 (thread-points by nq, scatter targets of three planes by
+// nx, their rows by ny), an offset in a level 2^31.  Boxes that fit a cluster's
+// shared memory, as every accepted box does, are far inside.
+inline bool level_box_fits(long long nx, long long ny, long long nxp, long long nq) {
+  const long long lim = 1LL << 32;
+  return nq * ny * nq < lim && 3 * ny * nx * nx < lim && 3 * ny * ny < lim && 3 * ny * nxp < (lim >> 1);
 }
 
 }  // namespace dd4dv

@@ -18,6 +18,10 @@ int main(int argc, char** argv) {
     for (int k : checkpoint_candidates(std::atoi(argv[2]), std::atoi(argv[3]))) std::printf("%d ", k);
     return 0;
   }
+  if (!std::strcmp(argv[1], "box")) {
+    std::printf("%d", level_box_fits(std::atoll(argv[2]), std::atoll(argv[3]), std::atoll(argv[4]), std::atoll(argv[5])));
+    return 0;
+  }
   SweepTimes t[2];
   double* f[8] = {&t[0].cluster_f, &t[0].cluster_a, &t[0].level_f, &t[0].level_a,
                   &t[1].cluster_f, &t[1].cluster_a, &t[1].level_f, &t[1].level_a};
@@ -61,3 +65,23 @@ def test_no_checkpoint_interval_is_timed_where_none_has_an_effect(run):
     assert run("ckpt", 1, 1) == ""
     for f, a in ((0, 0), (1, 0), (0, 1)):
         assert run("ckpt", f, a).split() == ["8", "16", "32"]
+
+
+def magic_quotient(a, d):
+    """mdiv(a, magic_of(d)) of csrc/point.cuh."""
+    m = 0 if d <= 1 else (0xFFFFFFFF // d + 1) & 0xFFFFFFFF
+    return (a * m) >> 32 if m else a
+
+
+@pytest.mark.parametrize("nx,ny,v,fits", [
+    (179, 85, 4, True), (2048, 1024, 1, False), (1024, 512, 1, True), (1025, 1365, 1, False), (1024, 1365, 1, True),
+    (5, 37837, 4, True), (5, 37838, 4, False), (4097, 86, 4, False), (4096, 85, 4, True),
+])
+def test_level_boxes_whose_quotients_are_exact(run, nx, ny, v, fits):
+    nq, nxp = (nx + v - 1) // v, (nx + 3) // 4 * 4
+    assert run("box", nx, ny, nxp, nq) == ("1" if fits else "0")
+    if fits:
+        for n, d in ((nq * ny, nq), (3 * ny * nx, nx), (3 * ny, ny)):
+            step = max(1, n // 4001)
+            for a in [*range(0, n, step), *range(max(0, n - 3 * d), n, max(1, d // 7)), n - 1, n - d - 1]:
+                assert magic_quotient(a, d) == a // d, (a, d)
