@@ -61,9 +61,6 @@ __device__ __forceinline__ void ldv(const T* p, T* x) {
   if constexpr (V == 4) {
     const float4 q = *reinterpret_cast<const float4*>(p);
     x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
-  } else if constexpr (V == 2) {
-    const float2 q = *reinterpret_cast<const float2*>(p);
-    x[0] = q.x; x[1] = q.y;
   } else {
     x[0] = *p;
   }
@@ -71,7 +68,6 @@ __device__ __forceinline__ void ldv(const T* p, T* x) {
 template <typename T, int V>
 __device__ __forceinline__ void stv(T* p, const T* x) {
   if constexpr (V == 4) *reinterpret_cast<float4*>(p) = make_float4(x[0], x[1], x[2], x[3]);
-  else if constexpr (V == 2) *reinterpret_cast<float2*>(p) = make_float2(x[0], x[1]);
   else *p = x[0];
 }
 

@@ -72,45 +72,11 @@ __device__ __forceinline__ double tz_val(const TzArgs& t, const double* Y, int v
 //   Dv = (1-alpha) ((v c)[j+q] - (v c)[j-q])
 //        + alpha/2 ((v c)[i+p,j+q] - (v c)[i+p,j-q] + (v c)[i-p,j+q] - (v c)[i-p,j-q])
 // with C = f + u tan(theta)/a at the point it multiplies (its own row's f, tan).
-__device__ void tz_F(const TzArgs& t, const double* Y, int j, int i, double& Fh, double& Fu, double& Fv) {
-  const int p = t.p, q = t.q;
-  const double al = t.alpha, sl = t.slon, st = t.slat, g = t.g;
-  const RowConst rc = t.rows[j];
-  const double c = rc.c, f = rc.f, tau = rc.tau;
-  const RowConst rN = t.rows[tz_resolve(t, j + q, i).j], rS = t.rows[tz_resolve(t, j - q, i).j];
-  const double h = tz_val(t, Y, 0, j, i), u = tz_val(t, Y, 1, j, i), v = tz_val(t, Y, 2, j, i);
-  const double C = f + u * tau;
-  double cor_u = (1.0 - al) * C * v;
-  double cor_v = (1.0 - al) * C * u;
-  if (al != 0.0) {
-    const double uEp = tz_val(t, Y, 1, j, i + p), uWp = tz_val(t, Y, 1, j, i - p);
-    cor_u += 0.5 * al * ((f + uEp * tau) * tz_val(t, Y, 2, j, i + p) + (f + uWp * tau) * tz_val(t, Y, 2, j, i - p));
-    const double uNq = tz_val(t, Y, 1, j + q, i), uSq = tz_val(t, Y, 1, j - q, i);
-    cor_v += 0.5 * al * ((rN.f + uNq * rN.tau) * uNq + (rS.f + uSq * rS.tau) * uSq);
-  }
-  Fu = -sl * u / c * (tz_val(t, Y, 1, j, i + 1) - tz_val(t, Y, 1, j, i - 1)) -
-       st * v * (tz_val(t, Y, 1, j + 1, i) - tz_val(t, Y, 1, j - 1, i)) -
-       sl * g / (p * c) * (tz_val(t, Y, 0, j, i + p) - tz_val(t, Y, 0, j, i - p)) + cor_u;
-  Fv = -sl * u / c * (tz_val(t, Y, 2, j, i + 1) - tz_val(t, Y, 2, j, i - 1)) -
-       st * v * (tz_val(t, Y, 2, j + 1, i) - tz_val(t, Y, 2, j - 1, i)) -
-       st * g / q * (tz_val(t, Y, 0, j + q, i) - tz_val(t, Y, 0, j - q, i)) - cor_v;
-  double du = (1.0 - al) * (tz_val(t, Y, 1, j, i + p) - tz_val(t, Y, 1, j, i - p));
-  double dv = (1.0 - al) * (tz_val(t, Y, 2, j + q, i) * rN.c - tz_val(t, Y, 2, j - q, i) * rS.c);
-  if (al != 0.0) {
-    du += 0.5 * al * (tz_val(t, Y, 1, j + q, i + p) - tz_val(t, Y, 1, j + q, i - p) +
-                      tz_val(t, Y, 1, j - q, i + p) - tz_val(t, Y, 1, j - q, i - p));
-    dv += 0.5 * al * (tz_val(t, Y, 2, j + q, i + p) * rN.c - tz_val(t, Y, 2, j - q, i + p) * rS.c +
-                      tz_val(t, Y, 2, j + q, i - p) * rN.c - tz_val(t, Y, 2, j - q, i - p) * rS.c);
-  }
-  Fh = -(sl * u / c * (tz_val(t, Y, 0, j, i + 1) - tz_val(t, Y, 0, j, i - 1)) +
-         st * v * (tz_val(t, Y, 0, j + 1, i) - tz_val(t, Y, 0, j - 1, i)) + sl * h / (p * c) * du +
-         st * h / (q * c) * dv);
-}
 
 // Partial derivatives of (F_h, F_u, F_v) at (j, i) with respect to every
 // state value they read: vis(out_var, in_var, row, col, coef) with the
 // location resolved through the periodic wrap and the wall mirror (a v read
-// through a mirror enters with the sign flipped).  Derived from tz_F term by
+// through a mirror enters with the sign flipped).  Derived from F above term by
 // term; a location read by several terms (p = 1 or q = 1) gets one entry
 // per term.
 template <typename Vis>
@@ -220,7 +186,7 @@ __device__ __forceinline__ int tz_row(int j, int s, int nlat, double& sg) {
   return r < 0 ? -1 - r : r >= nlat ? 2 * nlat - 1 - r : r;
 }
 
-// out = cx X + cy (Y + dt F(Y)), the tendencies of tz_F with the row records
+// out = cx X + cy (Y + dt F(Y)), the tendencies F above with the row records
 __global__ void __launch_bounds__(kTzThreads) tz_stage_kernel(TzArgs t, const double* X, const double* Y, double* out,
                                                               double cx, double cy) {
   const TzPt m(t);
