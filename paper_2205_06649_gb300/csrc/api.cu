@@ -128,7 +128,7 @@ struct dd4dv_ctx {
   double* scal_d = nullptr;
   double* scal_h = nullptr;   // pinned
   int* err_d = nullptr;
-  int* late_h = nullptr;      // pinned, written by the device: a lost copy (see ring_lost in level.cu)
+  int* late_h = nullptr;      // (in counter_h) written by the device: a lost copy (see ring_lost in level.cu)
   int vblocks = 8;
   bool fwd_pending = false;
   LbState* lbst_h = nullptr;  // pinned
@@ -1782,7 +1782,6 @@ dd4dv_ctx::~dd4dv_ctx() {
   cudaFree(scal_d);
   cudaFree(err_d);
   cudaFreeHost(counter_h);
-  cudaFreeHost(late_h);
   cudaFreeHost(phase_h);
   cudaFreeHost(scal_h);
   cudaFree(ptraj_io);
@@ -1900,10 +1899,10 @@ dd4dv_status dd4dv_create(const dd4dv_model* model, void* cuda_stream, dd4dv_ctx
     ctx->counter_d = dalloc<int>(ctx, 4);
     ctx->scal_d = dalloc<double>(ctx, 8);
     ctx->err_d = dalloc<int>(ctx, 1);
-    if (cudaMallocHost(&ctx->counter_h, 4 * sizeof(int)) != cudaSuccess ||
-        cudaMallocHost(&ctx->scal_h, 8 * sizeof(double)) != cudaSuccess ||
-        cudaMallocHost(&ctx->late_h, sizeof(int)) != cudaSuccess)
+    if (cudaMallocHost(&ctx->counter_h, 8 * sizeof(int)) != cudaSuccess ||
+        cudaMallocHost(&ctx->scal_h, 8 * sizeof(double)) != cudaSuccess)
       fail(ctx, DD4DV_ENOMEM, "pinned host allocation failed");
+    ctx->late_h = ctx->counter_h + 4;
     *ctx->late_h = 0;
     CK(cudaMemcpyAsync(ctx->rows_d, ctx->rows_h.data(), m.nlat * sizeof(RowConst),
                        cudaMemcpyHostToDevice, ctx->st));

@@ -980,15 +980,17 @@ cudaError_t launch_global_stage(const double* x, const double* y, double* out, d
 // 768 x 384 (67.6 / 63.7) and 1024 x 512 (114.3 / 105.3) the stage kernels run.
 GlobalStepPlan global_step_plan(int nlon, int nlat) {
   GlobalStepPlan best;
-  const double per = 16.0 / 32.0 / 2.07e3;   // us per FP64 thread instruction of an SM
-  const double stages = 13.0 + 96.0 * (double)nlon * nlat / 152.0 * per;
+  int sms = 152, dev = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const double per = 16.0 / 32.0 / 2.07e3;   // us per FP64 thread instruction of an SM (2.07 GHz)
+  const double stages = 13.0 + 96.0 * (double)nlon * nlat / sms * per;
   double least = stages;
   for (int tx = 16; tx <= 128; tx += 8)
     for (int ty = 4; ty <= 40; ++ty) {
       if (step_smem(tx, ty) > 110 * 1024 || tx - 8 >= nlon || ty - 1 >= nlat) continue;
       const long long n = (long long)((nlon + tx - 1) / tx) * ((nlat + ty - 1) / ty);
       const double work = 28.0 * (tx + 4) * (ty + 4) + 34.0 * (tx + 2) * (ty + 2) + 34.0 * tx * ty;
-      const double cost = 6.0 + (double)((n + 151) / 152) * work * per;
+      const double cost = 6.0 + (double)((n + sms - 1) / sms) * work * per;
       if (cost < least) {
         least = cost;
         best.tx = tx;

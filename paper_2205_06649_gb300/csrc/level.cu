@@ -10,7 +10,9 @@
 //   * FP64: 28-47 FP64 instructions per point take 16 SM cycles per warp each;
 //     the 15-36 loads of a point are a tenth of that, so plain loads through L1
 //     keep the FP64 pipe fed, and every SM works until the grid's end.  Bound:
-//     the FP64 pipe (about 90 % of its rate with the overlap terms counted).
+//     the FP64 pipe, 83-88 % of its rate inside a launch of 2.9 million points
+//     (profiles/level_sweeps_fp64.md), 57-58 % over the short launches of the medium
+//     workload (14-28 us each, some 5 of them start, first loads and last tiles).
 //   * FP32: a thread takes four neighbouring columns with 16-byte loads.  Bound:
 //     latency of the loads (forward HBM at 55 % of its measured rate); groups of
 //     boxes sized for L2, strips marching north with rows kept in registers, one
@@ -21,9 +23,10 @@
 // A tile is a run of points of one box (flat over rows, so that every lane has
 // one); tiles are ordered longest window first, so the boxes still running at
 // step l are a prefix and the grid shrinks with them.  CTAs of 128 threads: with
-// 256 the last wave of a 175,000-point level left a fifth of the SMs idle (FP64
-// evaluation of 64 boxes 3.33 ms, with 128 3.07 ms).  Launches overlap their
-// set-up with the end of the launch before (programmatic dependent launch).
+// 256 the last wave of a 175,000-point level leaves more of the SMs idle (FP64, 64
+// boxes, forward / adjoint 1.93 / 2.43 ms, with 128 1.83 / 2.23; FP32, 645,000 points
+// a level 1.75 / 3.32, with 128 1.73 / 3.20).  Launches overlap their set-up with the
+// end of the launch before (programmatic dependent launch).
 //
 // Measured against the cluster sweeps with the launch shapes that the library
 // chooses (forward / adjoint, ms):
@@ -31,8 +34,8 @@
 //     9.6 / 13.5; FP64: 102.8 / 156.7 -> 76.0 / 92.5 (a part of it from the FP64
 //     adjoint's point function, without which the level sweeps took 77 / 112)
 //   one 128-step window of the large workload (256 boxes), FP32: 15.4 / 29.6 -> 9.3 / 13.9
-//   differentiation workload (FP32, 16-step checkpoints): 1.68 / 4.91 -> 1.72 / 3.18
-//   medium workload (FP64, 64 boxes, 184,000 points): 1.82 / 2.31 -> 1.82 / 2.16
+//   differentiation workload (FP32, 16-step checkpoints): 1.68 / 4.92 -> 1.73 / 3.20
+//   medium workload (FP64, 64 boxes, 175,000 points): 1.86 / 2.32 -> 1.83 / 2.23
 //
 // The arithmetic per point is that of sweep.cu (point.cuh), so trajectories,
 // stage states and gradients are the same bit for bit; J differs by the order
@@ -690,9 +693,10 @@ __global__ void __launch_bounds__(kLvThreads) lv_export_kernel(const LvArgs<T> a
 // ring of slots in shared memory: bulk copies for the rows and their constants,
 // 4-byte copies for the ghosts, one barrier a slot, no barrier between the
 // computing warps.  What is in flight no longer depends on the registers.
-// Bound: instruction issue (45-48 % of the slots, 560 instructions for a warp's
-// 128 points) and the wait for a slot.  Phases 1, 2, 3 of 2.9 million points:
-// 40.6, 39.5, 63.8 -> 30.7, 27.4, 57.3 us; adjoint sweep of the batching
+// Bound: instruction issue (44-48 % of the slots, 550 to 600 instructions for a warp's
+// 128 points in phases 1 and 2) and the wait for a slot.  Phase 3 takes 128 registers
+// a thread and spills 56 bytes.  Phases 1, 2, 3 of 2.9 million points: 40.6, 39.5,
+// 63.8 -> 30.9, 27.8, 52.0 us; adjoint sweep of the batching
 // workload 17.6 -> 13.5 ms, of a 128-step window of the large workload 17.7 ->
 // 13.9 ms.  With the copies made by a computing warp and a CTA barrier a tile
 // the same sweep took 16.7 ms; the row constants read through L1 (small beside

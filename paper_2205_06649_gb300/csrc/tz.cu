@@ -15,8 +15,10 @@
 // The tangent-linear stage is built from one list of partial derivatives per
 // point (tz_jacobian: for each value of the state that F at the point reads,
 // d F_out / d value_in).  The adjoint stage gathers the transposed list: a point
-// collects, term by term, what the points that read it send back, so there are
-// no atomic additions and the result does not depend on their order.
+// collects, term by term, what the points that read it send back, without atomic
+// additions.  (The observation forcing is still scattered by FP64 atomics, in
+// tz_obs_scatter_kernel: where observations share a corner, the last bits of a
+// gradient depend on their order.)
 // Bound: launch latency on small grids (8 launches a step of about 3 us), the
 // FP64 pipe on large ones.  Row constants hold every quotient (launch_tz_rows):
 // the divisions were most of the FP64 work.  256 x 128 points, 128 steps,
