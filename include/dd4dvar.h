@@ -452,7 +452,8 @@ dd4dv_status dd4dv_stage1_stored(const dd4dv_ctx* ctx, int* n_subs, double* pt_s
  * with the decomposition (cluster 0, or -1 where they measure faster), give the
  * same trajectories and gradients bit for bit and J up to the order of its
  * partial sums, and give way to the cluster sweeps when a variant other than 0
- * or a launch shape (dd4dv_set_sweep_config) is set.  The environment variable
+ * or a launch shape (dd4dv_set_sweep_config) is set, or when another allocation
+ * of the context needs their scratch.  The environment variable
  * DD4DV_LEVEL_MIN_POINTS, read by dd4dv_set_decomposition, replaces the number
  * of points from which they are chosen.  Four more are for tests:
  * DD4DV_LEVEL_ROUNDS replaces the points (FP32: groups of four) that a thread takes,

@@ -1032,18 +1032,26 @@ void split_box(LvTile t, int rounds, std::vector<LvTile>& out) {
   }
 }
 
+// Tiles per step, from the windows of a list's boxes.
+std::vector<int> per_step(const std::vector<LvTile>& tiles, int maxL) {
+  std::vector<int> n(maxL, 0);
+  for (const LvTile& t : tiles)
+    if (t.L > 0) ++n[t.L - 1];
+  for (int l = maxL - 2; l >= 0; --l) n[l] += n[l + 1];
+  return n;
+}
+
 // Counts of a list of tiles (longest window first): tiles, pipelined tiles and
 // boxes per step or level, and each box's accumulator slots (tile_off).
 void count_tiles(LvPlan& g, const std::vector<LvTile>& tiles, const std::vector<LvTile>& ring_tiles, int maxL,
                  int n_sub, std::vector<int>* tile_off) {
   g.tiles = (int)tiles.size();
-  g.n_tile.assign(maxL, 0);
-  g.n_ring.assign(maxL, 0);
+  g.n_tile = per_step(tiles, maxL);
+  g.n_ring = per_step(ring_tiles, maxL);
   g.n_box.assign(maxL + 1, 0);
   tile_off->assign(2 * n_sub, 0);
   for (size_t i = 0; i < tiles.size(); ++i) {
     const LvTile& t = tiles[i];
-    for (int l = 0; l < t.L; ++l) ++g.n_tile[l];
     int* slots = &(*tile_off)[2 * t.s];
     if (t.p0 == 0) {   // a box's first tile
       slots[0] = (int)i * kLvThreads;
@@ -1051,8 +1059,6 @@ void count_tiles(LvPlan& g, const std::vector<LvTile>& tiles, const std::vector<
     }
     slots[1] += kLvThreads;
   }
-  for (const LvTile& t : ring_tiles)
-    for (int l = 0; l < t.L; ++l) ++g.n_ring[l];
 }
 
 // Moves a list to the device (set's buffers) and into set.
@@ -1298,9 +1304,7 @@ void own_level_set(dd4dv_ctx* ctx) {
   const bool one_round = o.fine_tiles && level_rounds<double>(pts) == 1;
   if (one_round) {
     g.fine = (int)fine.size();
-    g.n_fine.assign(maxL, 0);
-    for (const LvTile& t : fine)
-      for (int l = 0; l < t.L; ++l) ++g.n_fine[l];
+    g.n_fine = per_step(fine, maxL);
     if (!fine.empty()) h2d(ctx, o.fine_tiles, fine.data(), fine.size() * sizeof(LvTile));
     g.fine_tiles = o.fine_tiles;
   }
